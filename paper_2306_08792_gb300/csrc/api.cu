@@ -100,6 +100,17 @@ size_t op_capacity(int64_t n, const gcr_params* p, int kinds) {
   return (size_t)(n * per);
 }
 
+PoolParts carve_parts(Carve& c, int na, int nb, int d, Elt elt, int kp, bool cross) {
+  const PoolPlan pl = pool_plan(na, nb, d, elt, kp, cross);
+  const size_t rows = (size_t)(cross ? 2 : 1) * na, entries = pool_part_entries(pl, na, cross);
+  PoolParts t;
+  t.v = c.take<float>(entries);
+  t.i = c.take<int>(entries);
+  t.cnt = c.take<int>((size_t)pl.splits * rows);
+  t.tau = c.take<uint32_t>(rows);
+  return t;
+}
+
 struct BuildWs {
   double* n64;
   float* n32;
@@ -109,8 +120,7 @@ struct BuildWs {
   float* anrm;
   float* pool_v;
   int* pool_i;
-  float* tau_x;        // paired GEMM splits: per-row thresholds of the two column halves
-  int* pair_cnt;
+  PoolParts parts;     // the tensor-core sweep's split buffers
   int* unc_count;
   int* unc_row;
   int* unc_kind;
@@ -167,12 +177,9 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.xr = bf ? c.take<char>(nn * d * es) : nullptr;
   t.enrm = bf ? c.take<float>(nn) : nullptr;
   t.anrm = bf ? c.take<float>(nn) : nullptr;
-  // 32-entry pools on the tensor-core path: room for the two column halves of paired GEMM splits
-  const bool pairable = bf && r.kp == 32;
-  t.pool_v = c.take<float>((size_t)(pairable ? 2 : 1) * kinds * nn * r.kp);
-  t.pool_i = c.take<int>((size_t)(pairable ? 2 : 1) * kinds * nn * r.kp);
-  t.tau_x = pairable ? c.take<float>((size_t)2 * kinds * nn) : nullptr;
-  t.pair_cnt = pairable ? c.take<int>((size_t)kinds * 4 * 2 * ((nn + 255) / 256)) : nullptr;
+  t.pool_v = c.take<float>((size_t)kinds * nn * r.kp);
+  t.pool_i = c.take<int>((size_t)kinds * nn * r.kp);
+  t.parts = bf ? carve_parts(c, (int)n, (int)n, d, elt_of(p), r.kp, kinds == 2) : PoolParts{};
   t.unc_count = c.take<int>(4);
   t.unc_row = c.take<int>((size_t)kinds * nn);
   t.unc_kind = c.take<int>((size_t)kinds * nn);
@@ -242,8 +249,8 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
   if (p->k > 0) {
     StageScope sc_(GCR_STAGE_SIM_GEMM, st);
     if (bf) {
-      GCR_CUDA_TRY(launch_umma_pool(w.xr, n, w.xr, n, d, elt, camp, p->cross_camera != 0, 1, r.kp, 1, w.pool_v,
-                                    w.pool_i, st, nullptr, w.tau_x, w.pair_cnt));
+      GCR_CUDA_TRY(launch_umma_pool(w.xr, n, w.xr, n, d, elt, camp, p->cross_camera != 0, 1, r.kp, w.parts,
+                                    w.pool_v, w.pool_i, st));
     } else {
       GCR_CUDA_TRY(launch_sgemm_pool(X, n, X, n, d, camp, r.kp, p->cross_camera != 0, 1, 1, w.pool_v, w.pool_i, st));
     }
@@ -623,8 +630,8 @@ struct ServeWs {
   float* enrm;
   float* anrm;
   RowScalars* sc;
-  float* part_v;
-  int* part_i;
+  PoolParts parts;     // the layer searches' split buffers (the FP32 path: its sorted lists in v
+  PoolParts parts_final;  // and i), and the final search's in the same memory
   float* pool_v;
   int* pool_i;
   int* unc_count;
@@ -664,7 +671,7 @@ int serve_kp_final(const gcr_params* p) {
   return K < 64 ? 64 : 128;
 }
 
-size_t carve_serve(Carve& c, int64_t b, int32_t d, const gcr_params* p, const Resolved& r, ServeWs* w) {
+size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params* p, const Resolved& r, ServeWs* w) {
   const size_t nb = (size_t)b;
   const bool bf = tensor_mode(p);
   const size_t es = elt_size(p);
@@ -678,8 +685,23 @@ size_t carve_serve(Carve& c, int64_t b, int32_t d, const gcr_params* p, const Re
   t.enrm = bf ? c.take<float>(nb) : nullptr;
   t.anrm = bf ? c.take<float>(nb) : nullptr;
   t.sc = c.take<RowScalars>(1);
-  t.part_v = c.take<float>((size_t)kServeMaxSplits * nb * kpmax);
-  t.part_i = c.take<int>((size_t)kServeMaxSplits * nb * kpmax);
+  if (bf) {
+    // one region for both pool sizes, as large as any smaller batch needs it (a batch of fewer row
+    // blocks is cut into more splits): a workspace sized for a batch serves every smaller one
+    size_t end = 0;
+    for (int64_t rows = std::min<int64_t>(b, 128);; rows = std::min<int64_t>(b, rows + 128)) {
+      Carve c1 = c, c2 = c;
+      t.parts = carve_parts(c1, (int)rows, (int)ng, d, elt_of(p), r.kp, false);
+      t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, elt_of(p), serve_kp_final(p), false);
+      end = std::max(end, std::max(c1.off, c2.off));
+      if (rows == b) break;
+    }
+    c.off = end;
+  } else {
+    t.parts.v = c.take<float>((size_t)kServeMaxSplits * nb * kpmax);
+    t.parts.i = c.take<int>((size_t)kServeMaxSplits * nb * kpmax);
+    t.parts_final = t.parts;
+  }
   t.pool_v = c.take<float>(nb * kpmax);
   t.pool_i = c.take<int>(nb * kpmax);
   t.unc_count = c.take<int>(4);
@@ -736,21 +758,19 @@ struct SeedSource {
 // Certified k nearest gallery rows for the b query rows xq: pool, merge, refine, band.
 // ball (may be NULL; tensor-core modes): workspace of the ball search of the rows the pools
 // cannot certify (without it, pools saturated with near-ties keep the 2 delta bound).
-int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp, const GallerySide& gs, int ng,
-              const ServeWs& w, unsigned long long* stats, int32_t* nbr, float* d2, cudaStream_t st,
+int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp, const PoolParts& parts,
+              const GallerySide& gs, int ng, const ServeWs& w, unsigned long long* stats, int32_t* nbr, float* d2, cudaStream_t st,
               const SeedSource& seed_src = SeedSource(), const BallArgs* ball = nullptr) {
   const bool bf = tensor_mode(p);
   const Elt elt = elt_of(p);
   const float* G = gs.G;
   const int rblocks = (b + 127) / 128;
-  const int splits = std::max(1, std::min(kServeMaxSplits, (152 + rblocks - 1) / rblocks));
   {
     StageScope sc_(GCR_STAGE_PREP, st, bf ? 2 : 2);
     GCR_CUDA_TRY(launch_row_stats(xq, b, d, w.n64, w.n32, bf ? w.qr : nullptr, elt, w.enrm, w.anrm, w.sc, st));
   }
   GCR_CUDA_TRY(cudaMemsetAsync(w.unc_count, 0, sizeof(int) * 4, st));
   GCR_CUDA_TRY(cudaMemsetAsync(w.band_cnt, 0, sizeof(int) * b, st));
-  int used_splits;
   // the split pools' admission floors (tensor-core modes), from the previous search's merged
   // pool, when given its rows' gallery lists, and a sample of the gallery
   const bool seeded = bf && (seed_src.prev_kp > 0 || seed_src.sample > 0) &&
@@ -767,16 +787,14 @@ int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp,
   {
     StageScope sc_(GCR_STAGE_SIM_GEMM, st, 2);
     if (bf) {
-      const int ntiles = (ng + 255) / 256;
-      used_splits = split_count(splits, ntiles);
-      GCR_CUDA_TRY(launch_umma_pool(w.qr, b, gs.Gr, ng, d, elt, nullptr, false, 0, kp, used_splits, w.part_v,
-                                    w.part_i, st, seeded ? w.seed : nullptr));
+      GCR_CUDA_TRY(launch_umma_pool(w.qr, b, gs.Gr, ng, d, elt, nullptr, false, 0, kp, parts, w.pool_v, w.pool_i, st,
+                                    seeded ? w.seed : nullptr));
     } else {
       const int ntiles = (ng + 127) / 128;
-      used_splits = split_count(splits, ntiles);
-      GCR_CUDA_TRY(launch_sgemm_pool(xq, b, G, ng, d, nullptr, kp, false, 0, used_splits, w.part_v, w.part_i, st));
+      const int used = split_count(std::max(1, std::min(kServeMaxSplits, (152 + rblocks - 1) / rblocks)), ntiles);
+      GCR_CUDA_TRY(launch_sgemm_pool(xq, b, G, ng, d, nullptr, kp, false, 0, used, parts.v, parts.i, st));
+      GCR_CUDA_TRY(launch_merge_splits(parts.v, parts.i, used, 1, b, kp, w.pool_v, w.pool_i, st));
     }
-    GCR_CUDA_TRY(launch_merge_splits(w.part_v, w.part_i, used_splits, 1, b, kp, w.pool_v, w.pool_i, st));
   }
   RefineArgs ra;
   std::memset(&ra, 0, sizeof(ra));
@@ -848,7 +866,7 @@ size_t carve_topk_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_
   r.kp = serve_kp_final(p);
   r.kinds = 1;
   TopkRerankWs t;
-  carve_serve(c, nq, d, p, r, &t.sw);
+  carve_serve(c, nq, ng, d, p, r, &t.sw);
   t.n64g = c.take<double>(ng);
   t.n32g = c.take<float>(ng);
   t.gr = bf ? c.take<char>((size_t)ng * d * elt_size(p)) : nullptr;
@@ -873,7 +891,7 @@ int topk_rerank_impl(const float* Xq, int64_t nq, const float* Xg, int64_t ng, i
   }
   GCR_CUDA_TRY(cudaMemsetAsync(w.sw.stats, 0, sizeof(unsigned long long) * GCR_STATS_LEN, st));
   const GallerySide gs{Xg, w.gr, w.n64g, w.scg, w.genrm, w.ganrm};
-  return serve_knn(Xq, (int)nq, d, p, p->topk_out, serve_kp_final(p), gs, (int)ng, w.sw, w.sw.stats, idx_out,
+  return serve_knn(Xq, (int)nq, d, p, p->topk_out, serve_kp_final(p), w.sw.parts_final, gs, (int)ng, w.sw, w.sw.stats, idx_out,
                    dist_out, st, SeedSource(), bf ? &w.ball : nullptr);
 }
 
@@ -1222,7 +1240,7 @@ size_t gcr_serve_workspace_size(int64_t b, int64_t ng, int32_t d, const gcr_para
   Resolved r;
   if (b < 1 || check_serve_params(p, ng, d, &r) != GCR_OK) return 0;
   Carve c(nullptr, 0);
-  return carve_serve(c, b, d, p, r, nullptr) + 256;
+  return carve_serve(c, b, ng, d, p, r, nullptr) + 256;
 }
 
 int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq, int64_t b, int32_t d,
@@ -1238,7 +1256,7 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
   if (!ws) return GCR_E_WORKSPACE;
   Carve cw(ws, ws_bytes);
   ServeWs w;
-  if (carve_serve(cw, b, d, p, r, &w) > ws_bytes) return GCR_E_WORKSPACE;
+  if (carve_serve(cw, b, ng, d, p, r, &w) > ws_bytes) return GCR_E_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   unsigned long long* stp = stats ? reinterpret_cast<unsigned long long*>(stats) : w.stats;
   const int nq = (int)b, n = (int)ng;
@@ -1258,7 +1276,7 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
         src.prev_kp = r.kp;
       else if (nq >= 32)
         src.sample = (int)std::min<int64_t>(ng, kSeedCandidates);
-      s = serve_knn(w.xq[cur], nq, d, p, p->k, r.kp, gallery_layer(g, t, n, d, elt_size(p)), n, w, stp, w.nbr, w.d2,
+      s = serve_knn(w.xq[cur], nq, d, p, p->k, r.kp, w.parts, gallery_layer(g, t, n, d, elt_size(p)), n, w, stp, w.nbr, w.d2,
                     st, src);
       if (s != GCR_OK) return s;
     }
@@ -1280,7 +1298,7 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
     if (p->topk_out > r.kp)
       src.sample = (int)std::min<int64_t>(ng, kSeedCandidates - (int64_t)r.kp * (1 + src.hop_k));
   }
-  return serve_knn(w.xq[cur], nq, d, p, p->topk_out, serve_kp_final(p), gallery_layer(g, p->T, n, d, elt_size(p)), n, w, stp,
+  return serve_knn(w.xq[cur], nq, d, p, p->topk_out, serve_kp_final(p), w.parts_final, gallery_layer(g, p->T, n, d, elt_size(p)), n, w, stp,
                    idx_out, dist_out, st, src);
 }
 

@@ -12,6 +12,10 @@ struct BallArgs;  // ball search of the pairs a pool could not certify (below)
 // Element type of the tensor-core GEMM operands: BF16 copies of the rows, or FP32 rows
 // rounded to TF32 (10 explicit mantissa bits, low 13 bits zero).
 enum class Elt : int { BF16 = 0, TF32 = 1 };
+// The device this library is written for: its SMs and L2 bytes size grids and workspaces (the
+// workspace queries run without a device).
+constexpr int kSMs = 152;
+constexpr double kL2Bytes = 126e6;
 inline size_t elt_bytes(Elt e) { return e == Elt::TF32 ? 4 : 2; }
 
 // Per-call scalars reduced over the rows of X (device memory).
@@ -45,18 +49,30 @@ cudaError_t launch_sgemm_dist(const float* Xq, int nq, const float* Xg, int ng, 
                               const float* nrm_q, const float* nrm_g, float* D, cudaStream_t st);
 
 // ---- umma.cu (tcgen05 path; operands BF16 or TF32)
-// Pools of S = A . B^T rows: [split][kind][na][kp], kp = 32, 64 or 128.
+// How a pool sweep is cut: the column splits of each 128-row block (tps column tiles each, in
+// the grid's order), whether clusters share the column tiles, and the buffers its splits leave.
+struct PoolPlan {
+  bool sel;          // selection buffers of cap slots (else sorted lists of cap = kp entries)
+  int cap, splits, tps;
+  bool deep;         // the four-stage variant of the 32-entry pools
+  bool split_first, cluster;
+};
+PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross);
+size_t pool_part_entries(const PoolPlan& p, int na, bool cross);
+struct PoolParts {   // scratch of one sweep
+  float* v;          // pool_part_entries
+  int* i;
+  int* cnt;          // splits * kinds * na
+  uint32_t* tau;     // kinds * na
+};
+// Pools [kind][na][kp] of the rows of S = A . B^T, kp = 32, 64 or 128, sorted best first and
+// padded with (-inf, -1): every score left out of a full pool is <= its last entry.
 // seed (may be NULL): per row of A an admission floor; every split keeps only scores above it,
-// so a merged pool may hold fewer than kp entries, and every score left out of it is <= the
-// floor or <= its last entry.
-// tau_x ([2][kinds][na] floats) and pair_cnt ([2 ceil(na / 256)][kinds][4] ints), both may be
-// NULL: for 32-entry pools without a seed and with splits = 1, where one 128-row A block per SM
-// would not fit in half the L2, two CTAs sweep the two column halves of each row block; pool_v
-// and pool_i then need room for two [kind][na][kp] regions, and the pools end in the first.
+// so a pool may hold fewer than kp entries, and every score left out of it is <= the floor or
+// <= its last entry.
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
-                             const int* cam, bool cross, int self_excl, int kp, int splits, float* pool_v,
-                             int* pool_i, cudaStream_t st, const float* seed = nullptr, float* tau_x = nullptr,
-                             int* pair_cnt = nullptr);
+                             const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
+                             float* pool_v, int* pool_i, cudaStream_t st, const float* seed = nullptr);
 // Pools of row blocks of the gathered matrix Y (rows x d, rounded operand) against column ranges
 // of Y: work item w = {first row, rows <= 128, first column, columns} of *n_items (<= max_items);
 // pool entry (s - col_bias[j], j), j a position in Y; column j == row skipped when self_excl;
@@ -322,6 +338,10 @@ cudaError_t launch_gcrv(const float* frames, int64_t F, int d, const int64_t* of
                         int ncam, float lambda, float* W, const GcrvWs& w, cudaStream_t st);
 
 // ---- serve.cu
+// Sorts and merges the S selection buffers of each (kind, row) ([S][kinds][na][cap], cnt entries)
+// into its pool [kinds][na][kp], best first, padded with (-inf, -1).
+cudaError_t launch_pool_finish(const float* pv, const int* pi, const int* cnt, int S, int kinds, int na, int cap, int kp,
+                               float* ov, int* oi, cudaStream_t st);
 cudaError_t launch_merge_splits(const float* pv, const int* pi, int S, int kinds, int na, int kp, float* ov, int* oi,
                                 cudaStream_t st);
 cudaError_t launch_query_step(const float* xq, int b, int d, const float* G, const float* deg, const int32_t* nbr,

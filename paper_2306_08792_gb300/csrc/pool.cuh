@@ -146,161 +146,269 @@ __device__ __forceinline__ void pool_flush(int lane, bool valid, PoolOwner& me, 
   }
 }
 
-// ---------------------------------------------------------------- lane-parallel heap pools
-// For 32-entry pools on the tensor-core path. Each row's pool is a heap of (score, index) pairs
-// in shared memory ordered by better(): the root is the worst entry kept, so once the heap holds
-// KP entries the admission threshold is the root's score (the same threshold as a sorted list's
-// last entry). Heaps and queues are slot-major, [slot][128 rows] of float2, so the lanes of a
-// warp (consecutive rows) always touch different bank pairs whatever slot each one is at. A lane
-// appends the scores that pass to its row's queue; when any lane's queue could overflow, every
-// lane drains its own queue into its own heap, so one pass serves the warp's 32 rows (the sorted
-// lists instead take one warp-wide merge per row, each waiting on a list in L2). At the end a
-// heapsort leaves each pool sorted best first, as the sorted lists are.
-constexpr int kHeapQ = 8;                  // queue slots per row
-constexpr uint32_t kHeapSlot = 128 * 8;    // bytes between consecutive slots of one row
+// ---------------------------------------------------------------- selection buffers
+// The pools of the tensor-core sweep (POOL mode of umma.cu). A row's candidates sit unsorted in
+// a buffer of CAP > KP slots in shared memory, owned by one lane: every score above the row's
+// threshold is appended, and when any lane of the warp runs short of room all its lanes compact
+// their buffers at once: a bisection over the buffered scores finds a value f with at least KP of
+// them above it, the others are dropped and f becomes the threshold. KP of the row's scores lie
+// above f, so nothing dropped at or below it can be among the row's KP best; after the sweep the
+// buffer holds all of them (and up to CAP - KP more), and pool_finish sorts and cuts it.
+// What bounds the sweep is the feed of the tensor core where rows are long, and the admissions
+// (about KP (1 + ln(columns / KP)) a row) where they are short. A heap, which these buffers
+// replaced for 32-entry pools, pays a chain of dependent shared-memory reads per admission; the
+// sorted lists of the larger pools paid a warp-wide merge through L2 per row and 28 admissions.
+// With column splits that fill the chip (pool_plan), similarity stage before and after: 201,000
+// rows of d = 512, 64-entry pools, 238 -> 180 ms for three layers; 7,001 rows of d = 1000 in
+// BF16, two graphs, 1.43 -> 0.57 ms; 800 rows of d = 128, two graphs, 150 -> 65 us; 512 queries
+// against 500,000 rows of d = 256, the 128-entry pools, 1.98 -> 0.57 ms.
+// Scores and columns are slot-major, [slot][128 rows], so a warp's lanes touch 32 different banks
+// whatever slot each is at; columns are 16-bit offsets from the split's first.
+// More slots, fewer compactions; what the ring (umma.cu) leaves. DEEP (32-entry pools of one
+// graph): 44 slots and a four-stage ring, where long rows make the sweep bound by its feed;
+// otherwise 96 slots and three stages.
+template <int KP, bool CROSS, bool DEEP = false>
+struct SelCap {
+  static constexpr int cap = KP == 32 ? (CROSS ? 48 : DEEP ? 44 : 96) : KP == 64 ? (CROSS ? 80 : 96) : 160;
+};
+constexpr int kSelMaxCols = 65536;         // columns per split (16-bit offsets)
+constexpr uint32_t kSelV = 128 * 4, kSelI = 128 * 2;  // bytes between consecutive slots
 
-__device__ __forceinline__ bool worse(float a, int ai, float b, int bi) { return a < b || (a == b && ai > bi); }
-
-__device__ __forceinline__ float2 heap_ld(uint32_t addr) {
-  float2 r;
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "r"(addr) : "memory");
+__device__ __forceinline__ float sel_ldv(uint32_t a) {
+  float r;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(r) : "r"(a) : "memory");
   return r;
 }
-__device__ __forceinline__ void heap_st(uint32_t addr, float2 v) {
-  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+// Unordered load, for sel_compact alone: the appends precede its (out-of-line) call, and its own
+// stores only go to slots it has read.
+__device__ __forceinline__ float sel_ldv_any(uint32_t a) {
+  float r;
+  asm("ld.shared.f32 %0, [%1];" : "=f"(r) : "r"(a));
+  return r;
+}
+// Order-preserving image of a buffered score (-0 as +0, so that equal scores have equal images).
+__device__ __forceinline__ uint32_t sel_image(uint32_t a) { return float_to_ordered(sel_ldv_any(a) + 0.f); }
+__device__ __forceinline__ uint32_t sel_ldi(uint32_t a) {
+  unsigned short r;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(r) : "r"(a) : "memory");
+  return r;
+}
+__device__ __forceinline__ void sel_st(uint32_t va, uint32_t ia, float v, uint32_t i) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(va), "f"(v) : "memory");
+  asm volatile("st.shared.u16 [%0], %1;" ::"r"(ia), "h"((unsigned short)i) : "memory");
 }
 
-struct HeapState {
-  float tau;
-  int len;
+struct SelState {
+  float tau;   // threshold: scores at or below it are dropped
+  float lo;    // every buffered score is above it (tau, but for what other splits raised it by)
+  float pub;   // a bound another split may drop at: KP of the row's scores are strictly above it
+  float sum;   // of the buffered scores
+  int cnt;
 };
 
-// Drains qcnt queued entries (queue slot 0 at qaddr) into the heap at haddr holding len entries.
-// An entry that no longer beats the root (the threshold rose since it was queued) is dropped.
-// Returns the new threshold (tau unchanged when nothing was queued) and length.
-template <int KP>
-__device__ __noinline__ HeapState heap_drain(uint32_t haddr, uint32_t qaddr, int qcnt, int len, float tau,
-                                             float floor) {
-  for (int i = 0; i < qcnt; ++i) {
-    const float2 e = heap_ld(qaddr + i * kHeapSlot);
-    const int ei = __float_as_int(e.y);
-    if (len < KP) {  // not full yet: sift up from the first free slot
-      int pos = len++;
-      while (pos > 0) {
-        const int par = (pos - 1) >> 1;
-        const float2 p = heap_ld(haddr + par * kHeapSlot);
-        if (!worse(e.x, ei, p.x, __float_as_int(p.y))) break;
-        heap_st(haddr + pos * kHeapSlot, p);
-        pos = par;
+// The buffered scores of a lane as its compaction reads them: in registers (-inf past the count)
+// up to 96 slots, else from shared memory 16 at a time. The tensor core's operand reads and the
+// TMA's writes take most of the shared memory's bandwidth while a compaction runs, so every
+// pass that stays in registers counts (15,000 cycles per compaction of 44 slots when each pass
+// read them again).
+template <int CAP, bool REGS = (CAP <= 96)>
+struct SelScores {
+  float v[CAP];
+  __device__ __forceinline__ void load(uint32_t va, int cnt) {
+#pragma unroll
+    for (int s = 0; s < CAP; ++s) v[s] = sel_ldv_any(va + s * kSelV);
+#pragma unroll
+    for (int s = 0; s < CAP; ++s) v[s] = s < cnt ? v[s] : -CUDART_INF_F;
+  }
+  // scores above p and their sum
+  __device__ __forceinline__ void count(float p, int& c, float& t) const {
+    int c4[4] = {0, 0, 0, 0};
+    float t4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int s = 0; s < CAP; ++s) {
+      const bool in = v[s] > p;
+      c4[s & 3] += in ? 1 : 0;
+      t4[s & 3] += in ? v[s] : 0.f;
+    }
+    c = (c4[0] + c4[1]) + (c4[2] + c4[3]);
+    t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
+  }
+  // bit s & 31 of word w = s >> 5: score s is above f
+  __device__ __forceinline__ void above(float f, uint32_t (&m)[(CAP + 31) / 32]) const {
+#pragma unroll
+    for (int w = 0; w < (CAP + 31) / 32; ++w) m[w] = 0u;
+#pragma unroll
+    for (int s = 0; s < CAP; ++s) m[s >> 5] |= (v[s] > f ? 1u : 0u) << (s & 31);
+  }
+};
+template <int CAP>
+struct SelScores<CAP, false> {
+  uint32_t va;
+  int cnt;
+  __device__ __forceinline__ void load(uint32_t a, int n) { va = a; cnt = n; }
+  __device__ __forceinline__ void count(float p, int& c, float& t) const {
+    int c4[4] = {0, 0, 0, 0};
+    float t4[4] = {0.f, 0.f, 0.f, 0.f};
+    static_assert(CAP % 16 == 0, "whole steps");
+#pragma unroll 1
+    for (int s0 = 0; s0 < CAP; s0 += 16) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = sel_ldv_any(va + (s0 + u) * kSelV);
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const bool in = v[u] > p && s0 + u < cnt;
+        c4[u & 3] += in ? 1 : 0;
+        t4[u & 3] += in ? v[u] : 0.f;
       }
-      heap_st(haddr + pos * kHeapSlot, e);
-    } else {  // full: replace the root if better, then sift down
-      const float2 root = heap_ld(haddr);
-      if (!worse(root.x, __float_as_int(root.y), e.x, ei)) continue;
-      int pos = 0;
-      for (;;) {
-        int c = 2 * pos + 1;
-        if (c >= KP) break;
-        float2 cv = heap_ld(haddr + c * kHeapSlot);
-        if (c + 1 < KP) {
-          const float2 c2 = heap_ld(haddr + (c + 1) * kHeapSlot);
-          if (worse(c2.x, __float_as_int(c2.y), cv.x, __float_as_int(cv.y))) {
-            cv = c2;
-            ++c;
+    }
+    c = (c4[0] + c4[1]) + (c4[2] + c4[3]);
+    t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
+  }
+  __device__ __forceinline__ void above(float f, uint32_t (&m)[(CAP + 31) / 32]) const {
+#pragma unroll
+    for (int w = 0; w < CAP / 32; ++w) {
+      uint32_t x = 0;
+#pragma unroll
+      for (int u = 0; u < 32; ++u) x |= (sel_ldv_any(va + (w * 32 + u) * kSelV) > f && w * 32 + u < cnt ? 1u : 0u) << u;
+      m[w] = x;
+    }
+  }
+};
+
+// Compacts the buffers of the warp's lanes (slot 0 at va / ia, cnt entries): a lane with more
+// than KP entries keeps KP to KP + kSlack of them (in any order), the others keep all. Every
+// lane of the warp calls it. The threshold is searched by pivots: the scores of a row's best few
+// hundred fall off about exponentially, so the first pivot is the quantile of an exponential
+// with their mean above the old threshold; the next ones are the mean of the scores still in
+// question, which splits them whatever their spread (a midpoint takes many more steps when a
+// few scores lie far above the rest). Five or six passes settle most warps.
+template <int KP, int CAP>
+__device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState st) {
+  constexpr int kSlack = (CAP - KP) / 4, W = (CAP + 31) / 32;
+  constexpr float kTarget = KP + 0.5f * kSlack;
+  const int cnt = st.cnt;
+  float tau = st.tau, pub = st.pub;
+  const bool act = cnt > KP;
+  SelScores<CAP> sc;
+  sc.load(va, cnt);
+  // scores in question lie in (a, b]: ca of the entries are above a (ca >= KP), cb above b
+  // (cb < KP); ta, tb are the sums of those
+  float a = st.lo, ta = st.sum, tb = 0.f;
+  int ca = cnt, cb = 0;
+  bool more = act;
+  for (int it = 0; it < 12 && __any_sync(GCR_FULL, more); ++it) {
+    float p = (ta - tb) / (float)max(1, ca - cb);
+    if (it == 0) {
+      const float q = a + (p - a) * __logf((float)ca / kTarget);
+      if (q > a && q < p) p = q;
+    }
+    int c;
+    float t;
+    sc.count(p, c, t);
+    if (more) {
+      if (c >= KP) {
+        more = c > KP + kSlack;
+        a = p;
+        ca = c;
+        ta = t;
+      } else {
+        cb = c;
+        tb = t;
+      }
+    }
+  }
+  float f = a;
+  uint32_t keep[W];
+  sc.above(act ? f : -CUDART_INF_F, keep);
+  float lo = st.lo, sum = act ? ta : st.sum;
+  int kept = act ? ca : cnt;
+  if (act) lo = f;
+  // Scores too close together for the pivots (ties, or infinities): the KP-th largest exactly,
+  // by a binary search on the order-preserving 32-bit images; of the entries equal to it those
+  // of the smallest columns are kept up to KP, as a sorted list would.
+  if (__any_sync(GCR_FULL, act && ca > KP + kSlack)) {
+    const bool ex = act && ca > KP + kSlack;
+    const int n = __reduce_max_sync(GCR_FULL, cnt);
+    uint32_t k = 0;
+    for (int bit = 31; bit >= 0; --bit) {
+      const uint32_t cand = k | (1u << bit);
+      int c = 0;
+      for (int s = 0; s < n; ++s) c += (s < cnt && sel_image(va + s * kSelV) >= cand) ? 1 : 0;
+      if (c >= KP) k = cand;
+    }
+    int larger = 0;
+    for (int s = 0; s < n; ++s) larger += (s < cnt && sel_image(va + s * kSelV) > k) ? 1 : 0;
+    uint32_t col = 0xffffu;  // the largest column offset kept among the equal ones
+    for (int bit = 15; bit >= 0; --bit) {
+      const uint32_t cand = col & ~(1u << bit);
+      int c = 0;
+      for (int s = 0; s < n; ++s)
+        c += (s < cnt && sel_image(va + s * kSelV) == k && sel_ldi(ia + s * kSelI) <= cand) ? 1 : 0;
+      if (larger + c >= KP) col = cand;
+    }
+    if (ex) {
+      float x = 0.f;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        uint32_t m = 0;
+        for (int u = 0; u < 32; ++u) {
+          const int s = w * 32 + u;
+          if (s < cnt) {
+            const uint32_t img = sel_image(va + s * kSelV);
+            if (img > k || (img == k && sel_ldi(ia + s * kSelI) <= col)) {
+              m |= 1u << u;
+              x += sel_ldv(va + s * kSelV);
+            }
           }
         }
-        if (!worse(cv.x, __float_as_int(cv.y), e.x, ei)) break;
-        heap_st(haddr + pos * kHeapSlot, cv);
-        pos = c;
+        keep[w] = m;
       }
-      heap_st(haddr + pos * kHeapSlot, e);
+      f = ordered_to_float(k);
+      lo = ordered_to_float(k - 1u);  // every entry kept is above the value below f
+      kept = KP;
+      sum = x;
     }
   }
-  if (qcnt > 0) tau = (len == KP) ? fmaxf(heap_ld(haddr).x, floor) : floor;
-  return HeapState{tau, len};
-}
-
-// Heapsort of the len entries at haddr (best first) and the row's KP-entry list written to lv /
-// li, padded with (-inf, -1) past len.
-template <int KP>
-__device__ __noinline__ void heap_emit(uint32_t haddr, int len, float* lv, int* li) {
-  for (int end = len - 1; end > 0; --end) {
-    const float2 root = heap_ld(haddr);
-    const float2 last = heap_ld(haddr + end * kHeapSlot);
-    const int lasti = __float_as_int(last.y);
-    heap_st(haddr + end * kHeapSlot, root);
-    int pos = 0;
-    for (;;) {
-      int c = 2 * pos + 1;
-      if (c >= end) break;
-      float2 cv = heap_ld(haddr + c * kHeapSlot);
-      if (c + 1 < end) {
-        const float2 c2 = heap_ld(haddr + (c + 1) * kHeapSlot);
-        if (worse(c2.x, __float_as_int(c2.y), cv.x, __float_as_int(cv.y))) {
-          cv = c2;
-          ++c;
-        }
-      }
-      if (!worse(cv.x, __float_as_int(cv.y), last.x, lasti)) break;
-      heap_st(haddr + pos * kHeapSlot, cv);
-      pos = c;
-    }
-    heap_st(haddr + pos * kHeapSlot, last);
+  if (act) {
+    tau = fmaxf(tau, f);  // another split may have raised it further
+    pub = fmaxf(pub, lo);
   }
-  for (int e = 0; e < KP; ++e) {
-    float v = -CUDART_INF_F;
-    int i = -1;
-    if (e < len) {
-      const float2 x = heap_ld(haddr + e * kHeapSlot);
-      v = x.x;
-      i = __float_as_int(x.y);
-    }
-    lv[e] = v;
-    li[e] = i;
+  // the kept entries past slot `kept` fill the holes before it
+  uint32_t hole = 0, mover = 0;  // what is left of the words being walked
+  int hw = -1, mw = -1;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    const int below = min(max(kept - 32 * w, 0), 32);
+    const uint32_t in = below == 32 ? GCR_FULL : (1u << below) - 1u;
+    const uint32_t h = ~keep[w] & in, m = keep[w] & ~in;
+    keep[w] = h | m;  // holes below slot `kept`, movers from it on
   }
-}
-
-// Paired column splits: the row's sorted list in this CTA's heap slots (own, best first, len
-// entries; slot e at own[e * 128]) merged with the other half's list (KP entries, best first,
-// padded with (-inf, -1), read through L2) into the KP best, written to (dv, di). The other
-// list is first copied to the scratch slots (same layout), so that dv may be the other list
-// itself. Each entry goes straight to its rank: its index in its own list plus the number of
-// entries of the other list that rank before it (a binary search; better() orders the two
-// lists' entries totally, so the ranks of all entries are distinct).
-template <int KP>
-__device__ __forceinline__ void pair_merge_lists(const float2* own, int len, const float* ov, const int* oi,
-                                                 float2* scratch, float* dv, int* di) {
-  for (int e = 0; e < KP; ++e) scratch[e * 128] = make_float2(__ldcg(ov + e), __int_as_float(__ldcg(oi + e)));
-  for (int i = 0; i < len; ++i) {
-    const float2 x = own[i * 128];
-    const int xi = __float_as_int(x.y);
-    int lo = 0, hi = KP;  // others before x: the first j with other[j] not better than x
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      const float2 y = scratch[mid * 128];
-      if (better(y.x, __float_as_int(y.y), x.x, xi)) lo = mid + 1;
-      else hi = mid;
+  auto next = [&](uint32_t& word, int& w, bool holes) -> int {
+    while (word == 0u) {
+      ++w;
+      if (w >= W) return -1;
+      const int below = min(max(kept - 32 * w, 0), 32);
+      const uint32_t in = below == 32 ? GCR_FULL : (1u << below) - 1u;
+      uint32_t x = 0;
+#pragma unroll
+      for (int q = 0; q < W; ++q)
+        if (q == w) x = keep[q];
+      word = holes ? (x & in) : (x & ~in);
     }
-    if (i + lo < KP) {
-      dv[i + lo] = x.x;
-      di[i + lo] = xi;
-    }
+    const int b = __ffs(word) - 1;
+    word &= word - 1u;
+    return 32 * w + b;
+  };
+  for (;;) {
+    const int h = next(hole, hw, true);
+    if (h < 0) break;
+    const int m = next(mover, mw, false);
+    if (m < 0) break;
+    sel_st(va + h * kSelV, ia + h * kSelI, sel_ldv(va + m * kSelV), sel_ldi(ia + m * kSelI));
   }
-  for (int j = 0; j < KP; ++j) {
-    const float2 y = scratch[j * 128];
-    const int yi = __float_as_int(y.y);
-    int lo = 0, hi = len;  // own entries before y
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      const float2 x = own[mid * 128];
-      if (better(x.x, __float_as_int(x.y), y.x, yi)) lo = mid + 1;
-      else hi = mid;
-    }
-    if (j + lo < KP) {
-      dv[j + lo] = y.x;
-      di[j + lo] = yi;
-    }
-  }
+  __syncwarp();
+  return SelState{tau, lo, pub, sum, kept};
 }
 
 }  // namespace gcr

@@ -35,8 +35,7 @@ namespace {
 constexpr int BM = 128;            // rows of A per tile (UMMA M)
 constexpr int BN = 256;            // rows of B per tile (UMMA N)
 constexpr int BKB = 128;           // K bytes per stage (one swizzle row): 64 BF16 / 32 TF32
-constexpr int NST = 3;             // pipeline stages of the modes with pool queues (POOL, GPOOL)
-constexpr int NST_MAX = 4;         // the others (no queues in shared memory)
+constexpr int NST_MAX = 4;         // pipeline stages where nothing else needs shared memory
 constexpr int A_BYTES = BM * BKB;
 constexpr int B_BYTES = BN * BKB;
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -44,6 +43,20 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr unsigned long long kTimeoutNs = 2000000000ull;
 
 enum Mode { POOL = 0, BAND = 1, DIST = 2, GRAM = 3, MUL = 4, GPOOL = 5 };
+
+// POOL runs on selection buffers, except cross-camera pools of 128 entries (two graphs' buffers
+// of 160 slots would leave room for one stage only): those, and GPOOL, keep sorted lists.
+template <int MODE, int KP, bool CROSS, bool DEEP>
+struct Cfg {
+  static constexpr bool kSel = MODE == POOL && !(KP == 128 && CROSS);
+  static constexpr bool kPool = MODE == POOL || MODE == GPOOL;
+  // ring stages: what the pools leave of the 227 KB
+  static constexpr int kStages = !kPool ? NST_MAX
+                                 : !kSel ? 3
+                                 : KP == 32 ? (DEEP ? 4 : 3)
+                                 : KP == 64 ? (CROSS ? 2 : 3)
+                                            : 2;
+};
 
 // ------------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -194,11 +207,12 @@ struct UmmaArgs {
   int d;
   int a_rows;     // rows of A (POOL: rows owning pools; DIST: nq; BAND: band capacity)
   int self_excl;  // skip column j == row i (A and B are the same matrix)
-  int tps;        // POOL: column tiles per split (grid.y = splits)
+  int tps;        // POOL: column tiles per split
   const int* cam;
   // POOL
-  float* pool_v;
-  int* pool_i;
+  float* pool_v;      // sorted lists [split][kind][a_rows][KP], or selection buffers
+  int* pool_i;        //   [split][kind][a_rows][cap] with part_cnt entries each
+  int* part_cnt;      // [split][kind][a_rows]
   const float* seed;  // per row of A, or NULL: admission floor of the row's split pools
   // BAND
   const int* count;
@@ -238,20 +252,15 @@ struct UmmaArgs {
   const int4* items;
   const int* n_items;
   const float* col_bias;
-  int vote;        // POOL: pick the kernel that skips groups of four scores below every row's
-                   // threshold by a vote (GPOOL always does)
-  int warm;        // POOL: admission floors from each row's first column tile (warm_floor)
-  // POOL with heap pools, paired splits: two CTAs per row block (grid.x = the 2 column splits,
-  // grid.y = row blocks, so both halves of a block run at the same time and the row blocks at
-  // work stay few enough for their A rows to stay in L2). Each writes its rows' thresholds to
-  // tau_x after every tile and raises its own to the other's (a threshold of either half is a
-  // score with KP of the row's scores at or above it); the warp that finishes second merges the
-  // two lists into the first split's pools.
-  int pair;
-  float* tau_x;    // [2][pools][a_rows], NaN-initialised (no threshold yet)
-  int* pair_cnt;   // [row blocks][pools][4], zero-initialised: finished warps per (block, pool, quad)
-  // POOL with heap pools: 2-CTA clusters of consecutive row blocks that take the same column
-  // tiles; each CTA loads its A block and one half of the B tile, and the half goes to both
+  // POOL: splits of one row block next to each other in the grid (grid.x = splits, grid.y = row
+  // blocks): they run at the same time, and fewer row blocks are at work, whose A rows then stay
+  // in L2. Otherwise grid.x = row blocks, so the first split of every block runs first.
+  int split_first;
+  // POOL with more than one split: per (kind, row) the order-preserving image of the best bound
+  // any split has published (KP of the row's scores are strictly above it; 0: none yet). Every
+  // split reads it before a tile and raises its own threshold to it.
+  uint32_t* tau_x;
+  // POOL: 2-CTA clusters of consecutive row blocks that take the same column tiles; each CTA loads its A block and one half of the B tile, and the half goes to both
   // CTAs by TMA multicast (tmB2: B in 128-row boxes), so a CTA reads two thirds of the bytes
   // per stage. Each MMA commit frees the stage in both CTAs (empty barriers count 2 arrivals).
   int mc;
@@ -309,22 +318,51 @@ struct Tiles {
   }
 };
 
-constexpr int kWarmIters = 6;  // bisection steps of warm_floor
+// Eligible scores of the tile above f (elig: a bit per column, all ones for most chunks).
+__device__ __forceinline__ int tile_count(uint32_t taddr, int ncol, const uint32_t (&elig)[BN / 32], float f) {
+  int cnt = 0;
+#pragma unroll
+  for (int ch = 0; ch < BN / 32; ++ch) {
+    if (ch * 32 < ncol) {
+      float v[32];
+      tmem_ld32(taddr + ch * 32, v);
+      if (__all_sync(GCR_FULL, elig[ch] == GCR_FULL)) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) cnt += v[c] > f ? 1 : 0;
+      } else {
+        uint32_t above = 0;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) above |= (v[c] > f ? 1u : 0u) << c;
+        cnt += __popc(above & elig[ch]);
+      }
+    }
+  }
+  return cnt;
+}
+
+// Upper quantile of the standard normal: z with P(Z > z) = q, to 3e-3 (Abramowitz and Stegun
+// 26.2.22). Only used to guess thresholds that are then verified by counting.
+__device__ __forceinline__ float normal_upper(float q) {
+  const float u = fminf(fmaxf(fminf(q, 1.f - q), 1e-6f), 0.5f);
+  const float t = sqrtf(-2.f * __logf(u));
+  const float z = t - (2.30753f + 0.27061f * t) / (1.f + t * (0.99229f + 0.04481f * t));
+  return q <= 0.5f ? z : -z;
+}
 
 // Admission floor of one row from the first column tile of its sweep. A pool starts empty, so
-// without a floor every score of that tile would enter the row's queue and the warp would merge
-// it about BN / 28 times before the threshold means anything. Bisection over the tile's eligible
-// scores (held in TMEM, read once per step) finds a value f with at least KP of them above it:
-// the row's KP best scores of the whole sweep all lie above f, so scores at or below f can be
-// dropped from the sweep, and the row's list still ends full with every score left out below its
-// last entry. The counts use the same values and the same eligibility (column < n, not the row
-// itself, another camera for the cross-camera pool) as the appends. -inf when the tile holds
-// KP eligible scores or fewer. All lanes run every step (the TMEM loads are warp-wide).
+// without a floor every score of that tile would be buffered. A value f with at least KP of the
+// tile's eligible scores above it is guessed from their mean and spread as if they were normal,
+// verified by counting them in TMEM, and corrected by the count: the row's KP best scores of the
+// whole sweep all lie above f, so scores at or below f can be dropped from the sweep. The counts
+// use the same values and the same eligibility (column < n, not the row itself, another camera
+// for the cross-camera pool) as the appends. -inf when the tile holds KP eligible scores or
+// fewer. Most warps need two or three counts where a bisection takes six (800 rows of d = 128:
+// 41,000 -> 25,000 cycles per CTA). All lanes run every step (the TMEM loads are warp-wide).
 template <int KP, bool CAMCHK>
 __device__ __noinline__ float warm_floor(uint32_t taddr, int cb0, int ncol, int n, int self_excl, int my_row,
                                          const int* __restrict__ cam, int my_cam, int lane) {
   uint32_t elig[BN / 32];
-  float lo_v = CUDART_INF_F, hi_v = -CUDART_INF_F;
+  float s1 = 0.f, s2 = 0.f, shift = 0.f, lo = CUDART_INF_F, hi = -CUDART_INF_F;
   int ne = 0;
 #pragma unroll
   for (int ch = 0; ch < BN / 32; ++ch) {
@@ -333,65 +371,70 @@ __device__ __noinline__ float warm_floor(uint32_t taddr, int cb0, int ncol, int 
       float v[32];
       tmem_ld32(taddr + ch * 32, v);
       const int cb = cb0 + ch * 32;
-      int ccam = 0;
-      if (CAMCHK) ccam = (cb + lane < n) ? cam[cb + lane] : -1;
+      uint32_t e = cb + 32 <= n ? GCR_FULL : (1u << (n - cb)) - 1u;
+      if (self_excl && my_row >= cb && my_row < cb + 32) e &= ~(1u << (my_row - cb));
+      if (CAMCHK) {
+        const int ccam = (cb + lane < n) ? cam[cb + lane] : -1;
+        uint32_t same = 0;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) same |= (__shfl_sync(GCR_FULL, ccam, c) == my_cam ? 1u : 0u) << c;
+        e &= ~same;
+      }
+      elig[ch] = e;
+      ne += __popc(e);
+      if (ch == 0) shift = v[0];  // sums of v - shift: the spread can be far below the mean
 #pragma unroll
       for (int c = 0; c < 32; ++c) {
-        const int cj = CAMCHK ? __shfl_sync(GCR_FULL, ccam, c) : 0;
-        const bool e = cb + c < n && !(self_excl && cb + c == my_row) && (!CAMCHK || cj != my_cam);
-        if (e) {
-          lo_v = fminf(lo_v, v[c]);
-          hi_v = fmaxf(hi_v, v[c]);
-          ++ne;
-          elig[ch] |= 1u << c;
-        }
+        const bool ok = (e >> c) & 1u;
+        const float x = v[c] - shift;
+        s1 += ok ? x : 0.f;
+        s2 += ok ? x * x : 0.f;
+        lo = ok ? fminf(lo, v[c]) : lo;
+        hi = ok ? fmaxf(hi, v[c]) : hi;
       }
     }
   }
   const bool active = ne > KP;
-  float f = -CUDART_INF_F;
-  float a = active ? lo_v : 0.f, b = active ? hi_v : 0.f;
+  const float inv = 1.f / (float)max(1, ne);
+  const float mean = s1 * inv, sd = sqrtf(fmaxf(0.f, s2 * inv - mean * mean));
+  const float goal = fminf(KP * 1.1f + 1.f, 0.5f * (float)(KP + ne));
+  const float zg = normal_upper(goal * inv);
+  float f = -CUDART_INF_F, x = mean + shift + zg * sd;
+  bool more = active;
 #pragma unroll 1
-  for (int it = 0; it < kWarmIters; ++it) {
-    const float mid = 0.5f * a + 0.5f * b;
-    int cnt = 0;
-#pragma unroll
-    for (int ch = 0; ch < BN / 32; ++ch) {
-      if (ch * 32 < ncol) {
-        float v[32];
-        tmem_ld32(taddr + ch * 32, v);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) cnt += (((elig[ch] >> c) & 1u) && v[c] > mid) ? 1 : 0;
+  for (int it = 0; it < 6 && __any_sync(GCR_FULL, more); ++it) {
+    if (!(x > lo && x < hi)) x = 0.5f * lo + 0.5f * hi;
+    const int c = tile_count(taddr, ncol, elig, x);
+    if (more) {
+      if (c >= KP) {
+        f = lo = x;
+        more = c > KP + KP / 4;
+      } else {
+        hi = x;
       }
-    }
-    if (cnt >= KP) {
-      f = mid;
-      a = mid;
-    } else {
-      b = mid;
+      x += (zg - normal_upper((float)max(c, 1) * inv)) * sd;
     }
   }
-  return active ? f : -CUDART_INF_F;
+  return f;
 }
 
 // MODE is a template parameter (not only a field of UmmaArgs) so that each mode's epilogue is
 // compiled alone: no per-value mode branches, and the POOL kernels need 88-90 registers instead
 // of 116-118 (similarity GEMM on crosscam 2.72 -> 2.65 ms per TF32 launch, 2.75 -> 2.48 BF16).
-template <int MODE, int KP, bool CROSS, bool VOTE = false>
-__global__ void __launch_bounds__(320, 1)
+template <int MODE, int KP, bool CROSS, bool DEEP = false>
+__global__ void __launch_bounds__(CROSS ? 320 : 192, 1)
 umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2, UmmaArgs a) {
   extern __shared__ __align__(1024) unsigned char dyn_raw[];
   // aligned by an offset from the shared array itself, so that every pointer derived from it
   // stays known as shared memory (queue appends compile to shared stores, not generic ones)
   unsigned char* dyn = dyn_raw + ((1024u - (smem_u32(dyn_raw) & 1023u)) & 1023u);
-  constexpr int NS = (MODE == POOL || MODE == GPOOL) ? NST : NST_MAX;  // ring stages
+  constexpr int NS = Cfg<MODE, KP, CROSS, DEEP>::kStages;                   // ring stages
   unsigned char* stages = dyn;                                        // NS * STAGE_BYTES
-  float2* qs = reinterpret_cast<float2*>(dyn + NS * STAGE_BYTES);    // [2][BM][kQCap] queues
-  // 32-entry pools of the per-value path: lane-parallel heaps ([2][KP][BM] float2, slot-major)
-  // and their queues ([2][kHeapQ][BM]) in place of the sorted lists' queues
-  constexpr bool HEAP = MODE == POOL && KP == 32 && !VOTE;
-  float2* hq = reinterpret_cast<float2*>(dyn + NS * STAGE_BYTES + 2 * KP * BM * sizeof(float2));
+  float2* qs = reinterpret_cast<float2*>(dyn + NS * STAGE_BYTES);    // [2][BM][kQCap] queues of the sorted lists
+  constexpr bool SEL = Cfg<MODE, KP, CROSS, DEEP>::kSel;                    // selection buffers instead
+  constexpr int CAP = SEL ? SelCap<KP, CROSS, DEEP>::cap : 1;
+  constexpr int KINDS = CROSS ? 2 : 1;
   __shared__ Bars bars;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -403,8 +446,8 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   const int mul_b0 = MODE == MUL ? max(0, a.mul_rowcam[blockIdx.y]) * a.n : 0;
 
   Tiles<MODE> tl;
-  tl.rb = (MODE == POOL && a.pair) ? (int)blockIdx.y : (int)blockIdx.x;
-  tl.split = (MODE == POOL && a.pair) ? (int)blockIdx.x : (int)blockIdx.y;
+  tl.rb = (MODE == POOL && a.split_first) ? (int)blockIdx.y : (int)blockIdx.x;
+  tl.split = (MODE == POOL && a.split_first) ? (int)blockIdx.x : (int)blockIdx.y;
   int nitems = 0;
   if (MODE == GPOOL) {
     nitems = *a.n_items;
@@ -550,10 +593,16 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     int my_kind = 0;
     const int qrow = kind * BM + r;
     const int sw = qrow & 31;
-    const uint32_t haddr = smem_u32(dyn + NS * STAGE_BYTES) + (uint32_t)((kind * KP * BM + r) * sizeof(float2));
-    const uint32_t qaddr = smem_u32(hq) + (uint32_t)((kind * kHeapQ * BM + r) * sizeof(float2));
-    float2* const hqp = hq + kind * kHeapQ * BM + r;  // this row's queue, slot s at hqp[s * BM]
-    const size_t pbase = ((size_t)tl.split * (CROSS ? 2 : 1) + kind) * a.a_rows * KP;
+    // selection buffers: scores [kind][slot][row], then column offsets
+    const uint32_t sva0 = smem_u32(dyn + NS * STAGE_BYTES) + (uint32_t)((kind * CAP * BM + r) * sizeof(float));
+    const uint32_t sia0 = smem_u32(dyn + NS * STAGE_BYTES) + (uint32_t)(KINDS * CAP * BM * sizeof(float)) +
+                         (uint32_t)((kind * CAP * BM + r) * sizeof(uint16_t));
+    uint32_t sva = sva0, sia = sia0;                       // the next free slot
+    const uint32_t sva_end = sva0 + (CAP - 4) * kSelV;     // past it a group of four may not fit
+    float ssum = 0.f;                                      // sum of the buffered scores
+    float pub = -CUDART_INF_F, pub_sent = -CUDART_INF_F;  // bound for the other splits
+    const bool idle = SEL && tl.rb * BM + quad * 32 >= a.a_rows;  // no row of this warp exists
+    const size_t pbase = ((size_t)tl.split * KINDS + kind) * a.a_rows * (SEL ? CAP : KP);
     float* pv = a.pool_v ? a.pool_v + pbase : nullptr;
     int* pi = a.pool_i ? a.pool_i + pbase : nullptr;
     if (MODE == POOL) {
@@ -566,14 +615,11 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     if (MODE == GPOOL) cur.start(a, nitems);
     bool g_valid = false;        // GPOOL: this thread's row belongs to the current item
     int g_row0 = 0, g_cend = 0;  // GPOOL: first row of the item, end of its columns
-    // paired splits: this row's threshold in the other half's sweep (read before the wait)
-    const bool pair_row = HEAP && a.pair && (kind == 0 || CROSS) && my_row < a.a_rows;
-    const size_t tx_mine = ((size_t)tl.split * (CROSS ? 2 : 1) + kind) * a.a_rows + (pair_row ? my_row : 0);
-    const size_t tx_other = ((size_t)(tl.split ^ 1) * (CROSS ? 2 : 1) + kind) * a.a_rows + (pair_row ? my_row : 0);
+    uint32_t* const tx = (SEL && a.tau_x && my_row >= 0 && my_row < a.a_rows) ? a.tau_x + (size_t)kind * a.a_rows + my_row : nullptr;
     for (int t = 0; t < tl.count; ++t) {
       const int buf = t & 1;
       const uint32_t use = t >> 1;
-      const float tau_other = pair_row ? __ldcg(a.tau_x + tx_other) : CUDART_NAN_F;
+      const uint32_t tau_other = tx ? __ldcg(tx) : 0u;
       if (!mbar_wait(&bars.tfull[buf], use & 1, abort_flag)) break;
       tc_fence_after();
       const int r0 = MODE == GPOOL ? cur.w.x : tl.row0(a, t);
@@ -612,24 +658,22 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
       const int cend = MODE == GPOOL ? g_cend : a.n;  // end of this tile's valid columns
       const int ncol = min(BN, cend - c0);
-      if (MODE == POOL && t == 0 && a.warm && (kind == 0 || CROSS)) {
+      if (MODE == POOL && t == 0 && !idle) {
         const uint32_t ta = tmem + lane_addr + buf * BN;
         const float f = (CROSS && kind == 1)
                             ? warm_floor<KP, true>(ta, c0, ncol, a.n, a.self_excl, my_row, a.cam, my_cam, lane)
                             : warm_floor<KP, false>(ta, c0, ncol, a.n, a.self_excl, my_row, a.cam, my_cam, lane);
         me.floor = fmaxf(me.floor, f);
         me.tau = fmaxf(me.tau, f);
+        if (my_row < a.a_rows) pub = f;
       }
-      if (pair_row) {  // fmaxf ignores the NaN of a threshold not yet written
-        me.floor = fmaxf(me.floor, tau_other);
-        me.tau = fmaxf(me.tau, tau_other);
-      }
+      if (tau_other) me.tau = fmaxf(me.tau, ordered_to_float(tau_other));
       // cross-camera pools: the column cameras of chunk ch + 1 are loaded while chunk ch is
       // processed, so one load latency per tile is exposed instead of one per chunk
       int cam_next = 0;
       if (MODE == POOL && CROSS && kind == 1) cam_next = (c0 + lane < a.n) ? a.cam[c0 + lane] : -1;
       for (int ch = 0; ch < BN / 32; ++ch) {
-        if (ch * 32 >= ncol) break;
+        if (ch * 32 >= ncol || idle) break;
         float v[32];
         tmem_ld32(tmem + lane_addr + buf * BN + ch * 32, v);
         const int cb = c0 + ch * 32;
@@ -656,124 +700,72 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
               const float m4 = fmaxf(fmaxf(v[4 * g], v[4 * g + 1]), fmaxf(v[4 * g + 2], v[4 * g + 3]));
-              if (!VOTE || __any_sync(GCR_FULL, m4 > me.tau)) {
+              if (__any_sync(GCR_FULL, m4 > me.tau)) {
                 pool_make_room<KP>(4, lane, me, r0w, kind * BM + quad * 32, qs, pv, pi);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                   const int cc = g * 4 + c;
                   const int cj = (CROSS && kind == 1) ? __shfl_sync(GCR_FULL, ccam, cc) : 0;
                   const bool eligible = !(CROSS && kind == 1) || cj != my_cam;
-                  if (VOTE) {
-                    if (eligible && v[cc] > me.tau) {
-                      myq[me.qcnt ^ sw] = make_float2(v[cc], __int_as_float(cb + cc));
-                      ++me.qcnt;
-                    }
-                  } else {
-                    pool_push(me, v[cc], cb + cc, eligible, myq, sw);  // branch-free append
+                  if (eligible && v[cc] > me.tau) {
+                    myq[me.qcnt ^ sw] = make_float2(v[cc], __int_as_float(cb + cc));
+                    ++me.qcnt;
                   }
                 }
               }
             }
           }
         } else if (MODE == POOL) {
-          if (kind == 0 || CROSS) {
-            int ccam = 0;
-            if (CROSS && kind == 1) ccam = cam_cur;
-            float2* myq = qs + qrow * kQCap;
-            const int r0w = tl.rb * BM + quad * 32;  // first row of this warp
-            if (VOTE) {
-              // Where few scores pass (a long sweep for the pool size, or admission floors),
-              // most groups of four fall below every row's threshold: one vote over the warp
-              // skips them. The chunk on the warp's diagonal (each row meets itself) and the
-              // ragged last chunk first get their excluded columns set to -inf. The queues get
-              // room every 4 values; votes and shuffles run on every lane.
-              if (cb + 32 > a.n || (a.self_excl && cb == r0w)) {
+          // Most groups of four scores fall below every row's threshold (floors from the first
+          // tile and from the other splits; thresholds only rise): one vote over the warp skips
+          // them. The chunk on the warp's diagonal (each row meets itself) and the ragged last
+          // chunk first get their excluded columns set to -inf; the global pool's warps compare
+          // against a camera no column has.
+          const int r0w = tl.rb * BM + quad * 32;  // first row of this warp
+          if (cb + 32 > a.n || (a.self_excl && cb == r0w)) {
 #pragma unroll
-                for (int c = 0; c < 32; ++c)
-                  if (cb + c >= a.n || (a.self_excl && cb + c == my_row)) v[c] = -CUDART_INF_F;
+            for (int c = 0; c < 32; ++c)
+              if (cb + c >= a.n || (a.self_excl && cb + c == my_row)) v[c] = -CUDART_INF_F;
+          }
+          const int ccam = (CROSS && kind == 1) ? cam_cur : 0;
+          const int cmp_cam = (CROSS && kind == 1) ? my_cam : -2;
+          const int off0 = cb - tl.split * a.tps * BN;  // 16-bit column offset of the chunk
+          float2* myq = qs + qrow * kQCap;
+#pragma unroll
+          for (int g = 0; g < 8; ++g) {
+            const float m4 = fmaxf(fmaxf(v[4 * g], v[4 * g + 1]), fmaxf(v[4 * g + 2], v[4 * g + 3]));
+            if (!__any_sync(GCR_FULL, m4 > me.tau)) continue;
+            if constexpr (SEL) {
+              if (__any_sync(GCR_FULL, sva > sva_end)) {
+                const SelState ss = sel_compact<KP, CAP>(
+                    sva0, sia0, SelState{me.tau, me.floor, pub, ssum, (int)((sva - sva0) / kSelV)});
+                me.tau = ss.tau;
+                me.floor = ss.lo;
+                sva = sva0 + ss.cnt * kSelV;
+                sia = sia0 + ss.cnt * kSelI;
+                pub = ss.pub;
+                ssum = ss.sum;
               }
 #pragma unroll
-              for (int g = 0; g < 8; ++g) {
-                const float m4 = fmaxf(fmaxf(v[4 * g], v[4 * g + 1]), fmaxf(v[4 * g + 2], v[4 * g + 3]));
-                if (__any_sync(GCR_FULL, m4 > me.tau)) {
-                  pool_make_room<KP>(4, lane, me, r0w, kind * BM + quad * 32, qs, pv, pi);
-#pragma unroll
-                  for (int c = 0; c < 4; ++c) {
-                    const int cc = g * 4 + c;
-                    // every lane of the warp (kind is the warp's) takes the camera of column cc
-                    const int cj = (CROSS && kind == 1) ? __shfl_sync(GCR_FULL, ccam, cc) : 0;
-                    if ((!(CROSS && kind == 1) || cj != my_cam) && v[cc] > me.tau) {
-                      myq[me.qcnt ^ sw] = make_float2(v[cc], __int_as_float(cb + cc));
-                      ++me.qcnt;
-                    }
-                  }
-                }
-              }
-            } else if (HEAP) {
-              // Per-value path with heap pools: a score that passes goes to the row's queue
-              // (a predicated shared store); every 4 values, if any lane's queue could not take
-              // 4 more, all lanes drain their queues into their heaps. A group of four that no
-              // row of the warp admits (its max at or below every lane's threshold; thresholds
-              // only rise, so none of it could enter later) is skipped after one vote: with
-              // first-tile floors and the paired halves' exchanged thresholds that is most
-              // groups past the first tiles. The excluded columns (past n, and each row itself
-              // on the warp's diagonal chunk) are set to -inf once per chunk; the global pool's
-              // warps compare against a camera no column has.
-              if (cb + 32 > a.n || (a.self_excl && cb == r0w)) {
-#pragma unroll
-                for (int c = 0; c < 32; ++c)
-                  if (cb + c >= a.n || (a.self_excl && cb + c == my_row)) v[c] = -CUDART_INF_F;
-              }
-              const int cmp_cam = (CROSS && kind == 1) ? my_cam : -2;
-#pragma unroll
-              for (int g = 0; g < 8; ++g) {
-                const float m4 = fmaxf(fmaxf(v[4 * g], v[4 * g + 1]), fmaxf(v[4 * g + 2], v[4 * g + 3]));
-                if (!__any_sync(GCR_FULL, m4 > me.tau)) continue;
-                if (__any_sync(GCR_FULL, me.qcnt > kHeapQ - 4)) {
-                  const HeapState hs = heap_drain<KP>(haddr, qaddr, me.qcnt, me.len, me.tau, me.floor);
-                  me.tau = hs.tau;
-                  me.len = hs.len;
-                  me.qcnt = 0;
-                }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                  const int cc = g * 4 + c;
-                  const int cj = CROSS ? __shfl_sync(GCR_FULL, ccam, cc) : 0;
-                  if (cj != cmp_cam && v[cc] > me.tau) {
-                    hqp[me.qcnt * BM] = make_float2(v[cc], __int_as_float(cb + cc));
-                    ++me.qcnt;
-                  }
+              for (int c = 0; c < 4; ++c) {
+                const int cc = g * 4 + c;
+                const int cj = CROSS ? __shfl_sync(GCR_FULL, ccam, cc) : 0;
+                if (cj != cmp_cam && v[cc] > me.tau) {
+                  sel_st(sva, sia, v[cc], off0 + cc);
+                  sva += kSelV;
+                  sia += kSelI;
+                  ssum += v[cc];
                 }
               }
             } else {
-              // Where many scores pass, every value goes through the branch-free append; the
-              // queues are checked every 4 values, so they fill to 28 of 32 slots before a merge
-              // (every 8: 24; measured 2.82 -> 2.73 ms per TF32 launch, every 2 is slower again).
-              // The excluded columns (past n, and each row itself on the warp's diagonal chunk)
-              // are set to -inf once per chunk, so the append tests only the score (and, in the
-              // cross-camera warps, the column's camera).
-              if (cb + 32 > a.n || (a.self_excl && cb == r0w)) {
+              pool_make_room<KP>(4, lane, me, r0w, kind * BM + quad * 32, qs, pv, pi);
 #pragma unroll
-                for (int c = 0; c < 32; ++c)
-                  if (cb + c >= a.n || (a.self_excl && cb + c == my_row)) v[c] = -CUDART_INF_F;
-              }
-              if (CROSS && kind == 1) {  // warp-uniform
-#pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                  pool_make_room<KP>(4, lane, me, r0w, kind * BM + quad * 32, qs, pv, pi);
-#pragma unroll
-                  for (int c = 0; c < 4; ++c) {
-                    const int cc = g * 4 + c;
-                    const int cj = __shfl_sync(GCR_FULL, ccam, cc);
-                    pool_push(me, v[cc], cb + cc, cj != my_cam, myq, sw);
-                  }
-                }
-              } else {
-#pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                  pool_make_room<KP>(4, lane, me, r0w, kind * BM + quad * 32, qs, pv, pi);
-#pragma unroll
-                  for (int c = 0; c < 4; ++c) pool_push(me, v[g * 4 + c], cb + g * 4 + c, true, myq, sw);
+              for (int c = 0; c < 4; ++c) {
+                const int cc = g * 4 + c;
+                const int cj = CROSS ? __shfl_sync(GCR_FULL, ccam, cc) : 0;
+                if (cj != cmp_cam && v[cc] > me.tau) {
+                  myq[me.qcnt ^ sw] = make_float2(v[cc], __int_as_float(cb + cc));
+                  ++me.qcnt;
                 }
               }
             }
@@ -828,35 +820,26 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars.tempty[buf]);
-      if (pair_row) __stcg(a.tau_x + tx_mine, me.tau);
+      if (tx && pub > pub_sent) {
+        atomicMax(tx, float_to_ordered(pub));
+        pub_sent = pub;
+      }
       if (g_last && (kind == 0 || CROSS))
         pool_flush<KP>(lane, g_valid, me, g_row0 + quad * 32, kind * BM + quad * 32, qs, pv, pi);
     }
-    if (MODE == POOL && (kind == 0 || CROSS) && !*abort_flag) {
-      if (HEAP) {
-        if (__any_sync(GCR_FULL, me.qcnt > 0)) {
-          const HeapState hs = heap_drain<KP>(haddr, qaddr, me.qcnt, me.len, me.tau, me.floor);
-          me.len = hs.len;
-          me.qcnt = 0;
-        }
-        if (my_row < a.a_rows) heap_emit<KP>(haddr, me.len, pv + (size_t)my_row * KP, pi + (size_t)my_row * KP);
-        if (a.pair) {
-          // the list is written: make it visible, count this warp, and merge if it is second
-          // (the stage buffers are idle by now and hold the other half's lists)
-          __threadfence();
-          __syncwarp();
-          int prev = 0;
-          if (lane == 0) prev = atomicAdd(a.pair_cnt + ((size_t)tl.rb * (CROSS ? 2 : 1) + kind) * 4 + quad, 1);
-          prev = __shfl_sync(GCR_FULL, prev, 0);
-          if (prev == 1) {
-            __threadfence();
-            const size_t ro = ((size_t)(tl.split ^ 1) * (CROSS ? 2 : 1) + kind) * a.a_rows * KP;  // the other half
-            const size_t r0s = (size_t)kind * a.a_rows * KP;                                   // split 0's pools
-            const float2* own = reinterpret_cast<const float2*>(dyn + NS * STAGE_BYTES) + kind * KP * BM + r;
-            float2* scratch = reinterpret_cast<float2*>(stages) + kind * KP * BM + r;
-            if (my_row < a.a_rows)
-              pair_merge_lists<KP>(own, me.len, a.pool_v + ro + (size_t)my_row * KP, a.pool_i + ro + (size_t)my_row * KP,
-                                   scratch, a.pool_v + r0s + (size_t)my_row * KP, a.pool_i + r0s + (size_t)my_row * KP);
+    if (MODE == POOL && !*abort_flag) {
+      if constexpr (SEL) {
+        if (my_row < a.a_rows) {
+          const int col0 = tl.split * a.tps * BN;
+          const int cnt = (int)((sva - sva0) / kSelV);
+          a.part_cnt[((size_t)tl.split * KINDS + kind) * a.a_rows + my_row] = cnt;
+          float4* ov = reinterpret_cast<float4*>(pv + (size_t)my_row * CAP);
+          int4* oi = reinterpret_cast<int4*>(pi + (size_t)my_row * CAP);
+          for (int s = 0; s < cnt; s += 4) {  // (slots past the count: never read)
+            const uint32_t va = sva0 + s * kSelV, ia = sia0 + s * kSelI;
+            ov[s >> 2] = make_float4(sel_ldv(va), sel_ldv(va + kSelV), sel_ldv(va + 2 * kSelV), sel_ldv(va + 3 * kSelV));
+            oi[s >> 2] = make_int4(col0 + (int)sel_ldi(ia), col0 + (int)sel_ldi(ia + kSelI),
+                                   col0 + (int)sel_ldi(ia + 2 * kSelI), col0 + (int)sel_ldi(ia + 3 * kSelI));
           }
         }
       } else {
@@ -929,19 +912,23 @@ cudaError_t make_map(CUtensorMap* m, const void* base, Elt elt, int rows, int d,
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-size_t smem_bytes(int mode, bool heap = false) {
-  if (mode != POOL && mode != GPOOL) return 1024 + (size_t)NST_MAX * STAGE_BYTES;
-  size_t s = 1024 + (size_t)NST * STAGE_BYTES;
-  if (heap) s += 2 * (32 + kHeapQ) * BM * sizeof(float2);
-  else s += 2 * BM * kQCap * (sizeof(float) + sizeof(int));
+template <int MODE, int KP, bool CROSS, bool DEEP>
+constexpr size_t smem_bytes() {
+  using C = Cfg<MODE, KP, CROSS, DEEP>;
+  size_t s = 1024 + (size_t)C::kStages * STAGE_BYTES;
+  if constexpr (C::kSel)
+    s += (size_t)(CROSS ? 2 : 1) * SelCap<KP, CROSS, DEEP>::cap * BM * (sizeof(float) + sizeof(uint16_t));
+  else if (C::kPool)
+    s += 2 * BM * kQCap * (sizeof(float) + sizeof(int));
   return s;
 }
 
-template <int MODE, int KP, bool CROSS, bool VOTE = false>
+template <int MODE, int KP, bool CROSS, bool DEEP = false>
 cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, const UmmaArgs& a, dim3 grid, cudaStream_t st,
                    const CUtensorMap* ta2 = nullptr, const CUtensorMap* tb2 = nullptr, dim3 cluster = dim3(1, 1, 1)) {
-  auto fn = umma_kernel<MODE, KP, CROSS, VOTE>;
-  const size_t smem = smem_bytes(a.mode, MODE == POOL && KP == 32 && !VOTE);
+  auto fn = umma_kernel<MODE, KP, CROSS, DEEP>;
+  constexpr size_t smem = smem_bytes<MODE, KP, CROSS, DEEP>();
+  static_assert(smem + sizeof(Bars) <= 232448, "shared memory of a CTA");
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (cluster.x * cluster.y * cluster.z == 1) {
@@ -977,37 +964,70 @@ int umma_read_and_clear_timeouts() {
   return h;
 }
 
+// A sweep's time in units of a column tile, per CTA: its tiles and the set-up, first-tile floor
+// and write-out around them (about 12 us against d / 64 * 0.25 us per tile, at least 0.8).
+PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross) {
+  PoolPlan p;
+  p.sel = !(kp == 128 && cross);
+  // eight K blocks or fewer per tile: a three-stage ring covers them
+  p.deep = kp == 32 && !cross && d * elt_bytes(elt) > 8 * BKB;
+  p.cap = !p.sel ? kp : kp == 32 ? (cross ? SelCap<32, true>::cap : p.deep ? SelCap<32, false, true>::cap : SelCap<32, false>::cap)
+                      : kp == 64 ? (cross ? SelCap<64, true>::cap : SelCap<64, false>::cap)
+                                 : SelCap<128, false>::cap;
+  const int ntiles = (nb + BN - 1) / BN, rblocks = (na + BM - 1) / BM;
+  const double tile_us = std::max(0.8, d * (double)elt_bytes(elt) / 128.0 * 0.25);
+  const double around = 12.0 / tile_us;
+  auto tps_of = [&](int s) { return (ntiles + s - 1) / s; };
+  int best = 1;
+  double best_t = 1e300;
+  for (int s = 1; s <= std::min(ntiles, kSMs); ++s) {
+    const int tps = tps_of(s);
+    if (s > 1 && (long)rblocks * (s - 1) > 16 * kSMs) break;  // past 16 waves nothing is left to even out
+    if (p.sel && (long)tps * BN > kSelMaxCols) continue;  // 16-bit column offsets
+    const int used = (ntiles + tps - 1) / tps;
+    const double waves = std::ceil((double)rblocks * used / kSMs);
+    const double t = waves * (tps + around);
+    if (t < best_t * 0.999) {
+      best_t = t;
+      best = s;
+    }
+  }
+  // more splits than SMs only for the 16-bit offsets (over kSelMaxCols columns per SM)
+  if (p.sel)
+    while ((long)tps_of(best) * BN > kSelMaxCols) ++best;
+  // Where one A block per SM would not fit in half the L2 (151 blocks of 128 x 2048 TF32 rows:
+  // 151 MB, re-read for every column tile), two CTAs sweep the halves of each block at the same
+  // time, so half as many blocks are at work.
+  const double live_a = (double)std::min(rblocks, kSMs) * BM * d * (double)elt_bytes(elt);
+  p.split_first = false;
+  if (best == 1 && ntiles >= 2 && live_a > 0.5 * kL2Bytes) {
+    best = 2;
+    p.split_first = true;
+  }
+  p.tps = tps_of(best);
+  p.splits = (ntiles + p.tps - 1) / p.tps;  // no split is left without a column tile
+  // 2-CTA clusters of row blocks share the column tiles (an even count: the last block of an odd
+  // one has no rows and only loads its half of the shared tiles, so not for few blocks)
+  p.cluster = p.sel && (rblocks % 2 == 0 || rblocks > 16);
+  return p;
+}
+
+size_t pool_part_entries(const PoolPlan& p, int na, bool cross) {
+  return (size_t)p.splits * (cross ? 2 : 1) * na * p.cap;
+}
+
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
-                             const int* cam, bool cross, int self_excl, int kp, int splits, float* pool_v,
-                             int* pool_i, cudaStream_t st, const float* seed, float* tau_x, int* pair_cnt) {
-  CUtensorMap ta, tb;
+                             const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
+                             float* pool_v, int* pool_i, cudaStream_t st, const float* seed) {
+  CUtensorMap ta, tb, tb_half;
   cudaError_t e = make_map(&ta, Ab, elt, na, d, BM);
   if (e != cudaSuccess) return e;
   e = make_map(&tb, Bb, elt, nb, d, BN);
   if (e != cudaSuccess) return e;
-  const int ntiles = (nb + BN - 1) / BN;
-  const int rblocks = (na + BM - 1) / BM;
-  // Paired splits (heap pools only) where the A blocks of one CTA per SM would not fit in half
-  // the L2: each CTA re-reads its A block for every column tile, and 151 blocks of 128 x 2048
-  // TF32 rows (151 MB) would otherwise come from DRAM every time.
-  int l2 = 0, nsm = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const double live_a = (double)std::min(rblocks, std::max(nsm, 1)) * BM * d * (double)elt_bytes(elt);
-  // expected share of a split's scores that enter a row's pool, in random order: about
-  // kp (1 + ln(columns / kp)) / columns; a vote pays where that is small (or with floors)
-  auto admit_share = [&](int tiles_per_split) {
-    const double cols = (double)std::min(nb, tiles_per_split * BN);
-    return cols > kp ? kp * (1.0 + std::log(cols / kp)) / cols : 1.0;
-  };
-  const bool pair = kp == 32 && !seed && tau_x && pair_cnt && splits <= 1 && ntiles >= 2 && l2 > 0 &&
-                    live_a > 0.5 * l2 && admit_share((ntiles + 1) / 2) >= 0.006;
-  if (pair) splits = 2;
-  if (splits < 1) splits = 1;
-  if (splits > ntiles) splits = ntiles;
-  const int tps = (ntiles + splits - 1) / splits;
-  splits = (ntiles + tps - 1) / tps;  // no split is left without a column tile
+  e = make_map(&tb_half, Bb, elt, nb, d, BN / 2);
+  if (e != cudaSuccess) return e;
+  const PoolPlan p = pool_plan(na, nb, d, elt, kp, cross);
+  const int rblocks = (na + BM - 1) / BM, kinds = cross ? 2 : 1;
   UmmaArgs a{};
   a.mode = POOL;
   a.tf32 = elt == Elt::TF32;
@@ -1015,52 +1035,29 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
   a.d = d;
   a.a_rows = na;
   a.self_excl = self_excl;
-  a.tps = tps;
+  a.tps = p.tps;
   a.cam = cam;
-  a.pool_v = pool_v;
-  a.pool_i = pool_i;
+  a.pool_v = parts.v;
+  a.pool_i = parts.i;
+  a.part_cnt = parts.cnt;
   a.seed = seed;
-  a.vote = (seed != nullptr || admit_share(tps) < 0.006) ? 1 : 0;
-  a.warm = 1;
-  dim3 grid(rblocks, splits);
-  // heap pools: 2-CTA clusters over row blocks (an even count: a last block past na has no
-  // rows and only loads its half of the shared B tiles)
-  const bool heap = kp == 32 && !a.vote;
-  const int rb_grid = heap ? (rblocks + 1) & ~1 : rblocks;
-  CUtensorMap tb_half;
-  dim3 cluster(1, 1, 1);
-  if (heap) {
-    e = make_map(&tb_half, Bb, elt, nb, d, BN / 2);
+  a.split_first = p.split_first;
+  if (p.sel && p.splits > 1) {
+    a.tau_x = parts.tau;
+    e = cudaMemsetAsync(parts.tau, 0, sizeof(uint32_t) * kinds * (size_t)na, st);
     if (e != cudaSuccess) return e;
-    a.mc = 1;
-    grid = dim3(rb_grid, splits);
-    cluster = dim3(2, 1, 1);
   }
-  if (pair) {  // no vote: the admission share was checked for these splits
-    const int pools = cross ? 2 : 1;
-    cudaError_t e2 = cudaMemsetAsync(tau_x, 0xFF, sizeof(float) * 2 * pools * (size_t)na, st);  // NaN
-    if (e2 == cudaSuccess) e2 = cudaMemsetAsync(pair_cnt, 0, sizeof(int) * (size_t)rb_grid * pools * 4, st);
-    if (e2 != cudaSuccess) return e2;
-    a.pair = 1;
-    a.tau_x = tau_x;
-    a.pair_cnt = pair_cnt;
-    grid = dim3(2, rb_grid);
-    cluster = dim3(1, 2, 1);
-  }
-  if (heap) {
-    return cross ? launch<POOL, 32, true>(ta, tb, a, grid, st, nullptr, &tb_half, cluster)
-                 : launch<POOL, 32, false>(ta, tb, a, grid, st, nullptr, &tb_half, cluster);
-  }
-  if (a.vote) {
-    if (kp == 32) return cross ? launch<POOL, 32, true, true>(ta, tb, a, grid, st) : launch<POOL, 32, false, true>(ta, tb, a, grid, st);
-    if (kp == 64) return cross ? launch<POOL, 64, true, true>(ta, tb, a, grid, st) : launch<POOL, 64, false, true>(ta, tb, a, grid, st);
-    if (kp == 128) return cross ? launch<POOL, 128, true, true>(ta, tb, a, grid, st) : launch<POOL, 128, false, true>(ta, tb, a, grid, st);
-    return cudaErrorInvalidValue;
-  }
-  if (kp == 32) return cross ? launch<POOL, 32, true>(ta, tb, a, grid, st) : launch<POOL, 32, false>(ta, tb, a, grid, st);
-  if (kp == 64) return cross ? launch<POOL, 64, true>(ta, tb, a, grid, st) : launch<POOL, 64, false>(ta, tb, a, grid, st);
-  if (kp == 128) return cross ? launch<POOL, 128, true>(ta, tb, a, grid, st) : launch<POOL, 128, false>(ta, tb, a, grid, st);
-  return cudaErrorInvalidValue;
+  const int rb_grid = p.cluster ? (rblocks + 1) & ~1 : rblocks;
+  const dim3 grid = p.split_first ? dim3(p.splits, rb_grid) : dim3(rb_grid, p.splits);
+  a.mc = p.cluster;
+  const dim3 cl = !p.cluster ? dim3(1, 1, 1) : p.split_first ? dim3(1, 2, 1) : dim3(2, 1, 1);
+  if (kp == 32) e = cross ? launch<POOL, 32, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : p.deep ? launch<POOL, 32, false, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : launch<POOL, 32, false>(ta, tb, a, grid, st, nullptr, &tb_half, cl);
+  else if (kp == 64) e = cross ? launch<POOL, 64, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : launch<POOL, 64, false>(ta, tb, a, grid, st, nullptr, &tb_half, cl);
+  else if (kp == 128) e = cross ? launch<POOL, 128, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : launch<POOL, 128, false>(ta, tb, a, grid, st, nullptr, &tb_half, cl);
+  else e = cudaErrorInvalidValue;
+  if (e != cudaSuccess) return e;
+  if (!p.sel) return launch_merge_splits(parts.v, parts.i, p.splits, kinds, na, kp, pool_v, pool_i, st);
+  return launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, na, p.cap, kp, pool_v, pool_i, st);
 }
 
 cudaError_t launch_umma_gpool(const void* Y, int rows, int d, Elt elt, const int* gcam, bool cross, int self_excl,
@@ -1085,12 +1082,11 @@ cudaError_t launch_umma_gpool(const void* Y, int rows, int d, Elt elt, const int
   a.items = items;
   a.n_items = n_items;
   a.col_bias = col_bias;
-  a.vote = 1;
   // persistent: one CTA per SM (the POOL shared memory allows one), items strided over the grid
   dim3 grid((unsigned)std::max(1, std::min(max_items, 152)));
-  if (kp == 32) return cross ? launch<GPOOL, 32, true, true>(ta, tb, a, grid, st) : launch<GPOOL, 32, false, true>(ta, tb, a, grid, st);
-  if (kp == 64) return cross ? launch<GPOOL, 64, true, true>(ta, tb, a, grid, st) : launch<GPOOL, 64, false, true>(ta, tb, a, grid, st);
-  if (kp == 128) return cross ? launch<GPOOL, 128, true, true>(ta, tb, a, grid, st) : launch<GPOOL, 128, false, true>(ta, tb, a, grid, st);
+  if (kp == 32) return cross ? launch<GPOOL, 32, true>(ta, tb, a, grid, st) : launch<GPOOL, 32, false>(ta, tb, a, grid, st);
+  if (kp == 64) return cross ? launch<GPOOL, 64, true>(ta, tb, a, grid, st) : launch<GPOOL, 64, false>(ta, tb, a, grid, st);
+  if (kp == 128) return cross ? launch<GPOOL, 128, true>(ta, tb, a, grid, st) : launch<GPOOL, 128, false>(ta, tb, a, grid, st);
   return cudaErrorInvalidValue;
 }
 

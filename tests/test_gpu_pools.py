@@ -1,0 +1,61 @@
+"""The candidate pools of the tensor-core sweep at the edges of their buffers and splits: kNN sets
+against the FP64 oracle (certified ties allowed, no other difference)."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(X, k, precision, pool=0, cam=None):
+    import paper_2306_08792_gb300 as gcr
+    X0 = gcr.gcr_normalize(torch.from_numpy(np.ascontiguousarray(X, dtype=np.float32)).cuda())
+    n = X0.shape[0]
+    p = gcr.default_params(k=k, precision=precision, pool=pool, cross_camera=0 if cam is None else 1, alpha=0.5)
+    G = gcr.gcr_build_graph(X0, p, None if cam is None else torch.from_numpy(cam.astype(np.int32)).cuda())
+    torch.cuda.synchronize()
+    X64 = X0.double().cpu().numpy()
+    r = parity.compare_knn(X64, np.arange(n), G.nbr.cpu().numpy(), k)
+    assert r["mismatched"] == 0, r
+    if cam is not None:
+        rc = parity.compare_knn(X64, np.arange(n), G.nbr_cr.cpu().numpy(), k, cam, cross=True)
+        assert rc["mismatched"] == 0, rc
+    assert G.stats_dict()["band_failed"] == 0
+
+
+# one tile and a column more, odd row blocks, splits of one and of several column tiles; pools of
+# 32 (long rows take the deep ring), 64 and 128 entries, one and two graphs
+@pytest.mark.parametrize("precision,n,d,k,pool,cams", [
+    ("tf32", 257, 64, 10, 32, 0), ("tf32", 257, 64, 31, 32, 5), ("tf32", 2305, 1024, 20, 0, 0),
+    ("tf32", 1537, 72, 40, 64, 0), ("tf32", 1537, 72, 40, 64, 4), ("bf16", 2817, 136, 15, 0, 6),
+    ("tf32", 1100, 40, 60, 128, 0), ("tf32", 1100, 40, 60, 128, 3), ("tf32", 5000, 256, 12, 0, 0)])
+def test_pool_sizes_and_splits(precision, n, d, k, pool, cams):
+    X, cam = workloads.random_unit_like(n + d, n, d, cams=max(cams, 1))
+    _check(X, k, precision, pool, cam if cams else None)
+
+
+@pytest.mark.parametrize("precision,k,pool", [("tf32", 12, 32), ("tf32", 30, 64), ("tf32", 50, 128), ("bf16", 20, 64)])
+def test_more_equal_scores_than_a_buffer_holds(precision, k, pool):
+    """200 copies of one row and 40 of another among 1,500: every score a copy gives is tied
+    far beyond the pool and its buffer."""
+    rng = np.random.default_rng(4)
+    X = rng.standard_normal((1500, 48)).astype(np.float32)
+    X[rng.choice(1500, 200, replace=False)] = X[0]
+    X[rng.choice(np.arange(1, 1500), 40, replace=False)] = X[1]
+    _check(X, k, precision, pool)
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_scores_that_rise_or_fall_along_the_columns(sign):
+    """Rows along an arc: for the last (first) rows every column tile beats all before it, so
+    that every score is appended once and the buffers are compacted as often as they can be."""
+    rng = np.random.default_rng(6)
+    n, d = 1800, 64
+    th = sign * np.linspace(0.0, 1.5, n)
+    X = 0.04 * rng.standard_normal((n, d))
+    X[:, 0] += np.cos(th)
+    X[:, 1] += np.sin(th)
+    _check(X, 20, "tf32")
