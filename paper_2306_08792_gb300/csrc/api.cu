@@ -100,8 +100,8 @@ size_t op_capacity(int64_t n, const gcr_params* p, int kinds) {
   return (size_t)(n * per);
 }
 
-PoolParts carve_parts(Carve& c, int na, int nb, int d, Elt elt, int kp, bool cross) {
-  const PoolPlan pl = pool_plan(na, nb, d, elt, kp, cross);
+PoolParts carve_parts(Carve& c, int na, int nb, int d, const gcr_params* p, int kp, bool cross) {
+  const PoolPlan pl = tensor_mode(p) ? pool_plan(na, nb, d, elt_of(p), kp, cross) : simt_pool_plan(na, nb, d, kp, cross);
   const size_t rows = (size_t)(cross ? 2 : 1) * na, entries = pool_part_entries(pl, na, cross);
   PoolParts t;
   t.v = c.take<float>(entries);
@@ -120,7 +120,7 @@ struct BuildWs {
   float* anrm;
   float* pool_v;
   int* pool_i;
-  PoolParts parts;     // the tensor-core sweep's split buffers
+  PoolParts parts;     // the sweep's split buffers
   int* unc_count;
   int* unc_row;
   int* unc_kind;
@@ -179,7 +179,7 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.anrm = bf ? c.take<float>(nn) : nullptr;
   t.pool_v = c.take<float>((size_t)kinds * nn * r.kp);
   t.pool_i = c.take<int>((size_t)kinds * nn * r.kp);
-  t.parts = bf ? carve_parts(c, (int)n, (int)n, d, elt_of(p), r.kp, kinds == 2) : PoolParts{};
+  t.parts = carve_parts(c, (int)n, (int)n, d, p, r.kp, kinds == 2);
   t.unc_count = c.take<int>(4);
   t.unc_row = c.take<int>((size_t)kinds * nn);
   t.unc_kind = c.take<int>((size_t)kinds * nn);
@@ -252,7 +252,8 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
       GCR_CUDA_TRY(launch_umma_pool(w.xr, n, w.xr, n, d, elt, camp, p->cross_camera != 0, 1, r.kp, w.parts,
                                     w.pool_v, w.pool_i, st));
     } else {
-      GCR_CUDA_TRY(launch_sgemm_pool(X, n, X, n, d, camp, r.kp, p->cross_camera != 0, 1, 1, w.pool_v, w.pool_i, st));
+      GCR_CUDA_TRY(launch_sgemm_pool(X, n, X, n, d, camp, r.kp, p->cross_camera != 0, 1, w.parts, w.pool_v, w.pool_i,
+                                     st));
     }
   }
 
@@ -630,8 +631,8 @@ struct ServeWs {
   float* enrm;
   float* anrm;
   RowScalars* sc;
-  PoolParts parts;     // the layer searches' split buffers (the FP32 path: its sorted lists in v
-  PoolParts parts_final;  // and i), and the final search's in the same memory
+  PoolParts parts;        // the layer searches' split buffers
+  PoolParts parts_final;  // and the final search's, in the same memory
   float* pool_v;
   int* pool_i;
   int* unc_count;
@@ -656,15 +657,6 @@ struct ServeWs {
   float* seed;         // per query: the admission floor of this search's split pools
 };
 
-constexpr int kServeMaxSplits = 152;
-
-// Column splits the pool launchers actually use for `want` splits of `ntiles` tiles.
-int split_count(int want, int ntiles) {
-  want = std::max(1, std::min(want, ntiles));
-  const int tps = (ntiles + want - 1) / want;
-  return (ntiles + tps - 1) / tps;
-}
-
 int serve_kp_final(const gcr_params* p) {
   const int K = p->topk_out;
   if (p->precision != GCR_PREC_BF16 && K < 32) return 32;
@@ -685,23 +677,17 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   t.enrm = bf ? c.take<float>(nb) : nullptr;
   t.anrm = bf ? c.take<float>(nb) : nullptr;
   t.sc = c.take<RowScalars>(1);
-  if (bf) {
-    // one region for both pool sizes, as large as any smaller batch needs it (a batch of fewer row
-    // blocks is cut into more splits): a workspace sized for a batch serves every smaller one
-    size_t end = 0;
-    for (int64_t rows = std::min<int64_t>(b, 128);; rows = std::min<int64_t>(b, rows + 128)) {
-      Carve c1 = c, c2 = c;
-      t.parts = carve_parts(c1, (int)rows, (int)ng, d, elt_of(p), r.kp, false);
-      t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, elt_of(p), serve_kp_final(p), false);
-      end = std::max(end, std::max(c1.off, c2.off));
-      if (rows == b) break;
-    }
-    c.off = end;
-  } else {
-    t.parts.v = c.take<float>((size_t)kServeMaxSplits * nb * kpmax);
-    t.parts.i = c.take<int>((size_t)kServeMaxSplits * nb * kpmax);
-    t.parts_final = t.parts;
+  // one region for both pool sizes, as large as any smaller batch needs it (a batch of fewer row
+  // blocks is cut into more splits): a workspace sized for a batch serves every smaller one
+  size_t end = 0;
+  for (int64_t rows = std::min<int64_t>(b, 128);; rows = std::min<int64_t>(b, rows + 128)) {
+    Carve c1 = c, c2 = c;
+    t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, r.kp, false);
+    t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, p, serve_kp_final(p), false);
+    end = std::max(end, std::max(c1.off, c2.off));
+    if (rows == b) break;
   }
+  c.off = end;
   t.pool_v = c.take<float>(nb * kpmax);
   t.pool_i = c.take<int>(nb * kpmax);
   t.unc_count = c.take<int>(4);
@@ -764,7 +750,6 @@ int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp,
   const bool bf = tensor_mode(p);
   const Elt elt = elt_of(p);
   const float* G = gs.G;
-  const int rblocks = (b + 127) / 128;
   {
     StageScope sc_(GCR_STAGE_PREP, st, bf ? 2 : 2);
     GCR_CUDA_TRY(launch_row_stats(xq, b, d, w.n64, w.n32, bf ? w.qr : nullptr, elt, w.enrm, w.anrm, w.sc, st));
@@ -790,10 +775,7 @@ int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp,
       GCR_CUDA_TRY(launch_umma_pool(w.qr, b, gs.Gr, ng, d, elt, nullptr, false, 0, kp, parts, w.pool_v, w.pool_i, st,
                                     seeded ? w.seed : nullptr));
     } else {
-      const int ntiles = (ng + 127) / 128;
-      const int used = split_count(std::max(1, std::min(kServeMaxSplits, (152 + rblocks - 1) / rblocks)), ntiles);
-      GCR_CUDA_TRY(launch_sgemm_pool(xq, b, G, ng, d, nullptr, kp, false, 0, used, parts.v, parts.i, st));
-      GCR_CUDA_TRY(launch_merge_splits(parts.v, parts.i, used, 1, b, kp, w.pool_v, w.pool_i, st));
+      GCR_CUDA_TRY(launch_sgemm_pool(xq, b, G, ng, d, nullptr, kp, false, 0, parts, w.pool_v, w.pool_i, st));
     }
   }
   RefineArgs ra;

@@ -35,11 +35,29 @@ cudaError_t launch_row_stats(const float* X, int n, int d, double* n64, float* n
                              cudaStream_t st);
 cudaError_t launch_split3(const float* X, int n, int d, int gallery_order, __nv_bfloat16* out, cudaStream_t st);
 
+// How a pool sweep is cut: the column splits of each 128-row block (tps column tiles each, in
+// the grid's order), whether clusters share the column tiles, and the buffers its splits leave.
+struct PoolPlan {
+  bool sel;          // selection buffers of cap slots (else sorted lists of cap = kp entries)
+  int cap, splits, tps;
+  bool deep;         // the four-stage variant of the 32-entry pools
+  bool split_first, cluster;
+};
+PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross);  // umma.cu
+size_t pool_part_entries(const PoolPlan& p, int na, bool cross);
+struct PoolParts {   // scratch of one sweep
+  float* v;          // pool_part_entries
+  int* i;
+  int* cnt;          // splits * kinds * na
+  uint32_t* tau;     // kinds * na
+};
+
 // ---- sgemm.cu
-size_t sgemm_pool_smem();
-// Pools of S = A . B^T rows: [split][kind][na][kp]; self_excl skips j == i (A == B).
+PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross);
+// As launch_umma_pool (below) on the CUDA cores; no seeds.
 cudaError_t launch_sgemm_pool(const float* A, int na, const float* B, int nb, int d, const int* cam, int kp,
-                              bool cross, int self_excl, int splits, float* pool_v, int* pool_i, cudaStream_t st);
+                              bool cross, int self_excl, const PoolParts& parts, float* pool_v, int* pool_i,
+                              cudaStream_t st);
 // Threshold rescan: rows X[band_row[u]] against all rows of Bm (n of them).
 cudaError_t launch_sgemm_band(const float* X, const float* Bm, int n, int d, const int* cam, int self_excl,
                               const int* count, int cap, const int* band_row, const int* band_kind,
@@ -49,22 +67,6 @@ cudaError_t launch_sgemm_dist(const float* Xq, int nq, const float* Xg, int ng, 
                               const float* nrm_q, const float* nrm_g, float* D, cudaStream_t st);
 
 // ---- umma.cu (tcgen05 path; operands BF16 or TF32)
-// How a pool sweep is cut: the column splits of each 128-row block (tps column tiles each, in
-// the grid's order), whether clusters share the column tiles, and the buffers its splits leave.
-struct PoolPlan {
-  bool sel;          // selection buffers of cap slots (else sorted lists of cap = kp entries)
-  int cap, splits, tps;
-  bool deep;         // the four-stage variant of the 32-entry pools
-  bool split_first, cluster;
-};
-PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross);
-size_t pool_part_entries(const PoolPlan& p, int na, bool cross);
-struct PoolParts {   // scratch of one sweep
-  float* v;          // pool_part_entries
-  int* i;
-  int* cnt;          // splits * kinds * na
-  uint32_t* tau;     // kinds * na
-};
 // Pools [kind][na][kp] of the rows of S = A . B^T, kp = 32, 64 or 128, sorted best first and
 // padded with (-inf, -1): every score left out of a full pool is <= its last entry.
 // seed (may be NULL): per row of A an admission floor; every split keeps only scores above it,

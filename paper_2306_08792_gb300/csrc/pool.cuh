@@ -150,7 +150,7 @@ __device__ __forceinline__ void pool_flush(int lane, bool valid, PoolOwner& me, 
 // The pools of the tensor-core sweep (POOL mode of umma.cu). A row's candidates sit unsorted in
 // a buffer of CAP > KP slots in shared memory, owned by one lane: every score above the row's
 // threshold is appended, and when any lane of the warp runs short of room all its lanes compact
-// their buffers at once: a bisection over the buffered scores finds a value f with at least KP of
+// their buffers at once: a search over the buffered scores finds a value f with at least KP of
 // them above it, the others are dropped and f becomes the threshold. KP of the row's scores lie
 // above f, so nothing dropped at or below it can be among the row's KP best; after the sweep the
 // buffer holds all of them (and up to CAP - KP more), and pool_finish sorts and cuts it.
@@ -283,7 +283,8 @@ struct SelScores<CAP, false> {
 // with their mean above the old threshold; the next ones are the mean of the scores still in
 // question, which splits them whatever their spread (a midpoint takes many more steps when a
 // few scores lie far above the rest). Five or six passes settle most warps.
-template <int KP, int CAP>
+// SUM: st.sum is given; else it is taken from the buffer.
+template <int KP, int CAP, bool SUM = true>
 __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState st) {
   constexpr int kSlack = (CAP - KP) / 4, W = (CAP + 31) / 32;
   constexpr float kTarget = KP + 0.5f * kSlack;
@@ -296,6 +297,10 @@ __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState 
   // (cb < KP); ta, tb are the sums of those
   float a = st.lo, ta = st.sum, tb = 0.f;
   int ca = cnt, cb = 0;
+  if constexpr (!SUM) {
+    int c;
+    sc.count(-CUDART_INF_F, c, ta);
+  }
   bool more = act;
   for (int it = 0; it < 12 && __any_sync(GCR_FULL, more); ++it) {
     float p = (ta - tb) / (float)max(1, ca - cb);
@@ -321,7 +326,7 @@ __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState 
   float f = a;
   uint32_t keep[W];
   sc.above(act ? f : -CUDART_INF_F, keep);
-  float lo = st.lo, sum = act ? ta : st.sum;
+  float lo = st.lo, sum = act ? ta : st.sum;  // (a lane that keeps all keeps its sum)
   int kept = act ? ca : cnt;
   if (act) lo = f;
   // Scores too close together for the pivots (ties, or infinities): the KP-th largest exactly,

@@ -1,18 +1,20 @@
 // FP32 similarity GEMM on CUDA cores (the plain FP32 reference path of the kNN search).
 //
 // s_ij = x_i . x_j (Sec. III-B: on unit rows ||x_i - x_j||^2 = 2 - 2 s_ij, so the k nearest
-// samples are the k largest scores) computed in 128 x 128 tiles, 256 threads, 8 x 8
+// samples are the k largest scores) computed in 128 x 128 tiles, 128 threads, 8 x 16
 // outputs per thread, each output a plain sequential FMA chain over d. That fixes the
 // error bound used by the certified refinement: |s^ - s| <= gamma_d * ||x_i|| ||x_j||,
 // gamma_d = d u / (1 - d u), u = 2^-24.
 //
 // Three epilogues share the tile loop:
-//   POOL  one CTA owns 128 rows and sweeps every column tile; the tile goes through
-//         shared memory into the streaming per-row pool (global graph: threads 0-127,
-//         cross-camera graph: threads 128-255).
+//   POOL  a CTA owns 128 rows and sweeps the column tiles of its split; the scores above a row's
+//         threshold go from the accumulators into the row's selection buffer (pool.cuh).
 //   BAND  one CTA owns a column tile and loops over blocks of gathered rows; every score
 //         at or above the row's threshold is appended to that row's band buffer.
 //   DIST  one CTA per (row tile, column tile): writes ||x_q||^2 + ||x_g||^2 - 2 s_qg.
+#include <algorithm>
+#include <cmath>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "pool.cuh"
@@ -24,76 +26,165 @@ using namespace simt;
 
 // ---------------------------------------------------------------------------------- POOL
 // S = A . B^T; rows of A own pools, columns are the rows of B. grid = (ceil(na / 128), splits):
-// split y sweeps column tiles [y * tps, (y + 1) * tps). Pools: [split][kind][na][KP].
-// With self_excl (A == B) the diagonal is skipped; the cross-camera graph needs A == B.
-template <int KP, bool CROSS>
-__global__ void __launch_bounds__(256, 1)
-sgemm_pool_kernel(const float* __restrict__ A, int na, const float* __restrict__ B, int nb, int d,
-                  const int* __restrict__ cam, int self_excl, int tps, float* __restrict__ pool_v,
-                  int* __restrict__ pool_i) {
-  __shared__ TileSmem sm;
-  extern __shared__ __align__(16) unsigned char dyn[];
-  float (*S)[SP] = reinterpret_cast<float (*)[SP]>(dyn);
-  float2* q = reinterpret_cast<float2*>(dyn + sizeof(float) * BM * SP);
-  __shared__ int cam_tile[BN];
+// split y sweeps column tiles [y * tps, (y + 1) * tps). GLOBAL / CROSS: which graphs' pools it
+// keeps; buffers [split][kind][na][cap], kind0 the first of its kinds among them. With self_excl
+// (A == B) the diagonal is skipped; the cross-camera graph needs A == B.
+//
+// Every thread tests its 128 scores of a tile against the rows' thresholds in shared memory and
+// appends those above (a slot by atomicAdd); few pass once the thresholds have risen. Then the
+// rows' owners (a lane per row and graph) compact the buffers that are nearly full. Scores that
+// found a buffer full are tested again after that, so a round always makes room or progress: a
+// compaction leaves at least three quarters of CAP - KP slots free. Two CTAs per SM (but for the
+// largest pools), so that one's epilogue runs beside the other's FMAs; the earlier kernel kept
+// one CTA per SM, one per 128 rows, and passed every score through shared memory to one thread per
+// row: 13,290 rows of d = 2048 32.2 -> 14.7 ms, 2,500 rows of d = 256 1.40 -> 0.23 ms.
+template <int KP, bool GLOBAL, bool CROSS>
+struct SimtPool {
+  static constexpr int kinds = (GLOBAL ? 1 : 0) + (CROSS ? 1 : 0);
+  static constexpr int cap = SelCap<KP, kinds == 2>::cap;
+  static constexpr size_t buf = (size_t)kinds * cap * BM * (sizeof(float) + sizeof(uint16_t));
+  static constexpr size_t smem = sizeof(TileSmem) + buf + sizeof(int) * BM * (3 * kinds + 2);
+  static constexpr int ctas = 2 * (smem + 1024) <= 228 * 1024 ? 2 : 1;
+};
 
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int ty = tid >> 4, tx = tid & 15;
+template <int KP, bool GLOBAL, bool CROSS>
+__global__ void __launch_bounds__(NT, SimtPool<KP, GLOBAL, CROSS>::ctas)
+sgemm_pool_kernel(const float* __restrict__ A, int na, const float* __restrict__ B, int nb, int d,
+                  const int* __restrict__ cam, int self_excl, int tps, int kinds_total, int kind0,
+                  float* __restrict__ part_v, int* __restrict__ part_i, int* __restrict__ part_cnt,
+                  uint32_t* __restrict__ tau_x) {
+  using P = SimtPool<KP, GLOBAL, CROSS>;
+  constexpr int KINDS = P::kinds, CAP = P::cap;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  TileSmem& sm = *reinterpret_cast<TileSmem*>(dyn);
+  unsigned char* buf = dyn + sizeof(TileSmem);   // scores [kind][slot][row], then column offsets
+  int* cnt_s = reinterpret_cast<int*>(buf + P::buf);          // [kind][row]
+  float* tau_s = reinterpret_cast<float*>(cnt_s + KINDS * BM);  // [kind][row]
+  int* camr_s = reinterpret_cast<int*>(tau_s + KINDS * BM);     // [row], [column]
+  int* camc_s = camr_s + BM;
+
+  const int tid = threadIdx.x;
   const int row0 = blockIdx.x * BM;
-  const int kind = tid >> 7;          // 0: global graph, 1: cross-camera graph
-  const int r = tid & 127;            // CTA-local row owned by this thread
-  const int row = row0 + r;
-  const bool valid = row < na && (kind == 0 || CROSS);
-  const int my_cam = (CROSS && row < na) ? cam[row] : 0;
-  PoolOwner me;
-  pool_init(me, valid);
-  const int qrow = kind * BM + r;     // queue row of this owner
-  const int sw = qrow & 31;
-  float2* my_q = q + qrow * kQCap;
-  const int kinds = CROSS ? 2 : 1;
-  const size_t pbase = ((size_t)blockIdx.y * kinds + kind) * na * KP;
-  float* pv = pool_v + pbase;
-  int* pi = pool_i + pbase;
-  const int warp_row0 = row0 + (r & ~31);
-  const int warp_qrow0 = qrow & ~31;
   const int arows = min(BM, na - row0);
   const int ntiles = (nb + BN - 1) / BN;
   const int t0 = blockIdx.y * tps, t1 = min(ntiles, t0 + tps);
+  const uint32_t bv = static_cast<uint32_t>(__cvta_generic_to_shared(buf));
+  const uint32_t bi = bv + (uint32_t)(KINDS * CAP * BM * sizeof(float));
+  // thread r owns row r, of every graph
+  const bool valid = tid < arows;
+  float tau[KINDS], lo[KINDS], pub[KINDS];
+#pragma unroll
+  for (int q = 0; q < KINDS; ++q) {
+    tau[q] = valid ? -CUDART_INF_F : CUDART_INF_F;
+    lo[q] = pub[q] = -CUDART_INF_F;
+    cnt_s[q * BM + tid] = 0;
+    tau_s[q * BM + tid] = tau[q];
+  }
+  if (CROSS) camr_s[tid] = tid < arows ? cam[row0 + tid] : -1;
 
-  float acc[8][8];
+  float acc[TM][TN];
   for (int t = t0; t < t1; ++t) {
     const int col0 = t * BN;
     const int brows = min(BN, nb - col0);
+#pragma unroll
+    for (int q = 0; q < KINDS; ++q) {
+      const uint32_t x = (valid && tau_x) ? __ldcg(tau_x + (size_t)(kind0 + q) * na + row0 + tid) : 0u;
+      if (x) tau_s[q * BM + tid] = tau[q] = fmaxf(tau[q], ordered_to_float(x));
+    }
+    if (CROSS) camc_s[tid] = tid < brows ? cam[col0 + tid] : -1;
     tile_mma(sm, A + (size_t)row0 * d, arows, nullptr, B + (size_t)col0 * d, brows, d, acc);
-    __syncthreads();  // every thread is past its reads of S (previous tile)
+    // (its barriers also publish the owners' thresholds and counts)
+    if (brows < BN || (self_excl && row0 < col0 + BN && col0 < row0 + BM)) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < 8; ++j) S[acc_row(ty, i)][acc_col(tx, j)] = acc[i][j];
-    if (CROSS && tid < BN) cam_tile[tid] = (col0 + tid < nb) ? cam[col0 + tid] : -1;
-    __syncthreads();
-    if (kind == 0 || CROSS) {
-      for (int c0 = 0; c0 < brows; c0 += 4) {  // queues fill to 28 of 32 before a merge
-        pool_make_room<KP>(4, lane, me, warp_row0, warp_qrow0, q, pv, pi);
+        for (int j = 0; j < TN; ++j) {
+          const int cc = acc_col(tid, j);
+          if (cc >= brows || (self_excl && col0 + cc == row0 + acc_row(tid, i))) acc[i][j] = -CUDART_INF_F;
+        }
+    }
+    const int off0 = (t - t0) * BN;
+    uint32_t done[KINDS][TM];  // per row a bit for each of its columns already appended
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int cc = c0 + c;
-          const int j = col0 + cc;
-          float v = S[r][cc];
-          bool ok = cc < brows && !(self_excl && j == row);
-          if (CROSS && kind == 1) ok = ok && cam_tile[cc] != my_cam;
-          pool_push(me, v, j, ok, my_q, sw);
+    for (int q = 0; q < KINDS; ++q)
+#pragma unroll
+      for (int i = 0; i < TM; ++i) done[q][i] = 0u;
+    for (;;) {
+      bool full = false;
+#pragma unroll
+      for (int q = 0; q < KINDS; ++q) {
+        const bool cross_kind = q == 1 || !GLOBAL;
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          const int r = acc_row(tid, i);
+          const float th = tau_s[q * BM + r];
+          float m = acc[i][0];
+#pragma unroll
+          for (int j = 1; j < TN; ++j) m = fmaxf(m, acc[i][j]);
+          if (m > th) {
+#pragma unroll
+            for (int j = 0; j < TN; ++j) {
+              const int cc = acc_col(tid, j);
+              if (acc[i][j] > th && !((done[q][i] >> j) & 1u) && !(cross_kind && camc_s[cc] == camr_s[r])) {
+                const int pos = atomicAdd(&cnt_s[q * BM + r], 1);
+                if (pos < CAP) {
+                  sel_st(bv + (uint32_t)(((q * CAP + pos) * BM + r) * sizeof(float)),
+                         bi + (uint32_t)(((q * CAP + pos) * BM + r) * sizeof(uint16_t)), acc[i][j], off0 + cc);
+                  done[q][i] |= 1u << j;
+                } else {
+                  full = true;
+                }
+              }
+            }
+          }
         }
       }
+      const int again = __syncthreads_or(full ? 1 : 0);
+#pragma unroll
+      for (int q = 0; q < KINDS; ++q) {
+        int n = min(cnt_s[q * BM + tid], CAP);
+        if (__any_sync(GCR_FULL, n > (again ? KP : CAP - (CAP - KP) / 2))) {
+          const SelState ss = sel_compact<KP, CAP, false>(bv + (uint32_t)((q * CAP * BM + tid) * sizeof(float)),
+                                                          bi + (uint32_t)((q * CAP * BM + tid) * sizeof(uint16_t)),
+                                                          SelState{tau[q], lo[q], pub[q], 0.f, n});
+          n = ss.cnt;
+          lo[q] = ss.lo;
+          // lo, not the threshold kept ties lie at: scores of a tile do not come in column order
+          tau[q] = fmaxf(tau[q], ss.lo);
+          tau_s[q * BM + tid] = tau[q];
+          if (valid && tau_x && ss.pub > pub[q])
+            atomicMax(tau_x + (size_t)(kind0 + q) * na + row0 + tid, float_to_ordered(ss.pub));
+          pub[q] = ss.pub;
+        }
+        cnt_s[q * BM + tid] = n;
+      }
+      if (!again) break;
+      __syncthreads();
     }
   }
-  if (kind == 0 || CROSS) pool_flush<KP>(lane, valid, me, warp_row0, warp_qrow0, q, pv, pi);
+  if (!valid) return;
+  const int c0 = t0 * BN;
+#pragma unroll
+  for (int q = 0; q < KINDS; ++q) {
+    const int cnt = cnt_s[q * BM + tid];
+    const size_t row = ((size_t)blockIdx.y * kinds_total + kind0 + q) * na + row0 + tid;
+    part_cnt[row] = cnt;
+    float4* ov = reinterpret_cast<float4*>(part_v + row * CAP);
+    int4* oi = reinterpret_cast<int4*>(part_i + row * CAP);
+    for (int s = 0; s < cnt; s += 4) {  // (slots past the count: never read)
+      const uint32_t va = bv + (uint32_t)(((q * CAP + s) * BM + tid) * sizeof(float));
+      const uint32_t ia = bi + (uint32_t)(((q * CAP + s) * BM + tid) * sizeof(uint16_t));
+      ov[s >> 2] = make_float4(sel_ldv(va), sel_ldv(va + kSelV), sel_ldv(va + 2 * kSelV), sel_ldv(va + 3 * kSelV));
+      oi[s >> 2] = make_int4(c0 + (int)sel_ldi(ia), c0 + (int)sel_ldi(ia + kSelI), c0 + (int)sel_ldi(ia + 2 * kSelI),
+                             c0 + (int)sel_ldi(ia + 3 * kSelI));
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------------- BAND
 // Rows to rescan: band_row[u] (sample index), band_kind[u], band_thr[u], u < *count.
 // grid.x = ceil(n / 128) column tiles; each CTA loops over the row blocks.
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(NT, 2)
 sgemm_band_kernel(const float* __restrict__ X, const float* __restrict__ Bm, int n, int d,
                   const int* __restrict__ cam, int self_excl,
                   const int* __restrict__ count, int cap, const int* __restrict__ band_row,
@@ -101,17 +192,17 @@ sgemm_band_kernel(const float* __restrict__ X, const float* __restrict__ Bm, int
                   int bcap, int* __restrict__ band_cnt, float* __restrict__ band_v,
                   int* __restrict__ band_i) {
   __shared__ TileSmem sm;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int tid = threadIdx.x;
   const int col0 = blockIdx.x * BN;
   const int brows = min(BN, n - col0);
   const int U = min(*count, cap);
-  float acc[8][8];
+  float acc[TM][TN];
   for (int u0 = 0; u0 < U; u0 += BM) {
     const int arows = min(BM, U - u0);
     tile_mma(sm, X, arows, band_row + u0, Bm + (size_t)col0 * d, brows, d, acc);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int ur = acc_row(ty, i);
+    for (int i = 0; i < TM; ++i) {
+      const int ur = acc_row(tid, i);
       if (ur >= arows) continue;
       const int u = u0 + ur;
       const int row = band_row[u];
@@ -119,8 +210,8 @@ sgemm_band_kernel(const float* __restrict__ X, const float* __restrict__ Bm, int
       const float thr = band_thr[u];
       const int rc = cam ? cam[row] : 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int cc = acc_col(tx, j);
+      for (int j = 0; j < TN; ++j) {
+        const int cc = acc_col(tid, j);
         const int col = col0 + cc;
         if (cc >= brows || (self_excl && col == row) || acc[i][j] < thr) continue;
         if (kind == 1 && cam[col] == rc) continue;
@@ -136,58 +227,113 @@ sgemm_band_kernel(const float* __restrict__ X, const float* __restrict__ Bm, int
 
 // ---------------------------------------------------------------------------------- DIST
 // D[q][g] = nq[q] + ng[g] - 2 s_qg (squared Euclidean distance), grid = (ceil(ng/128), ceil(nq/128)).
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(NT, 2)
 sgemm_dist_kernel(const float* __restrict__ Xq, int nq, const float* __restrict__ Xg, int ng,
                   int d, const float* __restrict__ nrm_q, const float* __restrict__ nrm_g,
                   float* __restrict__ D) {
   __shared__ TileSmem sm;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int tid = threadIdx.x;
   const int q0 = blockIdx.y * BM, g0 = blockIdx.x * BN;
   const int arows = min(BM, nq - q0), brows = min(BN, ng - g0);
-  float acc[8][8];
+  float acc[TM][TN];
   tile_mma(sm, Xq + (size_t)q0 * d, arows, nullptr, Xg + (size_t)g0 * d, brows, d, acc);
+  // four consecutive columns of a row at a time, as one 16-byte store where the rows allow it
+  const bool wide = (ng & 3) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int qr = acc_row(ty, i);
+  for (int i = 0; i < TM; ++i) {
+    const int qr = acc_row(tid, i);
     if (qr >= arows) continue;
     const float a = nrm_q[q0 + qr];
     float* out = D + (size_t)(q0 + qr) * ng + g0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int gc = acc_col(tx, j);
-      if (gc < brows) out[gc] = a + nrm_g[g0 + gc] - 2.f * acc[i][j];
+    for (int h = 0; h < TN / 4; ++h) {
+      const int gc = acc_col(tid, 4 * h);
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = gc + j < brows ? a + nrm_g[g0 + gc + j] - 2.f * acc[i][4 * h + j] : 0.f;
+      if (wide && gc + 4 <= brows) {
+        *reinterpret_cast<float4*>(out + gc) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (gc + j < brows) out[gc + j] = v[j];
+      }
     }
   }
 }
 
 // ---------------------------------------------------------------------------------- launchers
-size_t sgemm_pool_smem() { return sizeof(float) * BM * SP + 2 * BM * kQCap * (sizeof(float) + sizeof(int)); }
+// CTAs of the sweep an SM holds (SimtPool::ctas), by pool size and graphs.
+static int simt_ctas(int kp, bool cross) { return kp == 128 || (kp == 64 && cross) ? 1 : 2; }
+
+// As pool_plan: splits whose CTAs fill the SMs evenly. A tile takes about 2 * 128 * 128 * d FMAs
+// at the SM's share; set-up, the first tile's rounds and the write-out about 20 us.
+PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
+  PoolPlan p{};
+  p.sel = true;
+  const bool two = kp == 128 && cross;  // two graphs of 128-entry pools: a sweep for each
+  p.cap = kp == 32 ? (cross ? SelCap<32, true>::cap : SelCap<32, false>::cap)
+          : kp == 64 ? (cross ? SelCap<64, true>::cap : SelCap<64, false>::cap)
+                     : SelCap<128, false>::cap;
+  const int ntiles = (nb + BN - 1) / BN, rblocks = (na + BM - 1) / BM;
+  const int slots = kSMs * simt_ctas(kp, cross && !two);
+  const double tile_us = d * 0.15, around = 20.0 / tile_us;
+  int best = 1;
+  double best_t = 1e300;
+  for (int s = 1; s <= ntiles; ++s) {
+    if (s > 1 && (long)rblocks * (s - 1) > 16 * slots) break;
+    const int tps = (ntiles + s - 1) / s;
+    if ((long)tps * BN > kSelMaxCols) continue;
+    const long ctas = (long)rblocks * ((ntiles + tps - 1) / tps);
+    const double t = std::ceil((double)ctas / slots) * (tps + around);
+    if (t < best_t * 0.97) {
+      best_t = t;
+      best = s;
+    }
+  }
+  while ((long)((ntiles + best - 1) / best) * BN > kSelMaxCols) ++best;
+  p.tps = (ntiles + best - 1) / best;
+  p.splits = (ntiles + p.tps - 1) / p.tps;
+  return p;
+}
+
+namespace {
+template <int KP, bool GLOBAL, bool CROSS>
+cudaError_t launch_simt(const PoolPlan& p, const float* A, int na, const float* B, int nb, int d, const int* cam,
+                        int self_excl, int kinds_total, int kind0, const PoolParts& parts, uint32_t* tau,
+                        cudaStream_t st) {
+  using P = SimtPool<KP, GLOBAL, CROSS>;
+  auto fn = sgemm_pool_kernel<KP, GLOBAL, CROSS>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::smem);
+  if (e != cudaSuccess) return e;
+  fn<<<dim3((na + BM - 1) / BM, p.splits), NT, P::smem, st>>>(A, na, B, nb, d, cam, self_excl, p.tps, kinds_total,
+                                                               kind0, parts.v, parts.i, parts.cnt, tau);
+  return cudaGetLastError();
+}
+}  // namespace
 
 cudaError_t launch_sgemm_pool(const float* A, int na, const float* B, int nb, int d, const int* cam, int kp,
-                              bool cross, int self_excl, int splits, float* pool_v, int* pool_i, cudaStream_t st) {
-  const int ntiles = (nb + BN - 1) / BN;
-  if (splits < 1) splits = 1;
-  if (splits > ntiles) splits = ntiles;
-  const int tps = (ntiles + splits - 1) / splits;
-  splits = (ntiles + tps - 1) / tps;  // no split is left without a column tile
-  dim3 grid((na + BM - 1) / BM, splits);
-  size_t smem = sgemm_pool_smem();
-#define GCR_POOL_CASE(KPV, CR)                                                                   \
-  {                                                                                              \
-    auto fn = sgemm_pool_kernel<KPV, CR>;                                                        \
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-    if (e != cudaSuccess) return e;                                                              \
-    fn<<<grid, 256, smem, st>>>(A, na, B, nb, d, cam, self_excl, tps, pool_v, pool_i);           \
-    return cudaGetLastError();                                                                   \
+                              bool cross, int self_excl, const PoolParts& parts, float* pool_v, int* pool_i,
+                              cudaStream_t st) {
+  const PoolPlan p = simt_pool_plan(na, nb, d, kp, cross);
+  const int kinds = cross ? 2 : 1;
+  uint32_t* tau = nullptr;
+  cudaError_t e = cudaSuccess;
+  if (p.splits > 1) {
+    tau = parts.tau;
+    e = cudaMemsetAsync(tau, 0, sizeof(uint32_t) * kinds * (size_t)na, st);
+    if (e != cudaSuccess) return e;
   }
-  if (kp == 32 && !cross) GCR_POOL_CASE(32, false)
-  if (kp == 32 && cross) GCR_POOL_CASE(32, true)
-  if (kp == 64 && !cross) GCR_POOL_CASE(64, false)
-  if (kp == 64 && cross) GCR_POOL_CASE(64, true)
-  if (kp == 128 && !cross) GCR_POOL_CASE(128, false)
-  if (kp == 128 && cross) GCR_POOL_CASE(128, true)
-#undef GCR_POOL_CASE
-  return cudaErrorInvalidValue;
+#define GCR_SIMT(KPV, G, C, K0) launch_simt<KPV, G, C>(p, A, na, B, nb, d, cam, self_excl, kinds, K0, parts, tau, st)
+  if (kp == 32) e = cross ? GCR_SIMT(32, true, true, 0) : GCR_SIMT(32, true, false, 0);
+  else if (kp == 64) e = cross ? GCR_SIMT(64, true, true, 0) : GCR_SIMT(64, true, false, 0);
+  else if (kp == 128) {
+    e = GCR_SIMT(128, true, false, 0);
+    if (e == cudaSuccess && cross) e = GCR_SIMT(128, false, true, 1);
+  } else return cudaErrorInvalidValue;
+#undef GCR_SIMT
+  if (e != cudaSuccess) return e;
+  return launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, na, p.cap, kp, pool_v, pool_i, st);
 }
 
 cudaError_t launch_sgemm_band(const float* X, const float* Bm, int n, int d, const int* cam, int self_excl,
@@ -195,7 +341,7 @@ cudaError_t launch_sgemm_band(const float* X, const float* Bm, int n, int d, con
                               const float* band_thr, int bcap, int* band_cnt, float* band_v, int* band_i,
                               cudaStream_t st) {
   dim3 grid((n + BN - 1) / BN);
-  sgemm_band_kernel<<<grid, 256, 0, st>>>(X, Bm, n, d, cam, self_excl, count, cap, band_row, band_kind, band_thr,
+  sgemm_band_kernel<<<grid, NT, 0, st>>>(X, Bm, n, d, cam, self_excl, count, cap, band_row, band_kind, band_thr,
                                           bcap, band_cnt, band_v, band_i);
   return cudaGetLastError();
 }
@@ -203,7 +349,7 @@ cudaError_t launch_sgemm_band(const float* X, const float* Bm, int n, int d, con
 cudaError_t launch_sgemm_dist(const float* Xq, int nq, const float* Xg, int ng, int d,
                               const float* nrm_q, const float* nrm_g, float* D, cudaStream_t st) {
   dim3 grid((ng + BN - 1) / BN, (nq + BM - 1) / BM);
-  sgemm_dist_kernel<<<grid, 256, 0, st>>>(Xq, nq, Xg, ng, d, nrm_q, nrm_g, D);
+  sgemm_dist_kernel<<<grid, NT, 0, st>>>(Xq, nq, Xg, ng, d, nrm_q, nrm_g, D);
   return cudaGetLastError();
 }
 

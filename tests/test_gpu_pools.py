@@ -59,3 +59,30 @@ def test_scores_that_rise_or_fall_along_the_columns(sign):
     X[:, 0] += np.cos(th)
     X[:, 1] += np.sin(th)
     _check(X, 20, "tf32")
+
+
+# FP32 sweep: one tile and a column more, ragged splits, 32-, 64- and 128-entry pools of one and
+# two graphs (two graphs of 128 entries take a sweep each), more ties than a buffer holds
+@pytest.mark.parametrize("n,d,k,pool,cams", [
+    (129, 20, 10, 32, 0), (257, 68, 31, 32, 5), (1537, 76, 40, 64, 0), (1537, 76, 40, 64, 4), (1100, 44, 60, 128, 0),
+    (1100, 44, 60, 128, 3), (5000, 260, 15, 0, 0)])
+def test_fp32_pool_sizes_and_splits(n, d, k, pool, cams):
+    X, cam = workloads.random_unit_like(n + d, n, d, cams=max(cams, 1))
+    _check(X, k, "fp32", pool, cam if cams else None)
+
+
+@pytest.mark.parametrize("k,pool", [(12, 32), (30, 64)])
+def test_fp32_equal_scores_go_to_the_smallest_columns(k, pool):
+    """600 copies of one row: no pool can certify its rows, and the ones kept are the exact
+    search's (ties to the smaller index)."""
+    import paper_2306_08792_gb300 as gcr
+    rng = np.random.default_rng(4)
+    X = rng.standard_normal((1500, 48)).astype(np.float32)
+    same = np.sort(rng.choice(np.arange(1, 1500), 600, replace=False))
+    X[same] = X[0]
+    same = np.concatenate([[0], same])
+    X0 = gcr.gcr_normalize(torch.from_numpy(X).cuda())
+    G = gcr.gcr_build_graph(X0, gcr.default_params(k=k, precision="fp32", pool=pool))
+    nbr = np.sort(G.nbr.cpu().numpy()[same], axis=1)
+    for t, i in enumerate(same):
+        assert np.array_equal(nbr[t], same[same != i][:k]), (t, nbr[t])
