@@ -102,12 +102,12 @@ size_t op_capacity(int64_t n, const gcr_params* p, int kinds) {
 
 PoolParts carve_parts(Carve& c, int na, int nb, int d, const gcr_params* p, int kp, bool cross) {
   const PoolPlan pl = tensor_mode(p) ? pool_plan(na, nb, d, elt_of(p), kp, cross) : simt_pool_plan(na, nb, d, kp, cross);
-  const size_t rows = (size_t)(cross ? 2 : 1) * na, entries = pool_part_entries(pl, na, cross);
+  const size_t rows = pool_part_rows(pl, na, cross);
   PoolParts t;
-  t.v = c.take<float>(entries);
-  t.i = c.take<int>(entries);
-  t.cnt = c.take<int>((size_t)pl.splits * rows);
-  t.tau = c.take<uint32_t>(rows);
+  t.v = c.take<float>(rows * pl.cap);
+  t.i = c.take<int>(rows * pl.cap);
+  t.cnt = c.take<int>(rows);
+  t.tau = c.take<uint32_t>((size_t)(cross ? 2 : 1) * na);
   return t;
 }
 
@@ -564,8 +564,6 @@ struct GalleryView {
   float* enrm;     // (T+1) x ng
   float* anrm;     // (T+1) x ng
   RowScalars* sc;  // T+1
-  int32_t* nbr;    // ng x k: the kNN lists of the last layer's graph (T >= 1, k >= 1); candidates
-                   // for the seeds of the final search's split pools
 };
 
 int check_serve_params(const gcr_params* p, int64_t ng, int32_t d, Resolved* r) {
@@ -590,7 +588,6 @@ size_t carve_gallery(Carve& c, int64_t ng, int32_t d, const gcr_params* p, Galle
   t.enrm = bf ? c.take<float>(L * n) : nullptr;
   t.anrm = bf ? c.take<float>(L * n) : nullptr;
   t.sc = c.take<RowScalars>(L);
-  t.nbr = c.take<int32_t>(n * std::max(p->k, 1));
   if (v) *v = t;
   return c.off;
 }
@@ -654,7 +651,6 @@ struct ServeWs {
   int32_t* nbr;
   float* d2;
   unsigned long long* stats;
-  float* seed;         // per query: the admission floor of this search's split pools
 };
 
 int serve_kp_final(const gcr_params* p) {
@@ -709,7 +705,6 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   t.nbr = c.take<int32_t>(nb * std::max(p->k, 1));
   t.d2 = c.take<float>(nb * std::max(p->k, 1));
   t.stats = c.take<unsigned long long>(GCR_STATS_LEN);
-  t.seed = c.take<float>(nb);
   if (w) *w = t;
   return c.off;
 }
@@ -731,22 +726,12 @@ GallerySide gallery_layer(const GalleryView& g, int layer, int ng, int d, size_t
                      g.enrm ? g.enrm + (size_t)layer * ng : nullptr, g.anrm ? g.anrm + (size_t)layer * ng : nullptr};
 }
 
-// Where the seeds of a search's split pools come from: the previous search's merged pool
-// (prev_kp per query, still in the workspace) and optionally the gallery lists hop (hop_k per row).
-// Both searches run on the same query rows (at different layers).
-struct SeedSource {
-  int prev_kp = 0;          // 0: no seed
-  const int32_t* hop = nullptr;
-  int hop_k = 0;
-  int sample = 0;           // evenly spaced gallery rows added to the candidates
-};
-
 // Certified k nearest gallery rows for the b query rows xq: pool, merge, refine, band.
 // ball (may be NULL; tensor-core modes): workspace of the ball search of the rows the pools
 // cannot certify (without it, pools saturated with near-ties keep the 2 delta bound).
 int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp, const PoolParts& parts,
               const GallerySide& gs, int ng, const ServeWs& w, unsigned long long* stats, int32_t* nbr, float* d2, cudaStream_t st,
-              const SeedSource& seed_src = SeedSource(), const BallArgs* ball = nullptr) {
+              const BallArgs* ball = nullptr) {
   const bool bf = tensor_mode(p);
   const Elt elt = elt_of(p);
   const float* G = gs.G;
@@ -756,24 +741,10 @@ int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp,
   }
   GCR_CUDA_TRY(cudaMemsetAsync(w.unc_count, 0, sizeof(int) * 4, st));
   GCR_CUDA_TRY(cudaMemsetAsync(w.band_cnt, 0, sizeof(int) * b, st));
-  // the split pools' admission floors (tensor-core modes), from the previous search's merged
-  // pool, when given its rows' gallery lists, and a sample of the gallery
-  const bool seeded = bf && (seed_src.prev_kp > 0 || seed_src.sample > 0) &&
-                      (long)seed_src.prev_kp * (1 + seed_src.hop_k) + seed_src.sample <= kSeedCandidates;
-  if (seeded) {
-    SeedArgs sa;
-    sa.xq = xq; sa.G = G; sa.b = b; sa.ng = ng; sa.d = d; sa.precision = p->precision;
-    sa.n64q = w.n64; sa.enrm = w.enrm; sa.anrm = w.anrm; sa.gsc = gs.sc;
-    sa.pool_i = seed_src.prev_kp > 0 ? w.pool_i : nullptr; sa.prev_kp = seed_src.prev_kp; sa.hop = seed_src.hop; sa.hop_k = seed_src.hop ? seed_src.hop_k : 0;
-    sa.sample = seed_src.sample; sa.k = k; sa.kp = kp; sa.seed = w.seed;
-    StageScope sc_(GCR_STAGE_PREP, st);
-    GCR_CUDA_TRY(launch_serve_seed(sa, st));
-  }
   {
     StageScope sc_(GCR_STAGE_SIM_GEMM, st, 2);
     if (bf) {
-      GCR_CUDA_TRY(launch_umma_pool(w.qr, b, gs.Gr, ng, d, elt, nullptr, false, 0, kp, parts, w.pool_v, w.pool_i, st,
-                                    seeded ? w.seed : nullptr));
+      GCR_CUDA_TRY(launch_umma_pool(w.qr, b, gs.Gr, ng, d, elt, nullptr, false, 0, kp, parts, w.pool_v, w.pool_i, st));
     } else {
       GCR_CUDA_TRY(launch_sgemm_pool(xq, b, G, ng, d, nullptr, kp, false, 0, parts, w.pool_v, w.pool_i, st));
     }
@@ -789,8 +760,7 @@ int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp,
   ra.unc_count = w.unc_count; ra.unc_row = w.unc_row; ra.unc_kind = w.unc_kind; ra.unc_thr = w.unc_thr;
   ra.stats = stats;
   ra.band_cnt = w.band_cnt; ra.band_v = w.band_v; ra.band_i = w.band_i; ra.bcap = kBandCap; ra.band_rows = b;
-  ra.floor = seeded ? w.seed : nullptr;
-  const bool use_ball = bf && ball != nullptr && !seeded;
+  const bool use_ball = bf && ball != nullptr;
   ra.skip_saturated = use_ball ? 0 : 1;
   ra.unc_dk = w.unc_dk;
   {
@@ -874,7 +844,7 @@ int topk_rerank_impl(const float* Xq, int64_t nq, const float* Xg, int64_t ng, i
   GCR_CUDA_TRY(cudaMemsetAsync(w.sw.stats, 0, sizeof(unsigned long long) * GCR_STATS_LEN, st));
   const GallerySide gs{Xg, w.gr, w.n64g, w.scg, w.genrm, w.ganrm};
   return serve_knn(Xq, (int)nq, d, p, p->topk_out, serve_kp_final(p), w.sw.parts_final, gs, (int)ng, w.sw, w.sw.stats, idx_out,
-                   dist_out, st, SeedSource(), bf ? &w.ball : nullptr);
+                   dist_out, st, bf ? &w.ball : nullptr);
 }
 
 // The whole re-ranking on device buffers (gcr_pipeline); hd (may be NULL) delivers the
@@ -1207,8 +1177,6 @@ int gcr_gallery_build(const float* Xg, int64_t ng, int32_t d, const gcr_params* 
     GCR_CUDA_TRY(launch_propagate(w.g.op_rowptr, w.g.op_len, w.g.op_col, w.g.op_val, cur, nxt, n, d,
                                   p->k > 0 ? w.g.row_order : nullptr, st));
   }
-  if (p->T >= 1 && p->k > 0)
-    GCR_CUDA_TRY(cudaMemcpyAsync(g.nbr, w.g.nbr, sizeof(int32_t) * (size_t)n * p->k, cudaMemcpyDeviceToDevice, st));
   for (int t = 0; t <= p->T; ++t) {
     GCR_CUDA_TRY(launch_row_stats(g.layers + (size_t)t * n * d, n, d, g.n64 + (size_t)t * n, g.n32 + (size_t)t * n,
                                   bf ? g.xr + (size_t)t * n * d * es : nullptr, elt_of(p),
@@ -1249,17 +1217,8 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
   int cur = 0;
   for (int t = 0; t < p->T; ++t) {
     if (p->k > 0) {
-      // every search after the first starts from the previous search's pool; the first one, for
-      // 32 queries or more, from a sample of the gallery (the seed kernel, one latency-bound CTA
-      // per query, costs more than it saves for fewer: measured 1.63 -> 1.76 ms per call at b = 1,
-      // 2.75 -> 2.37 ms at b = 64 on a 500,000 x 256 gallery)
-      SeedSource src;
-      if (t > 0)
-        src.prev_kp = r.kp;
-      else if (nq >= 32)
-        src.sample = (int)std::min<int64_t>(ng, kSeedCandidates);
       s = serve_knn(w.xq[cur], nq, d, p, p->k, r.kp, w.parts, gallery_layer(g, t, n, d, elt_size(p)), n, w, stp, w.nbr, w.d2,
-                    st, src);
+                    st);
       if (s != GCR_OK) return s;
     }
     StageScope sc_(GCR_STAGE_PROPAGATE, st);
@@ -1267,21 +1226,8 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
                                    w.d2, p->k, p->gamma, p->symmetric, w.xq[cur ^ 1], st));
     cur ^= 1;
   }
-  // the final search starts from the last layer search's pool, those rows' gallery lists and,
-  // when it must certify more rows than that pool holds, a sample of the gallery (the lists
-  // mostly lead back into the pool's own clusters)
-  SeedSource src;
-  if (p->T >= 1 && p->k > 0) {
-    src.prev_kp = r.kp;
-    if (r.kp * (1 + p->k) <= kSeedCandidates) {
-      src.hop = g.nbr;
-      src.hop_k = p->k;
-    }
-    if (p->topk_out > r.kp)
-      src.sample = (int)std::min<int64_t>(ng, kSeedCandidates - (int64_t)r.kp * (1 + src.hop_k));
-  }
   return serve_knn(w.xq[cur], nq, d, p, p->topk_out, serve_kp_final(p), w.parts_final, gallery_layer(g, p->T, n, d, elt_size(p)), n, w, stp,
-                   idx_out, dist_out, st, src);
+                   idx_out, dist_out, st);
 }
 
 size_t gcr_pipeline_workspace_size(int64_t n, int64_t nq, int32_t d, const gcr_params* p) {

@@ -42,19 +42,20 @@ struct PoolPlan {
   int cap, splits, tps;
   bool deep;         // the four-stage variant of the 32-entry pools
   bool split_first, cluster;
+  int sample_tiles;  // column tiles of the sample sweep that gives the rows their floors (0: none)
 };
 PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross);  // umma.cu
-size_t pool_part_entries(const PoolPlan& p, int na, bool cross);
+size_t pool_part_rows(const PoolPlan& p, int na, bool cross);
 struct PoolParts {   // scratch of one sweep
-  float* v;          // pool_part_entries
+  float* v;          // pool_part_rows * cap
   int* i;
-  int* cnt;          // splits * kinds * na
+  int* cnt;          // pool_part_rows
   uint32_t* tau;     // kinds * na
 };
 
 // ---- sgemm.cu
 PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross);
-// As launch_umma_pool (below) on the CUDA cores; no seeds.
+// As launch_umma_pool (below) on the CUDA cores.
 cudaError_t launch_sgemm_pool(const float* A, int na, const float* B, int nb, int d, const int* cam, int kp,
                               bool cross, int self_excl, const PoolParts& parts, float* pool_v, int* pool_i,
                               cudaStream_t st);
@@ -69,12 +70,9 @@ cudaError_t launch_sgemm_dist(const float* Xq, int nq, const float* Xg, int ng, 
 // ---- umma.cu (tcgen05 path; operands BF16 or TF32)
 // Pools [kind][na][kp] of the rows of S = A . B^T, kp = 32, 64 or 128, sorted best first and
 // padded with (-inf, -1): every score left out of a full pool is <= its last entry.
-// seed (may be NULL): per row of A an admission floor; every split keeps only scores above it,
-// so a pool may hold fewer than kp entries, and every score left out of it is <= the floor or
-// <= its last entry.
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
                              const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
-                             float* pool_v, int* pool_i, cudaStream_t st, const float* seed = nullptr);
+                             float* pool_v, int* pool_i, cudaStream_t st);
 // Pools of row blocks of the gathered matrix Y (rows x d, rounded operand) against column ranges
 // of Y: work item w = {first row, rows <= 128, first column, columns} of *n_items (<= max_items);
 // pool entry (s - col_bias[j], j), j a position in Y; column j == row skipped when self_excl;
@@ -145,39 +143,12 @@ struct RefineArgs {
   int bcap;
   int band_rows;            // capacity of the band buffers (rows beyond it are not rescanned)
   const int* order;         // processing order of the rows (NULL: 0..n-1); results do not depend on it
-  const float* floor;       // per row (kinds == 1), or NULL: the admission floor the pools were
-                            // searched with (a bound on every score left out of a short pool)
 };
 cudaError_t launch_refine_pool(const RefineArgs& a, cudaStream_t st);
 // Refinement of the grouped pools of the ball search (ball.cu): each queued pair of a searched
 // group is certified in the centred coordinates of its ball (result written, counted in
 // GCR_STAT_BALL) or handed on to the band queue bq_* with its original threshold.
 cudaError_t launch_refine_ball(const RefineArgs& a, const BallArgs& b, cudaStream_t st);
-// Split-pool seeds of the serving search (see refine.cu): for each of the b query rows of xq,
-// an admission floor for its search against the gallery G, from the FP32 scores of the distinct
-// rows of the row's previous pool (prev_kp entries of pool_i), of their hop lists (hop_k per
-// gallery row, when hop != NULL) and of the sample rows floor(i * ng / sample), i < sample:
-// below the approximate score of every candidate among the best min(valid, kp), so that the
-// search keeps at least that many. -inf when fewer than k distinct candidates.
-constexpr int kSeedCandidates = 4096;  // prev_kp * (1 + hop_k) + sample must not exceed this
-struct SeedArgs {
-  const float* xq;          // b x d query rows of this search (FP32)
-  const float* G;           // ng x d gallery rows of this search (FP32)
-  int b, ng, d, precision;
-  const double* n64q;       // ||x_q||^2
-  const float* enrm;        // rounding statistics of the query rows (tensor-core modes)
-  const float* anrm;
-  const RowScalars* gsc;    // maxima over the gallery rows
-  const int* pool_i;        // b x prev_kp (NULL when prev_kp == 0)
-  int prev_kp;
-  const int32_t* hop;       // ng x hop_k, or NULL
-  int hop_k;
-  int sample;               // evenly spaced gallery rows added to the candidates (0..ng)
-  int k;                    // neighbours this search must certify
-  int kp;                   // pool size of this search
-  float* seed;              // b
-};
-cudaError_t launch_serve_seed(const SeedArgs& a, cudaStream_t st);
 cudaError_t launch_refine_band(const RefineArgs& a, cudaStream_t st);
 // Cluster-local row order from the pools (first k candidates): order[0..n) is a permutation.
 cudaError_t launch_row_order(const int* pool_i, int n, int kp, int k, int* key, int* cnt, int* off, int* fill,

@@ -28,23 +28,37 @@ constexpr double kU32rz = 1.1920928955078125e-07; // 2^-23 (truncating accumulat
 
 __device__ __forceinline__ double gamma_n(double h, double u) { return h * u / (1.0 - h * u); }
 
-// ---- warp list of 32*P entries, entry e = p*32 + lane: key sig (desc), index id, value val
+// sigma as a signed 64-bit integer of the same order: the sorts compare integers (FP64 compares
+// run at 1/64 of the FP32 rate on this GPU). sigma is never -0 (a difference from +0 or more).
+__device__ __forceinline__ long long sig_key(double s) {
+  const long long i = __double_as_longlong(s);
+  return i ^ ((i >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double key_sig(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+__device__ __forceinline__ bool better_k(long long a, int ai, long long b, int bi) {
+  return a > b || (a == b && ai < bi);
+}
+constexpr long long kNoKey = (long long)0x800fffffffffffffull;  // sig_key(-inf)
+
+// ---- warp list of 32*P entries, entry e = p*32 + lane: sigma (desc, as a key), index, dot product
 template <int P>
 struct WList {
-  double sig[P];
+  long long key[P];
   int id[P];
-  double val[P];
+  float val[P];
 };
 
 template <int P>
 __device__ __forceinline__ double wl_sig(const WList<P>& L, int e) {
-  double r = 0;
+  long long r = 0;
 #pragma unroll
   for (int p = 0; p < P; ++p) {
-    double t = __shfl_sync(GCR_FULL, L.sig[p], e & 31);
+    const long long t = __shfl_sync(GCR_FULL, L.key[p], e & 31);
     if ((e >> 5) == p) r = t;
   }
-  return r;
+  return key_sig(r);
 }
 template <int P>
 __device__ __forceinline__ int wl_id(const WList<P>& L, int e) {
@@ -57,7 +71,24 @@ __device__ __forceinline__ int wl_id(const WList<P>& L, int e) {
   return r;
 }
 
-// Descending bitonic sort of the whole list by (sig, smaller id first).
+template <int P>
+__device__ __forceinline__ void wl_swap(WList<P>& L, int a, int b) {
+  const long long k = L.key[a]; L.key[a] = L.key[b]; L.key[b] = k;
+  const int i = L.id[a]; L.id[a] = L.id[b]; L.id[b] = i;
+  const float v = L.val[a]; L.val[a] = L.val[b]; L.val[b] = v;
+}
+// The better (worse) of a lane's entry p and its partner's at lane distance stride.
+template <int P>
+__device__ __forceinline__ void wl_exchange(WList<P>& L, int p, int stride, bool keep_better) {
+  const long long ok = __shfl_xor_sync(GCR_FULL, L.key[p], stride);
+  const int oi = __shfl_xor_sync(GCR_FULL, L.id[p], stride);
+  const float ov = __shfl_xor_sync(GCR_FULL, L.val[p], stride);
+  // the ids of two entries differ, or both are empty: "not better" is "worse or the same"
+  const bool take = better_k(ok, oi, L.key[p], L.id[p]) == keep_better;
+  if (take) { L.key[p] = ok; L.id[p] = oi; L.val[p] = ov; }
+}
+
+// Descending bitonic sort of the whole list by (sigma, smaller id first).
 template <int P>
 __device__ __forceinline__ void wl_sort(WList<P>& L, int lane) {
   constexpr int N = 32 * P;
@@ -70,29 +101,17 @@ __device__ __forceinline__ void wl_sort(WList<P>& L, int lane) {
         for (int p = 0; p < P; ++p) {
           const int q2 = p ^ (stride >> 5);
           if (q2 > p) {
-            const int s = p * 32 + lane;
-            const bool desc = (s & size) == 0;
-            const bool sw = desc ? better_d(L.sig[q2], L.id[q2], L.sig[p], L.id[p])
-                                 : better_d(L.sig[p], L.id[p], L.sig[q2], L.id[q2]);
-            if (sw) {
-              double ts = L.sig[p]; L.sig[p] = L.sig[q2]; L.sig[q2] = ts;
-              int ti = L.id[p]; L.id[p] = L.id[q2]; L.id[q2] = ti;
-              double tv = L.val[p]; L.val[p] = L.val[q2]; L.val[q2] = tv;
-            }
+            const bool desc = ((p * 32 + lane) & size) == 0;
+            if (desc ? better_k(L.key[q2], L.id[q2], L.key[p], L.id[p])
+                     : better_k(L.key[p], L.id[p], L.key[q2], L.id[q2]))
+              wl_swap(L, p, q2);
           }
         }
       } else {
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-          double os = __shfl_xor_sync(GCR_FULL, L.sig[p], stride);
-          int oi = __shfl_xor_sync(GCR_FULL, L.id[p], stride);
-          double ov = __shfl_xor_sync(GCR_FULL, L.val[p], stride);
           const int s = p * 32 + lane;
-          const bool desc = (s & size) == 0;
-          const bool lower = (s & stride) == 0;
-          const bool take = (lower == desc) ? better_d(os, oi, L.sig[p], L.id[p])
-                                            : better_d(L.sig[p], L.id[p], os, oi);
-          if (take) { L.sig[p] = os; L.id[p] = oi; L.val[p] = ov; }
+          wl_exchange(L, p, stride, ((s & stride) == 0) == ((s & size) == 0));
         }
       }
     }
@@ -101,50 +120,23 @@ __device__ __forceinline__ void wl_sort(WList<P>& L, int lane) {
 
 // Merge a sorted-descending chunk of 32 (one per lane) into a sorted list of 32P: keeps the top 32P.
 template <int P>
-__device__ __forceinline__ void wl_merge(WList<P>& L, double cs, int ci, double cv, int lane) {
-  double rs = __shfl_sync(GCR_FULL, cs, 31 - lane);
-  int ri = __shfl_sync(GCR_FULL, ci, 31 - lane);
-  double rv = __shfl_sync(GCR_FULL, cv, 31 - lane);
-  if (better_d(rs, ri, L.sig[P - 1], L.id[P - 1])) { L.sig[P - 1] = rs; L.id[P - 1] = ri; L.val[P - 1] = rv; }
+__device__ __forceinline__ void wl_merge(WList<P>& L, const WList<1>& C, int lane) {
+  const long long rk = __shfl_sync(GCR_FULL, C.key[0], 31 - lane);
+  const int ri = __shfl_sync(GCR_FULL, C.id[0], 31 - lane);
+  const float rv = __shfl_sync(GCR_FULL, C.val[0], 31 - lane);
+  if (better_k(rk, ri, L.key[P - 1], L.id[P - 1])) { L.key[P - 1] = rk; L.id[P - 1] = ri; L.val[P - 1] = rv; }
 #pragma unroll
   for (int stride = 16 * P; stride >= 32; stride >>= 1) {
 #pragma unroll
     for (int p = 0; p < P; ++p) {
       const int q2 = p ^ (stride >> 5);
-      if (q2 > p && better_d(L.sig[q2], L.id[q2], L.sig[p], L.id[p])) {
-        double ts = L.sig[p]; L.sig[p] = L.sig[q2]; L.sig[q2] = ts;
-        int ti = L.id[p]; L.id[p] = L.id[q2]; L.id[q2] = ti;
-        double tv = L.val[p]; L.val[p] = L.val[q2]; L.val[q2] = tv;
-      }
+      if (q2 > p && better_k(L.key[q2], L.id[q2], L.key[p], L.id[p])) wl_swap(L, p, q2);
     }
   }
 #pragma unroll
   for (int p = 0; p < P; ++p) {
 #pragma unroll
-    for (int stride = 16; stride > 0; stride >>= 1) {
-      double os = __shfl_xor_sync(GCR_FULL, L.sig[p], stride);
-      int oi = __shfl_xor_sync(GCR_FULL, L.id[p], stride);
-      double ov = __shfl_xor_sync(GCR_FULL, L.val[p], stride);
-      const bool lower = (lane & stride) == 0;
-      const bool take = lower ? better_d(os, oi, L.sig[p], L.id[p]) : better_d(L.sig[p], L.id[p], os, oi);
-      if (take) { L.sig[p] = os; L.id[p] = oi; L.val[p] = ov; }
-    }
-  }
-}
-
-__device__ __forceinline__ void sort32_d(double& s, int& i, double& v, int lane) {
-#pragma unroll
-  for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      double os = __shfl_xor_sync(GCR_FULL, s, stride);
-      int oi = __shfl_xor_sync(GCR_FULL, i, stride);
-      double ov = __shfl_xor_sync(GCR_FULL, v, stride);
-      const bool desc = (lane & size) == 0 || size == 32;
-      const bool lower = (lane & stride) == 0;
-      const bool take = (lower == desc) ? better_d(os, oi, s, i) : better_d(s, i, os, oi);
-      if (take) { s = os; i = oi; v = ov; }
-    }
+    for (int stride = 16; stride > 0; stride >>= 1) wl_exchange(L, p, stride, (lane & stride) == 0);
   }
 }
 
@@ -214,10 +206,13 @@ __device__ __forceinline__ double dot_f64(const float* __restrict__ X, int d, co
   return warp_sum_d(acc);
 }
 
-// Re-scores entries [0, r) of L in FP32 (entry e's index is L.id), setting sig and val.
-template <int VPL, int P>
-__device__ __forceinline__ void rescore(const RefineArgs& a, const float* __restrict__ xi, WList<P>& L, int r, int lane) {
-  for (int e0 = 0; e0 < r; e0 += 4) {
+// Re-scores entries [0, r) of L in FP32 (entry e's index is L.id), setting key and val. With more
+// than one warp on the row (every warp holds the list) each takes every W-th group of four and
+// the results meet in shared memory (sval: 32 P floats).
+template <int VPL, int P, int W = 1>
+__device__ __forceinline__ void rescore(const RefineArgs& a, const float* __restrict__ xi, WList<P>& L, int r, int lane,
+                                        int warp = 0, float* sval = nullptr) {
+  for (int e0 = 4 * warp; e0 < r; e0 += 4 * W) {
     int j[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
@@ -231,13 +226,27 @@ __device__ __forceinline__ void rescore(const RefineArgs& a, const float* __rest
     for (int t = 0; t < 4; ++t) {
       const int e = e0 + t;
       if (e < r) {
+        if constexpr (W > 1) {
+          if (lane == 0) sval[e] = s[t];
+        } else {
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-          if (e == p * 32 + lane) {
-            L.val[p] = (double)s[t];
-            L.sig[p] = (double)s[t] - 0.5 * a.n64B[j[t]];
-          }
+          for (int p = 0; p < P; ++p)
+            if (e == p * 32 + lane) {
+              L.val[p] = s[t];
+              L.key[p] = sig_key((double)s[t] - 0.5 * a.n64B[j[t]]);
+            }
         }
+      }
+    }
+  }
+  if constexpr (W > 1) {
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      const int e = p * 32 + lane;
+      if (e < r) {
+        L.val[p] = sval[e];
+        L.key[p] = sig_key((double)sval[e] - 0.5 * a.n64B[L.id[p]]);
       }
     }
   }
@@ -256,8 +265,12 @@ __device__ void finalize(const RefineArgs& a, const float* __restrict__ xi, WLis
   const double n_i = a.n64[frow];
   int acnt = kk, zcnt = kk;
   int rank[P];
+  double val[P];
 #pragma unroll
-  for (int p = 0; p < P; ++p) rank[p] = 0;
+  for (int p = 0; p < P; ++p) {
+    rank[p] = 0;
+    val[p] = (double)L.val[p];
+  }
   if (r > kk) {
     const double sig_next = wl_sig(L, kk);
     const double sig_k = wl_sig(L, kk - 1);
@@ -266,8 +279,9 @@ __device__ void finalize(const RefineArgs& a, const float* __restrict__ xi, WLis
 #pragma unroll
     for (int p = 0; p < P; ++p) {
       const int e = p * 32 + lane;
-      acnt += __popc(__ballot_sync(GCR_FULL, e < kk && L.sig[p] - eps > sig_next + eps));
-      zcnt += __popc(__ballot_sync(GCR_FULL, e < r && L.sig[p] + eps >= sig_k - eps));
+      const double sig = key_sig(L.key[p]);
+      acnt += __popc(__ballot_sync(GCR_FULL, e < kk && sig - eps > sig_next + eps));
+      zcnt += __popc(__ballot_sync(GCR_FULL, e < r && sig + eps >= sig_k - eps));
     }
     if (acnt < kk) {
       // FP64 for the ambiguous entries [acnt, zcnt)
@@ -280,7 +294,7 @@ __device__ void finalize(const RefineArgs& a, const float* __restrict__ xi, WLis
 #pragma unroll
         for (int p = 0; p < P; ++p) {
           if (e == p * 32 + lane) {
-            L.val[p] = dot;
+            val[p] = dot;
             sig64[p] = dot - 0.5 * a.n64B[j];
           }
         }
@@ -322,7 +336,7 @@ __device__ void finalize(const RefineArgs& a, const float* __restrict__ xi, WLis
     else if (e >= acnt && e < zcnt && acnt < kk && rank[p] < kk - acnt) slot = acnt + rank[p];
     if (slot >= 0) {
       const int j = L.id[p];
-      double dd = n_i + a.n64B[j] - 2.0 * L.val[p];
+      double dd = n_i + a.n64B[j] - 2.0 * val[p];
       onbr[slot] = idmap ? idmap[j] : j;
       od2[slot] = (float)(dd > 0.0 ? dd : 0.0);
     }
@@ -349,12 +363,18 @@ __device__ __forceinline__ void bounds(const RefineArgs& a, int row, int vpl, do
   eps = gamma_n((double)(4 * vpl + 6), kU32) * b_i * sc.bmax * (1.0 + 1e-6);
 }
 
-// One warp per (row, kind).
-template <int VPL, int P>
+// One warp per (row, kind); W = 8: a block of eight warps per (row, kind), for batches too small
+// to fill the GPU with a warp each (the re-scoring of a 100-best list is 25 or more dependent
+// rounds of gathers for one warp): the warps share the re-scoring, warp 0 does the rest. One
+// query's 128-entry pool 147 -> 47 us, 512 queries' 175 -> 85; but 1,600 pools of 32 entries 58 ->
+// 92, so small pools take it only up to four pairs per SM.
+template <int VPL, int P, int W>
 __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
   constexpr int KP = 32 * P;
-  const int lane = threadIdx.x & 31;
-  const long wid = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  __shared__ float sval[W > 1 ? KP : 1];
+  const int lane = threadIdx.x & 31, warp = W > 1 ? threadIdx.x >> 5 : 0;
+  const long wid = W > 1 ? (long)blockIdx.x : (long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const bool lead = lane == 0 && warp == 0;
   if (wid >= (long)a.n * a.kinds) return;
   const int kind = (int)(wid / a.n);
   const int row = a.order ? a.order[wid % a.n] : (int)(wid % a.n);
@@ -367,21 +387,21 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
   for (int p = 0; p < P; ++p) {
     pval[p] = pv[p * 32 + lane];
     L.id[p] = pi[p * 32 + lane];
-    L.sig[p] = -CUDART_INF;
-    L.val[p] = 0.0;
+    L.key[p] = kNoKey;
+    L.val[p] = 0.f;
     mvalid += __popc(__ballot_sync(GCR_FULL, L.id[p] >= 0));
   }
-  if (lane == 0 && a.stats) atomicAdd(&a.stats[GCR_STAT_ROWS], 1ull);
+  if (lead && a.stats) atomicAdd(&a.stats[GCR_STAT_ROWS], 1ull);
   if (mvalid == 0) {
-    for (int s = lane; s < a.k; s += 32) {
+    for (int s = threadIdx.x & (W > 1 ? 255 : 31); s < a.k; s += W > 1 ? 256 : 32) {
       a.nbr[kind][(size_t)row * a.k + s] = -1;
       a.d2[kind][(size_t)row * a.k + s] = CUDART_INF_F;
     }
-    if (lane == 0 && a.stats && a.k > 0) atomicAdd(&a.stats[GCR_STAT_CLAMPED], 1ull);
+    if (lead && a.stats && a.k > 0) atomicAdd(&a.stats[GCR_STAT_CLAMPED], 1ull);
     return;
   }
   const int kk = min(a.k, mvalid);
-  if (kk < a.k && lane == 0 && a.stats) atomicAdd(&a.stats[GCR_STAT_CLAMPED], 1ull);
+  if (kk < a.k && lead && a.stats) atomicAdd(&a.stats[GCR_STAT_CLAMPED], 1ull);
   if (kk == 0) return;
   auto pool_at = [&](int e) {
     float r = 0.f;
@@ -393,11 +413,9 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
     return r;
   };
   const float s_k = pool_at(kk - 1);
-  // bound on every approximate score left out of the pool: its last entry when full, else the
-  // admission floor it was searched with (-inf: nothing was left out)
-  const float fl = a.floor ? a.floor[row] : -CUDART_INF_F;
+  // bound on every approximate score left out of a full pool (nothing is left out of another)
   const bool full = mvalid == KP;
-  const float tau = full ? pool_at(KP - 1) : fl;
+  const float tau = full ? pool_at(KP - 1) : -CUDART_INF_F;
   double delta, eps;
   RowScalars sc;
   bounds<P>(a, row, VPL, delta, eps, sc);
@@ -406,7 +424,8 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
 #pragma unroll
   for (int p = 0; p < P; ++p) r += __popc(__ballot_sync(GCR_FULL, L.id[p] >= 0 && (double)pval[p] >= thr));
   const float* xi = a.X + (size_t)row * a.d;
-  rescore<VPL, P>(a, xi, L, r, lane);
+  rescore<VPL, P, W>(a, xi, L, r, lane, warp, sval);
+  if (W > 1 && warp != 0) return;
   if (lane == 0 && a.stats) atomicAdd(&a.stats[GCR_STAT_RESCORED], (unsigned long long)r);
   wl_sort<P>(L, lane);
   const double sig_k = wl_sig(L, kk - 1);
@@ -414,7 +433,7 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
   // most n_i - 2 (sig_k - eps) (the local scale the ball search groups rows by)
   const float dk = __double2float_ru(fmax(0.0, a.n64[row] - 2.0 * (sig_k - eps)) * (1.0 + 1e-9));
   if (a.dk_all && lane == 0) a.dk_all[(size_t)kind * a.n + row] = dk;
-  if (full || fl > -CUDART_INF_F) {
+  if (full) {
     const bool cert = (sig_k - eps) > ((double)tau + delta - 0.5 * sc.nmin);
     // Saturated pool: the density of the pool's lower half, extrapolated over the band's
     // window below tau (about 2*delta wide), predicts more than 512 band entries, so the
@@ -424,7 +443,7 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
     const float mid = pool_at(KP / 2);
     const double dens = (KP / 2) / fmax((double)mid - (double)tau, 1e-30);
     const double below = fmax(0.0, 2.0 * delta + 0.5 * (sc.nmax - sc.nmin) - ((double)s_k - (double)tau));
-    const bool dense = full && KP + dens * below > 512.0;
+    const bool dense = KP + dens * below > 512.0;
     const bool saturated = a.skip_saturated && dense;
     if (!cert && lane == 0) {
       if (a.stats) atomicAdd(&a.stats[GCR_STAT_UNCERTIFIED], 1ull);
@@ -474,6 +493,76 @@ __device__ __forceinline__ float band_kth(const float* __restrict__ bv, int cnt,
 // rule as the pool refinement), and only they are re-scored. Capped at 85 registers (three
 // blocks per SM): the band's long candidate loops gain more from resident warps than they lose
 // to the few spills (measured 0.98 -> 0.80 ms per step on the cross-camera workload).
+// W = 8: a block of eight warps per pair for small batches (at most kSmallRows rows), which share
+// the re-scoring: the selected entries are listed first, re-scored into shared memory, and merged
+// by warp 0.
+constexpr int kSmallRows = 16 * kSMs;
+
+template <int VPL, int P>
+__global__ void __launch_bounds__(256) refine_band_block_kernel(RefineArgs a) {
+  __shared__ int ids[512];
+  __shared__ float val[512];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int U = *a.unc_count;
+  for (int u = blockIdx.x; u < U; u += gridDim.x) {
+    const int row = a.unc_row[u], kind = a.unc_kind[u];
+    const int cnt = u < a.band_rows ? a.band_cnt[u] : a.bcap + 1;
+    if (cnt > a.bcap || cnt > 512) {
+      if (threadIdx.x == 0 && a.stats) atomicAdd(&a.stats[GCR_STAT_BAND_FAILED], 1ull);
+      continue;
+    }
+    double delta, eps;
+    RowScalars sc;
+    bounds<P>(a, row, VPL, delta, eps, sc);
+    const float* xi = a.X + (size_t)row * a.d;
+    const int* bi = a.band_i + (size_t)u * a.bcap;
+    const float* bv = a.band_v + (size_t)u * a.bcap;
+    const int kb = min(a.k, cnt);
+    const double thr = kb > 0 ? (double)band_kth(bv, cnt, kb, lane) - 2.0 * delta - 0.5 * (sc.nmax - sc.nmin)
+                              : -CUDART_INF;
+    // every warp lists the selected entries in band order (the same values to the same slots)
+    int total = 0;
+    for (int c0 = 0; c0 < cnt; c0 += 32) {
+      const int e = c0 + lane;
+      const bool s = e < cnt && (double)bv[e] >= thr;
+      const unsigned m = __ballot_sync(GCR_FULL, s);
+      if (s) ids[total + __popc(m & ((1u << lane) - 1u))] = bi[e];
+      total += __popc(m);
+    }
+    __syncthreads();
+    for (int e0 = 4 * warp; e0 < total; e0 += 32) {
+      int j[4];
+      float s[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) j[t] = e0 + t < total ? ids[e0 + t] : -1;
+      dot4_f32<VPL>(a.XB, a.d, xi, j, lane, s);
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (lane == 0 && e0 + t < total) val[e0 + t] = s[t];
+    }
+    __syncthreads();
+    if (warp == 0) {
+      WList<P> L;
+#pragma unroll
+      for (int p = 0; p < P; ++p) { L.key[p] = kNoKey; L.id[p] = 0x7fffffff; L.val[p] = 0.f; }
+      for (int e0 = 0; e0 < total; e0 += 32) {
+        const int e = e0 + lane;
+        WList<1> C;
+        C.id[0] = e < total ? ids[e] : 0x7fffffff;
+        C.val[0] = e < total ? val[e] : 0.f;
+        C.key[0] = e < total ? sig_key((double)val[e] - 0.5 * a.n64B[ids[e]]) : kNoKey;
+        wl_sort(C, lane);
+        wl_merge<P>(L, C, lane);
+      }
+      if (lane == 0 && a.stats) atomicAdd(&a.stats[GCR_STAT_RESCORED], (unsigned long long)total);
+      const int r = min(total, 32 * P);
+      const int kk = min(a.k, r);
+      finalize<VPL, P>(a, xi, L, r, kk, eps, row, row, kind, lane);
+    }
+    __syncthreads();
+  }
+}
+
 template <int VPL, int P>
 __global__ void __launch_bounds__(256, 3) refine_band_kernel(RefineArgs a) {
   __shared__ int sel_ids[8][64];
@@ -494,7 +583,7 @@ __global__ void __launch_bounds__(256, 3) refine_band_kernel(RefineArgs a) {
     const float* xi = a.X + (size_t)row * a.d;
     WList<P> L;
 #pragma unroll
-    for (int p = 0; p < P; ++p) { L.sig[p] = -CUDART_INF; L.id[p] = 0x7fffffff; L.val[p] = 0.0; }
+    for (int p = 0; p < P; ++p) { L.key[p] = kNoKey; L.id[p] = 0x7fffffff; L.val[p] = 0.f; }
     const int* bi = a.band_i + (size_t)u * a.bcap;
     const float* bv = a.band_v + (size_t)u * a.bcap;
     const int kb = min(a.k, cnt);
@@ -517,12 +606,12 @@ __global__ void __launch_bounds__(256, 3) refine_band_kernel(RefineArgs a) {
         const int take = min(nsel, 32);
         WList<1> C;
         C.id[0] = lane < take ? sb[lane] : -1;
-        C.sig[0] = -CUDART_INF;
-        C.val[0] = 0.0;
+        C.key[0] = kNoKey;
+        C.val[0] = 0.f;
         rescore<VPL, 1>(a, xi, C, take, lane);
         if (C.id[0] < 0) C.id[0] = 0x7fffffff;
-        sort32_d(C.sig[0], C.id[0], C.val[0], lane);
-        wl_merge<P>(L, C.sig[0], C.id[0], C.val[0], lane);
+        wl_sort(C, lane);
+        wl_merge<P>(L, C, lane);
         total += take;
         const int rem = nsel - take;
         const int v = lane < rem ? sb[take + lane] : 0;
@@ -577,8 +666,8 @@ __device__ void refine_ball_one(const RefineArgs& a, const BallArgs& b, int u, i
   for (int q = 0; q < P; ++q) {
     pval[q] = pv[q * 32 + lane];
     L.id[q] = pi[q * 32 + lane];
-    L.sig[q] = -CUDART_INF;
-    L.val[q] = 0.0;
+    L.key[q] = kNoKey;
+    L.val[q] = 0.f;
     mvalid += __popc(__ballot_sync(GCR_FULL, L.id[q] >= 0));
   }
   const int kk = min(a.k, mvalid);
@@ -665,162 +754,27 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ src, long w16, cons
   }
 }
 
+template <int VPL, int P>
+void launch_pool_w(const RefineArgs& a, long pairs, cudaStream_t st) {
+  if (pairs <= (P == 4 ? kSmallRows : 4 * kSMs)) refine_pool_kernel<VPL, P, 8><<<(unsigned)pairs, 256, 0, st>>>(a);
+  else refine_pool_kernel<VPL, P, 1><<<(unsigned)((pairs + 7) / 8), 256, 0, st>>>(a);
+}
+
 template <int P>
 cudaError_t launch_pool_vpl(const RefineArgs& a, cudaStream_t st) {
-  const long warps = (long)a.n * a.kinds;
-  dim3 grid((unsigned)((warps + 7) / 8));
+  const long pairs = (long)a.n * a.kinds;
   const int vpl = (a.d + 127) / 128;
-  if (vpl <= 1) refine_pool_kernel<1, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 2) refine_pool_kernel<2, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 4) refine_pool_kernel<4, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 8) refine_pool_kernel<8, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 16) refine_pool_kernel<16, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 32) refine_pool_kernel<32, P><<<grid, 256, 0, st>>>(a);
+  if (vpl <= 1) launch_pool_w<1, P>(a, pairs, st);
+  else if (vpl <= 2) launch_pool_w<2, P>(a, pairs, st);
+  else if (vpl <= 4) launch_pool_w<4, P>(a, pairs, st);
+  else if (vpl <= 8) launch_pool_w<8, P>(a, pairs, st);
+  else if (vpl <= 16) launch_pool_w<16, P>(a, pairs, st);
+  else if (vpl <= 32) launch_pool_w<32, P>(a, pairs, st);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
 }  // namespace
-
-// ---------------------------------------------------------------------------- split-pool seeds
-// Serving splits the gallery sweep of a query batch over many CTAs, and each split's pool starts
-// empty: most of the search's time goes to filling those pools. A seed s_q lets every split
-// admit only scores above it. It comes from distinct gallery rows j scored here in FP32 (the
-// rows of the query's previous pool, their gallery kNN lists and, where there is no previous
-// pool or it cannot supply k rows, an evenly spaced sample of the gallery, whose best scores
-// bound the sweep's quantile at about (k - graph candidates) / sample from below): with valid
-// such rows, V =
-// min(valid, kp) and S the V-th best of their scores, each within eps of the exact dot product,
-// and delta the certified bound of the GEMM's approximate scores (the same delta the refinement
-// uses), V rows have an approximate score >= S - eps - delta, so the search keeps at least V
-// entries above s_q = (S - eps - delta - (spread of the gallery's squared norms) / 2, rounded
-// down, one ulp lower). A pool may then hold fewer than kp entries; the refinement takes s_q as
-// the bound on every score left out of it and certifies (or rescans) the row as for a full
-// pool. With fewer than k candidates the seed is -inf and the row is searched unseeded.
-constexpr int kSeedCap = kSeedCandidates;  // candidate slots per query
-
-// Ascending bitonic sort of n (a power of two, <= kSeedCap) values in shared memory; the block's
-// threads share the compare-exchanges. KEY_DESC sorts descending instead.
-template <typename T, bool DESC>
-__device__ void block_bitonic(T* v, int n) {
-  for (int size = 2; size <= n; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int e = threadIdx.x; e < (n >> 1); e += blockDim.x) {
-        const int lo = 2 * e - (e & (stride - 1));
-        const int hi = lo + stride;
-        const bool up = ((lo & size) == 0) != DESC;
-        const T a = v[lo], b = v[hi];
-        if ((a > b) == up) { v[lo] = b; v[hi] = a; }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__global__ void __launch_bounds__(1024) serve_seed_kernel(SeedArgs a) {
-  __shared__ int cand[kSeedCap];
-  __shared__ float score[kSeedCap];
-  __shared__ int s_valid;
-  const int q = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int per = 1 + (a.hop ? a.hop_k : 0);
-  const int total1 = a.prev_kp * per;
-  const int total = total1 + a.sample;
-  int N = 32;
-  while (N < total) N <<= 1;
-  // candidates: the previous pool's rows, each followed by its hop list, then the evenly spaced
-  // sample rows floor(i * ng / sample) (absent entries: INT_MAX)
-  for (int e = t; e < N; e += blockDim.x) {
-    int j = -1;
-    if (e < total1) {
-      const int p = e / per, h = e % per;
-      const int j0 = a.pool_i[(size_t)q * a.prev_kp + p];
-      j = h == 0 ? j0 : (j0 >= 0 && j0 < a.ng ? a.hop[(size_t)j0 * a.hop_k + h - 1] : -1);
-    } else if (e < total) {
-      j = (int)((long)(e - total1) * a.ng / a.sample);
-    }
-    cand[e] = (j >= 0 && j < a.ng) ? j : INT_MAX;
-  }
-  if (t == 0) s_valid = 0;
-  __syncthreads();
-  block_bitonic<int, false>(cand, N);
-  // FP32 score of each distinct candidate (duplicates and absent slots: -inf); each warp takes
-  // four candidates at a time (their row loads in flight together), each lane a sequential chain
-  // over its slice, then the butterfly
-  const int vpl = (a.d + 127) / 128;
-  const float* x = a.xq + (size_t)q * a.d;
-  int nv = 0;
-  for (int e0 = warp * 4; e0 < N; e0 += (blockDim.x >> 5) * 4) {
-    int j[4];
-    bool ok[4];
-    float acc[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int e = e0 + c;
-      j[c] = cand[e];
-      ok[c] = j[c] != INT_MAX && (e == 0 || cand[e - 1] != j[c]);
-      acc[c] = 0.f;
-    }
-    for (int v = 0; v < vpl; ++v) {
-      const int off = v * 128 + lane * 4;
-      if (off < a.d) {
-        const float4 xv = *reinterpret_cast<const float4*>(x + off);
-        float4 gv[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          gv[c] = ok[c] ? *reinterpret_cast<const float4*>(a.G + (size_t)j[c] * a.d + off) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          acc[c] = fmaf(xv.x, gv[c].x, acc[c]);
-          acc[c] = fmaf(xv.y, gv[c].y, acc[c]);
-          acc[c] = fmaf(xv.z, gv[c].z, acc[c]);
-          acc[c] = fmaf(xv.w, gv[c].w, acc[c]);
-        }
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      acc[c] = warp_sum(acc[c]);
-      nv += ok[c] ? 1 : 0;
-      if (lane == 0) score[e0 + c] = ok[c] ? acc[c] : -CUDART_INF_F;
-    }
-  }
-  if (lane == 0 && nv) atomicAdd(&s_valid, nv);
-  __syncthreads();
-  const int valid = s_valid;
-  block_bitonic<float, true>(score, N);
-  if (t != 0) return;
-  if (valid < a.k || a.k < 1) {
-    a.seed[q] = -CUDART_INF_F;
-    return;
-  }
-  RowScalars sc = *a.gsc;
-  const double bmax = sqrt(sc.nmax) * (1.0 + 1e-12);
-  const double b_i = sqrt(a.n64q[q]);
-  double delta;
-  if (a.precision == GCR_PREC_FP32) {
-    delta = gamma_n((double)a.d, kU32) * b_i * bmax;
-  } else {
-    const double ai = a.anrm[q], ei = a.enrm[q];
-    delta = ai * sc.emax + ei * bmax + gamma_n((double)a.d + 32.0, kU32rz) * ai * sc.amax;
-  }
-  delta *= 1.0 + 1e-6;
-  const double eps = gamma_n((double)(4 * vpl + 6), kU32) * b_i * bmax * (1.0 + 1e-6);
-  // below the approximate score of each of the best V candidates (their exact scores are within
-  // eps of these, their approximate ones within delta of the exact), with the spread of the
-  // gallery's squared norms as slack for ranking by distance rather than by score
-  const int V = valid < a.kp ? valid : a.kp;
-  const double th = (double)score[V - 1] - eps - delta - 0.5 * (sc.nmax - sc.nmin);
-  a.seed[q] = nextafterf(__double2float_rd(th), -CUDART_INF_F);
-}
-
-cudaError_t launch_serve_seed(const SeedArgs& a, cudaStream_t st) {
-  const long total = (long)a.prev_kp * (1 + (a.hop ? a.hop_k : 0)) + a.sample;
-  if (total > kSeedCap || total < 1 || a.prev_kp < 0 || (a.prev_kp > 0 && !a.pool_i) || a.kp < 1 || a.k < 1 ||
-      a.k > a.kp || a.b < 1 || a.sample < 0 || a.sample > a.ng)
-    return cudaErrorInvalidValue;
-  serve_seed_kernel<<<a.b, 1024, 0, st>>>(a);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_refine_pool(const RefineArgs& a, cudaStream_t st) {
   if (a.kp == 32) return launch_pool_vpl<1>(a, st);
@@ -829,16 +783,23 @@ cudaError_t launch_refine_pool(const RefineArgs& a, cudaStream_t st) {
   return cudaErrorInvalidValue;
 }
 
+template <int VPL, int P>
+void launch_band_w(const RefineArgs& a, cudaStream_t st) {
+  if (a.band_rows <= kSmallRows)
+    refine_band_block_kernel<VPL, P><<<std::min(a.band_rows, kSMs * 4), 256, 0, st>>>(a);
+  else
+    refine_band_kernel<VPL, P><<<kSMs * 4, 256, 0, st>>>(a);
+}
+
 template <int P>
 cudaError_t launch_band_p(const RefineArgs& a, cudaStream_t st) {
-  dim3 grid(152 * 4);
   const int vpl = (a.d + 127) / 128;
-  if (vpl <= 1) refine_band_kernel<1, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 2) refine_band_kernel<2, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 4) refine_band_kernel<4, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 8) refine_band_kernel<8, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 16) refine_band_kernel<16, P><<<grid, 256, 0, st>>>(a);
-  else if (vpl <= 32) refine_band_kernel<32, P><<<grid, 256, 0, st>>>(a);
+  if (vpl <= 1) launch_band_w<1, P>(a, st);
+  else if (vpl <= 2) launch_band_w<2, P>(a, st);
+  else if (vpl <= 4) launch_band_w<4, P>(a, st);
+  else if (vpl <= 8) launch_band_w<8, P>(a, st);
+  else if (vpl <= 16) launch_band_w<16, P>(a, st);
+  else if (vpl <= 32) launch_band_w<32, P>(a, st);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

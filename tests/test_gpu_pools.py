@@ -86,3 +86,22 @@ def test_fp32_equal_scores_go_to_the_smallest_columns(k, pool):
     nbr = np.sort(G.nbr.cpu().numpy()[same], axis=1)
     for t, i in enumerate(same):
         assert np.array_equal(nbr[t], same[same != i][:k]), (t, nbr[t])
+
+
+@pytest.mark.parametrize("K,d", [(20, 64), (20, 520), (60, 64), (100, 64)])
+def test_sampled_floors_of_a_wide_search(K, d):
+    """300 queries against 60,001 rows: few row blocks and long splits, so a sample sweep gives the
+    rows their floors (32- (both rings), 64- and 128-entry pools). A block of near-copies of some
+    queries sits where the evenly spaced sample steps over it."""
+    import paper_2306_08792_gb300 as gcr
+    g = torch.Generator(device="cuda").manual_seed(K + d)
+    G = torch.randn(60001, d, generator=g, device="cuda")
+    Q = torch.randn(300, d, generator=g, device="cuda")
+    G[1:59000:59][:200] = Q[:200] + 0.1 * torch.randn(200, d, generator=g, device="cuda")
+    G, Q = gcr.gcr_normalize(G), gcr.gcr_normalize(Q)
+    idx, dist = gcr.gcr_rerank(Q, G, gcr.default_params(precision="tf32", topk_out=K))
+    ref = torch.cdist(Q.double(), G.double()).square()
+    v, o = torch.topk(ref, K + 1, dim=1, largest=False)
+    assert torch.allclose(dist.double(), v[:, :K], atol=2e-6, rtol=0)
+    clear = v[:, K] - v[:, K - 1] > 1e-9
+    assert torch.equal(idx[clear].long().sort(1)[0], o[clear, :K].sort(1)[0])
