@@ -135,10 +135,10 @@ typedef struct {
   int32_t* op_col;    /* [op_capacity]                                              */
   float*   op_val;    /* [op_capacity]                                              */
   int64_t* stats;     /* [GCR_STATS_LEN] device counters (may be NULL)              */
-  int32_t* row_order; /* [n] optional (may be NULL): filled by gcr_build_graph with a
-                         cluster-local order of the rows (rows sharing their nearest
-                         candidates end up adjacent), used by gcr_propagate to walk the
-                         rows in that order. Results do not depend on it.             */
+  int32_t* row_order; /* [n] optional (may be NULL): filled by gcr_build_graph with an order of
+                         the rows, used by gcr_propagate to walk them (cluster-local, rows
+                         sharing their nearest candidates adjacent, where the features do not
+                         fit in half of L2). Results do not depend on it.             */
 } gcr_graph;
 
 /* ------------------------------------------------------------------ utilities */
@@ -174,11 +174,11 @@ int gcr_normalize(const float* X_in, float* X_out, int64_t n, int32_t d, gcr_str
  * exact: every candidate whose score lies within the certified error bound of the
  * k-th is re-scored in FP32 and, where FP32 cannot separate two candidates, in FP64;
  * exact FP64 ties go to the smaller index.
- * Part of the work (the cross-camera graph's transpose, the propagation's row order) runs
- * on helper streams that the call forks from `stream` and joins back into it by events
- * (one set per device, created on the first such call and kept): `stream` still orders
- * the whole call, and once a first call on the device has created them, later calls can
- * be captured in a CUDA graph (the fork and join become graph dependencies).
+ * For rows that do not fit in half of L2, the propagation's row order is computed on a helper
+ * stream that the call forks from `stream` and joins back into it by events (one set per
+ * device, created on the first such call and kept): `stream` still orders the whole call, and
+ * once a first call on the device has created them, later calls can be captured in a CUDA graph
+ * (the fork and join become graph dependencies).
  * cam: device int32[n], required when cross_camera = 1, else may be NULL.
  * Errors: GCR_E_INVALID (n < 1, k out of range, gamma <= 0, alpha outside [0,1],
  * pool <= k, missing arrays), GCR_E_UNSUPPORTED (d % 4, d % 8 with BF16 or TF32,

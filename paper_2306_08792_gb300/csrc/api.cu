@@ -44,6 +44,9 @@ struct StageScope {
 
 constexpr int kBandCap = 512;        // band entries kept per rescanned (row, graph)
 
+// Whether a feature matrix fits in half of L2: its rows need no processing order then.
+bool in_l2(int64_t n, int32_t d) { return (double)n * d * sizeof(float) <= 0.5 * kL2Bytes; }
+
 struct Resolved {
   int kp;
   int kinds;
@@ -132,7 +135,6 @@ struct BuildWs {
   int* bq_kind;
   float* bq_thr;
   int* bq_flag;
-  int* bq_pos;
   int* band_cnt;
   float* band_v;
   int* band_i;
@@ -150,7 +152,8 @@ struct BuildWs {
   double* inv;
   int* long_list;
   int* long_count;
-  int* scan_tmp2;      // the second graph's transpose scratch (built on a second stream)
+  size_t zero_n;
+  int* scan_tmp2;      // the second graph's transpose scratch
   int* long_list2;
   unsigned long long* stats;
   int* err;
@@ -180,7 +183,9 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.pool_v = c.take<float>((size_t)kinds * nn * r.kp);
   t.pool_i = c.take<int>((size_t)kinds * nn * r.kp);
   t.parts = carve_parts(c, (int)n, (int)n, d, p, r.kp, kinds == 2);
-  t.unc_count = c.take<int>(4);
+  t.unc_count = c.take<int>(8 + (size_t)band_rows);
+  t.err = t.unc_count + 4;
+  t.band_cnt = t.unc_count + 8;
   t.unc_row = c.take<int>((size_t)kinds * nn);
   t.unc_kind = c.take<int>((size_t)kinds * nn);
   t.unc_thr = c.take<float>((size_t)kinds * nn);
@@ -191,8 +196,6 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.bq_kind = c.take<int>((size_t)kinds * nn);
   t.bq_thr = c.take<float>((size_t)kinds * nn);
   t.bq_flag = c.take<int>((size_t)kinds * nn);
-  t.bq_pos = c.take<int>((size_t)kinds * nn + 1);
-  t.band_cnt = c.take<int>(band_rows);
   t.band_v = c.take<float>((size_t)band_rows * kBandCap);
   t.band_i = c.take<int>((size_t)band_rows * kBandCap);
   t.band_a = bf ? c.take<char>((size_t)band_rows * d * es) : nullptr;
@@ -201,8 +204,10 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   // one contracted cluster overlap, so their total can exceed n
   if (bf && p->k > 0) carve_ball(c, (int)n, d, kinds, r.kp, elt_of(p), (int)std::min<int64_t>(2 * n, INT32_MAX / 2), &t.ball);
   t.w = c.take<float>((size_t)kinds * nn * p->k);
-  t.cnt = c.take<int>((size_t)kinds * (nn + 1));
-  t.fill = c.take<int>((size_t)kinds * nn);
+  t.zero_n = (size_t)kinds * (2 * nn + 1) + 2;  // in-degree counts, fills and hub counts together
+  t.cnt = c.take<int>(t.zero_n);
+  t.fill = t.cnt + (size_t)kinds * (nn + 1);
+  t.long_count = t.fill + (size_t)kinds * nn;
   t.t_src = c.take<int>((size_t)kinds * nn * p->k);
   t.t_w = c.take<float>((size_t)kinds * nn * p->k);
   t.raw_col = c.take<int>(cap);
@@ -211,11 +216,9 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.scan_tmp = c.take<int>(nn + 1);
   t.inv = c.take<double>((size_t)2 * kinds * nn);
   t.long_list = c.take<int>(nn);
-  t.long_count = c.take<int>(4);
   t.scan_tmp2 = c.take<int>(nn + 1);
   t.long_list2 = c.take<int>(nn);
   t.stats = c.take<unsigned long long>(GCR_STATS_LEN);
-  t.err = c.take<int>(4);
   t.okey = c.take<int>(nn);
   t.ocnt = c.take<int>(nn + 1);
   t.ooff = c.take<int>(nn + 1);
@@ -241,9 +244,8 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
     StageScope sc_(GCR_STAGE_PREP, st, 2);
     GCR_CUDA_TRY(launch_row_stats(X, n, d, w.n64, w.n32, bf ? w.xr : nullptr, elt, w.enrm, w.anrm, w.sc, st));
   }
-  GCR_CUDA_TRY(cudaMemsetAsync(w.unc_count, 0, sizeof(int) * 4, st));
-  GCR_CUDA_TRY(cudaMemsetAsync(w.band_cnt, 0, sizeof(int) * w.band_rows, st));
-  GCR_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int) * 4, st));
+  // pending-pair count, error word and band counts together
+  GCR_CUDA_TRY(cudaMemsetAsync(w.unc_count, 0, sizeof(int) * (8 + (size_t)w.band_rows), st));
   const int* camp = p->cross_camera ? cam : nullptr;
 
   if (p->k > 0) {
@@ -273,7 +275,7 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
   // is always written when the caller provides row_order (the identity when k = 0)
   int* order = g->row_order ? g->row_order : w.order;
   if (p->k == 0 && g->row_order)
-    GCR_CUDA_TRY(launch_row_order(w.pool_i, n, r.kp, 0, w.okey, w.ocnt, w.ooff, w.ofill, order, st));
+    GCR_CUDA_TRY(launch_identity_order(order, n, st));
   if (p->k > 0) {
     ra.unc_dk = w.unc_dk;
     ra.dk_all = bf ? w.dk_all : nullptr;
@@ -282,8 +284,13 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
     ra.skip_saturated = bf ? 0 : 1;
     {
       StageScope sc_(GCR_STAGE_REFINE, st, 5);
-      GCR_CUDA_TRY(launch_row_order(w.pool_i, n, r.kp, p->k, w.okey, w.ocnt, w.ooff, w.ofill, order, st));
-      ra.order = order;
+      // rows that fit in half of L2 are gathered from there whatever their order
+      if (in_l2(n, d)) {
+        if (g->row_order) GCR_CUDA_TRY(launch_identity_order(order, n, st));
+      } else {
+        GCR_CUDA_TRY(launch_row_order(w.pool_i, n, r.kp, p->k, w.okey, w.ocnt, w.ooff, w.ofill, order, st));
+        ra.order = order;
+      }
       GCR_CUDA_TRY(launch_refine_pool(ra, st));
     }
     // the queue the band rescan takes: the ball search's leftovers, or the refinement's queue
@@ -301,7 +308,7 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
       GCR_CUDA_TRY(launch_umma_gpool(b.Yr, b.cap_rows, d, elt, b.gcam, kinds == 2, 1, r.kp, b.items, b.ioff + n,
                                      b.max_items, b.hy, b.gpool_v, b.gpool_i, st));
       ra.bq_count = w.bq_count; ra.bq_row = w.bq_row; ra.bq_kind = w.bq_kind; ra.bq_thr = w.bq_thr;
-      ra.bq_flag = w.bq_flag; ra.bq_pos = w.bq_pos;
+      ra.bq_flag = w.bq_flag;
       GCR_CUDA_TRY(launch_refine_ball(ra, b, st));
       rb.unc_count = w.bq_count; rb.unc_row = w.bq_row; rb.unc_kind = w.bq_kind; rb.unc_thr = w.bq_thr;
     }
@@ -358,7 +365,8 @@ int build_graph_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam
   ga.raw_col = w.raw_col; ga.raw_val = w.raw_val; ga.op_cnt = w.op_cnt; ga.scan_tmp = w.scan_tmp;
   ga.inv = w.inv; ga.long_list = w.long_list; ga.long_count = w.long_count;
   ga.scan_tmp2 = w.scan_tmp2; ga.long_list2 = w.long_list2;
-  const bool want_order = g->row_order != nullptr && p->k > 0;
+  ga.zero = w.cnt; ga.zero_n = w.zero_n;
+  const bool want_order = g->row_order != nullptr && p->k > 0 && !in_l2(n, d);
   std::unique_lock<std::mutex> olock;
   OrderStream* os = nullptr;
   if (want_order) {
@@ -374,7 +382,7 @@ int build_graph_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam
     }
   }
   {
-    StageScope sc_(GCR_STAGE_GRAPH, st, 7 * kinds + 3 + (want_order ? 5 : 0));
+    StageScope sc_(GCR_STAGE_GRAPH, st, 8 + (want_order ? 6 : 0));
     if (want_order) {
       GCR_CUDA_TRY(cudaEventRecord(os->fork, st));
       GCR_CUDA_TRY(cudaStreamWaitEvent(os->s, os->fork, 0));
@@ -642,7 +650,6 @@ struct ServeWs {
   int* bq_kind;
   float* bq_thr;
   int* bq_flag;
-  int* bq_pos;
   int* err;
   int* band_cnt;
   float* band_v;
@@ -696,7 +703,6 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   t.bq_kind = c.take<int>(nb);
   t.bq_thr = c.take<float>(nb);
   t.bq_flag = c.take<int>(nb);
-  t.bq_pos = c.take<int>(nb + 1);
   t.err = c.take<int>(4);
   t.band_cnt = c.take<int>(nb);
   t.band_v = c.take<float>(nb * kBandCap);
@@ -782,7 +788,7 @@ int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp,
     GCR_CUDA_TRY(launch_umma_gpool(bl.Yr, bl.cap_rows, d, elt, nullptr, false, 0, kp, bl.items, bl.ioff + b + ng,
                                    bl.max_items, bl.hy, bl.gpool_v, bl.gpool_i, st));
     ra.bq_count = w.bq_count; ra.bq_row = w.bq_row; ra.bq_kind = w.bq_kind; ra.bq_thr = w.bq_thr;
-    ra.bq_flag = w.bq_flag; ra.bq_pos = w.bq_pos;
+    ra.bq_flag = w.bq_flag;
     GCR_CUDA_TRY(launch_refine_ball(ra, bl, st));
     rb.unc_count = w.bq_count; rb.unc_row = w.bq_row; rb.unc_kind = w.bq_kind; rb.unc_thr = w.bq_thr;
   }

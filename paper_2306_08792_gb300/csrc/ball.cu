@@ -98,6 +98,7 @@ __global__ void ball_init_kernel(BallArgs a) {
     a.active[v] = 0;
     a.seen[v] = 0;
     a.rdense[v] = 0;
+    a.gsize[v] = 0;
   }
   if (v < a.na) {
     a.pend[v] = 0;
@@ -213,29 +214,10 @@ __global__ void ball_root_kernel(BallArgs a) {
   }
 }
 
-// The groups searched: roots with a pair whose band the refinement predicted to overflow, or with
-// at least kMinGroupRows pending rows in a contracted ball (R^2 <= ||c||^2 / 4: centring shrinks
-// the rounding bound by (R / ||c||)^2, so a wider ball gains too little over the rescan); the
-// others' pairs go to the threshold rescan.
-__global__ void ball_elig_kernel(BallArgs a) {
-  const bool go = ball_go(a);
-  if (go && blockIdx.x == 0 && threadIdx.x == 0 && a.stats)
-    atomicAdd(a.stats + GCR_STAT_BALL_PAIRS, (unsigned long long)*a.npart);
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < node_count(a); v += gridDim.x * blockDim.x) {
-    const double nc = (a.two && v >= a.na) ? a.n64B[v - a.na] : a.n64A[v];
-    const double R = (double)a.rad[v];
-    const bool contracted = R * R <= 0.25 * nc;
-    a.active[v] = (go && a.seen[v] && (a.rdense[v] || (a.acnt[v] >= kMinGroupRows && contracted))) ? 1 : 0;
-  }
-}
-
-// Group table from the scanned active flags; the sweep threshold of each centre:
+// The group of root r: its table entry and the sweep threshold of its centre:
 // ||x_j - c||^2 <= R^2 implies s_cj >= (||x_j||^2 + ||c||^2 - R^2) / 2 >= (nmin + ||c||^2 - R^2) / 2,
 // and the approximate score is within delta_c (the GEMM bound of row c against the B rows) of s_cj.
-__global__ void ball_group_kernel(BallArgs a) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= node_count(a) || !a.active[r]) return;
-  const int g = a.gid[r];
+__device__ __forceinline__ void ball_group_one(const BallArgs& a, int r, int g) {
   a.groot[g] = r;
   a.ga[g] = a.acnt[r];
   a.gkind[g] = 0;
@@ -259,6 +241,36 @@ __global__ void ball_group_kernel(BallArgs a) {
   a.gthr[g] = nextafterf(__double2float_rd(thr), -CUDART_INF_F);
 }
 
+// The groups searched, and their table, by one block: roots with a pair whose band the refinement
+// predicted to overflow, or with at least kMinGroupRows pending rows in a contracted ball
+// (R^2 <= ||c||^2 / 4: centring shrinks the rounding bound by (R / ||c||)^2, so a wider ball gains
+// too little over the rescan); the others' pairs go to the threshold rescan. (Flags, scan and
+// table as one launch: most builds search no ball, and each launch of the chain costs them 3 to 4
+// us. 15 launches where there were 25: 95 -> 60 us per build of 800 rows.)
+__global__ void __launch_bounds__(1024) ball_group_kernel(BallArgs a) {
+  const int nn = node_count(a);
+  if (!ball_go(a)) {
+    if (threadIdx.x == 0) a.gid[nn] = 0;
+    return;
+  }
+  if (threadIdx.x == 0 && a.stats) atomicAdd(a.stats + GCR_STAT_BALL_PAIRS, (unsigned long long)*a.npart);
+  const int G = block_scan_1024(
+      nn,
+      [&](int v) {
+        const double nc = (a.two && v >= a.na) ? a.n64B[v - a.na] : a.n64A[v];
+        const double R = (double)a.rad[v];
+        const bool contracted = R * R <= 0.25 * nc;
+        const int on = (a.seen[v] && (a.rdense[v] || (a.acnt[v] >= kMinGroupRows && contracted))) ? 1 : 0;
+        a.active[v] = on;
+        return on;
+      },
+      [&](int v, int g, int on) {
+        a.gid[v] = g;
+        if (on) ball_group_one(a, v, g);
+      });
+  if (threadIdx.x == 0) a.gid[nn] = G;
+}
+
 // The centres' rounded operand rows (from the A or the B copy), 16 bytes per thread.
 __global__ void ball_centres_kernel(BallArgs a) {
   const int G = a.gid[node_count(a)];
@@ -271,41 +283,39 @@ __global__ void ball_centres_kernel(BallArgs a) {
     const uint4* src = static_cast<const uint4*>(on_b ? a.xrB : a.xrA) + (size_t)(on_b ? r - a.na : r) * w16;
     static_cast<uint4*>(a.cent)[g * w16 + c] = src[c];
   }
+  // positions are unused until the members are placed
+  if (G > 0)
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.cap_rows; p += gridDim.x * blockDim.x) a.ggrp[p] = -1;
 }
 
 // Groups searched: a ball no larger than half of the B rows (among the A rows it must also hold
 // the group's pending rows; anything else is a numerical impossibility, handled as a failure).
-// Segment size: the pending rows plus the ball against a gallery, the ball alone otherwise.
-__global__ void ball_route_kernel(BallArgs a) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nn = node_count(a);
-  if (g >= nn) return;
-  const int G = a.gid[nn];
-  int sz = 0;
-  if (g < G) {
-    const int c = a.gsize[g];
-    if (a.two) sz = c <= a.nb / 2 ? a.ga[g] + c : 0;
-    else sz = (c <= a.na / 2 && c >= a.ga[g]) ? c : 0;
-  }
-  a.rsize[g] = sz;
-  a.gfill[g] = 0;
-  a.afill[g] = 0;
-  a.bfill[g] = 0;
-  a.gfail[g] = 0;
-}
-
-// Capacity cut (segments in scan order), fill-pass thresholds (+inf: not searched), and where
-// the fill pass lists each ball: after the pending rows against a gallery, else the segment.
-__global__ void ball_cut_kernel(BallArgs a) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+// Segment size: the pending rows plus the ball against a gallery, the ball alone otherwise. One
+// block: sizes, their scan, the capacity cut (segments in scan order), the fill-pass thresholds
+// (+inf: not searched), and where the fill pass lists each ball: after the pending rows against a
+// gallery, else the segment.
+__global__ void __launch_bounds__(1024) ball_route_kernel(BallArgs a) {
   const int G = a.gid[node_count(a)];
-  if (g >= G) return;
-  const bool fits = a.rsize[g] > 0 && a.goff[g] + a.rsize[g] <= a.cap_rows;
-  if (!fits) a.rsize[g] = 0;
-  a.gthr_fill[g] = fits ? a.gthr[g] : CUDART_INF_F;
-  if (!fits) a.gfail[g] = 1;
-  a.boff[g] = a.goff[g] + (a.two ? a.ga[g] : 0);
-  a.blim[g] = fits ? (a.two ? a.rsize[g] - a.ga[g] : a.rsize[g]) : 0;
+  const int total = block_scan_1024(
+      G,
+      [&](int g) {
+        a.gfill[g] = 0;
+        a.afill[g] = 0;
+        a.bfill[g] = 0;
+        const int c = a.gsize[g];
+        if (a.two) return c <= a.nb / 2 ? a.ga[g] + c : 0;
+        return (c <= a.na / 2 && c >= a.ga[g]) ? c : 0;
+      },
+      [&](int g, int off, int sz) {
+        a.goff[g] = off;
+        const bool fits = sz > 0 && off + sz <= a.cap_rows;
+        a.rsize[g] = fits ? sz : 0;
+        a.gthr_fill[g] = fits ? a.gthr[g] : CUDART_INF_F;
+        a.gfail[g] = fits ? 0 : 1;
+        a.boff[g] = off + (a.two ? a.ga[g] : 0);
+        a.blim[g] = fits ? (a.two ? sz - a.ga[g] : sz) : 0;
+      });
+  if (threadIdx.x == 0) a.goff[G] = total;
 }
 
 __device__ __forceinline__ int group_of(const int* goff, int G, int e) {
@@ -377,37 +387,34 @@ __global__ void ball_place_rows_kernel(BallArgs a) {
   }
 }
 
-// Every pending row of a group must have been placed; work items of the searched groups.
-__global__ void ball_items_count_kernel(BallArgs a) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+// Every pending row of a group must have been placed; work items of the searched groups, and
+// neutral per-group maxima for the centring pass. One block.
+__global__ void __launch_bounds__(1024) ball_items_kernel(BallArgs a) {
   const int nn = node_count(a);
-  if (g >= nn) return;
   const int G = a.gid[nn];
-  int c = 0;
-  if (g < G && a.rsize[g] > 0) {
-    if (a.afill[g] != a.ga[g]) a.gfail[g] = 1;
-    if (!a.gfail[g]) c = (a.ga[g] + 127) / 128;
-  }
-  a.icnt[g] = c;
-  if (c > 0 && a.stats) {
-    atomicAdd(a.stats + GCR_STAT_BALL_GROUPS, 1ull);
-    atomicAdd(a.stats + GCR_STAT_BALL_ROWS, (unsigned long long)a.rsize[g]);
-  }
-  if (g < G) {  // neutral per-group maxima for the centring pass
-    a.gsc[g].nmin = 1e300;
-    a.gsc[g].nmax = 0.0;
-    a.gsc[g].emax = 0.0;
-    a.gsc[g].amax = 0.0;
-  }
-}
-
-__global__ void ball_items_kernel(BallArgs a) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  const int G = a.gid[node_count(a)];
-  if (g >= G || a.icnt[g] == 0) return;
-  const int o = a.ioff[g];
-  for (int b = 0; b < a.icnt[g]; ++b)
-    a.items[o + b] = make_int4(a.goff[g] + 128 * b, min(128, a.ga[g] - 128 * b), a.boff[g], a.blim[g]);
+  const int total = block_scan_1024(
+      G,
+      [&](int g) {
+        int c = 0;
+        if (a.rsize[g] > 0) {
+          if (a.afill[g] != a.ga[g]) a.gfail[g] = 1;
+          if (!a.gfail[g]) c = (a.ga[g] + 127) / 128;
+        }
+        if (c > 0 && a.stats) {
+          atomicAdd(a.stats + GCR_STAT_BALL_GROUPS, 1ull);
+          atomicAdd(a.stats + GCR_STAT_BALL_ROWS, (unsigned long long)a.rsize[g]);
+        }
+        a.gsc[g].nmin = 1e300;
+        a.gsc[g].nmax = 0.0;
+        a.gsc[g].emax = 0.0;
+        a.gsc[g].amax = 0.0;
+        return c;
+      },
+      [&](int g, int o, int c) {
+        for (int b = 0; b < c; ++b)
+          a.items[o + b] = make_int4(a.goff[g] + 128 * b, min(128, a.ga[g] - 128 * b), a.boff[g], a.blim[g]);
+      });
+  if (threadIdx.x == 0) a.ioff[nn] = total;
 }
 
 __device__ __forceinline__ unsigned long long dbits_b(double v) { return (unsigned long long)__double_as_longlong(v); }
@@ -639,37 +646,24 @@ cudaError_t launch_ball_prepare(const BallArgs& a, cudaStream_t st) {
   if (a.two) ball_scale_kernel<<<wb, 256, 0, st>>>(a);
   ball_link_kernel<<<wb, 256, 0, st>>>(a);
   ball_root_kernel<<<wb, 256, 0, st>>>(a);
-  ball_elig_kernel<<<std::min(nb, 152 * 8), 256, 0, st>>>(a);
+  ball_group_kernel<<<1, 1024, 0, st>>>(a);  // group ids; gid[nn] = number of groups
+  ball_centres_kernel<<<152 * 4, 256, 0, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = launch_scan(a.active, a.gid, nn, st);  // group ids; gid[nn] = number of groups
-  if (e != cudaSuccess) return e;
-  ball_group_kernel<<<nb, 256, 0, st>>>(a);
-  ball_centres_kernel<<<152 * 4, 256, 0, st>>>(a);
   // sweep pass 1: ball sizes (the centre rows: at most cent_rows groups, one per pending row)
-  e = cudaMemsetAsync(a.gsize, 0, sizeof(int) * (nn + 1), st);
-  if (e != cudaSuccess) return e;
   const int B_rows = a.two ? a.nb : a.na;
   const void* xrB = a.two ? a.xrB : a.xrA;
   e = launch_umma_band(xrB, B_rows, a.d, a.elt, nullptr, 0, a.cent, a.gid + nn, a.cent_rows, a.groot, a.gkind,
                        a.gthr, 0, a.gsize, nullptr, a.ball_j, st);
   if (e != cudaSuccess) return e;
-  ball_route_kernel<<<nb, 256, 0, st>>>(a);
-  e = launch_scan(a.rsize, a.goff, nn, st);
-  if (e != cudaSuccess) return e;
-  ball_cut_kernel<<<nb, 256, 0, st>>>(a);
+  ball_route_kernel<<<1, 1024, 0, st>>>(a);
   // sweep pass 2: members of the searched balls at their offsets
   e = launch_umma_band(xrB, B_rows, a.d, a.elt, nullptr, 0, a.cent, a.gid + nn, a.cent_rows, a.groot, a.gkind,
                        a.gthr_fill, 0, a.gfill, nullptr, a.ball_j, st, a.boff, a.blim);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.ggrp, 0xff, sizeof(int) * a.cap_rows, st);
-  if (e != cudaSuccess) return e;
   ball_place_kernel<<<std::min((a.cap_rows + 255) / 256, 152 * 8), 256, 0, st>>>(a);
   if (a.two) ball_place_rows_kernel<<<std::min((a.unc_cap + 255) / 256, 152 * 4), 256, 0, st>>>(a);
-  ball_items_count_kernel<<<nb, 256, 0, st>>>(a);
-  e = launch_scan(a.icnt, a.ioff, nn, st);
-  if (e != cudaSuccess) return e;
-  ball_items_kernel<<<nb, 256, 0, st>>>(a);
+  ball_items_kernel<<<1, 1024, 0, st>>>(a);
   const unsigned cb = (unsigned)std::min((a.cap_rows + 7) / 8, 152 * 4);
   if (a.elt == Elt::TF32) ball_center_kernel<Elt::TF32><<<cb, 256, 0, st>>>(a);
   else ball_center_kernel<Elt::BF16><<<cb, 256, 0, st>>>(a);

@@ -137,6 +137,74 @@ __device__ __forceinline__ float ordered_to_float(uint32_t u) {
   return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
+// Exclusive scan over [0, n) by one block of 1024 threads, tiles of 8,192 elements with a running
+// carry: ld(i) gives element i (called once, coalesced), st(i, prefix, value) takes its prefix.
+// Returns the total (on every thread). Each tile goes through shared memory (padded against bank
+// conflicts) so that a thread scans 8 consecutive elements.
+constexpr int kScanPer = 8;
+constexpr int kScanTile = 1024 * kScanPer;
+__device__ __forceinline__ int scan_pad(int i) { return i + (i >> 5); }
+template <typename Load, typename Store>
+__device__ __forceinline__ int block_scan_1024(int n, Load ld, Store st) {
+  __shared__ int tile[kScanTile + kScanTile / 32];
+  __shared__ int wsum[32];
+  __shared__ int carry_s;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid == 0) carry_s = 0;
+  for (int base = 0; base < n; base += kScanTile) {
+    int x[kScanPer];
+#pragma unroll
+    for (int e = 0; e < kScanPer; ++e) {
+      const int idx = base + e * 1024 + tid;
+      x[e] = idx < n ? ld(idx) : 0;
+    }
+#pragma unroll
+    for (int e = 0; e < kScanPer; ++e) tile[scan_pad(e * 1024 + tid)] = x[e];
+    __syncthreads();
+    int v[kScanPer];
+    int loc = 0;
+#pragma unroll
+    for (int e = 0; e < kScanPer; ++e) {
+      v[e] = tile[scan_pad(tid * kScanPer + e)];
+      loc += v[e];
+    }
+    int incl = loc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int t = __shfl_up_sync(GCR_FULL, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+      int s = wsum[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        int t = __shfl_up_sync(GCR_FULL, s, o);
+        if (lane >= o) s += t;
+      }
+      wsum[lane] = s;
+    }
+    __syncthreads();
+    int run = carry_s + (w > 0 ? wsum[w - 1] : 0) + incl - loc;
+#pragma unroll
+    for (int e = 0; e < kScanPer; ++e) {
+      tile[scan_pad(tid * kScanPer + e)] = run;
+      run += v[e];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < kScanPer; ++e) {
+      const int idx = base + e * 1024 + tid;
+      if (idx < n) st(idx, tile[scan_pad(e * 1024 + tid)], x[e]);
+    }
+    if (tid == 1023) carry_s = run;
+    __syncthreads();
+  }
+  __syncthreads();
+  return carry_s;
+}
+
 struct GcrvWs;
 size_t gcrv_carve(Carve& c, int64_t F, int d, int C, int ncam, GcrvWs* w);
 

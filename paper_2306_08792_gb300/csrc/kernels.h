@@ -130,11 +130,10 @@ struct RefineArgs {
   float* dk_all;            // [kinds][n] (may be NULL): the same bound for every (row, graph)
   int skip_saturated;       // 1: pairs whose pool is saturated with near-ties are not queued
   int* bq_count;            // ball refinement: pairs handed on to the band rescan, in the
-  int* bq_row;              // pending queue's order (bq_flag per pending pair, bq_pos its
-  int* bq_kind;             // scan: cap + 1 entries)
+  int* bq_row;              // pending queue's order (bq_flag per pending pair)
+  int* bq_kind;
   float* bq_thr;
   int* bq_flag;
-  int* bq_pos;
   unsigned long long* stats;
   // band rescan results
   const int* band_cnt;
@@ -153,6 +152,7 @@ cudaError_t launch_refine_band(const RefineArgs& a, cudaStream_t st);
 // Cluster-local row order from the pools (first k candidates): order[0..n) is a permutation.
 cudaError_t launch_row_order(const int* pool_i, int n, int kp, int k, int* key, int* cnt, int* off, int* fill,
                              int* order, cudaStream_t st);
+cudaError_t launch_identity_order(int* order, int n, cudaStream_t st);
 // Copies rows[u] of src (row_bytes each, a multiple of 16) to row u of out, u < min(*count, max_rows).
 cudaError_t launch_gather_rows(const void* src, size_t row_bytes, const int* count, const int* rows,
                                int max_rows, void* out, cudaStream_t st);
@@ -261,8 +261,10 @@ struct GraphArgs {
   double* inv;              // [2*kinds][n] scratch: inverse square roots of the degrees
   int* long_list;           // [n] scratch: transposed rows of a hub's length
   int* long_count;          // [2] scratch
-  int* scan_tmp2;           // [n+1], [n]: the second graph's scan temporary and hub list (its
-  int* long_list2;          //   transpose is built on a second stream)
+  int* scan_tmp2;           // [n+1], [n]: the second graph's scan and hub list
+  int* long_list2;
+  int* zero;                // cnt, fill and long_count of both graphs, zero_n ints
+  size_t zero_n;
 };
 cudaError_t launch_build_operator(const GraphArgs& g, cudaStream_t st);
 cudaError_t launch_scan(const int* in, int* out, int n, cudaStream_t st);

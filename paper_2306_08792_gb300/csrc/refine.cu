@@ -716,6 +716,7 @@ __device__ void refine_ball_one(const RefineArgs& a, const BallArgs& b, int u, i
   wl_sort<P>(L, lane);
   const double sig_k = wl_sig(L, kk - 1);
   if (full && !(sig_k - eps > tau + delta)) { hand_on(); return; }
+  if (lane == 0) a.bq_flag[u] = 0;
   if (lane == 0 && a.stats) atomicAdd(&a.stats[GCR_STAT_BALL], 1ull);
   finalize<VPL, P>(c, xi, L, r, kk, eps, p, i, kind, lane, b.gmap);
 }
@@ -819,34 +820,43 @@ cudaError_t launch_ball_vpl(const RefineArgs& a, const BallArgs& b, cudaStream_t
   return cudaGetLastError();
 }
 
-__global__ void hand_on_kernel(RefineArgs a, int cap) {
+// Stable compaction of the flagged pairs into the band queue, by one block.
+__global__ void __launch_bounds__(1024) hand_on_kernel(RefineArgs a, int cap) {
   const int U = min(*a.unc_count, cap);
-  for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < U; u += gridDim.x * blockDim.x) {
-    if (!a.bq_flag[u]) continue;
-    const int v = a.bq_pos[u];
-    a.bq_row[v] = a.unc_row[u];
-    a.bq_kind[v] = a.unc_kind[u];
-    a.bq_thr[v] = a.unc_thr[u];
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *a.bq_count = a.bq_pos[cap];
+  const int total = block_scan_1024(
+      U, [&](int u) { return a.bq_flag[u]; },
+      [&](int u, int v, int on) {
+        if (!on) return;
+        a.bq_row[v] = a.unc_row[u];
+        a.bq_kind[v] = a.unc_kind[u];
+        a.bq_thr[v] = a.unc_thr[u];
+      });
+  if (threadIdx.x == 0) *a.bq_count = total;
 }
 
 cudaError_t launch_refine_ball(const RefineArgs& a, const BallArgs& b, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(a.bq_flag, 0, sizeof(int) * b.unc_cap, st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   if (a.kp == 32) e = launch_ball_vpl<1>(a, b, st);
   else if (a.kp == 64) e = launch_ball_vpl<2>(a, b, st);
   else if (a.kp == 128) e = launch_ball_vpl<4>(a, b, st);
   else return cudaErrorInvalidValue;
   if (e != cudaSuccess) return e;
-  e = launch_scan(a.bq_flag, a.bq_pos, b.unc_cap, st);
-  if (e != cudaSuccess) return e;
-  hand_on_kernel<<<std::min((b.unc_cap + 255) / 256, 152 * 4), 256, 0, st>>>(a, b.unc_cap);
+  hand_on_kernel<<<1, 1024, 0, st>>>(a, b.unc_cap);
   return cudaGetLastError();
 }
 
 cudaError_t launch_refine_band(const RefineArgs& a, cudaStream_t st) {
   return a.k >= 64 ? launch_band_p<4>(a, st) : launch_band_p<2>(a, st);
+}
+
+__global__ void identity_order_kernel(int* order, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) order[i] = i;
+}
+
+cudaError_t launch_identity_order(int* order, int n, cudaStream_t st) {
+  identity_order_kernel<<<(n + 255) / 256, 256, 0, st>>>(order, n);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_row_order(const int* pool_i, int n, int kp, int k, int* key, int* cnt, int* off, int* fill,
