@@ -409,15 +409,10 @@ int check_graph(const gcr_graph* g, int kinds, int k) {
 
 struct RerankWs {
   float* D;
-  double* n64q;
-  double* n64g;
   float* nq;
   float* ng;
-  RowScalars* sc;
   __nv_bfloat16* qb;
   __nv_bfloat16* gb;
-  float* dummy;
-  int* err;
 };
 
 // Top-K re-ranking through the certified pool search: used when 1 <= topk_out <= 127 and
@@ -429,15 +424,10 @@ bool rerank_uses_pool(const gcr_params* p, int64_t ng) {
 size_t carve_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, bool bf, RerankWs* w) {
   RerankWs t;
   t.D = c.take<float>((size_t)nq * ng);
-  t.n64q = c.take<double>(nq);
-  t.n64g = c.take<double>(ng);
   t.nq = c.take<float>(nq);
   t.ng = c.take<float>(ng);
-  t.sc = c.take<RowScalars>(2);
   t.qb = bf ? c.take<__nv_bfloat16>((size_t)nq * 3 * d) : nullptr;
   t.gb = bf ? c.take<__nv_bfloat16>((size_t)ng * 3 * d) : nullptr;
-  t.dummy = c.take<float>(2 * (size_t)std::max(nq, ng));
-  t.err = c.take<int>(4);
   if (w) *w = t;
   return c.off;
 }
@@ -459,18 +449,10 @@ int rerank_impl(const float* Xq, int64_t nq, const float* Xg, int64_t ng, int32_
   // the distance GEMM of both tensor-core modes runs on compensated BF16 operands
   const bool bf = tensor_mode(p);
   const int K = p->topk_out > 0 ? (int)std::min<int64_t>(p->topk_out, ng) : (int)ng;
-  const size_t mx = (size_t)std::max(nq, ng);
   {
-    StageScope sc_(GCR_STAGE_PREP, st, bf ? 6 : 4);
-    GCR_CUDA_TRY(launch_row_stats(Xq, (int)nq, d, w.n64q, w.nq, nullptr, Elt::BF16, w.dummy, w.dummy + mx, w.sc, st));
-    GCR_CUDA_TRY(
-        launch_row_stats(Xg, (int)ng, d, w.n64g, w.ng, nullptr, Elt::BF16, w.dummy, w.dummy + mx, w.sc + 1, st));
-    if (bf) {
-      GCR_CUDA_TRY(launch_split3(Xq, (int)nq, d, 0, w.qb, st));
-      GCR_CUDA_TRY(launch_split3(Xg, (int)ng, d, 1, w.gb, st));
-    }
+    StageScope sc_(GCR_STAGE_PREP, st);
+    GCR_CUDA_TRY(launch_rerank_prep(Xq, (int)nq, Xg, (int)ng, d, w.nq, w.ng, w.qb, w.gb, st));
   }
-  if (bf) GCR_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int) * 4, st));
   const int64_t chunk = hd ? hd->chunk_rows : nq;
   for (int64_t q0 = 0, c = 0; q0 < nq; q0 += chunk, ++c) {
     const int nc = (int)std::min<int64_t>(chunk, nq - q0);

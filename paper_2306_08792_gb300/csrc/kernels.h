@@ -33,7 +33,9 @@ cudaError_t launch_normalize(const float* X_in, float* X_out, int64_t n, int d, 
 cudaError_t launch_row_stats(const float* X, int n, int d, double* n64, float* n32,
                              void* xr, Elt elt, float* enrm, float* anrm, RowScalars* sc,
                              cudaStream_t st);
-cudaError_t launch_split3(const float* X, int n, int d, int gallery_order, __nv_bfloat16* out, cudaStream_t st);
+// Squared norms of query and gallery rows and (qb != NULL, d % 8 == 0) their compensated BF16 operands.
+cudaError_t launch_rerank_prep(const float* Xq, int nq, const float* Xg, int ng, int d, float* n32q, float* n32g,
+                               __nv_bfloat16* qb, __nv_bfloat16* gb, cudaStream_t st);
 
 // How a pool sweep is cut: the column splits of each 128-row block (tps column tiles each, in
 // the grid's order), whether clusters share the column tiles, and the buffers its splits leave.

@@ -105,3 +105,21 @@ def test_sampled_floors_of_a_wide_search(K, d):
     assert torch.allclose(dist.double(), v[:, :K], atol=2e-6, rtol=0)
     clear = v[:, K] - v[:, K - 1] > 1e-9
     assert torch.equal(idx[clear].long().sort(1)[0], o[clear, :K].sort(1)[0])
+
+
+@pytest.mark.parametrize("ng", [1, 33, 64, 65, 256, 257, 511, 513, 1024, 1025, 2049])
+def test_ranking_of_short_galleries(ng):
+    """The bitonic network (to 256 keys) and the radix sort's small sizes, with exact ties."""
+    import paper_2306_08792_gb300 as gcr
+    rng = np.random.default_rng(ng)
+    G = rng.standard_normal((ng, 40)).astype(np.float32)
+    G[rng.choice(ng, ng // 4, replace=False)] = G[0]
+    Q = rng.standard_normal((5, 40)).astype(np.float32)
+    Xq, Xg = (gcr.gcr_normalize(torch.from_numpy(a).cuda()) for a in (Q, G))
+    idx, dist = (t.cpu().numpy() for t in gcr.gcr_rerank(Xq, Xg, gcr.default_params(topk_out=0)))
+    assert np.array_equal(np.sort(idx, axis=1), np.broadcast_to(np.arange(ng), idx.shape))
+    step = np.diff(dist, axis=1)
+    assert np.all(step >= 0) and np.all(np.diff(idx, axis=1)[step == 0] > 0)
+    D = torch.cdist(Xq.double(), Xg.double()).square().cpu().numpy()
+    # FP32 products of 40 terms: 40 * 2^-24, and the rounding of the distance
+    assert np.max(np.abs(np.take_along_axis(D, idx, axis=1) - dist)) < 2 * 40 * 2.0 ** -24 + 3 * 2.0 ** -23
