@@ -55,6 +55,8 @@ struct Resolved {
 // The tensor-core modes (BF16, TF32) search on rounded operand copies; FP32 runs on the CUDA cores.
 bool tensor_mode(const gcr_params* p) { return p->precision != GCR_PREC_FP32; }
 Elt elt_of(const gcr_params* p) { return p->precision == GCR_PREC_TF32 ? Elt::TF32 : Elt::BF16; }
+// Operands of the serving searches (normalised rows, no ball search): TF32's values in 16 bits.
+Elt serve_elt(const gcr_params* p) { return p->precision == GCR_PREC_TF32 ? Elt::F16 : Elt::BF16; }
 size_t elt_size(const gcr_params* p) { return elt_bytes(elt_of(p)); }
 
 int check_precision(const gcr_params* p, int32_t d) {
@@ -103,8 +105,8 @@ size_t op_capacity(int64_t n, const gcr_params* p, int kinds) {
   return (size_t)(n * per);
 }
 
-PoolParts carve_parts(Carve& c, int na, int nb, int d, const gcr_params* p, int kp, bool cross) {
-  const PoolPlan pl = tensor_mode(p) ? pool_plan(na, nb, d, elt_of(p), kp, cross) : simt_pool_plan(na, nb, d, kp, cross);
+PoolParts carve_parts(Carve& c, int na, int nb, int d, const gcr_params* p, Elt elt, int kp, bool cross) {
+  const PoolPlan pl = tensor_mode(p) ? pool_plan(na, nb, d, elt, kp, cross) : simt_pool_plan(na, nb, d, kp, cross);
   const size_t rows = pool_part_rows(pl, na, cross);
   PoolParts t;
   t.v = c.take<float>(rows * pl.cap);
@@ -182,7 +184,7 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.anrm = bf ? c.take<float>(nn) : nullptr;
   t.pool_v = c.take<float>((size_t)kinds * nn * r.kp);
   t.pool_i = c.take<int>((size_t)kinds * nn * r.kp);
-  t.parts = carve_parts(c, (int)n, (int)n, d, p, r.kp, kinds == 2);
+  t.parts = carve_parts(c, (int)n, (int)n, d, p, elt_of(p), r.kp, kinds == 2);
   t.unc_count = c.take<int>(8 + (size_t)band_rows);
   t.err = t.unc_count + 4;
   t.band_cnt = t.unc_count + 8;
@@ -262,7 +264,7 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
   RefineArgs ra;
   std::memset(&ra, 0, sizeof(ra));
   ra.X = X; ra.XB = X; ra.n = n; ra.d = d; ra.k = p->k; ra.kinds = kinds; ra.precision = p->precision;
-  ra.n64 = w.n64; ra.n64B = w.n64; ra.enrm = w.enrm; ra.anrm = w.anrm; ra.sc = w.sc;
+  ra.n64 = w.n64; ra.n64B = w.n64; ra.enrm = w.enrm; ra.anrm = w.anrm; ra.sc = w.sc; ra.scale = 1.f;
   ra.pool_v = w.pool_v; ra.pool_i = w.pool_i; ra.kp = r.kp;
   ra.nbr[0] = g->nbr; ra.d2[0] = g->nbr_d2;
   ra.nbr[1] = kinds == 2 ? g->nbr_cr : g->nbr;
@@ -574,7 +576,7 @@ size_t carve_gallery(Carve& c, int64_t ng, int32_t d, const gcr_params* p, Galle
   t.deg = c.take<float>((size_t)(p->T > 0 ? p->T : 1) * n);
   t.n64 = c.take<double>(L * n);
   t.n32 = c.take<float>(L * n);
-  t.xr = bf ? c.take<char>(L * n * d * elt_size(p)) : nullptr;
+  t.xr = bf ? c.take<char>(L * n * d * elt_bytes(serve_elt(p))) : nullptr;
   t.enrm = bf ? c.take<float>(L * n) : nullptr;
   t.anrm = bf ? c.take<float>(L * n) : nullptr;
   t.sc = c.take<RowScalars>(L);
@@ -648,10 +650,11 @@ int serve_kp_final(const gcr_params* p) {
   return K < 64 ? 64 : 128;
 }
 
-size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params* p, const Resolved& r, ServeWs* w) {
+size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params* p, Elt elt, const Resolved& r,
+                   ServeWs* w) {
   const size_t nb = (size_t)b;
   const bool bf = tensor_mode(p);
-  const size_t es = elt_size(p);
+  const size_t es = elt_bytes(elt);
   const int kpmax = std::max(r.kp, serve_kp_final(p));
   ServeWs t;
   t.xq[0] = c.take<float>(nb * d);
@@ -667,8 +670,8 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   size_t end = 0;
   for (int64_t rows = std::min<int64_t>(b, 128);; rows = std::min<int64_t>(b, rows + 128)) {
     Carve c1 = c, c2 = c;
-    t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, r.kp, false);
-    t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, p, serve_kp_final(p), false);
+    t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, elt, r.kp, false);
+    t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, p, elt, serve_kp_final(p), false);
     end = std::max(end, std::max(c1.off, c2.off));
     if (rows == b) break;
   }
@@ -717,11 +720,10 @@ GallerySide gallery_layer(const GalleryView& g, int layer, int ng, int d, size_t
 // Certified k nearest gallery rows for the b query rows xq: pool, merge, refine, band.
 // ball (may be NULL; tensor-core modes): workspace of the ball search of the rows the pools
 // cannot certify (without it, pools saturated with near-ties keep the 2 delta bound).
-int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp, const PoolParts& parts,
+int serve_knn(const float* xq, int b, int d, const gcr_params* p, Elt elt, int k, int kp, const PoolParts& parts,
               const GallerySide& gs, int ng, const ServeWs& w, unsigned long long* stats, int32_t* nbr, float* d2, cudaStream_t st,
               const BallArgs* ball = nullptr) {
   const bool bf = tensor_mode(p);
-  const Elt elt = elt_of(p);
   const float* G = gs.G;
   {
     StageScope sc_(GCR_STAGE_PREP, st, bf ? 2 : 2);
@@ -742,6 +744,7 @@ int serve_knn(const float* xq, int b, int d, const gcr_params* p, int k, int kp,
   ra.X = xq; ra.XB = G; ra.n = b; ra.d = d; ra.k = k; ra.kinds = 1; ra.precision = p->precision;
   ra.n64 = w.n64; ra.n64B = gs.n64;
   ra.enrm = w.enrm; ra.anrm = w.anrm; ra.sc = gs.sc;
+  ra.scale = elt == Elt::F16 ? kF16Scale * kF16Scale : 1.f;
   ra.pool_v = w.pool_v; ra.pool_i = w.pool_i; ra.kp = kp;
   ra.nbr[0] = ra.nbr[1] = nbr;
   ra.d2[0] = ra.d2[1] = d2;
@@ -806,7 +809,7 @@ size_t carve_topk_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_
   r.kp = serve_kp_final(p);
   r.kinds = 1;
   TopkRerankWs t;
-  carve_serve(c, nq, ng, d, p, r, &t.sw);
+  carve_serve(c, nq, ng, d, p, elt_of(p), r, &t.sw);
   t.n64g = c.take<double>(ng);
   t.n32g = c.take<float>(ng);
   t.gr = bf ? c.take<char>((size_t)ng * d * elt_size(p)) : nullptr;
@@ -831,7 +834,7 @@ int topk_rerank_impl(const float* Xq, int64_t nq, const float* Xg, int64_t ng, i
   }
   GCR_CUDA_TRY(cudaMemsetAsync(w.sw.stats, 0, sizeof(unsigned long long) * GCR_STATS_LEN, st));
   const GallerySide gs{Xg, w.gr, w.n64g, w.scg, w.genrm, w.ganrm};
-  return serve_knn(Xq, (int)nq, d, p, p->topk_out, serve_kp_final(p), w.sw.parts_final, gs, (int)ng, w.sw, w.sw.stats, idx_out,
+  return serve_knn(Xq, (int)nq, d, p, elt_of(p), p->topk_out, serve_kp_final(p), w.sw.parts_final, gs, (int)ng, w.sw, w.sw.stats, idx_out,
                    dist_out, st, bf ? &w.ball : nullptr);
 }
 
@@ -1151,7 +1154,8 @@ int gcr_gallery_build(const float* Xg, int64_t ng, int32_t d, const gcr_params* 
   cudaStream_t st = (cudaStream_t)stream;
   const int n = (int)ng;
   const bool bf = tensor_mode(p);
-  const size_t es = elt_size(p);
+  const Elt elt = serve_elt(p);
+  const size_t es = elt_bytes(elt);
   GCR_CUDA_TRY(launch_normalize(Xg, g.layers, ng, d, st));
   for (int t = 0; t < p->T; ++t) {
     float* cur = g.layers + (size_t)t * n * d;
@@ -1167,7 +1171,7 @@ int gcr_gallery_build(const float* Xg, int64_t ng, int32_t d, const gcr_params* 
   }
   for (int t = 0; t <= p->T; ++t) {
     GCR_CUDA_TRY(launch_row_stats(g.layers + (size_t)t * n * d, n, d, g.n64 + (size_t)t * n, g.n32 + (size_t)t * n,
-                                  bf ? g.xr + (size_t)t * n * d * es : nullptr, elt_of(p),
+                                  bf ? g.xr + (size_t)t * n * d * es : nullptr, elt,
                                   bf ? g.enrm + (size_t)t * n : nullptr,
                                   bf ? g.anrm + (size_t)t * n : nullptr, g.sc + t, st));
   }
@@ -1178,7 +1182,7 @@ size_t gcr_serve_workspace_size(int64_t b, int64_t ng, int32_t d, const gcr_para
   Resolved r;
   if (b < 1 || check_serve_params(p, ng, d, &r) != GCR_OK) return 0;
   Carve c(nullptr, 0);
-  return carve_serve(c, b, ng, d, p, r, nullptr) + 256;
+  return carve_serve(c, b, ng, d, p, serve_elt(p), r, nullptr) + 256;
 }
 
 int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq, int64_t b, int32_t d,
@@ -1194,7 +1198,7 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
   if (!ws) return GCR_E_WORKSPACE;
   Carve cw(ws, ws_bytes);
   ServeWs w;
-  if (carve_serve(cw, b, ng, d, p, r, &w) > ws_bytes) return GCR_E_WORKSPACE;
+  if (carve_serve(cw, b, ng, d, p, serve_elt(p), r, &w) > ws_bytes) return GCR_E_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   unsigned long long* stp = stats ? reinterpret_cast<unsigned long long*>(stats) : w.stats;
   const int nq = (int)b, n = (int)ng;
@@ -1205,7 +1209,7 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
   int cur = 0;
   for (int t = 0; t < p->T; ++t) {
     if (p->k > 0) {
-      s = serve_knn(w.xq[cur], nq, d, p, p->k, r.kp, w.parts, gallery_layer(g, t, n, d, elt_size(p)), n, w, stp, w.nbr, w.d2,
+      s = serve_knn(w.xq[cur], nq, d, p, serve_elt(p), p->k, r.kp, w.parts, gallery_layer(g, t, n, d, elt_bytes(serve_elt(p))), n, w, stp, w.nbr, w.d2,
                     st);
       if (s != GCR_OK) return s;
     }
@@ -1214,7 +1218,7 @@ int gcr_serve(const void* state, size_t state_bytes, int64_t ng, const float* Xq
                                    w.d2, p->k, p->gamma, p->symmetric, w.xq[cur ^ 1], st));
     cur ^= 1;
   }
-  return serve_knn(w.xq[cur], nq, d, p, p->topk_out, serve_kp_final(p), w.parts_final, gallery_layer(g, p->T, n, d, elt_size(p)), n, w, stp,
+  return serve_knn(w.xq[cur], nq, d, p, serve_elt(p), p->topk_out, serve_kp_final(p), w.parts_final, gallery_layer(g, p->T, n, d, elt_bytes(serve_elt(p))), n, w, stp,
                    idx_out, dist_out, st);
 }
 

@@ -9,9 +9,17 @@ namespace gcr {
 struct Carve;     // bump allocator over a caller's workspace (common.cuh)
 struct BallArgs;  // ball search of the pairs a pool could not certify (below)
 
-// Element type of the tensor-core GEMM operands: BF16 copies of the rows, or FP32 rows
-// rounded to TF32 (10 explicit mantissa bits, low 13 bits zero).
-enum class Elt : int { BF16 = 0, TF32 = 1 };
+// Element type of the tensor-core GEMM operands: BF16 copies of the rows; FP32 rows rounded to
+// TF32 (10 explicit mantissa bits, low 13 bits zero); or F16, which holds the same TF32-rounded
+// values times kF16Scale: TF32 and FP16 have the same 10 explicit mantissa bits, and unit rows
+// times 2^14 stay below FP16's largest number and keep all 11 significant bits down to elements of
+// 2^-28 (the largest of a unit row is at least 2^-6). The GEMM reads half the bytes and runs at
+// twice the kind::tf32 rate; its scores are kF16Scale^2 times the products of the rows. The
+// serving searches use it, whose rows are always normalised and whose distances come from the
+// FP32 rows whichever way a neighbour was certified. The offline graphs keep TF32: their scores
+// decide, to the last bit, which pairs the ball search takes, and its distances round otherwise.
+enum class Elt : int { BF16 = 0, TF32 = 1, F16 = 2 };
+constexpr float kF16Scale = 16384.f;
 // The device this library is written for: its SMs and L2 bytes size grids and workspaces (the
 // workspace queries run without a device).
 constexpr int kSMs = 152;
@@ -28,7 +36,7 @@ struct RowScalars {
 
 // ---- prep.cu
 cudaError_t launch_normalize(const float* X_in, float* X_out, int64_t n, int d, cudaStream_t st);
-// xr (may be NULL): the rounded operand copy (BF16, or TF32 held as FP32) written alongside
+// xr (may be NULL): the rounded operand copy (BF16, F16 of unit rows, or TF32 held as FP32) written alongside
 // the rounding-error norms enrm and the norms of the rounded rows anrm.
 cudaError_t launch_row_stats(const float* X, int n, int d, double* n64, float* n32,
                              void* xr, Elt elt, float* enrm, float* anrm, RowScalars* sc,
@@ -69,7 +77,7 @@ cudaError_t launch_sgemm_band(const float* X, const float* Bm, int n, int d, con
 cudaError_t launch_sgemm_dist(const float* Xq, int nq, const float* Xg, int ng, int d,
                               const float* nrm_q, const float* nrm_g, float* D, cudaStream_t st);
 
-// ---- umma.cu (tcgen05 path; operands BF16 or TF32)
+// ---- umma.cu (tcgen05 path; operands BF16, F16 or TF32; scores and thresholds in the operands' scale)
 // Pools [kind][na][kp] of the rows of S = A . B^T, kp = 32, 64 or 128, sorted best first and
 // padded with (-inf, -1): every score left out of a full pool is <= its last entry.
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
@@ -117,6 +125,7 @@ struct RefineArgs {
   const float* enrm;        // rounding statistics of the rows of X (tensor-core paths)
   const float* anrm;
   const RowScalars* sc;     // maxima over the rows of XB
+  float scale;              // of the pools' and the band's scores (a power of two)
   const float* pool_v;      // [kinds][n][kp]
   const int* pool_i;
   int kp;

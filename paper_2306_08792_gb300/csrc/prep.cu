@@ -1,5 +1,6 @@
 // Row normalisation (S0) and the per-row statistics used by the certified kNN search.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 
@@ -33,8 +34,8 @@ __global__ void normalize_kernel(const float* __restrict__ X_in, float* __restri
 }
 
 // n64[i] = ||x_i||^2 (float-float accumulation, combined in FP64), n32[i] = its FP32 rounding;
-// with xr != NULL also the rounded operand copy xr = round(x) (BF16 round-to-nearest-even, or
-// TF32 as above, held as FP32), enrm[i] >= ||round(x_i) - x_i|| and anrm[i] >= ||round(x_i)||
+// with xr != NULL also the rounded operand copy xr = round(x) (BF16 round-to-nearest-even; TF32
+// as above, held as FP32; or F16, the TF32-rounded value times kF16Scale), enrm[i] >= ||round(x_i) - x_i|| and anrm[i] >= ||round(x_i)||
 // (FP32 sums rounded up by a relative margin that covers their own accumulation error: at most
 // (d/32 + 5) * 2^-24 < 1e-3 for d <= 4096). Each difference round(x) - x is exact in FP32.
 // The min / max of those over the rows go to sc: every value is non-negative, so the bit
@@ -75,6 +76,15 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const float* __restrict_
           o[1] = __halves2bfloat162(b2, b3);
           f0 = __bfloat162float(b0); f1 = __bfloat162float(b1);
           f2 = __bfloat162float(b2); f3 = __bfloat162float(b3);
+        } else if constexpr (E == Elt::F16) {
+          const __half2 h01 = __floats2half2_rn(round_tf32(x.x) * kF16Scale, round_tf32(x.y) * kF16Scale);
+          const __half2 h23 = __floats2half2_rn(round_tf32(x.z) * kF16Scale, round_tf32(x.w) * kF16Scale);
+          uint2 o;
+          o.x = *reinterpret_cast<const unsigned*>(&h01);
+          o.y = *reinterpret_cast<const unsigned*>(&h23);
+          *reinterpret_cast<uint2*>(static_cast<__half*>(xr) + (size_t)row * d + 4 * v) = o;
+          f0 = __low2float(h01) * (1.f / kF16Scale); f1 = __high2float(h01) * (1.f / kF16Scale);
+          f2 = __low2float(h23) * (1.f / kF16Scale); f3 = __high2float(h23) * (1.f / kF16Scale);
         } else {
           f0 = round_tf32(x.x); f1 = round_tf32(x.y);
           f2 = round_tf32(x.z); f3 = round_tf32(x.w);
@@ -190,7 +200,9 @@ cudaError_t launch_row_stats(const float* X, int n, int d, double* n64, float* n
   if (e != cudaSuccess) return e;
   // 8 rows per block per pass; one wave of 6 blocks (40 registers a thread) on each of the 152 SMs
   const int blocks = std::max(1, std::min((n + 7) / 8, 152 * 6));
-  if (elt == Elt::TF32)
+  if (elt == Elt::F16)
+    row_stats_kernel<Elt::F16><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc);
+  else if (elt == Elt::TF32)
     row_stats_kernel<Elt::TF32><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc);
   else
     row_stats_kernel<Elt::BF16><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc);

@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
   int mvalid = 0;
 #pragma unroll
   for (int p = 0; p < P; ++p) {
-    pval[p] = pv[p * 32 + lane];
+    pval[p] = pv[p * 32 + lane] / a.scale;  // (exact: a power of two)
     L.id[p] = pi[p * 32 + lane];
     L.key[p] = kNoKey;
     L.val[p] = 0.f;
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
         const int u = atomicAdd(a.unc_count, 1);
         a.unc_row[u] = row;
         a.unc_kind[u] = kind;
-        a.unc_thr[u] = __double2float_rd(sig_k - eps + 0.5 * sc.nmin - delta);
+        a.unc_thr[u] = __double2float_rd(sig_k - eps + 0.5 * sc.nmin - delta) * a.scale;
         // negative (never -0): the pair's band is predicted to overflow
         if (a.unc_dk) a.unc_dk[u] = dense ? -fmaxf(dk, 1e-30f) : dk;
       }
@@ -518,7 +518,9 @@ __global__ void __launch_bounds__(256) refine_band_block_kernel(RefineArgs a) {
     const int* bi = a.band_i + (size_t)u * a.bcap;
     const float* bv = a.band_v + (size_t)u * a.bcap;
     const int kb = min(a.k, cnt);
-    const double thr = kb > 0 ? (double)band_kth(bv, cnt, kb, lane) - 2.0 * delta - 0.5 * (sc.nmax - sc.nmin)
+    // (in the scale of the band's scores)
+    const double thr = kb > 0 ? (double)band_kth(bv, cnt, kb, lane) -
+                                    (2.0 * delta + 0.5 * (sc.nmax - sc.nmin)) * (double)a.scale
                               : -CUDART_INF;
     // every warp lists the selected entries in band order (the same values to the same slots)
     int total = 0;
@@ -587,7 +589,9 @@ __global__ void __launch_bounds__(256, 3) refine_band_kernel(RefineArgs a) {
     const int* bi = a.band_i + (size_t)u * a.bcap;
     const float* bv = a.band_v + (size_t)u * a.bcap;
     const int kb = min(a.k, cnt);
-    const double thr = kb > 0 ? (double)band_kth(bv, cnt, kb, lane) - 2.0 * delta - 0.5 * (sc.nmax - sc.nmin)
+    // (in the scale of the band's scores)
+    const double thr = kb > 0 ? (double)band_kth(bv, cnt, kb, lane) -
+                                    (2.0 * delta + 0.5 * (sc.nmax - sc.nmin)) * (double)a.scale
                               : -CUDART_INF;
     // selected entries are staged per warp (at most 31 left over + 32 new) and re-scored 32 at
     // a time

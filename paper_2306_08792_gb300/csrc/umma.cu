@@ -1,8 +1,8 @@
 // Similarity GEMM on the 5th-generation tensor cores (tcgen05), sm_103a.
 //
-// S = A . B^T with A, B row-major (K = d contiguous, "K-major"), either BF16 or FP32 rows
-// rounded to TF32: A holds 128 rows of X, B 256 rows. Per CTA:
-//   warp 0        TMA producer: 128-byte K blocks (64 BF16 or 32 TF32 elements) of A (128 rows)
+// S = A . B^T with A, B row-major (K = d contiguous, "K-major"), BF16 or scaled FP16 rows or FP32
+// rows rounded to TF32: A holds 128 rows of X, B 256 rows. Per CTA:
+//   warp 0        TMA producer: 128-byte K blocks (64 16-bit or 32 TF32 elements) of A (128 rows)
 //                 and B (256 rows) into a 3-stage shared-memory ring (128-byte swizzle),
 //                 mbarrier transaction counts;
 //   warp 1        allocates 512 TMEM columns (two 128 x 256 FP32 accumulators) and, from one
@@ -123,17 +123,19 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
   d |= (uint64_t)2 << 61;                          // layout: 128-byte swizzle
   return d;
 }
-// Instruction descriptors: D = F32 (bits 4-5 = 1), A and B formats (bits 7-9, 10-12: BF16 = 1
-// under kind::f16, TF32 = 2 under kind::tf32), both K-major, N >> 3 (bits 17-22), M >> 4
+// Instruction descriptors: D = F32 (bits 4-5 = 1), A and B formats (bits 7-9, 10-12: F16 = 0 and
+// BF16 = 1 under kind::f16, TF32 = 2 under kind::tf32), both K-major, N >> 3 (bits 17-22), M >> 4
 // (bits 24-28); N = 256, M = 128.
 constexpr uint32_t kIdescShape = ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 constexpr uint32_t kIdescBf16 = (1u << 4) | (1u << 7) | (1u << 10) | kIdescShape;
+constexpr uint32_t kIdescF16 = (1u << 4) | kIdescShape;
 constexpr uint32_t kIdescTf32 = (1u << 4) | (2u << 7) | (2u << 10) | kIdescShape;
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accum) {
+__device__ __forceinline__ void umma_16bit(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accum) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(kIdescBf16), "r"(accum));
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum));
 }
 __device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accum) {
   asm volatile(
@@ -202,7 +204,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 // ------------------------------------------------------------------------ kernel
 struct UmmaArgs {
   int mode;
-  int tf32;       // operands: 0 BF16 (kind::f16), 1 TF32 held as FP32 (kind::tf32)
+  int tf32;       // operands: 0 16-bit (kind::f16), 1 TF32 held as FP32 (kind::tf32)
+  uint32_t idesc; // instruction descriptor of 16-bit operands
   int n;          // rows of B (columns of S)
   int d;
   int a_rows;     // rows of A (POOL: rows owning pools; DIST: nq; BAND: band capacity)
@@ -570,7 +573,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             for (int k = 0; k < 4; ++k) umma_tf32(dcol, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), (kb | k) != 0);
           } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) umma_bf16(dcol, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), (kb | k) != 0);
+            for (int k = 0; k < 4; ++k) umma_16bit(dcol, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), a.idesc, (kb | k) != 0);
           }
           if (MODE == POOL && a.mc) umma_commit_mc(&bars.empty[s], (uint16_t)0x3);
           else umma_commit(&bars.empty[s]);
@@ -911,7 +914,10 @@ cudaError_t make_map(CUtensorMap* m, const void* base, Elt elt, int rows, int d,
   cuuint64_t strides[1] = {(cuuint64_t)step * d * es};
   cuuint32_t box[2] = {(cuuint32_t)(BKB / es), (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(m, elt == Elt::TF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+  CUresult r = fn(m,
+                  elt == Elt::TF32  ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                  : elt == Elt::F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                    : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                   const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -1055,6 +1061,7 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
   UmmaArgs a{};
   a.mode = POOL;
   a.tf32 = elt == Elt::TF32;
+  a.idesc = elt == Elt::F16 ? kIdescF16 : kIdescBf16;
   a.n = nb;
   a.d = d;
   a.a_rows = na;
@@ -1116,6 +1123,7 @@ cudaError_t launch_umma_gpool(const void* Y, int rows, int d, Elt elt, const int
   UmmaArgs a{};
   a.mode = GPOOL;
   a.tf32 = elt == Elt::TF32;
+  a.idesc = elt == Elt::F16 ? kIdescF16 : kIdescBf16;
   a.n = rows;
   a.d = d;
   a.a_rows = rows;
@@ -1146,6 +1154,7 @@ cudaError_t launch_umma_band(const void* Xb, int n, int d, Elt elt, const int* c
   UmmaArgs a{};
   a.mode = BAND;
   a.tf32 = elt == Elt::TF32;
+  a.idesc = elt == Elt::F16 ? kIdescF16 : kIdescBf16;
   a.n = n;
   a.d = d;
   a.a_rows = cap;
@@ -1179,6 +1188,7 @@ cudaError_t launch_umma_dist(const __nv_bfloat16* Qb, int nq, const __nv_bfloat1
   if (e != cudaSuccess) return e;
   UmmaArgs a{};
   a.mode = DIST;
+  a.idesc = kIdescBf16;
   a.n = ng;
   a.d = d;
   a.a_rows = nq;
@@ -1208,6 +1218,7 @@ cudaError_t launch_umma_gram(const __nv_bfloat16* zt_hi, const __nv_bfloat16* zt
   if (e != cudaSuccess) return e;
   UmmaArgs a{};
   a.mode = GRAM;
+  a.idesc = kIdescBf16;
   a.n = d;
   a.d = 64;  // unused: the K extent of a tile comes from gram_knum
   a.a_rows = d;
