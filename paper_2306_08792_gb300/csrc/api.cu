@@ -58,6 +58,12 @@ Elt elt_of(const gcr_params* p) { return p->precision == GCR_PREC_TF32 ? Elt::TF
 // Operands of the serving searches (normalised rows, no ball search): TF32's values in 16 bits.
 Elt serve_elt(const gcr_params* p) { return p->precision == GCR_PREC_TF32 ? Elt::F16 : Elt::BF16; }
 size_t elt_size(const gcr_params* p) { return elt_bytes(elt_of(p)); }
+// The first layer of a large offline problem (see Elt): from about 0.4 ms of TF32 sweep, of which
+// F16 saves more than the 11 launches (25 us) that the repetition costs when it is not needed.
+// 19,281 rows of d = 2048: the sweep 1.9 -> 1.0 ms; 201,000 of d = 512: 58 -> 39 ms.
+bool f16_first(const gcr_params* p, const Resolved& r, int64_t n, int32_t d) {
+  return p->precision == GCR_PREC_TF32 && p->k > 0 && !(r.kp == 128 && r.kinds == 2) && 2.0 * (double)n * (double)n * d > 3e11;
+}
 
 int check_precision(const gcr_params* p, int32_t d) {
   if (p->precision != GCR_PREC_FP32 && p->precision != GCR_PREC_BF16 && p->precision != GCR_PREC_TF32)
@@ -121,11 +127,15 @@ struct BuildWs {
   float* n32;
   RowScalars* sc;
   void* xr;            // rounded operand copy (tensor-core modes)
+  void* xr16;          // the first layer's F16 copy (f16_first), its repetition flag and counters
+  int* repeat;
+  unsigned long long* saved;
   float* enrm;
   float* anrm;
   float* pool_v;
   int* pool_i;
   PoolParts parts;     // the sweep's split buffers
+  PoolParts parts16;
   int* unc_count;
   int* unc_row;
   int* unc_kind;
@@ -180,11 +190,22 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.n32 = c.take<float>(nn);
   t.sc = c.take<RowScalars>(1);
   t.xr = bf ? c.take<char>(nn * d * es) : nullptr;
+  const bool f16 = f16_first(p, r, n, d);
+  t.xr16 = f16 ? c.take<char>(nn * d * 2) : nullptr;
+  t.repeat = f16 ? c.take<int>(1) : nullptr;
+  t.saved = f16 ? c.take<unsigned long long>(GCR_STATS_LEN) : nullptr;
   t.enrm = bf ? c.take<float>(nn) : nullptr;
   t.anrm = bf ? c.take<float>(nn) : nullptr;
   t.pool_v = c.take<float>((size_t)kinds * nn * r.kp);
   t.pool_i = c.take<int>((size_t)kinds * nn * r.kp);
-  t.parts = carve_parts(c, (int)n, (int)n, d, p, elt_of(p), r.kp, kinds == 2);
+  {
+    Carve c16 = c;
+    t.parts = carve_parts(c, (int)n, (int)n, d, p, elt_of(p), r.kp, kinds == 2);
+    if (f16) {  // one region for both searches
+      t.parts16 = carve_parts(c16, (int)n, (int)n, d, p, Elt::F16, r.kp, kinds == 2);
+      c.off = std::max(c.off, c16.off);
+    }
+  }
   t.unc_count = c.take<int>(8 + (size_t)band_rows);
   t.err = t.unc_count + 4;
   t.band_cnt = t.unc_count + 8;
@@ -232,19 +253,27 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
 }
 
 // The certified kNN search of Eq. 4 / Eq. 8 (S1-S3): writes g->nbr / nbr_d2 (and the
-// cross-camera lists), g->row_order when given, and the search counters.
+// cross-camera lists), g->row_order when given, and the search counters. first: the rows are the
+// normalised input of a first layer (f16_first may apply).
 int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const gcr_params* p, const Resolved& r,
-             gcr_graph* g, const BuildWs& w, cudaStream_t st) {
+             gcr_graph* g, const BuildWs& w, bool first, cudaStream_t st) {
   const int n = (int)n64_;
   const int kinds = r.kinds;
   const bool bf = tensor_mode(p);
+  const bool f16 = first && f16_first(p, r, n64_, d);
   const Elt elt = elt_of(p);
   unsigned long long* stats = g->stats ? reinterpret_cast<unsigned long long*>(g->stats) : w.stats;
   if (!g->stats) GCR_CUDA_TRY(cudaMemsetAsync(w.stats, 0, sizeof(unsigned long long) * GCR_STATS_LEN, st));
 
   {
     StageScope sc_(GCR_STAGE_PREP, st, 2);
-    GCR_CUDA_TRY(launch_row_stats(X, n, d, w.n64, w.n32, bf ? w.xr : nullptr, elt, w.enrm, w.anrm, w.sc, st));
+    if (f16) {
+      GCR_CUDA_TRY(launch_row_stats(X, n, d, w.n64, w.n32, w.xr16, Elt::F16, w.enrm, w.anrm, w.sc, st));
+      GCR_CUDA_TRY(cudaMemcpyAsync(w.saved, stats, sizeof(unsigned long long) * GCR_STATS_LEN,
+                                   cudaMemcpyDeviceToDevice, st));
+    } else {
+      GCR_CUDA_TRY(launch_row_stats(X, n, d, w.n64, w.n32, bf ? w.xr : nullptr, elt, w.enrm, w.anrm, w.sc, st));
+    }
   }
   // pending-pair count, error word and band counts together
   GCR_CUDA_TRY(cudaMemsetAsync(w.unc_count, 0, sizeof(int) * (8 + (size_t)w.band_rows), st));
@@ -252,7 +281,10 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
 
   if (p->k > 0) {
     StageScope sc_(GCR_STAGE_SIM_GEMM, st);
-    if (bf) {
+    if (f16) {
+      GCR_CUDA_TRY(launch_umma_pool(w.xr16, n, w.xr16, n, d, Elt::F16, camp, p->cross_camera != 0, 1, r.kp, w.parts16,
+                                    w.pool_v, w.pool_i, st));
+    } else if (bf) {
       GCR_CUDA_TRY(launch_umma_pool(w.xr, n, w.xr, n, d, elt, camp, p->cross_camera != 0, 1, r.kp, w.parts,
                                     w.pool_v, w.pool_i, st));
     } else {
@@ -264,7 +296,7 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
   RefineArgs ra;
   std::memset(&ra, 0, sizeof(ra));
   ra.X = X; ra.XB = X; ra.n = n; ra.d = d; ra.k = p->k; ra.kinds = kinds; ra.precision = p->precision;
-  ra.n64 = w.n64; ra.n64B = w.n64; ra.enrm = w.enrm; ra.anrm = w.anrm; ra.sc = w.sc; ra.scale = 1.f;
+  ra.n64 = w.n64; ra.n64B = w.n64; ra.enrm = w.enrm; ra.anrm = w.anrm; ra.sc = w.sc; ra.scale = f16 ? kF16Scale * kF16Scale : 1.f;
   ra.pool_v = w.pool_v; ra.pool_i = w.pool_i; ra.kp = r.kp;
   ra.nbr[0] = g->nbr; ra.d2[0] = g->nbr_d2;
   ra.nbr[1] = kinds == 2 ? g->nbr_cr : g->nbr;
@@ -295,6 +327,21 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
       }
       GCR_CUDA_TRY(launch_refine_pool(ra, st));
     }
+    // F16: where a ball search would run, everything again on TF32 (decided on the device: the
+    // launches below return at once otherwise)
+    RefineArgs r16 = ra;  // the rescan of a search that stays on F16
+    const Gate again{f16 ? w.repeat : nullptr, 1};
+    if (f16) {
+      StageScope sc_(GCR_STAGE_SIM_GEMM, st, 7);
+      GCR_CUDA_TRY(launch_search_gate(w.unc_row, w.unc_dk, w.unc_count, kinds * n, w.n64, w.saved, stats, w.repeat, st));
+      GCR_CUDA_TRY(launch_row_stats(X, n, d, w.n64, w.n32, w.xr, elt, w.enrm, w.anrm, w.sc, st, again));
+      GCR_CUDA_TRY(launch_umma_pool(w.xr, n, w.xr, n, d, elt, camp, p->cross_camera != 0, 1, r.kp, w.parts, w.pool_v,
+                                    w.pool_i, st, again));
+      ra.scale = 1.f;
+      ra.gate = again;
+      GCR_CUDA_TRY(launch_refine_pool(ra, st));
+      ra.gate = Gate();
+    }
     // the queue the band rescan takes: the ball search's leftovers, or the refinement's queue
     RefineArgs rb = ra;
     if (bf) {
@@ -315,12 +362,24 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
       rb.unc_count = w.bq_count; rb.unc_row = w.bq_row; rb.unc_kind = w.bq_kind; rb.unc_thr = w.bq_thr;
     }
     // threshold rescan of the pairs still uncertified
-    StageScope sc_(GCR_STAGE_BAND, st, bf ? 3 : 2);
+    StageScope sc_(GCR_STAGE_BAND, st, f16 ? 6 : bf ? 3 : 2);
+    if (f16) {
+      r16.gate = Gate{w.repeat, 0};
+      r16.unc_count = rb.unc_count; r16.unc_row = rb.unc_row; r16.unc_kind = rb.unc_kind; r16.unc_thr = rb.unc_thr;
+      GCR_CUDA_TRY(launch_gather_rows(w.xr16, (size_t)d * 2, rb.unc_count, rb.unc_row, w.band_rows, w.band_a, st,
+                                      r16.gate));
+      GCR_CUDA_TRY(launch_umma_band(w.xr16, n, d, Elt::F16, camp, 1, w.band_a, rb.unc_count, w.band_rows, rb.unc_row,
+                                    rb.unc_kind, rb.unc_thr, kBandCap, w.band_cnt, w.band_v, w.band_i, st, nullptr,
+                                    nullptr, r16.gate));
+      GCR_CUDA_TRY(launch_refine_band(r16, st));
+      rb.gate = again;
+    }
     if (bf) {
       GCR_CUDA_TRY(launch_gather_rows(w.xr, (size_t)d * elt_bytes(elt), rb.unc_count, rb.unc_row, w.band_rows,
-                                      w.band_a, st));
+                                      w.band_a, st, again));
       GCR_CUDA_TRY(launch_umma_band(w.xr, n, d, elt, camp, 1, w.band_a, rb.unc_count, w.band_rows, rb.unc_row,
-                                    rb.unc_kind, rb.unc_thr, kBandCap, w.band_cnt, w.band_v, w.band_i, st));
+                                    rb.unc_kind, rb.unc_thr, kBandCap, w.band_cnt, w.band_v, w.band_i, st, nullptr,
+                                    nullptr, again));
     } else {
       GCR_CUDA_TRY(launch_sgemm_band(X, X, n, d, camp, 1, rb.unc_count, w.band_rows, rb.unc_row, rb.unc_kind,
                                      rb.unc_thr, kBandCap, w.band_cnt, w.band_v, w.band_i, st));
@@ -342,10 +401,10 @@ OrderStream g_order_side[kMaxOrderDevices];
 std::mutex g_order_mu;
 
 int build_graph_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const gcr_params* p,
-                     const Resolved& r, gcr_graph* g, const BuildWs& w, cudaStream_t st) {
+                     const Resolved& r, gcr_graph* g, const BuildWs& w, bool first, cudaStream_t st) {
   const int n = (int)n64_;
   const int kinds = r.kinds;
-  const int s = knn_impl(X, n64_, d, cam, p, r, g, w, st);
+  const int s = knn_impl(X, n64_, d, cam, p, r, g, w, first, st);
   if (s != GCR_OK) return s;
 
   GraphArgs ga;
@@ -855,7 +914,7 @@ int pipeline_impl(const float* X, int64_t n, int64_t nq, int32_t d, const int32_
     Carve cb(w.inner, w.inner_bytes);
     BuildWs bw;
     carve_build(cb, n, d, p, r, &bw);
-    s = build_graph_impl(cur, n, d, cam, p, r, &w.g, bw, st);
+    s = build_graph_impl(cur, n, d, cam, p, r, &w.g, bw, t == 0, st);
     if (s != GCR_OK) return s;
     {
       StageScope sc_(GCR_STAGE_PROPAGATE, st);
@@ -1044,7 +1103,7 @@ int gcr_build_graph(const float* X, int64_t n, int32_t d, const int32_t* cam, co
   Carve c(ws, ws_bytes);
   BuildWs w;
   if (carve_build(c, n, d, p, r, &w) > ws_bytes) return GCR_E_WORKSPACE;
-  return build_graph_impl(X, n, d, cam, p, r, g, w, (cudaStream_t)stream);
+  return build_graph_impl(X, n, d, cam, p, r, g, w, false, (cudaStream_t)stream);
 }
 
 int gcr_propagate(const gcr_graph* g, const float* X_in, float* X_out, int64_t n, int32_t d, gcr_stream_t stream) {
@@ -1163,7 +1222,7 @@ int gcr_gallery_build(const float* Xg, int64_t ng, int32_t d, const gcr_params* 
     Carve cb(w.inner, w.inner_bytes);
     BuildWs bw;
     carve_build(cb, ng, d, p, r, &bw);
-    s = build_graph_impl(cur, ng, d, nullptr, p, r, &w.g, bw, st);
+    s = build_graph_impl(cur, ng, d, nullptr, p, r, &w.g, bw, t == 0, st);
     if (s != GCR_OK) return s;
     GCR_CUDA_TRY(launch_layer_degree(w.g.deg_r, w.g.deg_c, n, p->symmetric, g.deg + (size_t)t * n, st));
     GCR_CUDA_TRY(launch_propagate(w.g.op_rowptr, w.g.op_len, w.g.op_col, w.g.op_val, cur, nxt, n, d,
@@ -1347,7 +1406,7 @@ int gcr_dsfp(const float* X, int64_t n, int32_t d, const gcr_params* p, float* X
     g.nbr = nbr;
     g.nbr_d2 = w.d2;
     g.stats = stats;
-    s = knn_impl(w.Xn, n, d, nullptr, p, r, &g, w.bw, st);
+    s = knn_impl(w.Xn, n, d, nullptr, p, r, &g, w.bw, true, st);
     if (s != GCR_OK) return s;
   }
   StageScope sc_(GCR_STAGE_PROPAGATE, st);

@@ -544,7 +544,35 @@ __global__ void order_scatter_kernel2(const int* root, const int* off, int n, in
   }
 }
 
+// The decision of ball_go over the pending pairs of a search, by one block.
+__global__ void __launch_bounds__(1024) search_gate_kernel(const int* __restrict__ unc_row, const float* __restrict__ unc_dk,
+                                                           int* unc_count, int unc_cap, const double* __restrict__ n64,
+                                                           const unsigned long long* __restrict__ saved,
+                                                           unsigned long long* stats, int* flag) {
+  const int U = min(*unc_count, unc_cap);
+  int part = 0, dense = 0;
+  for (int u0 = 0; u0 < U; u0 += 1024) {
+    const int u = u0 + threadIdx.x;
+    const float dk = u < U ? unc_dk[u] : CUDART_INF_F;
+    const bool in = u < U && ball_participates(dk, n64[unc_row[u]]);
+    part += __syncthreads_count(in);
+    dense += __syncthreads_count(in && dk < 0.f);
+  }
+  const bool go = dense > 0 || part >= kMinBallPairs;
+  if (threadIdx.x == 0) *flag = go ? 1 : 0;
+  if (!go) return;
+  __syncthreads();
+  if (threadIdx.x == 0) *unc_count = 0;
+  if (threadIdx.x < GCR_STATS_LEN) stats[threadIdx.x] = saved[threadIdx.x];
+}
+
 }  // namespace
+
+cudaError_t launch_search_gate(const int* unc_row, const float* unc_dk, int* unc_count, int unc_cap, const double* n64,
+                               const unsigned long long* saved, unsigned long long* stats, int* flag, cudaStream_t st) {
+  search_gate_kernel<<<1, 1024, 0, st>>>(unc_row, unc_dk, unc_count, unc_cap, n64, saved, stats, flag);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_cluster_order(const int32_t* nbr, const float* d2, const double* n64, int n, int d, int k,
                                  const int* prev_key, int* parent, int* root, int* csize, int* cnt, int* off,

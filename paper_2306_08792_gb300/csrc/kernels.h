@@ -16,8 +16,10 @@ struct BallArgs;  // ball search of the pairs a pool could not certify (below)
 // 2^-28 (the largest of a unit row is at least 2^-6). The GEMM reads half the bytes and runs at
 // twice the kind::tf32 rate; its scores are kF16Scale^2 times the products of the rows. The
 // serving searches use it, whose rows are always normalised and whose distances come from the
-// FP32 rows whichever way a neighbour was certified. The offline graphs keep TF32: their scores
-// decide, to the last bit, which pairs the ball search takes, and its distances round otherwise.
+// FP32 rows whichever way a neighbour was certified. In an offline graph the scores decide, to the
+// last bit, which pairs the ball search takes, whose distances round otherwise: the first layer
+// of a large problem is searched on F16, and again on TF32 should a ball search turn out to run;
+// the other layers, which propagation has contracted, on TF32.
 enum class Elt : int { BF16 = 0, TF32 = 1, F16 = 2 };
 constexpr float kF16Scale = 16384.f;
 // The device this library is written for: its SMs and L2 bytes size grids and workspaces (the
@@ -25,6 +27,13 @@ constexpr float kF16Scale = 16384.f;
 constexpr int kSMs = 152;
 constexpr double kL2Bytes = 126e6;
 inline size_t elt_bytes(Elt e) { return e == Elt::TF32 ? 4 : 2; }
+
+// A kernel's launch condition, decided on the device: it runs when flag is NULL or *flag == want.
+struct Gate {
+  const int* flag = nullptr;
+  int want = 0;
+};
+__device__ __forceinline__ bool gate_shut(const Gate& g) { return g.flag && *g.flag != g.want; }
 
 // Per-call scalars reduced over the rows of X (device memory).
 struct RowScalars {
@@ -40,7 +49,7 @@ cudaError_t launch_normalize(const float* X_in, float* X_out, int64_t n, int d, 
 // the rounding-error norms enrm and the norms of the rounded rows anrm.
 cudaError_t launch_row_stats(const float* X, int n, int d, double* n64, float* n32,
                              void* xr, Elt elt, float* enrm, float* anrm, RowScalars* sc,
-                             cudaStream_t st);
+                             cudaStream_t st, Gate gate = Gate());
 // Squared norms of query and gallery rows and (qb != NULL, d % 8 == 0) their compensated BF16 operands.
 cudaError_t launch_rerank_prep(const float* Xq, int nq, const float* Xg, int ng, int d, float* n32q, float* n32g,
                                __nv_bfloat16* qb, __nv_bfloat16* gb, cudaStream_t st);
@@ -82,7 +91,7 @@ cudaError_t launch_sgemm_dist(const float* Xq, int nq, const float* Xg, int ng, 
 // padded with (-inf, -1): every score left out of a full pool is <= its last entry.
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
                              const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
-                             float* pool_v, int* pool_i, cudaStream_t st);
+                             float* pool_v, int* pool_i, cudaStream_t st, Gate gate = Gate());
 // Pools of row blocks of the gathered matrix Y (rows x d, rounded operand) against column ranges
 // of Y: work item w = {first row, rows <= 128, first column, columns} of *n_items (<= max_items);
 // pool entry (s - col_bias[j], j), j a position in Y; column j == row skipped when self_excl;
@@ -97,7 +106,7 @@ cudaError_t launch_umma_band(const void* Xb, int n, int d, Elt elt, const int* c
                              const void* Ab, const int* count, int cap, const int* band_row,
                              const int* band_kind, const float* band_thr, int bcap, int* band_cnt, float* band_v,
                              int* band_i, cudaStream_t st, const int* band_off = nullptr,
-                             const int* band_lim = nullptr);
+                             const int* band_lim = nullptr, Gate gate = Gate());
 cudaError_t launch_umma_dist(const __nv_bfloat16* Qb, int nq, const __nv_bfloat16* Gb, int ng, int d,
                              const float* nrm_q, const float* nrm_g, float* D, cudaStream_t st);
 // G_s = Z_s Z_s^T + lambda n_s I for every camera s (d x d, FP32, [ncam][d][d]), Z the
@@ -152,6 +161,7 @@ struct RefineArgs {
   const int* band_i;
   int bcap;
   int band_rows;            // capacity of the band buffers (rows beyond it are not rescanned)
+  Gate gate;
   const int* order;         // processing order of the rows (NULL: 0..n-1); results do not depend on it
 };
 cudaError_t launch_refine_pool(const RefineArgs& a, cudaStream_t st);
@@ -166,7 +176,12 @@ cudaError_t launch_row_order(const int* pool_i, int n, int kp, int k, int* key, 
 cudaError_t launch_identity_order(int* order, int n, cudaStream_t st);
 // Copies rows[u] of src (row_bytes each, a multiple of 16) to row u of out, u < min(*count, max_rows).
 cudaError_t launch_gather_rows(const void* src, size_t row_bytes, const int* count, const int* rows,
-                               int max_rows, void* out, cudaStream_t st);
+                               int max_rows, void* out, cudaStream_t st, Gate gate = Gate());
+// After a search on F16 operands: *flag = 1 where the ball search would run on its pending pairs
+// (see ball.cu); the pending queue is then emptied and the counters set back to `saved`, for
+// the search to be repeated on TF32 operands.
+cudaError_t launch_search_gate(const int* unc_row, const float* unc_dk, int* unc_count, int unc_cap, const double* n64,
+                               const unsigned long long* saved, unsigned long long* stats, int* flag, cudaStream_t st);
 
 // ---- ball.cu: certified search of the pending (row, graph) pairs inside balls shared by
 // groups of them, in coordinates centred on each ball (see ball.cu)
@@ -327,7 +342,7 @@ cudaError_t launch_gcrv(const float* frames, int64_t F, int d, const int64_t* of
 // Sorts and merges the S selection buffers of each (kind, row) ([S][kinds][na][cap], cnt entries)
 // into its pool [kinds][na][kp], best first, padded with (-inf, -1).
 cudaError_t launch_pool_finish(const float* pv, const int* pi, const int* cnt, int S, int kinds, int na, int cap, int kp,
-                               float* ov, int* oi, cudaStream_t st);
+                               float* ov, int* oi, cudaStream_t st, Gate gate = Gate());
 cudaError_t launch_merge_splits(const float* pv, const int* pi, int S, int kinds, int na, int kp, float* ov, int* oi,
                                 cudaStream_t st);
 cudaError_t launch_query_step(const float* xq, int b, int d, const float* G, const float* deg, const int32_t* nbr,

@@ -44,7 +44,8 @@ __global__ void normalize_kernel(const float* __restrict__ X_in, float* __restri
 // over the grid so that each block folds many rows before its four atomics.
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
 
-__global__ void row_scalars_init_kernel(RowScalars* __restrict__ sc) {
+__global__ void row_scalars_init_kernel(RowScalars* __restrict__ sc, Gate gate) {
+  if (gate_shut(gate)) return;
   sc->nmin = 1e300;
   sc->nmax = 0.0;
   sc->emax = 0.0;
@@ -55,7 +56,9 @@ template <Elt E>
 __global__ void __launch_bounds__(256) row_stats_kernel(const float* __restrict__ X, int n, int d,
                                                         double* __restrict__ n64, float* __restrict__ n32,
                                                         void* __restrict__ xr, float* __restrict__ enrm,
-                                                        float* __restrict__ anrm, RowScalars* __restrict__ sc) {
+                                                        float* __restrict__ anrm, RowScalars* __restrict__ sc,
+                                                        Gate gate) {
+  if (gate_shut(gate)) return;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int d4 = d >> 2;
   double nmin = 1e300, nmax = 0.0, emax = 0.0, amax = 0.0;
@@ -194,18 +197,18 @@ cudaError_t launch_normalize(const float* X_in, float* X_out, int64_t n, int d, 
 
 cudaError_t launch_row_stats(const float* X, int n, int d, double* n64, float* n32,
                              void* xr, Elt elt, float* enrm, float* anrm, RowScalars* sc,
-                             cudaStream_t st) {
-  row_scalars_init_kernel<<<1, 1, 0, st>>>(sc);
+                             cudaStream_t st, Gate gate) {
+  row_scalars_init_kernel<<<1, 1, 0, st>>>(sc, gate);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // 8 rows per block per pass; one wave of 6 blocks (40 registers a thread) on each of the 152 SMs
   const int blocks = std::max(1, std::min((n + 7) / 8, 152 * 6));
   if (elt == Elt::F16)
-    row_stats_kernel<Elt::F16><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc);
+    row_stats_kernel<Elt::F16><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc, gate);
   else if (elt == Elt::TF32)
-    row_stats_kernel<Elt::TF32><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc);
+    row_stats_kernel<Elt::TF32><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc, gate);
   else
-    row_stats_kernel<Elt::BF16><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc);
+    row_stats_kernel<Elt::BF16><<<blocks, 256, 0, st>>>(X, n, d, n64, n32, xr, enrm, anrm, sc, gate);
   return cudaGetLastError();
 }
 

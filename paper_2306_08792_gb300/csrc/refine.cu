@@ -375,6 +375,7 @@ __global__ void __launch_bounds__(256, 4) refine_pool_kernel(RefineArgs a) {
   const int lane = threadIdx.x & 31, warp = W > 1 ? threadIdx.x >> 5 : 0;
   const long wid = W > 1 ? (long)blockIdx.x : (long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const bool lead = lane == 0 && warp == 0;
+  if (gate_shut(a.gate)) return;
   if (wid >= (long)a.n * a.kinds) return;
   const int kind = (int)(wid / a.n);
   const int row = a.order ? a.order[wid % a.n] : (int)(wid % a.n);
@@ -503,6 +504,7 @@ __global__ void __launch_bounds__(256) refine_band_block_kernel(RefineArgs a) {
   __shared__ int ids[512];
   __shared__ float val[512];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (gate_shut(a.gate)) return;
   const int U = *a.unc_count;
   for (int u = blockIdx.x; u < U; u += gridDim.x) {
     const int row = a.unc_row[u], kind = a.unc_kind[u];
@@ -570,6 +572,7 @@ __global__ void __launch_bounds__(256, 3) refine_band_kernel(RefineArgs a) {
   __shared__ int sel_ids[8][64];
   const int lane = threadIdx.x & 31;
   int* sb = sel_ids[threadIdx.x >> 5];
+  if (gate_shut(a.gate)) return;
   const int U = *a.unc_count;
   const int nw = gridDim.x * 8;
   for (int u = blockIdx.x * 8 + (threadIdx.x >> 5); u < U; u += nw) {
@@ -751,7 +754,8 @@ __global__ void order_scatter_kernel(const int* __restrict__ key, const int* __r
 
 // Row gather in 16-byte units: w16 units per row.
 __global__ void gather_rows_kernel(const uint4* __restrict__ src, long w16, const int* __restrict__ count,
-                                   const int* __restrict__ rows, int max_rows, uint4* __restrict__ out) {
+                                   const int* __restrict__ rows, int max_rows, uint4* __restrict__ out, Gate gate) {
+  if (gate_shut(gate)) return;
   const int U = min(*count, max_rows);
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < (long)U * w16; t += (long)gridDim.x * blockDim.x) {
     const long u = t / w16, c = t % w16;
@@ -877,10 +881,10 @@ cudaError_t launch_row_order(const int* pool_i, int n, int kp, int k, int* key, 
 }
 
 cudaError_t launch_gather_rows(const void* src, size_t row_bytes, const int* count, const int* rows,
-                               int max_rows, void* out, cudaStream_t st) {
+                               int max_rows, void* out, cudaStream_t st, Gate gate) {
   if (row_bytes % 16) return cudaErrorInvalidValue;
   gather_rows_kernel<<<152 * 4, 256, 0, st>>>(static_cast<const uint4*>(src), (long)(row_bytes / 16), count, rows,
-                                              max_rows, static_cast<uint4*>(out));
+                                              max_rows, static_cast<uint4*>(out), gate);
   return cudaGetLastError();
 }
 

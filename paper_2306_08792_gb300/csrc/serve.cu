@@ -124,7 +124,8 @@ __device__ __forceinline__ void merge_chunk(float (&b)[KP / 32], int (&bi)[KP / 
 template <int KP, int W>
 __global__ void __launch_bounds__(W > 1 ? 32 * W : 256) pool_finish_kernel(
     const float* __restrict__ pv, const int* __restrict__ pi, const int* __restrict__ cnt, int S, long rows, int cap,
-    float* __restrict__ ov, int* __restrict__ oi) {
+    float* __restrict__ ov, int* __restrict__ oi, Gate gate) {
+  if (gate_shut(gate)) return;
   constexpr int P = KP / 32, NW = W > 1 ? W : 8;
   __shared__ float stv[NW][64];
   __shared__ int sti[NW][64];
@@ -288,20 +289,20 @@ cudaError_t launch_merge_splits(const float* pv, const int* pi, int S, int kinds
 
 template <int KP>
 static void pool_finish(const float* pv, const int* pi, const int* cnt, int S, long rows, int cap, float* ov, int* oi,
-                        cudaStream_t st) {
+                        cudaStream_t st, Gate gate) {
   // a warp per row; a block per row where there are many splits' buffers to merge, with more
   // warps where the rows alone do not fill the GPU
-  if (S <= 8) pool_finish_kernel<KP, 1><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi);
-  else if (rows >= 4 * kSMs) pool_finish_kernel<KP, 8><<<(unsigned)rows, 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi);
-  else pool_finish_kernel<KP, 16><<<(unsigned)rows, 512, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi);
+  if (S <= 8) pool_finish_kernel<KP, 1><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
+  else if (rows >= 4 * kSMs) pool_finish_kernel<KP, 8><<<(unsigned)rows, 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
+  else pool_finish_kernel<KP, 16><<<(unsigned)rows, 512, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
 }
 
 cudaError_t launch_pool_finish(const float* pv, const int* pi, const int* cnt, int S, int kinds, int na, int cap, int kp,
-                               float* ov, int* oi, cudaStream_t st) {
+                               float* ov, int* oi, cudaStream_t st, Gate gate) {
   const long rows = (long)kinds * na;
-  if (kp == 32) pool_finish<32>(pv, pi, cnt, S, rows, cap, ov, oi, st);
-  else if (kp == 64) pool_finish<64>(pv, pi, cnt, S, rows, cap, ov, oi, st);
-  else if (kp == 128) pool_finish<128>(pv, pi, cnt, S, rows, cap, ov, oi, st);
+  if (kp == 32) pool_finish<32>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
+  else if (kp == 64) pool_finish<64>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
+  else if (kp == 128) pool_finish<128>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

@@ -270,6 +270,7 @@ struct UmmaArgs {
   // CTAs by TMA multicast (tmB2: B in 128-row boxes), so a CTA reads two thirds of the bytes
   // per stage. Each MMA commit frees the stage in both CTAs (empty barriers count 2 arrivals).
   int mc;
+  Gate gate;       // POOL, BAND: whether this launch runs
 };
 
 struct __align__(8) Bars {
@@ -443,6 +444,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   constexpr int KINDS = CROSS ? 2 : 1;
   __shared__ Bars bars;
 
+  if ((MODE == POOL || MODE == BAND) && gate_shut(a.gate)) return;  // (every CTA alike, before any barrier)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bk = a.tf32 ? BKB / 4 : BKB / 2;  // K elements per stage
   // K blocks per tile (GRAM: three passes over the camera's frame blocks)
@@ -1048,7 +1050,7 @@ size_t pool_part_rows(const PoolPlan& p, int na, bool cross) {
 
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
                              const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
-                             float* pool_v, int* pool_i, cudaStream_t st) {
+                             float* pool_v, int* pool_i, cudaStream_t st, Gate gate) {
   CUtensorMap ta, tb, tb_half;
   cudaError_t e = make_map(&ta, Ab, elt, na, d, BM);
   if (e != cudaSuccess) return e;
@@ -1072,6 +1074,7 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
   a.pool_i = parts.i;
   a.part_cnt = parts.cnt;
   a.split_first = p.split_first;
+  a.gate = gate;
   if (p.sample_tiles && !self_excl) {
     // every step-th row; the sample's pools end in pool_v, whose last entries are the floors
     const int rows = p.sample_tiles * BN, step = nb / rows;
@@ -1088,7 +1091,7 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
         : kp == 64 ? launch<POOL, 64, false>(ta, sb, sa, sg, st)
                    : launch<POOL, 128, false>(ta, sb, sa, sg, st);
     if (e == cudaSuccess)
-      e = launch_pool_finish(parts.v, parts.i, parts.cnt, splits, 1, na, p.cap, kp, pool_v, pool_i, st);
+      e = launch_pool_finish(parts.v, parts.i, parts.cnt, splits, 1, na, p.cap, kp, pool_v, pool_i, st, gate);
     if (e != cudaSuccess) return e;
     a.seed = pool_v + kp - 1;
     a.seed_ld = kp;
@@ -1108,7 +1111,7 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
   else e = cudaErrorInvalidValue;
   if (e != cudaSuccess) return e;
   if (!p.sel) return launch_merge_splits(parts.v, parts.i, p.splits, kinds, na, kp, pool_v, pool_i, st);
-  return launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, na, p.cap, kp, pool_v, pool_i, st);
+  return launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, na, p.cap, kp, pool_v, pool_i, st, gate);
 }
 
 cudaError_t launch_umma_gpool(const void* Y, int rows, int d, Elt elt, const int* gcam, bool cross, int self_excl,
@@ -1145,7 +1148,7 @@ cudaError_t launch_umma_gpool(const void* Y, int rows, int d, Elt elt, const int
 cudaError_t launch_umma_band(const void* Xb, int n, int d, Elt elt, const int* cam, int self_excl,
                              const void* Ab, const int* count, int cap, const int* band_row,
                              const int* band_kind, const float* band_thr, int bcap, int* band_cnt, float* band_v,
-                             int* band_i, cudaStream_t st, const int* band_off, const int* band_lim) {
+                             int* band_i, cudaStream_t st, const int* band_off, const int* band_lim, Gate gate) {
   CUtensorMap ta, tb;
   cudaError_t e = make_map(&ta, Ab, elt, cap, d, BM);
   if (e != cudaSuccess) return e;
@@ -1171,6 +1174,7 @@ cudaError_t launch_umma_band(const void* Xb, int n, int d, Elt elt, const int* c
   a.band_i = band_i;
   a.band_off = band_off;
   a.band_lim = band_lim;
+  a.gate = gate;
   // the row tiles (known only on the device) are strided over grid.y so that the grid covers
   // the GPU about twice even when the columns give few tiles
   const int gx = (n + BN - 1) / BN;
