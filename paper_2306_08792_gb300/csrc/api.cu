@@ -58,10 +58,11 @@ Elt elt_of(const gcr_params* p) { return p->precision == GCR_PREC_TF32 ? Elt::TF
 // Operands of the serving searches (normalised rows, no ball search): TF32's values in 16 bits.
 Elt serve_elt(const gcr_params* p) { return p->precision == GCR_PREC_TF32 ? Elt::F16 : Elt::BF16; }
 size_t elt_size(const gcr_params* p) { return elt_bytes(elt_of(p)); }
-// The first layer of a large offline problem (see Elt): from about 0.4 ms of TF32 sweep, of which
-// F16 saves more than the 11 launches (25 us) that the repetition costs when it is not needed.
-// 19,281 rows of d = 2048: the sweep 1.9 -> 1.0 ms; 201,000 of d = 512: 58 -> 39 ms.
-bool f16_first(const gcr_params* p, const Resolved& r, int64_t n, int32_t d) {
+// Large offline problems of normalised rows (see Elt): from about 0.4 ms of TF32 sweep, of which F16
+// saves more than the 11 launches (25 us) that the repetition costs when it is not needed, and
+// the probe of a later layer (40 us). 19,281 rows of d = 2048: the sweep 1.9 -> 1.0 ms with one
+// graph, 2.2 -> 1.2 with two; 201,000 of d = 512: 58 -> 39 ms.
+bool f16_search(const gcr_params* p, const Resolved& r, int64_t n, int32_t d) {
   return p->precision == GCR_PREC_TF32 && p->k > 0 && !(r.kp == 128 && r.kinds == 2) && 2.0 * (double)n * (double)n * d > 3e11;
 }
 
@@ -127,7 +128,7 @@ struct BuildWs {
   float* n32;
   RowScalars* sc;
   void* xr;            // rounded operand copy (tensor-core modes)
-  void* xr16;          // the first layer's F16 copy (f16_first), its repetition flag and counters
+  void* xr16;          // the first layer's F16 copy (f16_search), its repetition flag and counters
   int* repeat;
   unsigned long long* saved;
   float* enrm;
@@ -135,7 +136,10 @@ struct BuildWs {
   float* pool_v;
   int* pool_i;
   PoolParts parts;     // the sweep's split buffers
-  PoolParts parts16;
+  PoolParts parts16;   // of the F16 search, and of its probe, whose pools are probe_v / probe_i
+  PoolParts parts_probe;
+  float* probe_v;
+  int* probe_i;
   int* unc_count;
   int* unc_row;
   int* unc_kind;
@@ -190,7 +194,7 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   t.n32 = c.take<float>(nn);
   t.sc = c.take<RowScalars>(1);
   t.xr = bf ? c.take<char>(nn * d * es) : nullptr;
-  const bool f16 = f16_first(p, r, n, d);
+  const bool f16 = f16_search(p, r, n, d);
   t.xr16 = f16 ? c.take<char>(nn * d * 2) : nullptr;
   t.repeat = f16 ? c.take<int>(1) : nullptr;
   t.saved = f16 ? c.take<unsigned long long>(GCR_STATS_LEN) : nullptr;
@@ -202,8 +206,12 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
     Carve c16 = c;
     t.parts = carve_parts(c, (int)n, (int)n, d, p, elt_of(p), r.kp, kinds == 2);
     if (f16) {  // one region for both searches
+      Carve cp = c16;
       t.parts16 = carve_parts(c16, (int)n, (int)n, d, p, Elt::F16, r.kp, kinds == 2);
-      c.off = std::max(c.off, c16.off);
+      t.probe_v = cp.take<float>((size_t)kProbeRows * r.kp);
+      t.probe_i = cp.take<int>((size_t)kProbeRows * r.kp);
+      t.parts_probe = carve_parts(cp, kProbeRows, (int)n, d, p, Elt::F16, r.kp, false);
+      c.off = std::max(c.off, std::max(c16.off, cp.off));
     }
   }
   t.unc_count = c.take<int>(8 + (size_t)band_rows);
@@ -252,15 +260,19 @@ size_t carve_build(Carve& c, int64_t n, int32_t d, const gcr_params* p, const Re
   return c.off;
 }
 
+// Rows of a search: any; unit rows of a first layer; unit rows of a later one, which propagation may
+// have contracted.
+enum class Rows { Any, First, Later };
+
 // The certified kNN search of Eq. 4 / Eq. 8 (S1-S3): writes g->nbr / nbr_d2 (and the
-// cross-camera lists), g->row_order when given, and the search counters. first: the rows are the
-// normalised input of a first layer (f16_first may apply).
+// cross-camera lists), g->row_order when given, and the search counters. rows: what is
+// known of X.
 int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const gcr_params* p, const Resolved& r,
-             gcr_graph* g, const BuildWs& w, bool first, cudaStream_t st) {
+             gcr_graph* g, const BuildWs& w, Rows rows, cudaStream_t st) {
   const int n = (int)n64_;
   const int kinds = r.kinds;
   const bool bf = tensor_mode(p);
-  const bool f16 = first && f16_first(p, r, n64_, d);
+  const bool f16 = rows != Rows::Any && f16_search(p, r, n64_, d);
   const Elt elt = elt_of(p);
   unsigned long long* stats = g->stats ? reinterpret_cast<unsigned long long*>(g->stats) : w.stats;
   if (!g->stats) GCR_CUDA_TRY(cudaMemsetAsync(w.stats, 0, sizeof(unsigned long long) * GCR_STATS_LEN, st));
@@ -282,8 +294,15 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
   if (p->k > 0) {
     StageScope sc_(GCR_STAGE_SIM_GEMM, st);
     if (f16) {
+      if (rows == Rows::Later && n >= 4 * kProbeRows) {
+        GCR_CUDA_TRY(launch_umma_pool(w.xr16, kProbeRows, w.xr16, n, d, Elt::F16, nullptr, false, 0, r.kp, w.parts_probe,
+                                      w.probe_v, w.probe_i, st, Gate(), n / kProbeRows));
+        GCR_CUDA_TRY(launch_search_probe(w.probe_v, kProbeRows, r.kp, p->k, d, w.sc, w.repeat, st));
+      } else {
+        GCR_CUDA_TRY(cudaMemsetAsync(w.repeat, 0, sizeof(int), st));
+      }
       GCR_CUDA_TRY(launch_umma_pool(w.xr16, n, w.xr16, n, d, Elt::F16, camp, p->cross_camera != 0, 1, r.kp, w.parts16,
-                                    w.pool_v, w.pool_i, st));
+                                    w.pool_v, w.pool_i, st, Gate{w.repeat, 0}));
     } else if (bf) {
       GCR_CUDA_TRY(launch_umma_pool(w.xr, n, w.xr, n, d, elt, camp, p->cross_camera != 0, 1, r.kp, w.parts,
                                     w.pool_v, w.pool_i, st));
@@ -325,7 +344,9 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
         GCR_CUDA_TRY(launch_row_order(w.pool_i, n, r.kp, p->k, w.okey, w.ocnt, w.ooff, w.ofill, order, st));
         ra.order = order;
       }
+      if (f16) ra.gate = Gate{w.repeat, 0};
       GCR_CUDA_TRY(launch_refine_pool(ra, st));
+      ra.gate = Gate();
     }
     // F16: where a ball search would run, everything again on TF32 (decided on the device: the
     // launches below return at once otherwise)
@@ -337,6 +358,8 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
       GCR_CUDA_TRY(launch_row_stats(X, n, d, w.n64, w.n32, w.xr, elt, w.enrm, w.anrm, w.sc, st, again));
       GCR_CUDA_TRY(launch_umma_pool(w.xr, n, w.xr, n, d, elt, camp, p->cross_camera != 0, 1, r.kp, w.parts, w.pool_v,
                                     w.pool_i, st, again));
+      if (!in_l2(n, d))
+        GCR_CUDA_TRY(launch_row_order(w.pool_i, n, r.kp, p->k, w.okey, w.ocnt, w.ooff, w.ofill, order, st, again));
       ra.scale = 1.f;
       ra.gate = again;
       GCR_CUDA_TRY(launch_refine_pool(ra, st));
@@ -401,10 +424,10 @@ OrderStream g_order_side[kMaxOrderDevices];
 std::mutex g_order_mu;
 
 int build_graph_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const gcr_params* p,
-                     const Resolved& r, gcr_graph* g, const BuildWs& w, bool first, cudaStream_t st) {
+                     const Resolved& r, gcr_graph* g, const BuildWs& w, Rows rows, cudaStream_t st) {
   const int n = (int)n64_;
   const int kinds = r.kinds;
-  const int s = knn_impl(X, n64_, d, cam, p, r, g, w, first, st);
+  const int s = knn_impl(X, n64_, d, cam, p, r, g, w, rows, st);
   if (s != GCR_OK) return s;
 
   GraphArgs ga;
@@ -914,7 +937,7 @@ int pipeline_impl(const float* X, int64_t n, int64_t nq, int32_t d, const int32_
     Carve cb(w.inner, w.inner_bytes);
     BuildWs bw;
     carve_build(cb, n, d, p, r, &bw);
-    s = build_graph_impl(cur, n, d, cam, p, r, &w.g, bw, t == 0, st);
+    s = build_graph_impl(cur, n, d, cam, p, r, &w.g, bw, t == 0 ? Rows::First : Rows::Later, st);
     if (s != GCR_OK) return s;
     {
       StageScope sc_(GCR_STAGE_PROPAGATE, st);
@@ -1103,7 +1126,7 @@ int gcr_build_graph(const float* X, int64_t n, int32_t d, const int32_t* cam, co
   Carve c(ws, ws_bytes);
   BuildWs w;
   if (carve_build(c, n, d, p, r, &w) > ws_bytes) return GCR_E_WORKSPACE;
-  return build_graph_impl(X, n, d, cam, p, r, g, w, false, (cudaStream_t)stream);
+  return build_graph_impl(X, n, d, cam, p, r, g, w, Rows::Any, (cudaStream_t)stream);
 }
 
 int gcr_propagate(const gcr_graph* g, const float* X_in, float* X_out, int64_t n, int32_t d, gcr_stream_t stream) {
@@ -1222,7 +1245,7 @@ int gcr_gallery_build(const float* Xg, int64_t ng, int32_t d, const gcr_params* 
     Carve cb(w.inner, w.inner_bytes);
     BuildWs bw;
     carve_build(cb, ng, d, p, r, &bw);
-    s = build_graph_impl(cur, ng, d, nullptr, p, r, &w.g, bw, t == 0, st);
+    s = build_graph_impl(cur, ng, d, nullptr, p, r, &w.g, bw, t == 0 ? Rows::First : Rows::Later, st);
     if (s != GCR_OK) return s;
     GCR_CUDA_TRY(launch_layer_degree(w.g.deg_r, w.g.deg_c, n, p->symmetric, g.deg + (size_t)t * n, st));
     GCR_CUDA_TRY(launch_propagate(w.g.op_rowptr, w.g.op_len, w.g.op_col, w.g.op_val, cur, nxt, n, d,
@@ -1406,7 +1429,7 @@ int gcr_dsfp(const float* X, int64_t n, int32_t d, const gcr_params* p, float* X
     g.nbr = nbr;
     g.nbr_d2 = w.d2;
     g.stats = stats;
-    s = knn_impl(w.Xn, n, d, nullptr, p, r, &g, w.bw, true, st);
+    s = knn_impl(w.Xn, n, d, nullptr, p, r, &g, w.bw, Rows::First, st);
     if (s != GCR_OK) return s;
   }
   StageScope sc_(GCR_STAGE_PROPAGATE, st);

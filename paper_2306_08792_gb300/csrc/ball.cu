@@ -544,11 +544,26 @@ __global__ void order_scatter_kernel2(const int* root, const int* off, int n, in
   }
 }
 
+__global__ void search_probe_kernel(const float* __restrict__ pool_v, int rows, int kp, int k, int d,
+                                    const RowScalars* __restrict__ sc, int* flag) {
+  const int r = threadIdx.x;
+  const float unscale = 1.f / (kF16Scale * kF16Scale);
+  bool hit = false;
+  if (r < rows && k < kp - 1) {
+    const float sk = pool_v[(size_t)r * kp + k] * unscale, last = pool_v[(size_t)r * kp + kp - 1] * unscale;
+    const float delta = 2.f * (float)sc->emax + (float)(d + 32) * 1.2e-7f;  // of the GEMM, unit rows
+    hit = 2.f - 2.f * sk <= 0.25f && sk - last < 1.2f * delta;
+  }
+  const int hits = __syncthreads_count(hit);
+  if (threadIdx.x == 0) *flag = hits >= 2 ? 1 : 0;
+}
+
 // The decision of ball_go over the pending pairs of a search, by one block.
 __global__ void __launch_bounds__(1024) search_gate_kernel(const int* __restrict__ unc_row, const float* __restrict__ unc_dk,
                                                            int* unc_count, int unc_cap, const double* __restrict__ n64,
                                                            const unsigned long long* __restrict__ saved,
                                                            unsigned long long* stats, int* flag) {
+  if (*flag) return;  // the probe has decided
   const int U = min(*unc_count, unc_cap);
   int part = 0, dense = 0;
   for (int u0 = 0; u0 < U; u0 += 1024) {
@@ -558,15 +573,20 @@ __global__ void __launch_bounds__(1024) search_gate_kernel(const int* __restrict
     part += __syncthreads_count(in);
     dense += __syncthreads_count(in && dk < 0.f);
   }
-  const bool go = dense > 0 || part >= kMinBallPairs;
-  if (threadIdx.x == 0) *flag = go ? 1 : 0;
-  if (!go) return;
+  if (dense == 0 && part < kMinBallPairs) return;
+  if (threadIdx.x == 0) *flag = 1;
   __syncthreads();
   if (threadIdx.x == 0) *unc_count = 0;
   if (threadIdx.x < GCR_STATS_LEN) stats[threadIdx.x] = saved[threadIdx.x];
 }
 
 }  // namespace
+
+cudaError_t launch_search_probe(const float* pool_v, int rows, int kp, int k, int d, const RowScalars* sc, int* flag,
+                                cudaStream_t st) {
+  search_probe_kernel<<<1, kProbeRows, 0, st>>>(pool_v, rows, kp, k, d, sc, flag);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_search_gate(const int* unc_row, const float* unc_dk, int* unc_count, int unc_cap, const double* n64,
                                const unsigned long long* saved, unsigned long long* stats, int* flag, cudaStream_t st) {

@@ -17,9 +17,10 @@ struct BallArgs;  // ball search of the pairs a pool could not certify (below)
 // twice the kind::tf32 rate; its scores are kF16Scale^2 times the products of the rows. The
 // serving searches use it, whose rows are always normalised and whose distances come from the
 // FP32 rows whichever way a neighbour was certified. In an offline graph the scores decide, to the
-// last bit, which pairs the ball search takes, whose distances round otherwise: the first layer
-// of a large problem is searched on F16, and again on TF32 should a ball search turn out to run;
-// the other layers, which propagation has contracted, on TF32.
+// last bit, which pairs the ball search takes, whose distances round otherwise: a large problem
+// is searched on F16, and again on TF32 should a ball search turn out to run; layers after the
+// first, which propagation may have contracted, first search 128 of their rows, and all of them
+// on TF32 at once where those foretell it.
 enum class Elt : int { BF16 = 0, TF32 = 1, F16 = 2 };
 constexpr float kF16Scale = 16384.f;
 // The device this library is written for: its SMs and L2 bytes size grids and workspaces (the
@@ -91,7 +92,7 @@ cudaError_t launch_sgemm_dist(const float* Xq, int nq, const float* Xg, int ng, 
 // padded with (-inf, -1): every score left out of a full pool is <= its last entry.
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
                              const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
-                             float* pool_v, int* pool_i, cudaStream_t st, Gate gate = Gate());
+                             float* pool_v, int* pool_i, cudaStream_t st, Gate gate = Gate(), int a_step = 1);
 // Pools of row blocks of the gathered matrix Y (rows x d, rounded operand) against column ranges
 // of Y: work item w = {first row, rows <= 128, first column, columns} of *n_items (<= max_items);
 // pool entry (s - col_bias[j], j), j a position in Y; column j == row skipped when self_excl;
@@ -172,14 +173,19 @@ cudaError_t launch_refine_ball(const RefineArgs& a, const BallArgs& b, cudaStrea
 cudaError_t launch_refine_band(const RefineArgs& a, cudaStream_t st);
 // Cluster-local row order from the pools (first k candidates): order[0..n) is a permutation.
 cudaError_t launch_row_order(const int* pool_i, int n, int kp, int k, int* key, int* cnt, int* off, int* fill,
-                             int* order, cudaStream_t st);
+                             int* order, cudaStream_t st, Gate gate = Gate());
 cudaError_t launch_identity_order(int* order, int n, cudaStream_t st);
 // Copies rows[u] of src (row_bytes each, a multiple of 16) to row u of out, u < min(*count, max_rows).
 cudaError_t launch_gather_rows(const void* src, size_t row_bytes, const int* count, const int* rows,
                                int max_rows, void* out, cudaStream_t st, Gate gate = Gate());
 // After a search on F16 operands: *flag = 1 where the ball search would run on its pending pairs
 // (see ball.cu); the pending queue is then emptied and the counters set back to `saved`, for
-// the search to be repeated on TF32 operands.
+// the search to be repeated on TF32 operands. Nothing is done where *flag is 1 already.
+// Whether a sample's pools (rows x kp scores in the F16 scale, the row itself among them) foretell
+// that: *flag = 1 where two or more rows are contracted and cannot be certified by a pool.
+constexpr int kProbeRows = 128;
+cudaError_t launch_search_probe(const float* pool_v, int rows, int kp, int k, int d, const RowScalars* sc, int* flag,
+                                cudaStream_t st);
 cudaError_t launch_search_gate(const int* unc_row, const float* unc_dk, int* unc_count, int unc_cap, const double* n64,
                                const unsigned long long* saved, unsigned long long* stats, int* flag, cudaStream_t st);
 

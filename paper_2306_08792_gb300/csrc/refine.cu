@@ -732,7 +732,8 @@ __device__ void refine_ball_one(const RefineArgs& a, const BallArgs& b, int u, i
 // candidates: rows of one tight cluster share it, so a counting sort by key puts them next to
 // each other and their (largely common) candidate rows are fetched from memory once.
 __global__ void order_key_kernel(const int* __restrict__ pool_i, int n, int kp, int k, int* __restrict__ key,
-                                 int* __restrict__ cnt) {
+                                 int* __restrict__ cnt, Gate gate) {
+  if (gate_shut(gate)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int m = i;
@@ -745,7 +746,8 @@ __global__ void order_key_kernel(const int* __restrict__ pool_i, int n, int kp, 
 }
 
 __global__ void order_scatter_kernel(const int* __restrict__ key, const int* __restrict__ off, int n,
-                                     int* __restrict__ fill, int* __restrict__ order) {
+                                     int* __restrict__ fill, int* __restrict__ order, Gate gate) {
+  if (gate_shut(gate)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int m = key[i];
@@ -868,15 +870,15 @@ cudaError_t launch_identity_order(int* order, int n, cudaStream_t st) {
 }
 
 cudaError_t launch_row_order(const int* pool_i, int n, int kp, int k, int* key, int* cnt, int* off, int* fill,
-                             int* order, cudaStream_t st) {
+                             int* order, cudaStream_t st, Gate gate) {
   cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int) * (n + 1), st);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(fill, 0, sizeof(int) * n, st);
   if (e != cudaSuccess) return e;
-  order_key_kernel<<<(n + 255) / 256, 256, 0, st>>>(pool_i, n, kp, k, key, cnt);
+  order_key_kernel<<<(n + 255) / 256, 256, 0, st>>>(pool_i, n, kp, k, key, cnt, gate);
   e = launch_scan(cnt, off, n, st);
   if (e != cudaSuccess) return e;
-  order_scatter_kernel<<<(n + 255) / 256, 256, 0, st>>>(key, off, n, fill, order);
+  order_scatter_kernel<<<(n + 255) / 256, 256, 0, st>>>(key, off, n, fill, order, gate);
   return cudaGetLastError();
 }
 

@@ -1050,9 +1050,9 @@ size_t pool_part_rows(const PoolPlan& p, int na, bool cross) {
 
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
                              const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
-                             float* pool_v, int* pool_i, cudaStream_t st, Gate gate) {
+                             float* pool_v, int* pool_i, cudaStream_t st, Gate gate, int a_step) {
   CUtensorMap ta, tb, tb_half;
-  cudaError_t e = make_map(&ta, Ab, elt, na, d, BM);
+  cudaError_t e = make_map(&ta, Ab, elt, na, d, BM, a_step);
   if (e != cudaSuccess) return e;
   e = make_map(&tb, Bb, elt, nb, d, BN);
   if (e != cudaSuccess) return e;

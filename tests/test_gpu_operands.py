@@ -39,3 +39,23 @@ def test_scaled_fp16_holds_the_tf32_rounded_value():
     big = x >= 2.0 ** -28
     assert np.array_equal(back[big], t[big].astype(np.float64))
     assert np.max(np.abs(back - t)) <= 2.0 ** -39
+
+
+@pytest.mark.parametrize("noise", [0.3, 0.02])
+def test_later_layers_equal_the_tf32_search(noise):
+    """Two layers of 20,000 rows of d = 512, by gcr_pipeline (later layers are probed, and searched
+    on 16-bit copies or on TF32) and layer by layer through gcr_build_graph (TF32): X_T and the
+    ranking are the same bits."""
+    import paper_2306_08792_gb300 as gcr
+    g = torch.Generator(device="cuda").manual_seed(5)
+    cent = torch.randn(400, 512, generator=g, device="cuda")
+    lab = torch.randint(0, 400, (20000,), generator=g, device="cuda")
+    X = cent[lab] + noise * torch.randn(20000, 512, generator=g, device="cuda")
+    p = gcr.default_params(k=20, T=2, precision="tf32", topk_out=50)
+    idx, dist, XT, st = gcr.gcr_pipeline(X, 500, p)
+    Y = gcr.gcr_normalize(X)
+    for _ in range(2):
+        Y = gcr.gcr_propagate(gcr.gcr_build_graph(Y, p), Y)
+    assert torch.equal(XT, Y)
+    i2, d2 = gcr.gcr_rerank(Y[:500].contiguous(), Y[500:].contiguous(), p)
+    assert torch.equal(idx, i2) and torch.equal(dist, d2)
