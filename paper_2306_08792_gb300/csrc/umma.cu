@@ -238,7 +238,7 @@ struct UmmaArgs {
   float* D;
   // GRAM: G_s = Z_s Z_s^T + lambda n_s I per camera s = blockIdx.z, Z = the transposed,
   // normalised frames (feature rows, frame columns) split as hi + lo in BF16; K blocks of 64
-  // frames [gram_kstart[s], + gram_knum[s]) run three times: hi.hi, hi.lo, lo.hi
+  // frames [gram_kstart[s], + gram_knum[s]) give hi.hi, hi.lo and lo.hi each
   const int64_t* gram_kstart;
   const int64_t* gram_knum;
   const int64_t* gram_nf;  // n_s
@@ -447,9 +447,9 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   if ((MODE == POOL || MODE == BAND) && gate_shut(a.gate)) return;  // (every CTA alike, before any barrier)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bk = a.tf32 ? BKB / 4 : BKB / 2;  // K elements per stage
-  // K blocks per tile (GRAM: three passes over the camera's frame blocks)
+  // K blocks per tile (GRAM, MUL: the hi operands' and the lo operands' of each block in turn)
   const int gram_kn = MODE == GRAM ? (int)a.gram_knum[blockIdx.z] : (a.d + bk - 1) / bk;
-  const int kb_count = (MODE == GRAM || MODE == MUL) ? 3 * gram_kn : (a.d + bk - 1) / bk;
+  const int kb_count = (MODE == GRAM || MODE == MUL) ? 2 * gram_kn : (a.d + bk - 1) / bk;
   // MUL: rows of camera s's G_s in the stacked G
   const int mul_b0 = MODE == MUL ? max(0, a.mul_rowcam[blockIdx.y]) * a.n : 0;
 
@@ -520,16 +520,11 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           if (!mbar_wait(&bars.empty[s], (round & 1) ^ 1, abort_flag)) break;
           unsigned char* sa = stages + s * STAGE_BYTES;
           mbar_arrive_expect_tx(&bars.full[s], STAGE_BYTES);
-          if (MODE == GRAM) {
-            const int pass = kb / gram_kn;
-            const int x = (int)((a.gram_kstart[blockIdx.z] + kb % gram_kn) * bk);
-            tma_load_2d(sa, pass == 2 ? &tmA2 : &tmA, &bars.full[s], x, r0);
-            tma_load_2d(sa + A_BYTES, pass == 1 ? &tmB2 : &tmB, &bars.full[s], x, c0);
-          } else if (MODE == MUL) {
-            const int pass = kb / gram_kn;
-            const int x = (kb % gram_kn) * bk;
-            tma_load_2d(sa, pass == 2 ? &tmA2 : &tmA, &bars.full[s], x, r0);
-            tma_load_2d(sa + A_BYTES, pass == 1 ? &tmB2 : &tmB, &bars.full[s], x, mul_b0 + c0);
+          if (MODE == GRAM || MODE == MUL) {
+            // even K blocks: the hi operands, odd ones: the lo operands of the same elements
+            const int x = MODE == GRAM ? (int)((a.gram_kstart[blockIdx.z] + (kb >> 1)) * bk) : (kb >> 1) * bk;
+            tma_load_2d(sa, (kb & 1) ? &tmA2 : &tmA, &bars.full[s], x, r0);
+            tma_load_2d(sa + A_BYTES, (kb & 1) ? &tmB2 : &tmB, &bars.full[s], x, mul_b0 + c0);
           } else {
             tma_load_2d(sa, &tmA, &bars.full[s], kb * bk, r0);
             if (MODE == POOL && a.mc) {
@@ -569,14 +564,33 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           tc_fence_after();
           const uint32_t sa = smem_u32(stages + s * STAGE_BYTES);
           const uint64_t ad = smem_desc(sa), bd = smem_desc(sa + A_BYTES);
-          // four MMAs per stage, +32 bytes (K=16 BF16 or K=8 TF32) inside the swizzle row
-          if (a.tf32) {
+          // four MMAs per stage, +32 bytes (16 16-bit elements or K=8 TF32) inside the swizzle row
+          auto mma4 = [&](uint64_t da, uint64_t db, bool accum) {
+            if (a.tf32) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) umma_tf32(dcol, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), (kb | k) != 0);
-          } else {
+              for (int k = 0; k < 4; ++k) umma_tf32(dcol, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), accum || k);
+            } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) umma_16bit(dcol, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), a.idesc, (kb | k) != 0);
+              for (int k = 0; k < 4; ++k)
+                umma_16bit(dcol, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), a.idesc, accum || k);
+            }
+          };
+          if (MODE == GRAM || MODE == MUL) {
+            // hi.hi as soon as the hi operands have landed; hi.lo and lo.hi with the lo ones, after
+            // which both stages are free: two operand loads per three products
+            static_assert(!(MODE == GRAM || MODE == MUL) || NS % 2 == 0, "hi and lo stages in pairs");
+            if (!(kb & 1)) {
+              mma4(ad, bd, kb != 0);
+              continue;
+            }
+            const uint32_t sh = smem_u32(stages + (s - 1) * STAGE_BYTES);
+            mma4(smem_desc(sh), bd, true);
+            mma4(ad, smem_desc(sh + A_BYTES), true);
+            umma_commit(&bars.empty[s - 1]);
+            umma_commit(&bars.empty[s]);
+            continue;
           }
+          mma4(ad, bd, kb != 0);
           if (MODE == POOL && a.mc) umma_commit_mc(&bars.empty[s], (uint16_t)0x3);
           else umma_commit(&bars.empty[s]);
         }
