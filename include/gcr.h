@@ -52,7 +52,8 @@ typedef enum {
   GCR_PREC_FP32 = 0, /* similarity GEMM on CUDA cores in FP32 (the reference path) */
   GCR_PREC_BF16 = 1, /* similarity GEMM on tcgen05 tensor cores, BF16 x BF16 -> FP32,
                         then boundary candidates re-scored in FP32 (FP64 for ties) */
-  GCR_PREC_TF32 = 2  /* as BF16 with the rows rounded to TF32 (kind::tf32): a rounding
+  GCR_PREC_TF32 = 2  /* as BF16 with the rows rounded to TF32 (kind::tf32, or kind::f16 on
+                        16-bit copies of the same values): a rounding
                         bound 8x tighter, so fewer candidates need the FP32 re-score.
                         Both tensor-core modes need d % 8 == 0 (BF16 also pool >= 64);
                         their certified re-score returns the neighbour sets of the exact

@@ -647,7 +647,6 @@ size_t carve_ball(Carve& c, int n, int d, int kinds, int kp, Elt elt, int cap_ro
   t.afill = c.take<int>(n);
   t.bfill = c.take<int>(n);
   t.gfail = c.take<int>(n);
-  t.icnt = c.take<int>(n + 1);
   t.ioff = c.take<int>(n + 1);
   t.gsc = c.take<RowScalars>(n);
   t.max_items = cap_rows / 128 + n + 1;  // sum over groups of ceil(pending rows / 128)
@@ -673,7 +672,7 @@ size_t carve_ball(Carve& c, int n, int d, int kinds, int kp, Elt elt, int cap_ro
     GCR_BALL_TAKE(ga); GCR_BALL_TAKE(gkind); GCR_BALL_TAKE(gthr); GCR_BALL_TAKE(gthr_fill); GCR_BALL_TAKE(gsize);
     GCR_BALL_TAKE(rsize); GCR_BALL_TAKE(goff); GCR_BALL_TAKE(boff); GCR_BALL_TAKE(blim); GCR_BALL_TAKE(gscale);
     GCR_BALL_TAKE(npart); GCR_BALL_TAKE(ndense); GCR_BALL_TAKE(gfill); GCR_BALL_TAKE(afill); GCR_BALL_TAKE(bfill);
-    GCR_BALL_TAKE(gfail); GCR_BALL_TAKE(icnt); GCR_BALL_TAKE(ioff); GCR_BALL_TAKE(gsc); GCR_BALL_TAKE(max_items);
+    GCR_BALL_TAKE(gfail); GCR_BALL_TAKE(ioff); GCR_BALL_TAKE(gsc); GCR_BALL_TAKE(max_items);
     GCR_BALL_TAKE(items); GCR_BALL_TAKE(ball_j); GCR_BALL_TAKE(gmap); GCR_BALL_TAKE(ggrp); GCR_BALL_TAKE(n64y);
     GCR_BALL_TAKE(hy); GCR_BALL_TAKE(enrm_y); GCR_BALL_TAKE(anrm_y); GCR_BALL_TAKE(gcam); GCR_BALL_TAKE(Y);
     GCR_BALL_TAKE(Yr); GCR_BALL_TAKE(gpool_v); GCR_BALL_TAKE(gpool_i); GCR_BALL_TAKE(cap_rows);

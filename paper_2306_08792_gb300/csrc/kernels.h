@@ -230,7 +230,7 @@ struct BallArgs {
   float* gscale;            // per B row (two = 1): its local scale
   int* npart;               // pending pairs taking part, and those predicted dense
   int* ndense;
-  int *groot, *ga, *gkind, *gsize, *rsize, *goff, *boff, *blim, *gfill, *afill, *bfill, *gfail, *icnt, *ioff;
+  int *groot, *ga, *gkind, *gsize, *rsize, *goff, *boff, *blim, *gfill, *afill, *bfill, *gfail, *ioff;
   float *gthr, *gthr_fill;
   RowScalars* gsc;          // per group: maxima over its positions
   int4* items;

@@ -1,8 +1,10 @@
 // Streaming per-row candidate pool for the kNN search of Eq. 4 / Eq. 8.
 //
 // The similarity tile S = X_rows . X_cols^T is produced column tile by column tile and
-// never stored. Each row has one owning thread (lane r of a warp owns row warp_row0 + r)
-// holding three registers:
+// never stored. Each row has one owning thread (lane r of a warp owns row warp_row0 + r).
+// Two forms. Selection buffers (SelCap and below, second half of this file) serve the searches.
+// Sorted lists, first, serve the ball search's groups and two graphs of 128-entry pools on the
+// tensor-core path; their owner holds three registers:
 //   tau   admission threshold: the KP-th best score seen so far (-inf until KP seen),
 //   qcnt  survivors queued in shared memory,
 //   len   entries in the row's list.

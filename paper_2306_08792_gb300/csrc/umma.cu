@@ -3,8 +3,9 @@
 // S = A . B^T with A, B row-major (K = d contiguous, "K-major"), BF16 or scaled FP16 rows or FP32
 // rows rounded to TF32: A holds 128 rows of X, B 256 rows. Per CTA:
 //   warp 0        TMA producer: 128-byte K blocks (64 16-bit or 32 TF32 elements) of A (128 rows)
-//                 and B (256 rows) into a 3-stage shared-memory ring (128-byte swizzle),
-//                 mbarrier transaction counts;
+//                 and B (256 rows) into a 2- to 4-stage shared-memory ring (128-byte
+//                 swizzle; as many stages as the pools leave room for), mbarrier transaction
+//                 counts;
 //   warp 1        allocates 512 TMEM columns (two 128 x 256 FP32 accumulators) and, from one
 //                 thread, issues tcgen05.mma (kind::f16 with K=16, or kind::tf32 with K=8;
 //                 M=128, N=256) for each K block,
