@@ -10,6 +10,8 @@
 //   asymmetric (Eq. 6): y = x_q / sqrt(r_q) + sum_j w_qj g_j / sqrt(r_q Dc_j), r_q = 1 + sum w
 // x_q <- normalise(y); finally the certified top-K of the gallery on G_T. Every step is per
 // query row, so a query's result does not depend on the other queries of its batch.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "pool.cuh"
@@ -114,27 +116,22 @@ __device__ __forceinline__ void merge_chunk(float (&b)[KP / 32], int (&bi)[KP / 
   for (int p = 0; p < P; ++p) warp_merge32_desc(b[p], bi[p], lane);
 }
 
-// The selection buffers of a (kind, row)'s S splits sorted into its pool. W = 1: a warp per row;
-// W > 1: a block of W warps per row, warp w taking the splits w, w + W, ..., then the warps'
-// lists merged pairwise. A warp streams its entries (the next 32 in flight while 32 are tested):
-// those that would enter its list so far are staged in shared memory and merged 32 at a time, so
-// past the first few splits most entries cost one comparison (one query, 152 splits: 260 -> 91 us
-// for a 128-entry pool, 65 -> 20 us for a 32-entry one, against sorting every chunk). The strict order makes the result
-// independent of the merge order.
-template <int KP, int W>
-__global__ void __launch_bounds__(W > 1 ? 32 * W : 256) pool_finish_kernel(
-    const float* __restrict__ pv, const int* __restrict__ pi, const int* __restrict__ cnt, int S, long rows, int cap,
-    float* __restrict__ ov, int* __restrict__ oi, Gate gate) {
+// The selection buffers of a (kind, row)'s S splits sorted into its pool, a warp per row (few
+// splits). The warp streams its entries (the next 32 in flight while 32 are tested): those that
+// would enter its list so far are staged in shared memory and merged 32 at a time, so past the
+// first few splits most entries cost one comparison. The strict order makes the result independent
+// of the merge order.
+template <int KP>
+__global__ void __launch_bounds__(256) pool_finish_kernel(const float* __restrict__ pv, const int* __restrict__ pi,
+                                                          const int* __restrict__ cnt, int S, long rows, int cap,
+                                                          float* __restrict__ ov, int* __restrict__ oi, Gate gate) {
   if (gate_shut(gate)) return;
-  constexpr int P = KP / 32, NW = W > 1 ? W : 8;
-  __shared__ float stv[NW][64];
-  __shared__ int sti[NW][64];
-  __shared__ float sv[W > 1 ? W : 1][W > 1 ? KP : 1];
-  __shared__ int si[W > 1 ? W : 1][W > 1 ? KP : 1];
+  constexpr int P = KP / 32;
+  __shared__ float stv[8][64];
+  __shared__ int sti[8][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long w = W > 1 ? (long)blockIdx.x : (long)blockIdx.x * 8 + warp;  // (kind, row)
-  if (W == 1 && w >= rows) return;
-  const int first = W > 1 ? warp : 0;
+  const long w = (long)blockIdx.x * 8 + warp;  // (kind, row)
+  if (w >= rows) return;
   float b[P];
   int bi[P];
 #pragma unroll
@@ -170,12 +167,12 @@ __global__ void __launch_bounds__(W > 1 ? 32 * W : 256) pool_finish_kernel(
   };
   float na = 0.f;  // the next chunk, in flight
   int ni = -1;
-  for (int s0 = first; s0 < S; s0 += 32 * W) {  // 32 of the warp's splits: a lane holds each count
-    const int sl = s0 + lane * W;
+  for (int s0 = 0; s0 < S; s0 += 32) {  // 32 splits: a lane holds each count
+    const int sl = s0 + lane;
     const int cl = sl < S ? cnt[(size_t)sl * rows + w] : 0;
-    for (int l = 0; l < 32 && s0 + l * W < S; ++l) {
+    for (int l = 0; l < 32 && s0 + l < S; ++l) {
       const int c = __shfl_sync(GCR_FULL, cl, l);
-      const size_t base = ((size_t)(s0 + l * W) * rows + w) * cap;
+      const size_t base = ((size_t)(s0 + l) * rows + w) * cap;
       for (int e0 = 0; e0 < c; e0 += 32) {
         const int e = e0 + lane;
         const float a = e < c ? pv[base + e] : 0.f;
@@ -188,26 +185,151 @@ __global__ void __launch_bounds__(W > 1 ? 32 * W : 256) pool_finish_kernel(
   }
   test(na, ni);
   if (staged > 0) merge_staged(staged);
-  if constexpr (W > 1) {
-    for (int step = 1; step < W; step <<= 1) {
-      // warps at odd multiples of step hand their lists to the warp step below
-      if ((warp & (2 * step - 1)) == step) {
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-          sv[warp][p * 32 + lane] = b[p];
-          si[warp][p * 32 + lane] = bi[p];
-        }
-      }
-      __syncthreads();
-      if ((warp & (2 * step - 1)) == 0 && warp + step < S) merge_list<KP>(b, bi, sv[warp + step], si[warp + step], lane);
-    }
-    if (warp != 0) return;
-  }
 #pragma unroll
   for (int p = 0; p < P; ++p) {
     ov[w * KP + p * 32 + lane] = b[p];
     oi[w * KP + p * 32 + lane] = bi[p];
   }
+}
+
+// The same from many splits' buffers, a block per row: the entries as 64-bit keys (score's image,
+// complement of the column: the strict order) in shared memory, narrowed to at most kSelKeep by
+// histograms of 256 equal parts of the keys' range (usually two or three), and these ranked by
+// counting. Merging sorted lists pairwise took about 110 shuffles per 32 entries and was bound by
+// them: 512 rows, 128-entry pools of 38 splits 139 -> 23 us, one row of 152 splits 46 -> 15 us (32
+// entries: 31 -> 14 and 20 -> 10).
+// Splits are taken in groups that fit the buffer; the best KP so far stay at its front.
+constexpr int kSelKeep = 256;
+constexpr int kSelThreads = 512;
+
+template <int KP>
+__global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float* __restrict__ pv,
+                                                                  const int* __restrict__ pi,
+                                                                  const int* __restrict__ cnt, int S, long rows,
+                                                                  int cap, int group, float* __restrict__ ov,
+                                                                  int* __restrict__ oi, Gate gate) {
+  static_assert(KP <= kSelKeep, "the kept entries hold the pool");
+  if (gate_shut(gate)) return;
+  extern __shared__ __align__(16) unsigned long long ent[];  // [KP + group * cap]
+  __shared__ unsigned long long keep[kSelKeep], s_min, s_max;
+  __shared__ int hist[256], part[kSelThreads], s_total, s_kept, s_bin, s_over;
+  constexpr int NW = kSelThreads / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long w = blockIdx.x;  // (kind, row)
+  int have = 0;
+  for (int s0 = 0; s0 < S; s0 += group) {
+    const int s1 = min(S, s0 + group);
+    if (tid == 0) { s_total = have; s_kept = 0; s_min = ~0ull; s_max = 0ull; }
+    __syncthreads();
+    unsigned long long mn = ~0ull, mx = 0ull;
+    for (int e = tid; e < have; e += kSelThreads) { mn = min(mn, ent[e]); mx = max(mx, ent[e]); }
+    for (int sb = s0 + warp; sb < s1; sb += NW * 32) {  // up to 32 splits of the warp: a lane holds each count
+      const int sl = sb + NW * lane;
+      const int cl = sl < s1 ? min(cnt[(size_t)sl * rows + w], cap) : 0;
+      int inc = cl;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(GCR_FULL, inc, o);
+        if (lane >= o) inc += y;
+      }
+      int at0 = 0;
+      if (lane == 31) at0 = atomicAdd(&s_total, inc);
+      at0 = __shfl_sync(GCR_FULL, at0, 31);
+      for (int l = 0; l < 32 && sb + NW * l < s1; ++l) {
+        const int c = __shfl_sync(GCR_FULL, cl, l), at = at0 + __shfl_sync(GCR_FULL, inc, l) - c;
+        const size_t base = ((size_t)(sb + NW * l) * rows + w) * cap;
+        for (int e = lane; e < c; e += 32) {
+          const unsigned long long key = ((unsigned long long)float_to_ordered(pv[base + e] + 0.f) << 32) |
+                                         (uint32_t)~pi[base + e];
+          ent[at + e] = key;
+          mn = min(mn, key);
+          mx = max(mx, key);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mn = min(mn, __shfl_xor_sync(GCR_FULL, mn, o));
+      mx = max(mx, __shfl_xor_sync(GCR_FULL, mx, o));
+    }
+    if (lane == 0) { atomicMin(&s_min, mn); atomicMax(&s_max, mx); }
+    __syncthreads();
+    const int E = s_total;
+    unsigned long long lo = s_min, hi = s_max;
+    if (E > kSelKeep) {
+      int need = KP, over = 0;  // the KP best: `over` above hi, `need` of those in [lo, hi]
+      for (;;) {                // block-uniform; every pass takes 8 bits off the range
+        const int shift = max(0, 56 - __clzll((long long)(hi - lo)));
+        if (tid < 256) hist[tid] = 0;
+        __syncthreads();
+        for (int e = tid; e < E; e += kSelThreads) {
+          const unsigned long long k = ent[e];
+          if (k >= lo && k <= hi) atomicAdd(&hist[(int)((k - lo) >> shift)], 1);
+        }
+        __syncthreads();
+        if (warp == 0) {  // the part that holds the need-th from above; lane l holds 8 parts
+          int c[8], tot = 0;
+#pragma unroll
+          for (int x = 0; x < 8; ++x) { c[x] = hist[255 - 8 * lane - x]; tot += c[x]; }
+          int inc = tot;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(GCR_FULL, inc, o);
+            if (lane >= o) inc += y;
+          }
+          int run = inc - tot;
+          if (run < need && inc >= need) {  // one lane
+            bool done = false;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+              if (!done && run + c[x] >= need) { s_bin = 255 - 8 * lane - x; s_over = run; done = true; }
+              run += c[x];
+            }
+          }
+        }
+        __syncthreads();
+        const int bin = s_bin, in = hist[bin];
+        need -= s_over;
+        over += s_over;
+        lo += (unsigned long long)bin << shift;
+        const unsigned long long width = (1ull << shift) - 1ull;
+        if (hi - lo > width) hi = lo + width;
+        if (over + in <= kSelKeep || shift == 0) break;
+        __syncthreads();  // hist and the result are read before the next pass clears them
+      }
+    }
+    // (E <= kSelKeep: lo is the smallest key and all are kept)
+    for (int e = tid; e < E; e += kSelThreads) {
+      const unsigned long long k = ent[e];
+      if (k >= lo) {
+        const int at = atomicAdd(&s_kept, 1);
+        if (at < kSelKeep) keep[at] = k;
+      }
+    }
+    __syncthreads();
+    const int n = min(s_kept, kSelKeep), half = (n + 1) / 2;
+    const int i = tid & (kSelKeep - 1), j0 = (tid >> 8) * half, j1 = min(n, j0 + half);
+    const unsigned long long k = i < n ? keep[i] : 0ull;
+    int r = 0;
+    if (i < n)
+      for (int j = j0; j < j1; ++j) r += keep[j] > k;
+    part[tid] = r;
+    __syncthreads();
+    have = min(n, KP);
+    if (tid < n) {
+      r = part[tid] + part[tid + kSelKeep];
+      if (r < KP) {
+        if (s1 < S) {
+          ent[r] = k;
+        } else {
+          ov[w * KP + r] = ordered_to_float((uint32_t)(k >> 32));
+          oi[w * KP + r] = (int)~(uint32_t)k;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  for (int r = have + tid; r < KP; r += kSelThreads) { ov[w * KP + r] = -CUDART_INF_F; oi[w * KP + r] = -1; }
 }
 
 // One warp per query: the query's row of the operator against the frozen layer, normalised.
@@ -288,23 +410,30 @@ cudaError_t launch_merge_splits(const float* pv, const int* pi, int S, int kinds
 }
 
 template <int KP>
-static void pool_finish(const float* pv, const int* pi, const int* cnt, int S, long rows, int cap, float* ov, int* oi,
-                        cudaStream_t st, Gate gate) {
-  // a warp per row; a block per row where there are many splits' buffers to merge, with more
-  // warps where the rows alone do not fill the GPU
-  if (S <= 8) pool_finish_kernel<KP, 1><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
-  else if (rows >= 4 * kSMs) pool_finish_kernel<KP, 8><<<(unsigned)rows, 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
-  else pool_finish_kernel<KP, 16><<<(unsigned)rows, 512, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
+static cudaError_t pool_finish(const float* pv, const int* pi, const int* cnt, int S, long rows, int cap, float* ov,
+                               int* oi, cudaStream_t st, Gate gate) {
+  if (S <= 8) {  // a warp per row
+    pool_finish_kernel<KP><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
+    return cudaGetLastError();
+  }
+  // a block per row: room for every split's buffer where a block has an SM to itself, for 6,144
+  // entries (four blocks per SM) where rows share one
+  const int room = rows <= kSMs ? 24576 : 6144;
+  const int group = std::max(1, std::min(S, room / cap));
+  const size_t smem = sizeof(unsigned long long) * ((size_t)KP + (size_t)group * cap);
+  cudaError_t e = cudaFuncSetAttribute(pool_select_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  pool_select_kernel<KP><<<(unsigned)rows, kSelThreads, smem, st>>>(pv, pi, cnt, S, rows, cap, group, ov, oi, gate);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_pool_finish(const float* pv, const int* pi, const int* cnt, int S, int kinds, int na, int cap, int kp,
                                float* ov, int* oi, cudaStream_t st, Gate gate) {
   const long rows = (long)kinds * na;
-  if (kp == 32) pool_finish<32>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
-  else if (kp == 64) pool_finish<64>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
-  else if (kp == 128) pool_finish<128>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (kp == 32) return pool_finish<32>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
+  if (kp == 64) return pool_finish<64>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
+  if (kp == 128) return pool_finish<128>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_query_step(const float* xq, int b, int d, const float* G, const float* deg, const int32_t* nbr,
