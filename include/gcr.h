@@ -295,7 +295,8 @@ int gcrv_mean_profiles(const float* frames, int64_t F, int32_t d, const int64_t*
  * computed and stored in advance the cost per query falls to O(N log N); this is that form:
  *  - gcr_gallery_build runs offline GCR (Eq. 3) on the gallery alone and stores, in the
  *    caller's state buffer (gcr_gallery_bytes), the layers G_0..G_T, the degrees of each
- *    layer's graph (D = (D_r + D_c)/2 of Eq. 7, or D_c of Eq. 6) and per-row statistics.
+ *    layer's graph (D = (D_r + D_c)/2 of Eq. 7, or D_c of Eq. 6), per-row statistics and the
+ *    kNN lists of the last layer's graph.
  *  - gcr_serve takes a batch of b raw queries (device float32 [b][d]) and, for t = 1..T,
  *    finds each query's certified k nearest rows of G_{t-1}, forms the query's row of the
  *    operator with the gallery frozen and no query-query edges

@@ -638,6 +638,7 @@ struct GalleryView {
   float* enrm;     // (T+1) x ng
   float* anrm;     // (T+1) x ng
   RowScalars* sc;  // T+1
+  int32_t* nbr;    // ng x k: the last layer's kNN lists (T >= 1)
 };
 
 int check_serve_params(const gcr_params* p, int64_t ng, int32_t d, Resolved* r) {
@@ -662,6 +663,7 @@ size_t carve_gallery(Carve& c, int64_t ng, int32_t d, const gcr_params* p, Galle
   t.enrm = bf ? c.take<float>(L * n) : nullptr;
   t.anrm = bf ? c.take<float>(L * n) : nullptr;
   t.sc = c.take<RowScalars>(L);
+  t.nbr = c.take<int32_t>(n * std::max(p->k, 1));
   if (v) *v = t;
   return c.off;
 }
@@ -1251,6 +1253,8 @@ int gcr_gallery_build(const float* Xg, int64_t ng, int32_t d, const gcr_params* 
     GCR_CUDA_TRY(launch_propagate(w.g.op_rowptr, w.g.op_len, w.g.op_col, w.g.op_val, cur, nxt, n, d,
                                   p->k > 0 ? w.g.row_order : nullptr, st));
   }
+  if (p->T >= 1 && p->k > 0)
+    GCR_CUDA_TRY(cudaMemcpyAsync(g.nbr, w.g.nbr, sizeof(int32_t) * (size_t)n * p->k, cudaMemcpyDeviceToDevice, st));
   for (int t = 0; t <= p->T; ++t) {
     GCR_CUDA_TRY(launch_row_stats(g.layers + (size_t)t * n * d, n, d, g.n64 + (size_t)t * n, g.n32 + (size_t)t * n,
                                   bf ? g.xr + (size_t)t * n * d * es : nullptr, elt,
