@@ -332,7 +332,10 @@ __global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float* _
   for (int r = have + tid; r < KP; r += kSelThreads) { ov[w * KP + r] = -CUDART_INF_F; oi[w * KP + r] = -1; }
 }
 
-// One warp per query: the query's row of the operator against the frozen layer, normalised.
+// One warp per query: the query's row of the operator against the frozen layer, normalised. Lanes
+// fetch 32 neighbours' indices, distances and degrees at once and the rows are gathered U at a time:
+// neighbour by neighbour, each step waited for three dependent loads (one query, k = 20, d = 256:
+// 28 -> 8 us). Sums keep the neighbours' order.
 template <int VPL>
 __global__ void __launch_bounds__(256) query_step_kernel(const float* __restrict__ xq, int b, int d,
                                                          const float* __restrict__ G, const float* __restrict__ deg,
@@ -342,10 +345,13 @@ __global__ void __launch_bounds__(256) query_step_kernel(const float* __restrict
   const int lane = threadIdx.x & 31;
   const int q = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (q >= b) return;
+  constexpr int U = VPL <= 2 ? 8 : VPL <= 4 ? 4 : VPL <= 8 ? 2 : 1;
   float wsum = 0.f;
-  for (int s = 0; s < k; ++s) {
-    const int j = nbr[(size_t)q * k + s];
-    if (j >= 0) wsum += expf(-d2[(size_t)q * k + s] / gamma);
+  for (int s0 = 0; s0 < k; s0 += 32) {
+    const int s = s0 + lane;
+    const int j = s < k ? nbr[(size_t)q * k + s] : -1;
+    const float w = j >= 0 ? expf(-d2[(size_t)q * k + s] / gamma) : 0.f;
+    for (unsigned m = __ballot_sync(GCR_FULL, j >= 0); m; m &= m - 1) wsum += __shfl_sync(GCR_FULL, w, __ffs(m) - 1);
   }
   const float Dq = symmetric ? 0.5f * (1.f + wsum + 1.f) : 1.f + wsum;
   const float cself = symmetric ? 1.f / Dq : 1.f / sqrtf(Dq);
@@ -359,19 +365,56 @@ __global__ void __launch_bounds__(256) query_step_kernel(const float* __restrict
       acc[v] = make_float4(cself * x.x, cself * x.y, cself * x.z, cself * x.w);
     }
   }
-  for (int s = 0; s < k; ++s) {
-    const int j = nbr[(size_t)q * k + s];
-    if (j < 0) continue;
-    const float w = expf(-d2[(size_t)q * k + s] / gamma);
-    const float c = symmetric ? 0.5f * w / sqrtf(Dq * deg[j]) : w / sqrtf(Dq * deg[j]);
-    const float* g = G + (size_t)j * d;
+  for (int s0 = 0; s0 < k; s0 += 32) {
+    const int s = s0 + lane;
+    const int j = s < k ? nbr[(size_t)q * k + s] : -1;
+    float c = 0.f;
+    if (j >= 0) {
+      const float w = expf(-d2[(size_t)q * k + s] / gamma);
+      c = symmetric ? 0.5f * w / sqrtf(Dq * deg[j]) : w / sqrtf(Dq * deg[j]);
+    }
+    if constexpr (U == 1) {  // long rows: the columns of one neighbour are loads enough in flight
+      for (unsigned m = __ballot_sync(GCR_FULL, j >= 0); m; m &= m - 1) {
+        const float cu = __shfl_sync(GCR_FULL, c, __ffs(m) - 1);
+        const float* g = G + (size_t)__shfl_sync(GCR_FULL, j, __ffs(m) - 1) * d;
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int off = v * 128 + lane * 4;
-      if (off < d) {
-        const float4 y = *reinterpret_cast<const float4*>(g + off);
-        acc[v].x = fmaf(c, y.x, acc[v].x); acc[v].y = fmaf(c, y.y, acc[v].y);
-        acc[v].z = fmaf(c, y.z, acc[v].z); acc[v].w = fmaf(c, y.w, acc[v].w);
+        for (int v = 0; v < VPL; ++v) {
+          const int off = v * 128 + lane * 4;
+          if (off < d) {
+            const float4 y = *reinterpret_cast<const float4*>(g + off);
+            acc[v].x = fmaf(cu, y.x, acc[v].x); acc[v].y = fmaf(cu, y.y, acc[v].y);
+            acc[v].z = fmaf(cu, y.z, acc[v].z); acc[v].w = fmaf(cu, y.w, acc[v].w);
+          }
+        }
+      }
+    } else {
+      for (unsigned m = __ballot_sync(GCR_FULL, j >= 0); m;) {
+        float4 y[U][VPL];
+        float cu[U];
+        int nu = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int l = m ? __ffs(m) - 1 : 0;
+          nu += m != 0;
+          m &= m - 1;  // (0 stays 0)
+          cu[u] = __shfl_sync(GCR_FULL, c, l);
+          const int ju = __shfl_sync(GCR_FULL, j, l);
+#pragma unroll
+          for (int v = 0; v < VPL; ++v) {
+            const int off = v * 128 + lane * 4;
+            if (u < nu && off < d) y[u][v] = *reinterpret_cast<const float4*>(G + (size_t)ju * d + off);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (u < nu) {
+#pragma unroll
+            for (int v = 0; v < VPL; ++v)
+              if (v * 128 + lane * 4 < d) {
+                acc[v].x = fmaf(cu[u], y[u][v].x, acc[v].x); acc[v].y = fmaf(cu[u], y[u][v].y, acc[v].y);
+                acc[v].z = fmaf(cu[u], y[u][v].z, acc[v].z); acc[v].w = fmaf(cu[u], y[u][v].w, acc[v].w);
+              }
+          }
       }
     }
   }
