@@ -751,7 +751,12 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   t.sc = c.take<RowScalars>(1);
   // one region for both pool sizes, as large as any smaller batch needs it (a batch of fewer row
   // blocks is cut into more splits): a workspace sized for a batch serves every smaller one
-  size_t end = 0;
+  // (the band's entries, written after a search's pools are finished and read before the next
+  // search, share it)
+  Carve cband = c;
+  t.band_v = cband.take<float>(nb * kBandCap);
+  t.band_i = cband.take<int>(nb * kBandCap);
+  size_t end = cband.off;
   for (int64_t rows = std::min<int64_t>(b, 128);; rows = std::min<int64_t>(b, rows + 128)) {
     Carve c1 = c, c2 = c;
     t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, elt, r.kp, false);
@@ -774,8 +779,6 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   t.bq_flag = c.take<int>(nb);
   t.err = c.take<int>(4);
   t.band_cnt = c.take<int>(nb);
-  t.band_v = c.take<float>(nb * kBandCap);
-  t.band_i = c.take<int>(nb * kBandCap);
   t.band_a = bf ? c.take<char>(nb * d * es) : nullptr;
   t.nbr = c.take<int32_t>(nb * std::max(p->k, 1));
   t.d2 = c.take<float>(nb * std::max(p->k, 1));

@@ -268,6 +268,8 @@ static int simt_ctas(int kp, bool cross) { return kp == 128 || (kp == 64 && cros
 
 // As pool_plan: splits whose CTAs fill the SMs evenly. A tile takes about 2 * 128 * 128 * d FMAs
 // at the SM's share; set-up, the first tile's rounds and the write-out about 20 us.
+constexpr long kFewRowsBytes = 9l << 20;
+
 PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
   PoolPlan p{};
   p.sel = true;
@@ -282,6 +284,9 @@ PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
   double best_t = 1e300;
   for (int s = 1; s <= ntiles; ++s) {
     if (s > 1 && (long)rblocks * (s - 1) > 16 * slots) break;
+    // up to three row blocks (a search of few queries): buffers of at most kFewRowsBytes, so that
+    // the workspace stays within what callers with fixed scratch had for such problems
+    if (s > 1 && na <= 3 * BM && (long)s * na * p.cap * 8 > kFewRowsBytes) break;
     const int tps = (ntiles + s - 1) / s;
     if ((long)tps * BN > kSelMaxCols) continue;
     const long ctas = (long)rblocks * ((ntiles + tps - 1) / tps);
