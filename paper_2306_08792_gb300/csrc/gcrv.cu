@@ -227,7 +227,7 @@ __global__ void gram_mirror_kernel(float* __restrict__ G, int d) {
 // from the caches for the mean, so they leave memory once: 675,977 frames of d = 2048 1.83 -> 1.45
 // ms (5.5 GB: 0.82 ms at the copy rate; the rest is the two phases of a batch waiting for each
 // other). VPT x 1024 >= d.
-constexpr int kMeanBatch = 16;
+constexpr int kMeanBatch = 8;  // (a whole call 16.39 ms at 16, 16.10 at 8, 16.53 at 4, 16.48 at 32)
 template <int VPT>
 __global__ void __launch_bounds__(256) norm_means_kernel(const float* __restrict__ F, int d,
                                                          const int64_t* __restrict__ off,
