@@ -1,4 +1,4 @@
-"""The frame passes of the profile vectors at the edges of their batches (16 frames) and column
+"""The frame passes of the profile vectors at the edges of their batches (8 frames) and column
 slices (512 and 1,024 floats)."""
 import numpy as np
 import pytest
