@@ -136,6 +136,12 @@ __device__ __forceinline__ uint32_t float_to_ordered(float f) {
 __device__ __forceinline__ float ordered_to_float(uint32_t u) {
   return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
+// The largest float that compares below f (finite or +inf). Below either zero that is the smallest
+// negative number: -0, whose image is one less than +0's, compares equal to +0.
+__device__ __forceinline__ float float_below(float f) {
+  const uint32_t k = float_to_ordered(f + 0.f);
+  return ordered_to_float(k - (k == 0x80000000u ? 2u : 1u));
+}
 
 // Exclusive scan over [0, n) by one block of 1024 threads, tiles of 8,192 elements with a running
 // carry: ld(i) gives element i (called once, coalesced), st(i, prefix, value) takes its prefix.

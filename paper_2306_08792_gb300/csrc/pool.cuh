@@ -372,7 +372,7 @@ __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState 
         keep[w] = m;
       }
       f = ordered_to_float(k);
-      lo = ordered_to_float(k - 1u);  // every entry kept is above the value below f
+      lo = float_below(f);  // every entry kept is above the value below f
       kept = KP;
       sum = x;
     }

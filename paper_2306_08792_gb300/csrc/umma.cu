@@ -634,7 +634,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       float floor = -CUDART_INF_F;
       if (valid && a.seed) floor = a.seed[(size_t)my_row * a.seed_ld];
       // strictly above the value below the floor
-      pool_init(me, valid, floor > -CUDART_INF_F ? ordered_to_float(float_to_ordered(floor + 0.f) - 1u) : floor);
+      pool_init(me, valid, floor > -CUDART_INF_F ? float_below(floor) : floor);
       if (CROSS && valid) my_cam = a.cam[my_row];
     }
     ItemCursor cur;

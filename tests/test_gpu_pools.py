@@ -123,3 +123,45 @@ def test_ranking_of_short_galleries(ng):
     D = torch.cdist(Xq.double(), Xg.double()).square().cpu().numpy()
     # FP32 products of 40 terms: 40 * 2^-24, and the rounding of the distance
     assert np.max(np.abs(np.take_along_axis(D, idx, axis=1) - dist)) < 2 * 40 * 2.0 ** -24 + 3 * 2.0 ** -23
+
+
+@pytest.mark.parametrize("precision", ["tf32", "bf16", "fp32"])
+@pytest.mark.parametrize("K", [10, 100])
+def test_wide_search_of_rows_that_meet_few_others(precision, K):
+    """Queries of which five gallery rows, or none, have a positive score: the sampled floor is zero, and
+    the rest of the list is the smallest indices among the rows of score zero (norms are exactly 1)."""
+    import paper_2306_08792_gb300 as gcr
+    ng = 300001
+    G = torch.zeros(ng, 64, device="cuda")
+    G[torch.arange(ng, device="cuda"), torch.arange(ng, device="cuda") % 32] = 1
+    near = torch.tensor([7, 50000, 123456, 250001, ng - 1], device="cuda")
+    G[near] = 0
+    G[near, 40] = 1
+    Q = torch.zeros(40, 64, device="cuda")
+    Q[1::2, 40] = 1  # the even ones are zero rows
+    idx, dist = gcr.gcr_rerank(Q, G, gcr.default_params(precision=precision, topk_out=K))
+    idx = idx.long().cpu()
+    all_rows = torch.arange(ng)
+    others = all_rows[~torch.isin(all_rows, near.cpu())]
+    assert torch.equal(idx[::2], all_rows[:K].expand(20, K))
+    assert torch.equal(idx[1::2], torch.cat([near.cpu(), others[:K - 5]]).expand(20, K))
+    assert torch.equal(dist[::2], torch.ones(20, K, device="cuda"))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "tf32", "bf16"])
+@pytest.mark.parametrize("k,pool", [(15, 0), (40, 64)])
+def test_rows_without_a_positive_score_take_the_smallest_columns(precision, k, pool):
+    """900 of 3,000 unit rows are orthogonal to all others: every score of theirs is zero, every
+    distance 2, and the ties go to the smaller index."""
+    import paper_2306_08792_gb300 as gcr
+    n = 3000
+    alone = np.sort(np.random.default_rng(8).choice(n, 900, replace=False))
+    col = np.arange(n) % 60
+    col[alone] = 60 + np.arange(900)
+    X = np.zeros((n, 960), dtype=np.float32)
+    X[np.arange(n), col] = 1
+    G = gcr.gcr_build_graph(torch.from_numpy(X).cuda(), gcr.default_params(k=k, precision=precision, pool=pool))
+    nbr = np.sort(G.nbr.cpu().numpy()[alone], axis=1)
+    first = np.arange(k + 1)
+    for t, i in enumerate(alone):
+        assert np.array_equal(nbr[t], first[first != i][:k]), (t, nbr[t])
