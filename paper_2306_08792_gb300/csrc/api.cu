@@ -112,9 +112,12 @@ size_t op_capacity(int64_t n, const gcr_params* p, int kinds) {
   return (size_t)(n * per);
 }
 
-PoolParts carve_parts(Carve& c, int na, int nb, int d, const gcr_params* p, Elt elt, int kp, bool cross) {
+// any_fewer: room for the buffers of every smaller search too, where the splits of few rows need it.
+PoolParts carve_parts(Carve& c, int na, int nb, int d, const gcr_params* p, Elt elt, int kp, bool cross,
+                      bool any_fewer = false) {
   const PoolPlan pl = tensor_mode(p) ? pool_plan(na, nb, d, elt, kp, cross) : simt_pool_plan(na, nb, d, kp, cross);
-  const size_t rows = pool_part_rows(pl, na, cross);
+  size_t rows = pool_part_rows(pl, na, cross);
+  if (any_fewer && !tensor_mode(p)) rows = std::max(rows, simt_part_rows_bound(na, nb, kp, cross));
   PoolParts t;
   t.v = c.take<float>(rows * pl.cap);
   t.i = c.take<int>(rows * pl.cap);
@@ -734,8 +737,9 @@ int serve_kp_final(const gcr_params* p) {
   return K < 64 ? 64 : 128;
 }
 
+// any_batch: room for every smaller batch too (what gcr_serve_workspace_size promises).
 size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params* p, Elt elt, const Resolved& r,
-                   ServeWs* w) {
+                   ServeWs* w, bool any_batch = true) {
   const size_t nb = (size_t)b;
   const bool bf = tensor_mode(p);
   const size_t es = elt_bytes(elt);
@@ -750,17 +754,17 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   t.anrm = bf ? c.take<float>(nb) : nullptr;
   t.sc = c.take<RowScalars>(1);
   // one region for both pool sizes, as large as any smaller batch needs it (a batch of fewer row
-  // blocks is cut into more splits): a workspace sized for a batch serves every smaller one
-  // (the band's entries, written after a search's pools are finished and read before the next
+  // blocks, in FP32 one of fewer rows, is cut into more splits): a workspace sized for a batch
+  // serves every smaller one (the band's entries, written after a search's pools are finished and read before the next
   // search, share it)
   Carve cband = c;
   t.band_v = cband.take<float>(nb * kBandCap);
   t.band_i = cband.take<int>(nb * kBandCap);
   size_t end = cband.off;
-  for (int64_t rows = std::min<int64_t>(b, 128);; rows = std::min<int64_t>(b, rows + 128)) {
+  for (int64_t rows = any_batch ? std::min<int64_t>(b, 128) : b;; rows = std::min<int64_t>(b, rows + 128)) {
     Carve c1 = c, c2 = c;
-    t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, elt, r.kp, false);
-    t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, p, elt, serve_kp_final(p), false);
+    t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, elt, r.kp, false, any_batch);
+    t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, p, elt, serve_kp_final(p), false, any_batch);
     end = std::max(end, std::max(c1.off, c2.off));
     if (rows == b) break;
   }
@@ -896,7 +900,7 @@ size_t carve_topk_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_
   r.kp = serve_kp_final(p);
   r.kinds = 1;
   TopkRerankWs t;
-  carve_serve(c, nq, ng, d, p, elt_of(p), r, &t.sw);
+  carve_serve(c, nq, ng, d, p, elt_of(p), r, &t.sw, false);
   t.n64g = c.take<double>(ng);
   t.n32g = c.take<float>(ng);
   t.gr = bf ? c.take<char>((size_t)ng * d * elt_size(p)) : nullptr;

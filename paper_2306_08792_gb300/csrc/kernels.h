@@ -75,6 +75,8 @@ struct PoolParts {   // scratch of one sweep
 
 // ---- sgemm.cu
 PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross);
+// Bound on pool_part_rows over all searches of min(na, 384) rows or fewer.
+size_t simt_part_rows_bound(int na, int nb, int kp, bool cross);
 // As launch_umma_pool (below) on the CUDA cores.
 cudaError_t launch_sgemm_pool(const float* A, int na, const float* B, int nb, int d, const int* cam, int kp,
                               bool cross, int self_excl, const PoolParts& parts, float* pool_v, int* pool_i,

@@ -269,14 +269,19 @@ static int simt_ctas(int kp, bool cross) { return kp == 128 || (kp == 64 && cros
 // As pool_plan: splits whose CTAs fill the SMs evenly. A tile takes about 2 * 128 * 128 * d FMAs
 // at the SM's share; set-up, the first tile's rounds and the write-out about 20 us.
 constexpr long kFewRowsBytes = 9l << 20;
+constexpr int kFewRows = 3 * BM;
+
+static int simt_cap(int kp, bool cross) {
+  return kp == 32 ? (cross ? SelCap<32, true>::cap : SelCap<32, false>::cap)
+         : kp == 64 ? (cross ? SelCap<64, true>::cap : SelCap<64, false>::cap)
+                    : SelCap<128, false>::cap;
+}
 
 PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
   PoolPlan p{};
   p.sel = true;
   const bool two = kp == 128 && cross;  // two graphs of 128-entry pools: a sweep for each
-  p.cap = kp == 32 ? (cross ? SelCap<32, true>::cap : SelCap<32, false>::cap)
-          : kp == 64 ? (cross ? SelCap<64, true>::cap : SelCap<64, false>::cap)
-                     : SelCap<128, false>::cap;
+  p.cap = simt_cap(kp, cross);
   const int ntiles = (nb + BN - 1) / BN, rblocks = (na + BM - 1) / BM;
   const int slots = kSMs * simt_ctas(kp, cross && !two);
   const double tile_us = d * 0.15, around = 20.0 / tile_us;
@@ -286,7 +291,7 @@ PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
     if (s > 1 && (long)rblocks * (s - 1) > 16 * slots) break;
     // up to three row blocks (a search of few queries): buffers of at most kFewRowsBytes, so that
     // the workspace stays within what callers with fixed scratch had for such problems
-    if (s > 1 && na <= 3 * BM && (long)s * na * p.cap * 8 > kFewRowsBytes) break;
+    if (s > 1 && na <= kFewRows && (long)s * na * p.cap * 8 > kFewRowsBytes) break;
     const int tps = (ntiles + s - 1) / s;
     if ((long)tps * BN > kSelMaxCols) continue;
     const long ctas = (long)rblocks * ((ntiles + tps - 1) / tps);
@@ -300,6 +305,18 @@ PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
   p.tps = (ntiles + best - 1) / best;
   p.splits = (ntiles + p.tps - 1) / p.tps;
   return p;
+}
+
+// The splits of few rows depend on the row count, not on its blocks alone: a smaller search can need
+// more. Its buffers are within kFewRowsBytes or what the 16-bit column offsets force, its splits at
+// most the column tiles and, up to two row blocks, the places on the chip (which one and two
+// blocks divide evenly: no cut of more waves is shorter).
+size_t simt_part_rows_bound(int na, int nb, int kp, bool cross) {
+  const long few = std::min(na, kFewRows), ntiles = (nb + BN - 1) / BN;
+  const long slots = kSMs * simt_ctas(kp, cross && kp != 128), forced = ((long)nb + kSelMaxCols - 1) / kSelMaxCols + 1;
+  long rows = std::min(kFewRowsBytes / (simt_cap(kp, cross) * 8), ntiles * few);
+  if (few <= 2 * BM) rows = std::min(rows, slots * std::min<long>(few, BM));
+  return (size_t)std::max(rows, std::min(forced, ntiles) * few);
 }
 
 namespace {
