@@ -114,11 +114,13 @@ size_t op_capacity(int64_t n, const gcr_params* p, int kinds) {
 
 // any_fewer: room for the buffers of every smaller search too, where the splits of few rows need it.
 PoolParts carve_parts(Carve& c, int na, int nb, int d, const gcr_params* p, Elt elt, int kp, bool cross,
-                      bool any_fewer = false) {
-  const PoolPlan pl = tensor_mode(p) ? pool_plan(na, nb, d, elt, kp, cross) : simt_pool_plan(na, nb, d, kp, cross);
+                      bool any_fewer = false, int max_splits = INT_MAX) {
+  const PoolPlan pl = tensor_mode(p) ? pool_plan(na, nb, d, elt, kp, cross, max_splits)
+                                     : simt_pool_plan(na, nb, d, kp, cross, max_splits);
   size_t rows = pool_part_rows(pl, na, cross);
   if (any_fewer && !tensor_mode(p)) rows = std::max(rows, simt_part_rows_bound(na, nb, kp, cross));
   PoolParts t;
+  t.plan = pl;
   t.v = c.take<float>(rows * pl.cap);
   t.i = c.take<int>(rows * pl.cap);
   t.cnt = c.take<int>(rows);
@@ -739,7 +741,7 @@ int serve_kp_final(const gcr_params* p) {
 
 // any_batch: room for every smaller batch too (what gcr_serve_workspace_size promises).
 size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params* p, Elt elt, const Resolved& r,
-                   ServeWs* w, bool any_batch = true) {
+                   ServeWs* w, bool any_batch = true, int max_splits = INT_MAX) {
   const size_t nb = (size_t)b;
   const bool bf = tensor_mode(p);
   const size_t es = elt_bytes(elt);
@@ -763,8 +765,8 @@ size_t carve_serve(Carve& c, int64_t b, int64_t ng, int32_t d, const gcr_params*
   size_t end = cband.off;
   for (int64_t rows = any_batch ? std::min<int64_t>(b, 128) : b;; rows = std::min<int64_t>(b, rows + 128)) {
     Carve c1 = c, c2 = c;
-    t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, elt, r.kp, false, any_batch);
-    t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, p, elt, serve_kp_final(p), false, any_batch);
+    t.parts = carve_parts(c1, (int)rows, (int)ng, d, p, elt, r.kp, false, any_batch, max_splits);
+    t.parts_final = carve_parts(c2, (int)rows, (int)ng, d, p, elt, serve_kp_final(p), false, any_batch, max_splits);
     end = std::max(end, std::max(c1.off, c2.off));
     if (rows == b) break;
   }
@@ -894,13 +896,14 @@ struct TopkRerankWs {
   BallArgs ball;       // ball search of the queries the pools cannot certify (tensor-core modes)
 };
 
-size_t carve_topk_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_params* p, TopkRerankWs* w) {
+size_t carve_topk_rerank_at(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_params* p, int max_splits,
+                            TopkRerankWs* w) {
   const bool bf = tensor_mode(p);
   Resolved r;
   r.kp = serve_kp_final(p);
   r.kinds = 1;
   TopkRerankWs t;
-  carve_serve(c, nq, ng, d, p, elt_of(p), r, &t.sw, false);
+  carve_serve(c, nq, ng, d, p, elt_of(p), r, &t.sw, false, max_splits);
   t.n64g = c.take<double>(ng);
   t.n32g = c.take<float>(ng);
   t.gr = bf ? c.take<char>((size_t)ng * d * elt_size(p)) : nullptr;
@@ -913,6 +916,27 @@ size_t carve_topk_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_
                      &t.ball, (int)ng);
   if (w) *w = t;
   return c.off;
+}
+
+// A search that fits gcr_rerank_noalloc's array with fewer splits of the sweep takes as many as fit
+// (few queries against 300,000 rows and more, whose norms fill much of the array): a callers' scratch
+// of that size goes on serving what it served when a split left a list and not a buffer.
+size_t carve_topk_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_params* p, TopkRerankWs* w) {
+  const size_t limit = GCR_RERANK_NOALLOC_SCRATCH_BYTES - 256;
+  auto need = [&](int m) {
+    Carve t(nullptr, 0);
+    return carve_topk_rerank_at(t, nq, ng, d, p, m, nullptr);
+  };
+  int lo = INT_MAX;
+  if (need(INT_MAX) > limit && need(1) <= limit) {
+    lo = 1;
+    for (int hi = 4096; hi - lo > 1;) {  // (a plan has at most about 2,500 splits)
+      const int mid = (lo + hi) / 2;
+      if (need(mid) <= limit) lo = mid;
+      else hi = mid;
+    }
+  }
+  return carve_topk_rerank_at(c, nq, ng, d, p, lo, w);
 }
 
 int topk_rerank_impl(const float* Xq, int64_t nq, const float* Xg, int64_t ng, int32_t d, const gcr_params* p,

@@ -1,5 +1,6 @@
 // Internal declarations shared by the GCR translation units (not part of the C ABI).
 #pragma once
+#include <limits.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -63,10 +64,13 @@ struct PoolPlan {
   bool deep;         // the four-stage variant of the 32-entry pools
   bool split_first, cluster;
   int sample_tiles;  // column tiles of the sample sweep that gives the rows their floors (0: none)
+  int sample_splits; // and its splits
 };
-PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross);  // umma.cu
+// max_splits: at most so many (but for what the 16-bit column offsets force), where scratch is short.
+PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross, int max_splits = INT_MAX);  // umma.cu
 size_t pool_part_rows(const PoolPlan& p, int na, bool cross);
-struct PoolParts {   // scratch of one sweep
+struct PoolParts {   // one sweep's plan and scratch
+  PoolPlan plan;
   float* v;          // pool_part_rows * cap
   int* i;
   int* cnt;          // pool_part_rows
@@ -74,7 +78,7 @@ struct PoolParts {   // scratch of one sweep
 };
 
 // ---- sgemm.cu
-PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross);
+PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross, int max_splits = INT_MAX);
 // Bound on pool_part_rows over all searches of min(na, 384) rows or fewer.
 size_t simt_part_rows_bound(int na, int nb, int kp, bool cross);
 // As launch_umma_pool (below) on the CUDA cores.

@@ -277,7 +277,7 @@ static int simt_cap(int kp, bool cross) {
                     : SelCap<128, false>::cap;
 }
 
-PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
+PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross, int max_splits) {
   PoolPlan p{};
   p.sel = true;
   const bool two = kp == 128 && cross;  // two graphs of 128-entry pools: a sweep for each
@@ -287,7 +287,7 @@ PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross) {
   const double tile_us = d * 0.15, around = 20.0 / tile_us;
   int best = 1;
   double best_t = 1e300;
-  for (int s = 1; s <= ntiles; ++s) {
+  for (int s = 1; s <= std::min(ntiles, max_splits); ++s) {
     if (s > 1 && (long)rblocks * (s - 1) > 16 * slots) break;
     // up to three row blocks (a search of few queries): buffers of at most kFewRowsBytes, so that
     // the workspace stays within what callers with fixed scratch had for such problems
@@ -337,7 +337,7 @@ cudaError_t launch_simt(const PoolPlan& p, const float* A, int na, const float* 
 cudaError_t launch_sgemm_pool(const float* A, int na, const float* B, int nb, int d, const int* cam, int kp,
                               bool cross, int self_excl, const PoolParts& parts, float* pool_v, int* pool_i,
                               cudaStream_t st) {
-  const PoolPlan p = simt_pool_plan(na, nb, d, kp, cross);
+  const PoolPlan& p = parts.plan;
   const int kinds = cross ? 2 : 1;
   uint32_t* tau = nullptr;
   cudaError_t e = cudaSuccess;

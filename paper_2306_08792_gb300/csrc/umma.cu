@@ -995,7 +995,7 @@ int umma_read_and_clear_timeouts() {
 
 // A sweep's time in units of a column tile, per CTA: its tiles and the set-up, first-tile floor
 // and write-out around them (about 12 us against d / 64 * 0.25 us per tile, at least 0.8).
-PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross) {
+PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross, int max_splits) {
   PoolPlan p;
   p.sel = !(kp == 128 && cross);
   // eight K blocks or fewer per tile: a three-stage ring covers them
@@ -1009,7 +1009,7 @@ PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross) {
   auto tps_of = [&](int s) { return (ntiles + s - 1) / s; };
   int best = 1;
   double best_t = 1e300;
-  for (int s = 1; s <= std::min(ntiles, kSMs); ++s) {
+  for (int s = 1; s <= std::min(std::min(ntiles, kSMs), max_splits); ++s) {
     const int tps = tps_of(s);
     if (s > 1 && (long)rblocks * (s - 1) > 16 * kSMs) break;  // past 16 waves nothing is left to even out
     if (p.sel && (long)tps * BN > kSelMaxCols) continue;  // 16-bit column offsets
@@ -1029,7 +1029,7 @@ PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross) {
   // time, so half as many blocks are at work.
   const double live_a = (double)std::min(rblocks, kSMs) * BM * d * (double)elt_bytes(elt);
   p.split_first = false;
-  if (best == 1 && ntiles >= 2 && live_a > 0.5 * kL2Bytes) {
+  if (best == 1 && std::min(ntiles, max_splits) >= 2 && live_a > 0.5 * kL2Bytes) {
     best = 2;
     p.split_first = true;
   }
@@ -1048,19 +1048,17 @@ PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross) {
   p.sample_tiles = 0;
   if (p.sel && !cross && p.splits >= 8 && p.tps >= 4) p.sample_tiles = std::max(16, std::min(64, ntiles / 16));
   if (p.sample_tiles * 2 > ntiles) p.sample_tiles = 0;
+  p.sample_splits = 0;
+  if (p.sample_tiles) {  // about one sample tile per CTA
+    const int tps = std::max((int)(((long)p.sample_tiles * rblocks + kSMs - 1) / kSMs),
+                             1 + (p.sample_tiles - 1) / max_splits);
+    p.sample_splits = (p.sample_tiles + tps - 1) / tps;
+  }
   return p;
 }
 
-// Splits of the sample sweep: about one sample tile per CTA.
-static int sample_splits(const PoolPlan& p, int na) {
-  const int rblocks = (na + BM - 1) / BM;
-  const int tps = (int)std::max<long>(1, ((long)p.sample_tiles * rblocks + kSMs - 1) / kSMs);
-  return (p.sample_tiles + tps - 1) / tps;
-}
-
 size_t pool_part_rows(const PoolPlan& p, int na, bool cross) {
-  const int splits = p.sample_tiles ? std::max(p.splits, sample_splits(p, na)) : p.splits;
-  return (size_t)splits * (cross ? 2 : 1) * na;
+  return (size_t)std::max(p.splits, p.sample_splits) * (cross ? 2 : 1) * na;
 }
 
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
@@ -1073,7 +1071,7 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
   if (e != cudaSuccess) return e;
   e = make_map(&tb_half, Bb, elt, nb, d, BN / 2);
   if (e != cudaSuccess) return e;
-  const PoolPlan p = pool_plan(na, nb, d, elt, kp, cross);
+  const PoolPlan& p = parts.plan;
   const int rblocks = (na + BM - 1) / BM, kinds = cross ? 2 : 1;
   UmmaArgs a{};
   a.mode = POOL;
@@ -1099,7 +1097,7 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
     UmmaArgs sa = a;
     sa.n = rows;
     sa.split_first = 0;
-    const int splits = sample_splits(p, na);
+    const int splits = p.sample_splits;
     sa.tps = (p.sample_tiles + splits - 1) / splits;
     const dim3 sg(rblocks, splits);
     e = kp == 32   ? (p.deep ? launch<POOL, 32, false, true>(ta, sb, sa, sg, st) : launch<POOL, 32, false>(ta, sb, sa, sg, st))

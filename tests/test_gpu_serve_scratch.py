@@ -22,3 +22,20 @@ def test_fp32_buckets_in_the_workspace_of_the_largest():
         i, d = G.query(torch.from_numpy(r.queries).cuda())
         assert np.array_equal(i.cpu().numpy(), r.idx)
         np.testing.assert_allclose(d.cpu().numpy(), r.dist, atol=1e-6, rtol=0)
+
+
+@pytest.mark.parametrize("nq,ng,topk", [(34, 577049, 10), (11, 791863, 63)])
+def test_top_k_in_the_static_scratch_with_fewer_splits(nq, ng, topk):
+    """The distances of the K nearest, in order, within 1e-5 (FP32 dot products of 32 terms), and
+    every index at its distance."""
+    import paper_2306_08792_gb300 as gcr
+    g = torch.Generator(device="cuda").manual_seed(nq)
+    q = gcr.gcr_normalize(torch.randn(nq, 32, generator=g, device="cuda"))
+    b = gcr.gcr_normalize(torch.randn(ng, 32, generator=g, device="cuda"))
+    idx = torch.empty(nq, topk, dtype=torch.int32, device="cuda")
+    dist = torch.empty(nq, topk, device="cuda")
+    gcr.gcr_rerank_noalloc(q, b, gcr.default_params(precision="fp32", topk_out=topk), idx, dist)
+    D = 2.0 - 2.0 * (q.double() @ b.double().T)
+    want = D.topk(topk, dim=1, largest=False).values
+    assert (D.gather(1, idx.long()) - want).abs().max() < 1e-5 and (dist.double() - want).abs().max() < 1e-5
+    assert all(len(set(r)) == topk for r in idx.cpu().tolist())
