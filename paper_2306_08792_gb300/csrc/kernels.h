@@ -57,12 +57,12 @@ cudaError_t launch_rerank_prep(const float* Xq, int nq, const float* Xg, int ng,
                                __nv_bfloat16* qb, __nv_bfloat16* gb, cudaStream_t st);
 
 // How a pool sweep is cut: the column splits of each 128-row block (tps column tiles each, in
-// the grid's order), whether clusters share the column tiles, and the buffers its splits leave.
+// the grid's order), and the buffers its splits leave.
 struct PoolPlan {
   bool sel;          // selection buffers of cap slots (else sorted lists of cap = kp entries)
   int cap, splits, tps;
   bool deep;         // the four-stage variant of the 32-entry pools
-  bool split_first, cluster;
+  bool split_first;
   int sample_tiles;  // column tiles of the sample sweep that gives the rows their floors (0: none)
   int sample_splits; // and its splits
 };

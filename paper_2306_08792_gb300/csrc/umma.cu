@@ -147,30 +147,6 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
-// 2-CTA clusters sharing B tiles: the commit arrives on the barrier at the same offset in every
-// CTA of the mask; the load writes the tile (and completes its bytes on the barrier) at the same
-// offsets in every CTA of the mask.
-__device__ __forceinline__ void umma_commit_mc(uint64_t* bar, uint16_t mask) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(smem_u32(bar)), "h"(mask)
-               : "memory");
-}
-__device__ __forceinline__ void tma_load_2d_mc(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y,
-                                               uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster"
-      " [%0], [%1, {%3, %4}], [%2], %5;"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "h"(mask)
-      : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 // Asynchronous TMEM load of 32 columns (one accumulator row per thread) ...
 __device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -267,10 +243,6 @@ struct UmmaArgs {
   // any split has published (KP of the row's scores are strictly above it; 0: none yet). Every
   // split reads it before a tile and raises its own threshold to it.
   uint32_t* tau_x;
-  // POOL: 2-CTA clusters of consecutive row blocks that take the same column tiles; each CTA loads its A block and one half of the B tile, and the half goes to both
-  // CTAs by TMA multicast (tmB2: B in 128-row boxes), so a CTA reads two thirds of the bytes
-  // per stage. Each MMA commit frees the stage in both CTAs (empty barriers count 2 arrivals).
-  int mc;
   Gate gate;       // POOL, BAND: whether this launch runs
 };
 
@@ -481,7 +453,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&bars.full[s], 1);
-      mbar_init(&bars.empty[s], (MODE == POOL && a.mc) ? 2 : 1);
+      mbar_init(&bars.empty[s], 1);
     }
     const int epi_warps = CROSS ? 8 : 4;
     for (int b = 0; b < 2; ++b) {
@@ -500,8 +472,6 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // clusters: every barrier of both CTAs is initialised before either CTA signals the other's
-  if (MODE == POOL && a.mc) cluster_sync_all();
   const uint32_t tmem = bars.tmem_base;
   volatile int* abort_flag = &bars.abort_flag;
 
@@ -528,13 +498,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             tma_load_2d(sa + A_BYTES, (kb & 1) ? &tmB2 : &tmB, &bars.full[s], x, mul_b0 + c0);
           } else {
             tma_load_2d(sa, &tmA, &bars.full[s], kb * bk, r0);
-            if (MODE == POOL && a.mc) {
-              const uint32_t cr = cluster_rank();
-              tma_load_2d_mc(sa + A_BYTES + cr * (B_BYTES / 2), &tmB2, &bars.full[s], kb * bk,
-                             c0 + (int)cr * (BN / 2), (uint16_t)0x3);
-            } else {
-              tma_load_2d(sa + A_BYTES, &tmB, &bars.full[s], kb * bk, c0);
-            }
+            tma_load_2d(sa + A_BYTES, &tmB, &bars.full[s], kb * bk, c0);
           }
         }
       }
@@ -592,8 +556,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             continue;
           }
           mma4(ad, bd, kb != 0);
-          if (MODE == POOL && a.mc) umma_commit_mc(&bars.empty[s], (uint16_t)0x3);
-          else umma_commit(&bars.empty[s]);
+          umma_commit(&bars.empty[s]);
         }
         if (ok) umma_commit(&bars.tfull[buf]);
       }
@@ -875,9 +838,6 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   }
   tc_fence_before();
   __syncthreads();
-  // clusters: neither CTA leaves while the other may still signal its barriers (its MMAs have
-  // drained by now) or write its stages
-  if (MODE == POOL && a.mc) cluster_sync_all();
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
@@ -954,29 +914,14 @@ constexpr size_t smem_bytes() {
 
 template <int MODE, int KP, bool CROSS, bool DEEP = false>
 cudaError_t launch(const CUtensorMap& ta, const CUtensorMap& tb, const UmmaArgs& a, dim3 grid, cudaStream_t st,
-                   const CUtensorMap* ta2 = nullptr, const CUtensorMap* tb2 = nullptr, dim3 cluster = dim3(1, 1, 1)) {
+                   const CUtensorMap* ta2 = nullptr, const CUtensorMap* tb2 = nullptr) {
   auto fn = umma_kernel<MODE, KP, CROSS, DEEP>;
   constexpr size_t smem = smem_bytes<MODE, KP, CROSS, DEEP>();
   static_assert(smem + sizeof(Bars) <= 232448, "shared memory of a CTA");
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  if (cluster.x * cluster.y * cluster.z == 1) {
-    fn<<<grid, CROSS ? 320 : 192, smem, st>>>(ta, tb, ta2 ? *ta2 : ta, tb2 ? *tb2 : tb, a);
-    return cudaGetLastError();
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(CROSS ? 320 : 192, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cluster.x;
-  at[0].val.clusterDim.y = cluster.y;
-  at[0].val.clusterDim.z = cluster.z;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fn, ta, tb, ta2 ? *ta2 : ta, tb2 ? *tb2 : tb, a);
+  fn<<<grid, CROSS ? 320 : 192, smem, st>>>(ta, tb, ta2 ? *ta2 : ta, tb2 ? *tb2 : tb, a);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -1035,9 +980,6 @@ PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross, int max_s
   }
   p.tps = tps_of(best);
   p.splits = (ntiles + p.tps - 1) / p.tps;  // no split is left without a column tile
-  // 2-CTA clusters of row blocks share the column tiles (an even count: the last block of an odd
-  // one has no rows and only loads its half of the shared tiles, so not for few blocks)
-  p.cluster = p.sel && (rblocks % 2 == 0 || rblocks > 16);
   // Many splits over long ranges (few rows against many columns): each split alone would admit
   // about kp (1 + ln(its columns / kp)) scores a row. A sweep of an evenly spaced sample of the
   // columns first bounds every row at about the (kp / share)-th best of all its scores, which
@@ -1064,12 +1006,10 @@ size_t pool_part_rows(const PoolPlan& p, int na, bool cross) {
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
                              const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
                              float* pool_v, int* pool_i, cudaStream_t st, Gate gate, int a_step) {
-  CUtensorMap ta, tb, tb_half;
+  CUtensorMap ta, tb;
   cudaError_t e = make_map(&ta, Ab, elt, na, d, BM, a_step);
   if (e != cudaSuccess) return e;
   e = make_map(&tb, Bb, elt, nb, d, BN);
-  if (e != cudaSuccess) return e;
-  e = make_map(&tb_half, Bb, elt, nb, d, BN / 2);
   if (e != cudaSuccess) return e;
   const PoolPlan& p = parts.plan;
   const int rblocks = (na + BM - 1) / BM, kinds = cross ? 2 : 1;
@@ -1114,13 +1054,13 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
     e = cudaMemsetAsync(parts.tau, 0, sizeof(uint32_t) * kinds * (size_t)na, st);
     if (e != cudaSuccess) return e;
   }
-  const int rb_grid = p.cluster ? (rblocks + 1) & ~1 : rblocks;
-  const dim3 grid = p.split_first ? dim3(p.splits, rb_grid) : dim3(rb_grid, p.splits);
-  a.mc = p.cluster;
-  const dim3 cl = !p.cluster ? dim3(1, 1, 1) : p.split_first ? dim3(1, 2, 1) : dim3(2, 1, 1);
-  if (kp == 32) e = cross ? launch<POOL, 32, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : p.deep ? launch<POOL, 32, false, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : launch<POOL, 32, false>(ta, tb, a, grid, st, nullptr, &tb_half, cl);
-  else if (kp == 64) e = cross ? launch<POOL, 64, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : launch<POOL, 64, false>(ta, tb, a, grid, st, nullptr, &tb_half, cl);
-  else if (kp == 128) e = cross ? launch<POOL, 128, true>(ta, tb, a, grid, st, nullptr, &tb_half, cl) : launch<POOL, 128, false>(ta, tb, a, grid, st, nullptr, &tb_half, cl);
+  const dim3 grid = p.split_first ? dim3(p.splits, rblocks) : dim3(rblocks, p.splits);
+  if (kp == 32)
+    e = cross    ? launch<POOL, 32, true>(ta, tb, a, grid, st)
+        : p.deep ? launch<POOL, 32, false, true>(ta, tb, a, grid, st)
+                 : launch<POOL, 32, false>(ta, tb, a, grid, st);
+  else if (kp == 64) e = cross ? launch<POOL, 64, true>(ta, tb, a, grid, st) : launch<POOL, 64, false>(ta, tb, a, grid, st);
+  else if (kp == 128) e = cross ? launch<POOL, 128, true>(ta, tb, a, grid, st) : launch<POOL, 128, false>(ta, tb, a, grid, st);
   else e = cudaErrorInvalidValue;
   if (e != cudaSuccess) return e;
   if (!p.sel) return launch_merge_splits(parts.v, parts.i, p.splits, kinds, na, kp, pool_v, pool_i, st);
