@@ -65,10 +65,13 @@ struct PoolPlan {
   bool split_first;
   int sample_tiles;  // column tiles of the sample sweep that gives the rows their floors (0: none)
   int sample_splits; // and its splits
+  int rows;          // rows swept at a time (all, or a multiple of 128): their splits' buffers share the scratch
 };
 // max_splits: at most so many (but for what the 16-bit column offsets force), where scratch is short.
 PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross, int max_splits = INT_MAX);  // umma.cu
 size_t pool_part_rows(const PoolPlan& p, int na, bool cross);
+// Rows of a sweep at a time, so that the splits' buffers take at most kPartBytes (or those of 128 rows).
+int pool_sweep_rows(const PoolPlan& p, int na, bool cross);
 struct PoolParts {   // one sweep's plan and scratch
   PoolPlan plan;
   float* v;          // pool_part_rows * cap
@@ -352,11 +355,12 @@ cudaError_t launch_gcrv(const float* frames, int64_t F, int d, const int64_t* of
 
 // ---- serve.cu
 // Sorts and merges the S selection buffers of each (kind, row) ([S][kinds][na][cap], cnt entries)
-// into its pool [kinds][na][kp], best first, padded with (-inf, -1).
+// into its pool, rows [row0, row0 + na) of [kinds][out_rows][kp], best first, padded with (-inf, -1).
 cudaError_t launch_pool_finish(const float* pv, const int* pi, const int* cnt, int S, int kinds, int na, int cap, int kp,
-                               float* ov, int* oi, cudaStream_t st, Gate gate = Gate());
+                               float* ov, int* oi, int out_rows, int row0, cudaStream_t st, Gate gate = Gate());
+// The same for sorted lists [S][kinds][na][kp].
 cudaError_t launch_merge_splits(const float* pv, const int* pi, int S, int kinds, int na, int kp, float* ov, int* oi,
-                                cudaStream_t st);
+                                int out_rows, int row0, cudaStream_t st);
 cudaError_t launch_query_step(const float* xq, int b, int d, const float* G, const float* deg, const int32_t* nbr,
                               const float* d2, int k, float gamma, int symmetric, float* out, cudaStream_t st);
 cudaError_t launch_layer_degree(const float* dr, const float* dc, int n, int symmetric, float* out, cudaStream_t st);

@@ -54,13 +54,19 @@ __device__ __forceinline__ void merge_list(float (&b)[KP / 32], int (&bi)[KP / 3
   }
 }
 
-// Merge S sorted pools per (kind, row) into one: pools [S][kinds][na][KP] -> [kinds][na][KP].
+// The pool of (kind, row) w = kind * na + row among [kinds][out_rows], the rows from row0 on.
+__device__ __forceinline__ size_t out_row(long w, int na, int out_rows, int row0) {
+  const long kind = w >= na ? 1 : 0;  // at most two graphs
+  return (size_t)(kind * out_rows + row0 + (w - kind * na));
+}
+
+// Merge S sorted pools per (kind, row) into one: pools [S][kinds][na][KP] -> [kinds][out_rows][KP].
 // One block of 8 warps per (kind, row): warp w merges splits w, w + 8, ..., then warp 0 merges
 // the 8 partial lists (the strict order makes the result independent of the merge order).
 template <int KP>
 __global__ void __launch_bounds__(256) merge_splits_kernel(const float* __restrict__ pv, const int* __restrict__ pi,
                                                            int S, int kinds, int na, float* __restrict__ ov,
-                                                           int* __restrict__ oi) {
+                                                           int* __restrict__ oi, int out_rows, int row0) {
   constexpr int P = KP / 32;
   __shared__ float sv[8][KP];
   __shared__ int si[8][KP];
@@ -86,10 +92,11 @@ __global__ void __launch_bounds__(256) merge_splits_kernel(const float* __restri
   __syncthreads();
   if (warp != 0) return;
   for (int v = 1; v < 8 && v < S; ++v) merge_list<KP>(b, bi, sv[v], si[v], lane);
+  const size_t out = out_row(w, na, out_rows, row0) * KP;
 #pragma unroll
   for (int p = 0; p < P; ++p) {
-    ov[w * KP + p * 32 + lane] = b[p];
-    oi[w * KP + p * 32 + lane] = bi[p];
+    ov[out + p * 32 + lane] = b[p];
+    oi[out + p * 32 + lane] = bi[p];
   }
 }
 
@@ -124,7 +131,8 @@ __device__ __forceinline__ void merge_chunk(float (&b)[KP / 32], int (&bi)[KP / 
 template <int KP>
 __global__ void __launch_bounds__(256) pool_finish_kernel(const float* __restrict__ pv, const int* __restrict__ pi,
                                                           const int* __restrict__ cnt, int S, long rows, int cap,
-                                                          float* __restrict__ ov, int* __restrict__ oi, Gate gate) {
+                                                          float* __restrict__ ov, int* __restrict__ oi, int part_rows,
+                                                          int out_rows, int row0, Gate gate) {
   if (gate_shut(gate)) return;
   constexpr int P = KP / 32;
   __shared__ float stv[8][64];
@@ -185,10 +193,11 @@ __global__ void __launch_bounds__(256) pool_finish_kernel(const float* __restric
   }
   test(na, ni);
   if (staged > 0) merge_staged(staged);
+  const size_t out = out_row(w, part_rows, out_rows, row0) * KP;
 #pragma unroll
   for (int p = 0; p < P; ++p) {
-    ov[w * KP + p * 32 + lane] = b[p];
-    oi[w * KP + p * 32 + lane] = bi[p];
+    ov[out + p * 32 + lane] = b[p];
+    oi[out + p * 32 + lane] = bi[p];
   }
 }
 
@@ -207,7 +216,8 @@ __global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float* _
                                                                   const int* __restrict__ pi,
                                                                   const int* __restrict__ cnt, int S, long rows,
                                                                   int cap, int group, float* __restrict__ ov,
-                                                                  int* __restrict__ oi, Gate gate) {
+                                                                  int* __restrict__ oi, int part_rows, int out_rows,
+                                                                  int row0, Gate gate) {
   static_assert(KP <= kSelKeep, "the kept entries hold the pool");
   if (gate_shut(gate)) return;
   extern __shared__ __align__(16) unsigned long long ent[];  // [KP + group * cap]
@@ -216,6 +226,7 @@ __global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float* _
   constexpr int NW = kSelThreads / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long w = blockIdx.x;  // (kind, row)
+  const size_t out = out_row(w, part_rows, out_rows, row0) * KP;
   int have = 0;
   for (int s0 = 0; s0 < S; s0 += group) {
     const int s1 = min(S, s0 + group);
@@ -322,14 +333,14 @@ __global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float* _
         if (s1 < S) {
           ent[r] = k;
         } else {
-          ov[w * KP + r] = ordered_to_float((uint32_t)(k >> 32));
-          oi[w * KP + r] = (int)~(uint32_t)k;
+          ov[out + r] = ordered_to_float((uint32_t)(k >> 32));
+          oi[out + r] = (int)~(uint32_t)k;
         }
       }
     }
     __syncthreads();
   }
-  for (int r = have + tid; r < KP; r += kSelThreads) { ov[w * KP + r] = -CUDART_INF_F; oi[w * KP + r] = -1; }
+  for (int r = have + tid; r < KP; r += kSelThreads) { ov[out + r] = -CUDART_INF_F; oi[out + r] = -1; }
 }
 
 // One warp per query: the query's row of the operator against the frozen layer, normalised. Lanes
@@ -443,20 +454,22 @@ __global__ void layer_degree_kernel(const float* __restrict__ dr, const float* _
 }  // namespace
 
 cudaError_t launch_merge_splits(const float* pv, const int* pi, int S, int kinds, int na, int kp, float* ov, int* oi,
-                                cudaStream_t st) {
+                                int out_rows, int row0, cudaStream_t st) {
   dim3 grid((unsigned)((long)kinds * na));  // one block per (kind, row)
-  if (kp == 32) merge_splits_kernel<32><<<grid, 256, 0, st>>>(pv, pi, S, kinds, na, ov, oi);
-  else if (kp == 64) merge_splits_kernel<64><<<grid, 256, 0, st>>>(pv, pi, S, kinds, na, ov, oi);
-  else if (kp == 128) merge_splits_kernel<128><<<grid, 256, 0, st>>>(pv, pi, S, kinds, na, ov, oi);
+  if (kp == 32) merge_splits_kernel<32><<<grid, 256, 0, st>>>(pv, pi, S, kinds, na, ov, oi, out_rows, row0);
+  else if (kp == 64) merge_splits_kernel<64><<<grid, 256, 0, st>>>(pv, pi, S, kinds, na, ov, oi, out_rows, row0);
+  else if (kp == 128) merge_splits_kernel<128><<<grid, 256, 0, st>>>(pv, pi, S, kinds, na, ov, oi, out_rows, row0);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
 template <int KP>
-static cudaError_t pool_finish(const float* pv, const int* pi, const int* cnt, int S, long rows, int cap, float* ov,
-                               int* oi, cudaStream_t st, Gate gate) {
+static cudaError_t pool_finish(const float* pv, const int* pi, const int* cnt, int S, int kinds, int na, int cap,
+                               float* ov, int* oi, int out_rows, int row0, cudaStream_t st, Gate gate) {
+  const long rows = (long)kinds * na;
   if (S <= 8) {  // a warp per row
-    pool_finish_kernel<KP><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, gate);
+    pool_finish_kernel<KP><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(pv, pi, cnt, S, rows, cap, ov, oi, na, out_rows,
+                                                                        row0, gate);
     return cudaGetLastError();
   }
   // a block per row: room for every split's buffer where a block has an SM to itself, for 6,144
@@ -466,16 +479,16 @@ static cudaError_t pool_finish(const float* pv, const int* pi, const int* cnt, i
   const size_t smem = sizeof(unsigned long long) * ((size_t)KP + (size_t)group * cap);
   cudaError_t e = cudaFuncSetAttribute(pool_select_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  pool_select_kernel<KP><<<(unsigned)rows, kSelThreads, smem, st>>>(pv, pi, cnt, S, rows, cap, group, ov, oi, gate);
+  pool_select_kernel<KP><<<(unsigned)rows, kSelThreads, smem, st>>>(pv, pi, cnt, S, rows, cap, group, ov, oi, na,
+                                                                     out_rows, row0, gate);
   return cudaGetLastError();
 }
 
 cudaError_t launch_pool_finish(const float* pv, const int* pi, const int* cnt, int S, int kinds, int na, int cap, int kp,
-                               float* ov, int* oi, cudaStream_t st, Gate gate) {
-  const long rows = (long)kinds * na;
-  if (kp == 32) return pool_finish<32>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
-  if (kp == 64) return pool_finish<64>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
-  if (kp == 128) return pool_finish<128>(pv, pi, cnt, S, rows, cap, ov, oi, st, gate);
+                               float* ov, int* oi, int out_rows, int row0, cudaStream_t st, Gate gate) {
+  if (kp == 32) return pool_finish<32>(pv, pi, cnt, S, kinds, na, cap, ov, oi, out_rows, row0, st, gate);
+  if (kp == 64) return pool_finish<64>(pv, pi, cnt, S, kinds, na, cap, ov, oi, out_rows, row0, st, gate);
+  if (kp == 128) return pool_finish<128>(pv, pi, cnt, S, kinds, na, cap, ov, oi, out_rows, row0, st, gate);
   return cudaErrorInvalidValue;
 }
 

@@ -25,9 +25,10 @@ namespace gcr {
 using namespace simt;
 
 // ---------------------------------------------------------------------------------- POOL
-// S = A . B^T; rows of A own pools, columns are the rows of B. grid = (ceil(na / 128), splits):
-// split y sweeps column tiles [y * tps, (y + 1) * tps). GLOBAL / CROSS: which graphs' pools it
-// keeps; buffers [split][kind][na][cap], kind0 the first of its kinds among them. With self_excl
+// S = A . B^T; rows of A own pools, columns are the rows of B. grid = (row blocks, splits): the
+// part_rows rows from r0 on, split y sweeps column tiles [y * tps, (y + 1) * tps). GLOBAL / CROSS: which
+// graphs' pools it keeps; buffers [split][kind][part_rows][cap], kind0 the first of its kinds among
+// them. With self_excl
 // (A == B) the diagonal is skipped; the cross-camera graph needs A == B.
 //
 // Every thread tests its 128 scores of a tile against the rows' thresholds in shared memory and
@@ -50,7 +51,7 @@ struct SimtPool {
 template <int KP, bool GLOBAL, bool CROSS>
 __global__ void __launch_bounds__(NT, SimtPool<KP, GLOBAL, CROSS>::ctas)
 sgemm_pool_kernel(const float* __restrict__ A, int na, const float* __restrict__ B, int nb, int d,
-                  const int* __restrict__ cam, int self_excl, int tps, int kinds_total, int kind0,
+                  const int* __restrict__ cam, int self_excl, int tps, int r0, int part_rows, int kinds_total, int kind0,
                   float* __restrict__ part_v, int* __restrict__ part_i, int* __restrict__ part_cnt,
                   uint32_t* __restrict__ tau_x) {
   using P = SimtPool<KP, GLOBAL, CROSS>;
@@ -64,7 +65,7 @@ sgemm_pool_kernel(const float* __restrict__ A, int na, const float* __restrict__
   int* camc_s = camr_s + BM;
 
   const int tid = threadIdx.x;
-  const int row0 = blockIdx.x * BM;
+  const int row0 = r0 + blockIdx.x * BM;
   const int arows = min(BM, na - row0);
   const int ntiles = (nb + BN - 1) / BN;
   const int t0 = blockIdx.y * tps, t1 = min(ntiles, t0 + tps);
@@ -167,7 +168,7 @@ sgemm_pool_kernel(const float* __restrict__ A, int na, const float* __restrict__
 #pragma unroll
   for (int q = 0; q < KINDS; ++q) {
     const int cnt = cnt_s[q * BM + tid];
-    const size_t row = ((size_t)blockIdx.y * kinds_total + kind0 + q) * na + row0 + tid;
+    const size_t row = ((size_t)blockIdx.y * kinds_total + kind0 + q) * part_rows + row0 - r0 + tid;
     part_cnt[row] = cnt;
     float4* ov = reinterpret_cast<float4*>(part_v + row * CAP);
     int4* oi = reinterpret_cast<int4*>(part_i + row * CAP);
@@ -304,6 +305,7 @@ PoolPlan simt_pool_plan(int na, int nb, int d, int kp, bool cross, int max_split
   while ((long)((ntiles + best - 1) / best) * BN > kSelMaxCols) ++best;
   p.tps = (ntiles + best - 1) / best;
   p.splits = (ntiles + p.tps - 1) / p.tps;
+  p.rows = pool_sweep_rows(p, na, cross);
   return p;
 }
 
@@ -322,14 +324,14 @@ size_t simt_part_rows_bound(int na, int nb, int kp, bool cross) {
 namespace {
 template <int KP, bool GLOBAL, bool CROSS>
 cudaError_t launch_simt(const PoolPlan& p, const float* A, int na, const float* B, int nb, int d, const int* cam,
-                        int self_excl, int kinds_total, int kind0, const PoolParts& parts, uint32_t* tau,
+                        int self_excl, int r0, int rows, int kinds_total, int kind0, const PoolParts& parts, uint32_t* tau,
                         cudaStream_t st) {
   using P = SimtPool<KP, GLOBAL, CROSS>;
   auto fn = sgemm_pool_kernel<KP, GLOBAL, CROSS>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::smem);
   if (e != cudaSuccess) return e;
-  fn<<<dim3((na + BM - 1) / BM, p.splits), NT, P::smem, st>>>(A, na, B, nb, d, cam, self_excl, p.tps, kinds_total,
-                                                               kind0, parts.v, parts.i, parts.cnt, tau);
+  fn<<<dim3((rows + BM - 1) / BM, p.splits), NT, P::smem, st>>>(A, na, B, nb, d, cam, self_excl, p.tps, r0, rows,
+                                                                 kinds_total, kind0, parts.v, parts.i, parts.cnt, tau);
   return cudaGetLastError();
 }
 }  // namespace
@@ -346,16 +348,22 @@ cudaError_t launch_sgemm_pool(const float* A, int na, const float* B, int nb, in
     e = cudaMemsetAsync(tau, 0, sizeof(uint32_t) * kinds * (size_t)na, st);
     if (e != cudaSuccess) return e;
   }
-#define GCR_SIMT(KPV, G, C, K0) launch_simt<KPV, G, C>(p, A, na, B, nb, d, cam, self_excl, kinds, K0, parts, tau, st)
-  if (kp == 32) e = cross ? GCR_SIMT(32, true, true, 0) : GCR_SIMT(32, true, false, 0);
-  else if (kp == 64) e = cross ? GCR_SIMT(64, true, true, 0) : GCR_SIMT(64, true, false, 0);
-  else if (kp == 128) {
-    e = GCR_SIMT(128, true, false, 0);
-    if (e == cudaSuccess && cross) e = GCR_SIMT(128, false, true, 1);
-  } else return cudaErrorInvalidValue;
+  for (int r0 = 0; r0 < na; r0 += p.rows) {
+    const int rows = std::min(p.rows, na - r0);
+#define GCR_SIMT(KPV, G, C, K0) \
+  launch_simt<KPV, G, C>(p, A, na, B, nb, d, cam, self_excl, r0, rows, kinds, K0, parts, tau, st)
+    if (kp == 32) e = cross ? GCR_SIMT(32, true, true, 0) : GCR_SIMT(32, true, false, 0);
+    else if (kp == 64) e = cross ? GCR_SIMT(64, true, true, 0) : GCR_SIMT(64, true, false, 0);
+    else if (kp == 128) {
+      e = GCR_SIMT(128, true, false, 0);
+      if (e == cudaSuccess && cross) e = GCR_SIMT(128, false, true, 1);
+    } else return cudaErrorInvalidValue;
 #undef GCR_SIMT
-  if (e != cudaSuccess) return e;
-  return launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, na, p.cap, kp, pool_v, pool_i, st);
+    if (e != cudaSuccess) return e;
+    e = launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, rows, p.cap, kp, pool_v, pool_i, na, r0, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_sgemm_band(const float* X, const float* Bm, int n, int d, const int* cam, int self_excl,

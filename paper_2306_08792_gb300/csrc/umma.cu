@@ -190,9 +190,11 @@ struct UmmaArgs {
   int tps;        // POOL: column tiles per split
   const int* cam;
   // POOL
-  float* pool_v;      // sorted lists [split][kind][a_rows][KP], or selection buffers
-  int* pool_i;        //   [split][kind][a_rows][cap] with part_cnt entries each
-  int* part_cnt;      // [split][kind][a_rows]
+  float* pool_v;      // sorted lists [split][kind][part_rows][KP], or selection buffers
+  int* pool_i;        //   [split][kind][part_rows][cap] with part_cnt entries each
+  int* part_cnt;      // [split][kind][part_rows]
+  int row0;           // the launch's rows of A: [row0, row0 + part_rows), row0 a multiple of BM
+  int part_rows;
   // per row of A (stride seed_ld), or NULL: KP of the row's scores are at or above it, so every
   // split keeps only scores at or above it (-inf: no floor)
   const float* seed;
@@ -427,7 +429,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   const int mul_b0 = MODE == MUL ? max(0, a.mul_rowcam[blockIdx.y]) * a.n : 0;
 
   Tiles<MODE> tl;
-  tl.rb = (MODE == POOL && a.split_first) ? (int)blockIdx.y : (int)blockIdx.x;
+  tl.rb = ((MODE == POOL && a.split_first) ? (int)blockIdx.y : (int)blockIdx.x) + (MODE == POOL ? a.row0 / BM : 0);
   tl.split = (MODE == POOL && a.split_first) ? (int)blockIdx.x : (int)blockIdx.y;
   int nitems = 0;
   if (MODE == GPOOL) {
@@ -588,9 +590,10 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     float ssum = 0.f;                                      // sum of the buffered scores
     float pub = -CUDART_INF_F, pub_sent = -CUDART_INF_F;  // bound for the other splits
     const bool idle = SEL && tl.rb * BM + quad * 32 >= a.a_rows;  // no row of this warp exists
-    const size_t pbase = ((size_t)tl.split * KINDS + kind) * a.a_rows * (SEL ? CAP : KP);
-    float* pv = a.pool_v ? a.pool_v + pbase : nullptr;
-    int* pi = a.pool_i ? a.pool_i + pbase : nullptr;
+    // of the launch's rows, indexed by the row of A
+    const ptrdiff_t part0 = (ptrdiff_t)((MODE == POOL ? tl.split : 0) * KINDS + kind) * a.part_rows - a.row0;
+    float* pv = a.pool_v ? a.pool_v + part0 * (SEL ? CAP : KP) : nullptr;
+    int* pi = a.pool_i ? a.pool_i + part0 * (SEL ? CAP : KP) : nullptr;
     if (MODE == POOL) {
       my_row = tl.rb * BM + r;
       const bool valid = my_row < a.a_rows;
@@ -821,7 +824,7 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (my_row < a.a_rows) {
           const int col0 = tl.split * a.tps * BN;
           const int cnt = (int)((sva - sva0) / kSelV);
-          a.part_cnt[((size_t)tl.split * KINDS + kind) * a.a_rows + my_row] = cnt;
+          a.part_cnt[part0 + my_row] = cnt;
           float4* ov = reinterpret_cast<float4*>(pv + (size_t)my_row * CAP);
           int4* oi = reinterpret_cast<int4*>(pi + (size_t)my_row * CAP);
           for (int s = 0; s < cnt; s += 4) {  // (slots past the count: never read)
@@ -940,6 +943,20 @@ int umma_read_and_clear_timeouts() {
 
 // A sweep's time in units of a column tile, per CTA: its tiles and the set-up, first-tile floor
 // and write-out around them (about 12 us against d / 64 * 0.25 us per tile, at least 0.8).
+// The 16-bit column offsets force a split per 65,536 columns, and the buffers of all splits of a row
+// wait for its pool: kept for all rows at once they grow with n^2 (4,000,000 rows of d = 64, 62
+// splits: 190 GB, where everything else takes 28). So the rows are swept in chunks whose buffers
+// share kPartBytes, which still hold 2,000 CTAs and more. 201,000 rows of d = 512 with four splits
+// of 64-entry pools (617 MB, three chunks), the whole three-layer call: 221.2 ms at once, 221.5 so.
+constexpr long kPartBytes = 256l << 20;
+int pool_sweep_rows(const PoolPlan& p, int na, bool cross) {
+  const long per_row = 8l * std::max(p.splits, p.sample_splits) * (cross ? 2 : 1) * p.cap;
+  const long most = std::max<long>(BM, kPartBytes / per_row / BM * BM);
+  if (na <= most) return na;
+  const long chunks = (na + most - 1) / most, rows = (na + chunks - 1) / chunks;
+  return (int)((rows + BM - 1) / BM * BM);
+}
+
 PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross, int max_splits) {
   PoolPlan p;
   p.sel = !(kp == 128 && cross);
@@ -996,23 +1013,35 @@ PoolPlan pool_plan(int na, int nb, int d, Elt elt, int kp, bool cross, int max_s
                              1 + (p.sample_tiles - 1) / max_splits);
     p.sample_splits = (p.sample_tiles + tps - 1) / tps;
   }
+  p.rows = pool_sweep_rows(p, na, cross);
   return p;
 }
 
 size_t pool_part_rows(const PoolPlan& p, int na, bool cross) {
-  return (size_t)std::max(p.splits, p.sample_splits) * (cross ? 2 : 1) * na;
+  return (size_t)std::max(p.splits, p.sample_splits) * (cross ? 2 : 1) * std::min(na, p.rows);
+}
+
+template <typename... T>
+static cudaError_t launch_pool_sweep(int kp, bool cross, bool deep, T&&... t) {
+  if (kp == 32)
+    return cross  ? launch<POOL, 32, true>(t...)
+           : deep ? launch<POOL, 32, false, true>(t...)
+                  : launch<POOL, 32, false>(t...);
+  if (kp == 64) return cross ? launch<POOL, 64, true>(t...) : launch<POOL, 64, false>(t...);
+  if (kp == 128) return cross ? launch<POOL, 128, true>(t...) : launch<POOL, 128, false>(t...);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int d, Elt elt,
                              const int* cam, bool cross, int self_excl, int kp, const PoolParts& parts,
                              float* pool_v, int* pool_i, cudaStream_t st, Gate gate, int a_step) {
-  CUtensorMap ta, tb;
+  CUtensorMap ta, tb, sb;
   cudaError_t e = make_map(&ta, Ab, elt, na, d, BM, a_step);
   if (e != cudaSuccess) return e;
   e = make_map(&tb, Bb, elt, nb, d, BN);
   if (e != cudaSuccess) return e;
   const PoolPlan& p = parts.plan;
-  const int rblocks = (na + BM - 1) / BM, kinds = cross ? 2 : 1;
+  const int kinds = cross ? 2 : 1;
   UmmaArgs a{};
   a.mode = POOL;
   a.tf32 = elt == Elt::TF32;
@@ -1028,23 +1057,14 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
   a.part_cnt = parts.cnt;
   a.split_first = p.split_first;
   a.gate = gate;
-  if (p.sample_tiles && !self_excl) {
-    // every step-th row; the sample's pools end in pool_v, whose last entries are the floors
-    const int rows = p.sample_tiles * BN, step = nb / rows;
-    CUtensorMap sb;
-    e = make_map(&sb, Bb, elt, rows, d, BN, step);
-    if (e != cudaSuccess) return e;
-    UmmaArgs sa = a;
-    sa.n = rows;
+  // every step-th row; the sample's pools end in pool_v, whose last entries are the floors
+  const bool sample = p.sample_tiles && !self_excl;
+  UmmaArgs sa = a;
+  if (sample) {
+    sa.n = p.sample_tiles * BN;
     sa.split_first = 0;
-    const int splits = p.sample_splits;
-    sa.tps = (p.sample_tiles + splits - 1) / splits;
-    const dim3 sg(rblocks, splits);
-    e = kp == 32   ? (p.deep ? launch<POOL, 32, false, true>(ta, sb, sa, sg, st) : launch<POOL, 32, false>(ta, sb, sa, sg, st))
-        : kp == 64 ? launch<POOL, 64, false>(ta, sb, sa, sg, st)
-                   : launch<POOL, 128, false>(ta, sb, sa, sg, st);
-    if (e == cudaSuccess)
-      e = launch_pool_finish(parts.v, parts.i, parts.cnt, splits, 1, na, p.cap, kp, pool_v, pool_i, st, gate);
+    sa.tps = (p.sample_tiles + p.sample_splits - 1) / p.sample_splits;
+    e = make_map(&sb, Bb, elt, sa.n, d, BN, nb / sa.n);
     if (e != cudaSuccess) return e;
     a.seed = pool_v + kp - 1;
     a.seed_ld = kp;
@@ -1054,17 +1074,26 @@ cudaError_t launch_umma_pool(const void* Ab, int na, const void* Bb, int nb, int
     e = cudaMemsetAsync(parts.tau, 0, sizeof(uint32_t) * kinds * (size_t)na, st);
     if (e != cudaSuccess) return e;
   }
-  const dim3 grid = p.split_first ? dim3(p.splits, rblocks) : dim3(rblocks, p.splits);
-  if (kp == 32)
-    e = cross    ? launch<POOL, 32, true>(ta, tb, a, grid, st)
-        : p.deep ? launch<POOL, 32, false, true>(ta, tb, a, grid, st)
-                 : launch<POOL, 32, false>(ta, tb, a, grid, st);
-  else if (kp == 64) e = cross ? launch<POOL, 64, true>(ta, tb, a, grid, st) : launch<POOL, 64, false>(ta, tb, a, grid, st);
-  else if (kp == 128) e = cross ? launch<POOL, 128, true>(ta, tb, a, grid, st) : launch<POOL, 128, false>(ta, tb, a, grid, st);
-  else e = cudaErrorInvalidValue;
-  if (e != cudaSuccess) return e;
-  if (!p.sel) return launch_merge_splits(parts.v, parts.i, p.splits, kinds, na, kp, pool_v, pool_i, st);
-  return launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, na, p.cap, kp, pool_v, pool_i, st, gate);
+  for (int r0 = 0; r0 < na; r0 += p.rows) {
+    const int rows = std::min(p.rows, na - r0), rblocks = (rows + BM - 1) / BM;
+    a.row0 = sa.row0 = r0;
+    a.part_rows = sa.part_rows = rows;
+    if (sample) {
+      e = launch_pool_sweep(kp, false, p.deep, ta, sb, sa, dim3(rblocks, p.sample_splits), st);
+      if (e == cudaSuccess)
+        e = launch_pool_finish(parts.v, parts.i, parts.cnt, p.sample_splits, 1, rows, p.cap, kp, pool_v, pool_i, na, r0,
+                               st, gate);
+      if (e != cudaSuccess) return e;
+    }
+    e = launch_pool_sweep(kp, cross, p.deep, ta, tb, a, p.split_first ? dim3(p.splits, rblocks) : dim3(rblocks, p.splits),
+                          st);
+    if (e != cudaSuccess) return e;
+    e = p.sel ? launch_pool_finish(parts.v, parts.i, parts.cnt, p.splits, kinds, rows, p.cap, kp, pool_v, pool_i, na, r0,
+                                   st, gate)
+              : launch_merge_splits(parts.v, parts.i, p.splits, kinds, rows, kp, pool_v, pool_i, na, r0, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_umma_gpool(const void* Y, int rows, int d, Elt elt, const int* gcam, bool cross, int self_excl,
@@ -1087,6 +1116,7 @@ cudaError_t launch_umma_gpool(const void* Y, int rows, int d, Elt elt, const int
   a.cam = gcam;
   a.pool_v = pool_v;
   a.pool_i = pool_i;
+  a.part_rows = rows;
   a.items = items;
   a.n_items = n_items;
   a.col_bias = col_bias;
