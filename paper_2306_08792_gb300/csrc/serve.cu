@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(256) pool_finish_kernel(const float* __restric
   int ni = -1;
   for (int s0 = 0; s0 < S; s0 += 32) {  // 32 splits: a lane holds each count
     const int sl = s0 + lane;
-    const int cl = sl < S ? cnt[(size_t)sl * rows + w] : 0;
+    const int cl = sl < S ? min(max(cnt[(size_t)sl * rows + w], 0), cap) : 0;
     for (int l = 0; l < 32 && s0 + l < S; ++l) {
       const int c = __shfl_sync(GCR_FULL, cl, l);
       const size_t base = ((size_t)(s0 + l) * rows + w) * cap;
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kSelThreads) pool_select_kernel(const float* _
     for (int e = tid; e < have; e += kSelThreads) { mn = min(mn, ent[e]); mx = max(mx, ent[e]); }
     for (int sb = s0 + warp; sb < s1; sb += NW * 32) {  // up to 32 splits of the warp: a lane holds each count
       const int sl = sb + NW * lane;
-      const int cl = sl < s1 ? min(cnt[(size_t)sl * rows + w], cap) : 0;
+      const int cl = sl < s1 ? min(max(cnt[(size_t)sl * rows + w], 0), cap) : 0;
       int inc = cl;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {

@@ -819,7 +819,18 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       if (g_last && (kind == 0 || CROSS))
         pool_flush<KP>(lane, g_valid, me, g_row0 + quad * 32, kind * BM + quad * 32, qs, pv, pi);
     }
-    if (MODE == POOL && !*abort_flag) {
+    // After a wait that ran out too: every count and list of the launch is written (with what was
+    // swept), so that what reads them stays within them; gcr_sync reports the timeout.
+    if (MODE == GPOOL && (kind == 0 || CROSS)) {
+      for (; cur.item < nitems; cur.item += gridDim.x, cur.load(a, nitems)) {  // items not finished: empty lists
+        if (r >= cur.w.y) continue;
+        for (int e = 0; e < KP; ++e) {
+          pv[(size_t)(cur.w.x + r) * KP + e] = -CUDART_INF_F;
+          pi[(size_t)(cur.w.x + r) * KP + e] = -1;
+        }
+      }
+    }
+    if (MODE == POOL) {
       if constexpr (SEL) {
         if (my_row < a.a_rows) {
           const int col0 = tl.split * a.tps * BN;

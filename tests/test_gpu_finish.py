@@ -1,5 +1,7 @@
 """The block-wide selection that ends a search of many splits: one block's worth of entries, several
 groups of splits, and more equal scores than it keeps."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -32,3 +34,34 @@ def test_top_k_of_many_splits(nq, ng, topk, copies):
     assert all(len(set(r)) == topk for r in idx.cpu().tolist())
     if copies >= topk:
         assert torch.equal(idx.long(), where[:topk].expand(nq, topk))
+
+
+class _Gate(ctypes.Structure):
+    _fields_ = [("flag", ctypes.c_void_p), ("want", ctypes.c_int)]
+
+
+@pytest.mark.parametrize("S", [3, 12])
+@pytest.mark.parametrize("kp,cap", [(32, 96), (128, 160)])
+def test_counts_are_held_to_the_buffers(S, kp, cap):
+    """Counts below zero or above the buffers' slots (a sweep that gave up a wait) are read as none
+    and as all of them; the pools are the best of what the buffers then hold."""
+    from paper_2306_08792_gb300 import _lib
+    fn = _lib.load()["_ZN3gcr18launch_pool_finishEPKfPKiS3_iiiiiPfPiiiP11CUstream_stNS_4GateE"]
+    fn.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int] * 5 + [ctypes.c_void_p] * 2 + [ctypes.c_int] * 2 + [
+        ctypes.c_void_p, _Gate]
+    rng = np.random.default_rng(S + kp)
+    kinds, rows = 2, 5
+    v = rng.standard_normal((S, kinds * rows, cap)).astype(np.float32)
+    i = (np.arange(S)[:, None, None] * 1000 + rng.permuted(np.tile(np.arange(cap), (S, kinds * rows, 1)), axis=2))
+    cnt = rng.choice([-2**31, -1, 0, 1, kp, cap, cap + 1, 2**31 - 1], size=(S, kinds * rows))
+    dv, di, dc = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (v, i.astype(np.int32), cnt.astype(np.int32)))
+    ov = torch.empty(kinds * rows, kp, device="cuda")
+    oi = torch.empty(kinds * rows, kp, dtype=torch.int32, device="cuda")
+    assert fn(dv.data_ptr(), di.data_ptr(), dc.data_ptr(), S, kinds, rows, cap, kp, ov.data_ptr(), oi.data_ptr(), rows,
+              0, torch.cuda.current_stream().cuda_stream, _Gate(None, 0)) == 0
+    for w in range(kinds * rows):
+        keep = [(-v[s, w, e], i[s, w, e]) for s in range(S) for e in range(min(max(int(cnt[s, w]), 0), cap))]
+        want = sorted(keep)[:kp]
+        got = oi[w].cpu().numpy()
+        assert np.array_equal(got[:len(want)], [c for _, c in want]) and np.all(got[len(want):] == -1)
+        assert np.array_equal(ov[w].cpu().numpy()[:len(want)], [-x for x, _ in want])
