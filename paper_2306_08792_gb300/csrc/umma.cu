@@ -612,7 +612,9 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       const int buf = t & 1;
       const uint32_t use = t >> 1;
       const uint32_t tau_other = tx ? __ldcg(tx) : 0u;
-      if (!mbar_wait(&bars.tfull[buf], use & 1, abort_flag)) break;
+      // the lanes stay together: one may find the tile ready while another finds the CTA aborting, and
+      // what follows (TMEM loads, votes, merges) needs the whole warp
+      if (!__all_sync(GCR_FULL, mbar_wait(&bars.tfull[buf], use & 1, abort_flag))) break;
       tc_fence_after();
       const int r0 = MODE == GPOOL ? cur.w.x : tl.row0(a, t);
       const int c0 = MODE == GPOOL ? cur.w.z + cur.ct * BN : tl.col0(a, t);
