@@ -346,7 +346,9 @@ int knn_impl(const float* X, int64_t n64_, int32_t d, const int32_t* cam, const 
       if (in_l2(n, d)) {
         if (g->row_order) GCR_CUDA_TRY(launch_identity_order(order, n, st));
       } else {
-        GCR_CUDA_TRY(launch_row_order(w.pool_i, n, r.kp, p->k, w.okey, w.ocnt, w.ooff, w.ofill, order, st));
+        // (where the probe has decided for TF32 the pools are not written yet: ordered below)
+        GCR_CUDA_TRY(launch_row_order(w.pool_i, n, r.kp, p->k, w.okey, w.ocnt, w.ooff, w.ofill, order, st,
+                                      f16 ? Gate{w.repeat, 0} : Gate()));
         ra.order = order;
       }
       if (f16) ra.gate = Gate{w.repeat, 0};
