@@ -222,13 +222,22 @@ __global__ void gram_mirror_kernel(float* __restrict__ G, int d) {
   }
 }
 
+__global__ void __launch_bounds__(256) frame_inv_norm_kernel(const float* __restrict__ F, int64_t nf, int d,
+                                                              float* __restrict__ inv) {
+  const int lane = threadIdx.x & 31;
+  const int64_t f = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (f >= nf) return;
+  const float s = frame_inv_norm(reinterpret_cast<const float4*>(F + f * d), d, lane);
+  if (lane == 0) inv[f] = s;
+}
+
 // inv[f] = 1/||x_f|| of the tracklet's frames and mu[row] = the mean of the normalised frames (Eq. 10);
 // padded rows are zero. The frames of a batch are read for their norms, a warp each, and again
 // from the caches for the mean, so they leave memory once: 675,977 frames of d = 2048 1.83 -> 1.45
 // ms (5.5 GB: 0.82 ms at the copy rate; the rest is the two phases of a batch waiting for each
-// other). VPT x 1024 >= d.
+// other). VPT x 1024 >= d. NORMS = false: inv is given (frame_inv_norm_kernel).
 constexpr int kMeanBatch = 8;  // (a whole call 16.39 ms at 16, 16.10 at 8, 16.53 at 4, 16.48 at 32)
-template <int VPT>
+template <int VPT, bool NORMS>
 __global__ void __launch_bounds__(256) norm_means_kernel(const float* __restrict__ F, int d,
                                                          const int64_t* __restrict__ off,
                                                          const int* __restrict__ perm, float* __restrict__ inv,
@@ -243,7 +252,32 @@ __global__ void __launch_bounds__(256) norm_means_kernel(const float* __restrict
   for (int v = 0; v < VPT; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c >= 0) {
     const int64_t b = off[c], e = off[c + 1];
-    for (int64_t f0 = b; f0 < e; f0 += kMeanBatch) {
+    if constexpr (!NORMS) {
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) {
+        const int a = v * 1024 + threadIdx.x * 4;
+        if (a >= d) break;
+        const float* src = F + a;
+        for (int64_t f0 = b; f0 < e; f0 += kMeanBatch) {  // a batch of frames in flight
+          float s[kMeanBatch];
+          float4 x[kMeanBatch];
+#pragma unroll
+          for (int j = 0; j < kMeanBatch; ++j) {
+            const int64_t f = min(f0 + j, e - 1);
+            s[j] = inv[f];
+            x[j] = *reinterpret_cast<const float4*>(src + f * d);
+          }
+#pragma unroll
+          for (int j = 0; j < kMeanBatch; ++j) {
+            if (f0 + j < e) {
+              acc[v].x = fmaf(x[j].x, s[j], acc[v].x); acc[v].y = fmaf(x[j].y, s[j], acc[v].y);
+              acc[v].z = fmaf(x[j].z, s[j], acc[v].z); acc[v].w = fmaf(x[j].w, s[j], acc[v].w);
+            }
+          }
+        }
+      }
+    }
+    for (int64_t f0 = b; NORMS && f0 < e; f0 += kMeanBatch) {
       const int nb = (int)min((int64_t)kMeanBatch, e - f0);
       for (int j = warp; j < nb; j += 8) {
         const float s = frame_inv_norm(reinterpret_cast<const float4*>(F + (f0 + j) * d), d, lane);
@@ -276,11 +310,29 @@ __global__ void __launch_bounds__(256) norm_means_kernel(const float* __restrict
   }
 }
 
-void launch_norm_means(const float* F, int d, const int64_t* off, const int* perm, int rows, float* inv, float* mu,
-                       cudaStream_t st) {
-  if (d <= 1024) norm_means_kernel<1><<<rows, 256, 0, st>>>(F, d, off, perm, inv, mu);
-  else if (d <= 2048) norm_means_kernel<2><<<rows, 256, 0, st>>>(F, d, off, perm, inv, mu);
-  else norm_means_kernel<4><<<rows, 256, 0, st>>>(F, d, off, perm, inv, mu);
+template <bool NORMS>
+void launch_means(const float* F, int d, const int64_t* off, const int* perm, int rows, float* inv, float* mu,
+                  cudaStream_t st) {
+  if (d <= 1024) norm_means_kernel<1, NORMS><<<rows, 256, 0, st>>>(F, d, off, perm, inv, mu);
+  else if (d <= 2048) norm_means_kernel<2, NORMS><<<rows, 256, 0, st>>>(F, d, off, perm, inv, mu);
+  else norm_means_kernel<4, NORMS><<<rows, 256, 0, st>>>(F, d, off, perm, inv, mu);
+}
+
+// C tracklets of F frames, a block each. Few tracklets leave most of the chip idle while their frames'
+// norms are taken, eight at a time with a barrier on either side: then the norms of all frames come
+// first, a warp each over the whole chip, and the means read them (the frames a second time, from L2
+// where they fit). One pass and two: 8 tracklets of 3,000 frames of d = 1,024 1,405 and 329 us, 64 of
+// 937 504 and 207, 200 of 300 250 and 150. From two blocks per SM on, or where the rows are long, one
+// pass is as fast as the separate kernels were: 304 of 197 172 against 184, 8 of 3,000 of d = 1,536
+// 2,168 against 2,216.
+void launch_norm_means(const float* F, int64_t nf, int d, const int64_t* off, const int* perm, int C, int rows,
+                       float* inv, float* mu, cudaStream_t st) {
+  if ((d <= 1024 && C < 2 * kSMs) || (long)C * d < 8192) {
+    frame_inv_norm_kernel<<<(unsigned)((nf + 7) / 8), 256, 0, st>>>(F, nf, d, inv);
+    launch_means<false>(F, d, off, perm, rows, inv, mu, st);
+  } else {
+    launch_means<true>(F, d, off, perm, rows, inv, mu, st);
+  }
 }
 
 // mu_s = (sum over the camera's tracklets of m_c mu_c) / n_s. 32 features per block; its 32 warps
@@ -490,7 +542,7 @@ cudaError_t launch_gcrv(const float* frames, int64_t F, int d, const int64_t* of
   Layout L{w.cam_cnt, w.cam_nf, w.blk0, w.perm, w.pos, w.fstart, w.foff, w.row_cam};
   layout_kernel<<<1, 1024, 0, st>>>(off, cam, C, ncam, w.rows_cap, L);
   frame_list_kernel<<<C, 128, 0, st>>>(off, C, w.fstart, w.flist);
-  launch_norm_means(frames, d, off, w.perm, w.rows_cap, w.inv, w.mu, st);
+  launch_norm_means(frames, F, d, off, w.perm, C, w.rows_cap, w.inv, w.mu, st);
   cam_means_kernel<<<dim3((d + 31) / 32, ncam), 1024, 0, st>>>(w.mu, d, off, w.perm, L, w.mu_cam);
   // G_s on the tensor cores: compensated BF16 operands of the transposed normalised frames
   zt_blocks_kernel<<<1, 32, 0, st>>>(w.cam_nf, ncam, w.kstart, w.knum);
@@ -516,7 +568,7 @@ cudaError_t launch_gcrv(const float* frames, int64_t F, int d, const int64_t* of
 
 cudaError_t launch_gcrv_means(const float* frames, int64_t F, int d, const int64_t* off, int C, float* inv, float* W,
                               cudaStream_t st) {
-  launch_norm_means(frames, d, off, nullptr, C, inv, W, st);
+  launch_norm_means(frames, F, d, off, nullptr, C, C, inv, W, st);
   return cudaGetLastError();
 }
 

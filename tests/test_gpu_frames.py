@@ -33,3 +33,15 @@ def test_profiles_and_means(d):
     nW, nWo = np.linalg.norm(W, axis=1, keepdims=True), np.linalg.norm(Wo, axis=1, keepdims=True)
     np.testing.assert_allclose(W / nW, Wo / nWo, atol=2e-5, rtol=0)
     np.testing.assert_allclose(nW, nWo, rtol=1e-4)
+
+
+@pytest.mark.parametrize("C,d", [(303, 68), (304, 68), (7, 1024), (5, 1636), (4, 2044), (2, 4092), (1, 4096), (2, 4096)])
+def test_means_of_few_long_and_of_many_tracklets(C, d):
+    """Both forms of the frame pass (norms first, or with the means) at the line between them, ragged."""
+    import paper_2306_08792_gb300 as gcr
+    rng = np.random.default_rng(C + d)
+    length = rng.integers(1, 60, size=C)
+    off = np.concatenate([[0], np.cumsum(length)]).astype(np.int64)
+    F = rng.standard_normal((off[-1], d)).astype(np.float32)
+    mu = gcr.gcrv_mean_profiles(torch.from_numpy(F).cuda(), torch.from_numpy(off).cuda()).double().cpu().numpy()
+    np.testing.assert_allclose(mu, oracle.mean_profiles(oracle.l2_normalize(F), off), atol=1e-6, rtol=0)
