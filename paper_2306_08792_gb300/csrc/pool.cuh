@@ -188,8 +188,6 @@ __device__ __forceinline__ float sel_ldv_any(uint32_t a) {
   asm("ld.shared.f32 %0, [%1];" : "=f"(r) : "r"(a));
   return r;
 }
-// Order-preserving image of a buffered score (-0 as +0, so that equal scores have equal images).
-__device__ __forceinline__ uint32_t sel_image(uint32_t a) { return float_to_ordered(sel_ldv_any(a) + 0.f); }
 __device__ __forceinline__ uint32_t sel_ldi(uint32_t a) {
   unsigned short r;
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(r) : "r"(a) : "memory");
@@ -235,12 +233,13 @@ struct SelScores {
     c = (c4[0] + c4[1]) + (c4[2] + c4[3]);
     t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
   }
-  // bit s & 31 of word w = s >> 5: score s is above f
+  // bit s & 31 of word w = s >> 5: score s is above f (EQ: is f)
+  template <bool EQ = false>
   __device__ __forceinline__ void above(float f, uint32_t (&m)[(CAP + 31) / 32]) const {
 #pragma unroll
     for (int w = 0; w < (CAP + 31) / 32; ++w) m[w] = 0u;
 #pragma unroll
-    for (int s = 0; s < CAP; ++s) m[s >> 5] |= (v[s] > f ? 1u : 0u) << (s & 31);
+    for (int s = 0; s < CAP; ++s) m[s >> 5] |= ((EQ ? v[s] == f : v[s] > f) ? 1u : 0u) << (s & 31);
   }
 };
 template <int CAP>
@@ -267,12 +266,16 @@ struct SelScores<CAP, false> {
     c = (c4[0] + c4[1]) + (c4[2] + c4[3]);
     t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
   }
+  template <bool EQ = false>
   __device__ __forceinline__ void above(float f, uint32_t (&m)[(CAP + 31) / 32]) const {
 #pragma unroll
     for (int w = 0; w < CAP / 32; ++w) {
       uint32_t x = 0;
-#pragma unroll
-      for (int u = 0; u < 32; ++u) x |= (sel_ldv_any(va + (w * 32 + u) * kSelV) > f && w * 32 + u < cnt ? 1u : 0u) << u;
+#pragma unroll(EQ ? 4 : 32)
+      for (int u = 0; u < 32; ++u) {
+        const float v = sel_ldv_any(va + (w * 32 + u) * kSelV);
+        x |= ((EQ ? v == f : v > f) && w * 32 + u < cnt ? 1u : 0u) << u;
+      }
       m[w] = x;
     }
   }
@@ -284,7 +287,14 @@ struct SelScores<CAP, false> {
 // hundred fall off about exponentially, so the first pivot is the quantile of an exponential
 // with their mean above the old threshold; the next ones are the mean of the scores still in
 // question, which splits them whatever their spread (a midpoint takes many more steps when a
-// few scores lie far above the rest). Five or six passes settle most warps.
+// few scores lie far above the rest). Five or six passes settle most warps. Where the mean no
+// longer splits them (ties, or infinities) the pivots go on as midpoints of the scores' order-
+// preserving images, which end at a threshold or, 32 passes on at most, at the score that the KP-th
+// largest ties with; of the entries equal to it those of the smallest columns are kept up to KP, as a
+// sorted list would, found by counting their columns' digits. (By a binary search for the score and
+// one for the column, each step through shared memory, such a compaction cost many usual ones: the
+// sweep of 13,290 rows of d = 512 with two non-zeros each, nearly all scores tied, took 4.5 ms in TF32,
+// 0.9 so, and 8.3 and 4.8 in FP32; of random rows 0.5 and 3.9.)
 // SUM: st.sum is given; else it is taken from the buffer.
 template <int KP, int CAP, bool SUM = true>
 __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState st) {
@@ -297,18 +307,23 @@ __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState 
   sc.load(va, cnt);
   // scores in question lie in (a, b]: ca of the entries are above a (ca >= KP), cb above b
   // (cb < KP); ta, tb are the sums of those
-  float a = st.lo, ta = st.sum, tb = 0.f;
+  float a = st.lo, b = CUDART_INF_F, ta = st.sum, tb = 0.f;
   int ca = cnt, cb = 0;
   if constexpr (!SUM) {
     int c;
     sc.count(-CUDART_INF_F, c, ta);
   }
   bool more = act;
-  for (int it = 0; it < 12 && __any_sync(GCR_FULL, more); ++it) {
+  for (int it = 0; __any_sync(GCR_FULL, more); ++it) {
     float p = (ta - tb) / (float)max(1, ca - cb);
     if (it == 0) {
       const float q = a + (p - a) * __logf((float)ca / kTarget);
       if (q > a && q < p) p = q;
+    }
+    if (it >= 12 || !(p > a && p < b)) {
+      const uint32_t ka = float_to_ordered(a), kb = float_to_ordered(b);  // (a < b: also as images)
+      if (kb - ka <= 1u) more = false;  // KP entries at b or above, fewer above it
+      p = ordered_to_float(ka + ((kb - ka) >> 1));
     }
     int c;
     float t;
@@ -320,61 +335,53 @@ __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState 
         ca = c;
         ta = t;
       } else {
+        b = p;
         cb = c;
         tb = t;
       }
     }
   }
-  float f = a;
+  const bool ex = act && ca > KP + kSlack;
+  float f = ex ? b : a;
   uint32_t keep[W];
   sc.above(act ? f : -CUDART_INF_F, keep);
   float lo = st.lo, sum = act ? ta : st.sum;  // (a lane that keeps all keeps its sum)
   int kept = act ? ca : cnt;
   if (act) lo = f;
-  // Scores too close together for the pivots (ties, or infinities): the KP-th largest exactly,
-  // by a binary search on the order-preserving 32-bit images; of the entries equal to it those
-  // of the smallest columns are kept up to KP, as a sorted list would.
-  if (__any_sync(GCR_FULL, act && ca > KP + kSlack)) {
-    const bool ex = act && ca > KP + kSlack;
-    const int n = __reduce_max_sync(GCR_FULL, cnt);
-    uint32_t k = 0;
-    for (int bit = 31; bit >= 0; --bit) {
-      const uint32_t cand = k | (1u << bit);
-      int c = 0;
-      for (int s = 0; s < n; ++s) c += (s < cnt && sel_image(va + s * kSelV) >= cand) ? 1 : 0;
-      if (c >= KP) k = cand;
-    }
-    int larger = 0;
-    for (int s = 0; s < n; ++s) larger += (s < cnt && sel_image(va + s * kSelV) > k) ? 1 : 0;
-    uint32_t col = 0xffffu;  // the largest column offset kept among the equal ones
-    for (int bit = 15; bit >= 0; --bit) {
-      const uint32_t cand = col & ~(1u << bit);
-      int c = 0;
-      for (int s = 0; s < n; ++s)
-        c += (s < cnt && sel_image(va + s * kSelV) == k && sel_ldi(ia + s * kSelI) <= cand) ? 1 : 0;
-      if (larger + c >= KP) col = cand;
-    }
-    if (ex) {
-      float x = 0.f;
+  if (__any_sync(GCR_FULL, ex)) {
+    uint32_t eq[W];
+    sc.template above<true>(f, eq);
+    int need = ex ? KP - cb : 0;  // of the entries equal to f, those of the smallest columns
+    uint32_t col = 0;             // the digits, from the top, of the largest of these columns
+    for (int shift = 12; shift >= 0; shift -= 4) {
+      unsigned long long n0 = 0, n1 = 0;  // entries of each digit, 8 bits a count
 #pragma unroll
-      for (int w = 0; w < W; ++w) {
-        uint32_t m = 0;
-        for (int u = 0; u < 32; ++u) {
-          const int s = w * 32 + u;
-          if (s < cnt) {
-            const uint32_t img = sel_image(va + s * kSelV);
-            if (img > k || (img == k && sel_ldi(ia + s * kSelI) <= col)) {
-              m |= 1u << u;
-              x += sel_ldv(va + s * kSelV);
-            }
+      for (int w = 0; w < W; ++w)
+        for (uint32_t m = ex ? eq[w] : 0u; m; m &= m - 1u) {
+          const uint32_t c = sel_ldi(ia + (32 * w + __ffs(m) - 1) * kSelI) >> shift, dg = c & 15u;
+          if (c >> 4 == col) {
+            if (dg < 8u) n0 += 1ull << (8u * dg);
+            else n1 += 1ull << (8u * (dg - 8u));
           }
         }
-        keep[w] = m;
+      uint32_t dg = 0;
+      for (; dg < 15u; ++dg) {
+        const int c = (int)((dg < 8u ? n0 >> (8u * dg) : n1 >> (8u * (dg - 8u))) & 255u);
+        if (c >= need) break;
+        need -= c;
       }
-      f = ordered_to_float(k);
+      col = col << 4 | dg;
+    }
+    if (ex) {
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        for (uint32_t m = eq[w]; m; m &= m - 1u) {
+          const int u = __ffs(m) - 1;
+          if (sel_ldi(ia + (32 * w + u) * kSelI) <= col) keep[w] |= 1u << u;
+        }
       lo = float_below(f);  // every entry kept is above the value below f
       kept = KP;
-      sum = x;
+      sum = tb + (float)(KP - cb) * f;
     }
   }
   if (act) {

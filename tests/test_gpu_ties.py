@@ -39,7 +39,7 @@ def _rows(kind, n, d):
     return gcr.gcr_normalize(X.contiguous())
 
 
-@pytest.mark.parametrize("precision", ["fp32"])
+@pytest.mark.parametrize("precision", ["fp32", "tf32"])
 def test_sweep_of_sparse_rows(precision):
     """13,290 rows of d = 512, against the sweep of random rows: 1.25 (FP32) and 1.9 times on one GB300,
     5.7 and 9.5 with tied compactions through shared memory and, in FP32, ties admitted by every tile."""
