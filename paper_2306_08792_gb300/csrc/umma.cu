@@ -780,6 +780,8 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const size_t at = (a.band_off ? (size_t)a.band_off[u] : (size_t)u * a.bcap) + pos;
                 if (a.band_v) a.band_v[at] = v[cc];
                 a.band_i[at] = j;
+              } else if (a.band_v) {
+                my_thr = CUDART_INF_F;  // past the band: what more there is need not be counted
               }
             }
           }

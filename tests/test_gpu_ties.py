@@ -47,3 +47,12 @@ def test_sweep_of_sparse_rows(precision):
     p = gcr.default_params(k=20, precision=precision)
     t = [_stage_ms(lambda X=_rows(kind, 13290, 512): gcr.gcr_build_graph(X, p), SIM) for kind in ("sparse", "random")]
     assert t[0] < 4.0 * t[1], t
+
+
+def test_band_rescan_that_overflows_in_any_row_order():
+    """20,000 rows that are copies of 8: every band overflows. Rows of one copy side by side count in
+    step; in any other order the rescan took 3.7 times as long while it counted every column, 1.75 now."""
+    import paper_2306_08792_gb300 as gcr
+    p = gcr.default_params(k=20, precision="tf32")
+    t = [_stage_ms(lambda X=_rows(kind, 20000, 256): gcr.gcr_build_graph(X, p), BAND) for kind in ("copies", "sorted copies")]
+    assert t[0] < 2.75 * t[1], t
