@@ -909,8 +909,8 @@ size_t carve_topk_rerank_at(Carve& c, int64_t nq, int64_t ng, int32_t d, const g
   t.n64g = c.take<double>(ng);
   t.n32g = c.take<float>(ng);
   t.gr = bf ? c.take<char>((size_t)ng * d * elt_size(p)) : nullptr;
-  t.genrm = c.take<float>(ng);
-  t.ganrm = c.take<float>(ng);
+  t.genrm = bf ? c.take<float>(ng) : nullptr;
+  t.ganrm = bf ? c.take<float>(ng) : nullptr;
   t.scg = c.take<RowScalars>(1);
   std::memset(&t.ball, 0, sizeof(t.ball));
   // gathered positions: each group's queries and its ball of gallery rows (balls may overlap)
@@ -922,16 +922,21 @@ size_t carve_topk_rerank_at(Carve& c, int64_t nq, int64_t ng, int32_t d, const g
 
 // A search that fits gcr_rerank_noalloc's array with fewer splits of the sweep takes as many as fit
 // (few queries against 300,000 rows and more, whose norms fill much of the array): a callers' scratch
-// of that size goes on serving what it served when a split left a list and not a buffer.
+// of that size goes on serving what it served when a split left a list and not a buffer. All of those
+// keep 50 CTAs at least: the array held 152 splits' lists of 32 to 128 entries a row, a third of a
+// buffer or more, besides 20 bytes of norms per gallery row where FP32 now has 12. A search that would
+// keep fewer never fitted and is not cut (the sweep of 11 queries over 829,000 rows of d = 64, cut to what
+// 20 bytes of norms a row left, 3.4 ms; 0.6 so).
 size_t carve_topk_rerank(Carve& c, int64_t nq, int64_t ng, int32_t d, const gcr_params* p, TopkRerankWs* w) {
   const size_t limit = GCR_RERANK_NOALLOC_SCRATCH_BYTES - 256;
+  const int least = (int)std::max<int64_t>(1, kSMs / 3 / ((nq + 127) / 128));
   auto need = [&](int m) {
     Carve t(nullptr, 0);
     return carve_topk_rerank_at(t, nq, ng, d, p, m, nullptr);
   };
   int lo = INT_MAX;
-  if (need(INT_MAX) > limit && need(1) <= limit) {
-    lo = 1;
+  if (need(INT_MAX) > limit && need(least) <= limit) {
+    lo = least;
     for (int hi = 4096; hi - lo > 1;) {  // (a plan has at most about 2,500 splits)
       const int mid = (lo + hi) / 2;
       if (need(mid) <= limit) lo = mid;

@@ -56,3 +56,16 @@ def test_band_rescan_that_overflows_in_any_row_order():
     p = gcr.default_params(k=20, precision="tf32")
     t = [_stage_ms(lambda X=_rows(kind, 20000, 256): gcr.gcr_build_graph(X, p), BAND) for kind in ("copies", "sorted copies")]
     assert t[0] < 2.75 * t[1], t
+
+
+def test_search_that_never_fitted_the_static_scratch_keeps_its_splits():
+    """11 queries of 829,000 rows: their norms nearly fill gcr_rerank_noalloc's array. Their sweep
+    takes no more than twice that of 700,000 rows, which leave room for all splits."""
+    import paper_2306_08792_gb300 as gcr
+    p = gcr.default_params(precision="fp32", topk_out=10)
+    t = []
+    for ng in (829000, 700000):
+        g = torch.Generator(device="cuda").manual_seed(2)
+        Q, X = (gcr.gcr_normalize(torch.randn(r, 64, generator=g, device="cuda")) for r in (11, ng))
+        t.append(_stage_ms(lambda: gcr.gcr_rerank(Q, X, p), SIM))
+    assert t[0] < 2.0 * t[1], t
