@@ -37,14 +37,6 @@ __device__ __forceinline__ void pool_init(PoolOwner& o, bool valid, float floor)
 }
 __device__ __forceinline__ void pool_init(PoolOwner& o, bool valid) { pool_init(o, valid, -CUDART_INF_F); }
 
-// Branch-free append: the candidate is always written into the next free slot and the count
-// only advances when it passes (ok and v > tau). The caller guarantees qcnt < kQCap before
-// every call (pool_make_room with room = values pushed before the next check).
-__device__ __forceinline__ void pool_push(PoolOwner& o, float v, int j, bool ok, float2* q, int sw) {
-  q[o.qcnt ^ sw] = make_float2(v, __int_as_float(j));
-  o.qcnt += (ok && v > o.tau) ? 1 : 0;
-}
-
 // Warp-cooperative merge of the queue of the row owned by lane `owner` into its list.
 // qv_row/qi_row: that row's queue; lv/li: that row's list (KP entries) in global memory.
 // Kept out of line (the merge is rare and large); takes and returns plain values so that the
@@ -118,8 +110,7 @@ __device__ __forceinline__ void pool_merge_apply(int owner, int lane, float* lv,
   }
 }
 
-// Merge every row of this warp whose queue could not take `room` more pushes (the branch-free
-// push writes one slot past the count, so the count must stay below kQCap - room).
+// Merge every row of this warp whose queue could not take `room` more entries.
 // row_of_lane0: global row of lane 0; qrow0: CTA-local queue row of lane 0.
 template <int KP>
 __device__ __forceinline__ void pool_make_room(int room, int lane, PoolOwner& me, int row_of_lane0,

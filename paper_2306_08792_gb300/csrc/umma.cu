@@ -401,8 +401,11 @@ __device__ __noinline__ float warm_floor(uint32_t taddr, int cb0, int ncol, int 
 }
 
 // MODE is a template parameter (not only a field of UmmaArgs) so that each mode's epilogue is
-// compiled alone: no per-value mode branches, and the POOL kernels need 88-90 registers instead
-// of 116-118 (similarity GEMM on crosscam 2.72 -> 2.65 ms per TF32 launch, 2.75 -> 2.48 BF16).
+// compiled alone, without mode branches per value: when it was introduced, on pools of sorted lists,
+// the similarity GEMM on crosscam went from 2.72 to 2.65 ms per TF32 launch and from 2.75 to 2.48 in
+// BF16. One CTA per SM leaves room for the 128 to 196 registers a thread that the selection buffers
+// take (they are compacted in registers); two graphs of 64 entries, at the 168 that 320 threads
+// leave, spill 40 bytes.
 template <int MODE, int KP, bool CROSS, bool DEEP = false>
 __global__ void __launch_bounds__(CROSS ? 320 : 192, 1)
 umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
