@@ -224,6 +224,15 @@ struct SelScores {
     c = (c4[0] + c4[1]) + (c4[2] + c4[3]);
     t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
   }
+  // the smallest and the largest score in (a, b]
+  __device__ __forceinline__ void range(float a, float b, float& mn, float& mx) const {
+#pragma unroll
+    for (int s = 0; s < CAP; ++s)
+      if (v[s] > a && v[s] <= b) {
+        mn = fminf(mn, v[s]);
+        mx = fmaxf(mx, v[s]);
+      }
+  }
   // bit s & 31 of word w = s >> 5: score s is above f (EQ: is f)
   template <bool EQ = false>
   __device__ __forceinline__ void above(float f, uint32_t (&m)[(CAP + 31) / 32]) const {
@@ -257,6 +266,16 @@ struct SelScores<CAP, false> {
     c = (c4[0] + c4[1]) + (c4[2] + c4[3]);
     t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
   }
+  __device__ __forceinline__ void range(float a, float b, float& mn, float& mx) const {
+#pragma unroll 8
+    for (int s = 0; s < CAP; ++s) {
+      const float v = sel_ldv_any(va + s * kSelV);
+      if (s < cnt && v > a && v <= b) {
+        mn = fminf(mn, v);
+        mx = fmaxf(mx, v);
+      }
+    }
+  }
   template <bool EQ = false>
   __device__ __forceinline__ void above(float f, uint32_t (&m)[(CAP + 31) / 32]) const {
 #pragma unroll
@@ -272,114 +291,9 @@ struct SelScores<CAP, false> {
   }
 };
 
-// Compacts the buffers of the warp's lanes (slot 0 at va / ia, cnt entries): a lane with more
-// than KP entries keeps KP to KP + kSlack of them (in any order), the others keep all. Every
-// lane of the warp calls it. The threshold is searched by pivots: the scores of a row's best few
-// hundred fall off about exponentially, so the first pivot is the quantile of an exponential
-// with their mean above the old threshold; the next ones are the mean of the scores still in
-// question, which splits them whatever their spread (a midpoint takes many more steps when a
-// few scores lie far above the rest). Five or six passes settle most warps. Where the mean no
-// longer splits them (ties, or infinities) the pivots go on as midpoints of the scores' order-
-// preserving images, which end at a threshold or, 32 passes on at most, at the score that the KP-th
-// largest ties with; of the entries equal to it those of the smallest columns are kept up to KP, as a
-// sorted list would, found by counting their columns' digits. (By a binary search for the score and
-// one for the column, each step through shared memory, such a compaction cost many usual ones: the
-// sweep of 13,290 rows of d = 512 with two non-zeros each, nearly all scores tied, took 4.5 ms in TF32,
-// 0.9 so, and 8.3 and 4.8 in FP32; of random rows 0.5 and 3.9.)
-// SUM: st.sum is given; else it is taken from the buffer.
-template <int KP, int CAP, bool SUM = true>
-__device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState st) {
-  constexpr int kSlack = (CAP - KP) / 4, W = (CAP + 31) / 32;
-  constexpr float kTarget = KP + 0.5f * kSlack;
-  const int cnt = st.cnt;
-  float tau = st.tau, pub = st.pub;
-  const bool act = cnt > KP;
-  SelScores<CAP> sc;
-  sc.load(va, cnt);
-  // scores in question lie in (a, b]: ca of the entries are above a (ca >= KP), cb above b
-  // (cb < KP); ta, tb are the sums of those
-  float a = st.lo, b = CUDART_INF_F, ta = st.sum, tb = 0.f;
-  int ca = cnt, cb = 0;
-  if constexpr (!SUM) {
-    int c;
-    sc.count(-CUDART_INF_F, c, ta);
-  }
-  bool more = act;
-  for (int it = 0; __any_sync(GCR_FULL, more); ++it) {
-    float p = (ta - tb) / (float)max(1, ca - cb);
-    if (it == 0) {
-      const float q = a + (p - a) * __logf((float)ca / kTarget);
-      if (q > a && q < p) p = q;
-    }
-    if (it >= 12 || !(p > a && p < b)) {
-      const uint32_t ka = float_to_ordered(a), kb = float_to_ordered(b);  // (a < b: also as images)
-      if (kb - ka <= 1u) more = false;  // KP entries at b or above, fewer above it
-      p = ordered_to_float(ka + ((kb - ka) >> 1));
-    }
-    int c;
-    float t;
-    sc.count(p, c, t);
-    if (more) {
-      if (c >= KP) {
-        more = c > KP + kSlack;
-        a = p;
-        ca = c;
-        ta = t;
-      } else {
-        b = p;
-        cb = c;
-        tb = t;
-      }
-    }
-  }
-  const bool ex = act && ca > KP + kSlack;
-  float f = ex ? b : a;
-  uint32_t keep[W];
-  sc.above(act ? f : -CUDART_INF_F, keep);
-  float lo = st.lo, sum = act ? ta : st.sum;  // (a lane that keeps all keeps its sum)
-  int kept = act ? ca : cnt;
-  if (act) lo = f;
-  if (__any_sync(GCR_FULL, ex)) {
-    uint32_t eq[W];
-    sc.template above<true>(f, eq);
-    int need = ex ? KP - cb : 0;  // of the entries equal to f, those of the smallest columns
-    uint32_t col = 0;             // the digits, from the top, of the largest of these columns
-    for (int shift = 12; shift >= 0; shift -= 4) {
-      unsigned long long n0 = 0, n1 = 0;  // entries of each digit, 8 bits a count
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-        for (uint32_t m = ex ? eq[w] : 0u; m; m &= m - 1u) {
-          const uint32_t c = sel_ldi(ia + (32 * w + __ffs(m) - 1) * kSelI) >> shift, dg = c & 15u;
-          if (c >> 4 == col) {
-            if (dg < 8u) n0 += 1ull << (8u * dg);
-            else n1 += 1ull << (8u * (dg - 8u));
-          }
-        }
-      uint32_t dg = 0;
-      for (; dg < 15u; ++dg) {
-        const int c = (int)((dg < 8u ? n0 >> (8u * dg) : n1 >> (8u * (dg - 8u))) & 255u);
-        if (c >= need) break;
-        need -= c;
-      }
-      col = col << 4 | dg;
-    }
-    if (ex) {
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-        for (uint32_t m = eq[w]; m; m &= m - 1u) {
-          const int u = __ffs(m) - 1;
-          if (sel_ldi(ia + (32 * w + u) * kSelI) <= col) keep[w] |= 1u << u;
-        }
-      lo = float_below(f);  // every entry kept is above the value below f
-      kept = KP;
-      sum = tb + (float)(KP - cb) * f;
-    }
-  }
-  if (act) {
-    tau = fmaxf(tau, f);  // another split may have raised it further
-    pub = fmaxf(pub, lo);
-  }
-  // the kept entries past slot `kept` fill the holes before it
+// The kept entries past slot `kept` fill the holes before it.
+template <int W>
+__device__ __forceinline__ void sel_close(uint32_t (&keep)[W], int kept, uint32_t va, uint32_t ia) {
   uint32_t hole = 0, mover = 0;  // what is left of the words being walked
   int hw = -1, mw = -1;
 #pragma unroll
@@ -413,7 +327,166 @@ __device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState 
     sel_st(va + h * kSelV, ia + h * kSelI, sel_ldv(va + m * kSelV), sel_ldi(ia + m * kSelI));
   }
   __syncwarp();
-  return SelState{tau, lo, pub, sum, kept};
+}
+
+// The scores a compaction's threshold lies among, (a, b]: ca of the entries are above a (ca >= KP), cb
+// above b (cb < KP); ta, tb are the sums of those.
+struct SelRange {
+  float a, b, ta, tb;
+  int ca, cb;
+};
+
+// The rest of a compaction whose pivots left some lane more than KP + kSlack entries: ties, or
+// infinities. The range is cut to the scores in it, which ends at once if they are all equal, and
+// halved by their order-preserving images, down to a threshold or to the score that the KP-th
+// largest ties with; of the entries equal to it those of the smallest columns are kept up to KP, as a
+// sorted list would, found by counting their columns' digits. A function of its own, so that the
+// pivots keep their registers. (By a binary search for the score and one for the column, each step
+// through shared memory, such a compaction cost many usual ones: the sweep of 13,290 rows of d = 512 with two non-zeros
+// each, nearly all scores tied, took 4.5 ms in TF32, 0.7 so, and 8.3 and 4.3 in FP32; of random rows 0.5
+// and 3.9.)
+template <int KP, int CAP>
+__device__ __noinline__ SelState sel_compact_ties(uint32_t va, uint32_t ia, SelState st, SelRange g) {
+  constexpr int kSlack = (CAP - KP) / 4, W = (CAP + 31) / 32;
+  const int cnt = st.cnt;
+  const bool act = cnt > KP;
+  SelScores<CAP> sc;
+  sc.load(va, cnt);
+  bool more = act && g.ca > KP + kSlack;
+  if (more) {
+    float mn = CUDART_INF_F, mx = -CUDART_INF_F;
+    sc.range(g.a, g.b, mn, mx);
+    g.a = float_below(mn);
+    g.b = mx;
+  }
+  while (__any_sync(GCR_FULL, more)) {
+    const uint32_t ka = float_to_ordered(g.a), kb = float_to_ordered(g.b);  // (a < b: also as images)
+    if (kb - ka <= 1u) more = false;  // KP entries at b or above, fewer above it
+    const float p = ordered_to_float(ka + ((kb - ka) >> 1));
+    int c;
+    float t;
+    sc.count(p, c, t);
+    if (more) {
+      if (c >= KP) {
+        more = c > KP + kSlack;
+        g.a = p;
+        g.ca = c;
+        g.ta = t;
+      } else {
+        g.b = p;
+        g.cb = c;
+        g.tb = t;
+      }
+    }
+  }
+  const bool ex = act && g.ca > KP + kSlack;
+  const float f = ex ? g.b : g.a;
+  uint32_t keep[W], eq[W];
+  sc.above(act ? f : -CUDART_INF_F, keep);
+  sc.template above<true>(f, eq);
+  int need = ex ? KP - g.cb : 0;  // of the entries equal to f, those of the smallest columns
+  uint32_t col = 0;               // the digits, from the top, of the largest of these columns
+  for (int shift = 12; shift >= 0; shift -= 4) {
+    unsigned long long n0 = 0, n1 = 0;  // entries of each digit, 8 bits a count
+#pragma unroll
+    for (int w = 0; w < W; ++w)
+#pragma unroll 8
+      for (int u = 0; u < (CAP - 32 * w < 32 ? CAP - 32 * w : 32); ++u) {
+        const uint32_t c = sel_ldi(ia + (32 * w + u) * kSelI) >> shift;
+        if (((eq[w] >> u) & 1u) && c >> 4 == col) {
+          const unsigned long long one = 1ull << (8u * (c & 7u));
+          if (c & 8u) n1 += one;
+          else n0 += one;
+        }
+      }
+    uint32_t dg = 0;
+    for (; dg < 15u; ++dg) {
+      const int c = (int)((dg < 8u ? n0 >> (8u * dg) : n1 >> (8u * (dg - 8u))) & 255u);
+      if (c >= need) break;
+      need -= c;
+    }
+    col = col << 4 | dg;
+  }
+  if (ex) {
+#pragma unroll
+    for (int w = 0; w < W; ++w)
+#pragma unroll 8
+      for (int u = 0; u < (CAP - 32 * w < 32 ? CAP - 32 * w : 32); ++u)
+        keep[w] |= (sel_ldi(ia + (32 * w + u) * kSelI) <= col ? eq[w] : 0u) & (1u << u);
+  }
+  if (act) {
+    st.lo = ex ? float_below(f) : f;  // (every tied entry kept is above the value below f)
+    st.cnt = ex ? KP : g.ca;
+    st.sum = ex ? g.tb + (float)(KP - g.cb) * f : g.ta;
+    st.tau = fmaxf(st.tau, f);  // another split may have raised it further
+    st.pub = fmaxf(st.pub, st.lo);
+  }
+  sel_close(keep, st.cnt, va, ia);
+  return st;
+}
+
+// Compacts the buffers of the warp's lanes (slot 0 at va / ia, cnt entries): a lane with more
+// than KP entries keeps KP to KP + kSlack of them (in any order), the others keep all. Every
+// lane of the warp calls it. The threshold is searched by pivots: the scores of a row's best few
+// hundred fall off about exponentially, so the first pivot is the quantile of an exponential
+// with their mean above the old threshold; the next ones are the mean of the scores still in
+// question, which splits them whatever their spread (a midpoint takes many more steps when a
+// few scores lie far above the rest). Five or six passes settle most warps; what a mean does not
+// split is left to sel_compact_ties.
+// SUM: st.sum is given; else it is taken from the buffer.
+template <int KP, int CAP, bool SUM = true>
+__device__ __noinline__ SelState sel_compact(uint32_t va, uint32_t ia, SelState st) {
+  constexpr int kSlack = (CAP - KP) / 4, W = (CAP + 31) / 32;
+  constexpr float kTarget = KP + 0.5f * kSlack;
+  const int cnt = st.cnt;
+  const bool act = cnt > KP;
+  SelScores<CAP> sc;
+  sc.load(va, cnt);
+  SelRange g{st.lo, CUDART_INF_F, st.sum, 0.f, cnt, 0};
+  if constexpr (!SUM) {
+    int c;
+    sc.count(-CUDART_INF_F, c, g.ta);
+  }
+  bool more = act;
+  for (int it = 0; it < 12 && __any_sync(GCR_FULL, more); ++it) {
+    float p = (g.ta - g.tb) / (float)max(1, g.ca - g.cb);
+    if (it == 0) {
+      const float q = g.a + (p - g.a) * __logf((float)g.ca / kTarget);
+      if (q > g.a && q < p) p = q;
+    }
+    int c;
+    float t;
+    sc.count(p, c, t);
+    if (more) {
+      if (c >= KP) {
+        more = c > KP + kSlack && (it == 0 || c < g.ca);
+        if (p > g.a) {
+          g.a = p;
+          g.ca = c;
+          g.ta = t;
+        }
+      } else {
+        more = it == 0 || c > g.cb;
+        if (p < g.b) {
+          g.b = p;
+          g.cb = c;
+          g.tb = t;
+        }
+      }
+    }
+  }
+  if (__any_sync(GCR_FULL, act && g.ca > KP + kSlack)) return sel_compact_ties<KP, CAP>(va, ia, st, g);
+  uint32_t keep[W];
+  sc.above(act ? g.a : -CUDART_INF_F, keep);
+  if (act) {
+    st.lo = g.a;
+    st.cnt = g.ca;
+    st.sum = g.ta;  // (a lane that keeps all keeps its sum)
+    st.tau = fmaxf(st.tau, g.a);  // another split may have raised it further
+    st.pub = fmaxf(st.pub, g.a);
+  }
+  sel_close(keep, st.cnt, va, ia);
+  return st;
 }
 
 }  // namespace gcr
