@@ -771,6 +771,9 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           if (kind == 0) {
             int ccam = 0;
             if (a.cam) ccam = (cb + lane < a.n) ? a.cam[cb + lane] : -1;
+            // the chunk's hits first, then one atomic for all of them: an atomic per hit waits for
+            // each in turn, and the lanes' rows meet their columns apart
+            uint32_t hit = 0u;
 #pragma unroll
             for (int cc = 0; cc < 32; ++cc) {
               const int j = cb + cc;
@@ -778,13 +781,24 @@ umma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
               const int cj = a.cam ? cjv : 0;
               if (u < 0 || j >= a.n || (a.self_excl && j == my_row) || v[cc] < my_thr) continue;
               if (my_kind == 1 && cj == my_cam) continue;
-              const int pos = atomicAdd(&a.band_cnt[u], 1);
-              if (pos < (a.band_lim ? a.band_lim[u] : a.bcap)) {
-                const size_t at = (a.band_off ? (size_t)a.band_off[u] : (size_t)u * a.bcap) + pos;
-                if (a.band_v) a.band_v[at] = v[cc];
-                a.band_i[at] = j;
-              } else if (a.band_v) {
-                my_thr = CUDART_INF_F;  // past the band: what more there is need not be counted
+              hit |= 1u << cc;
+            }
+            if (hit) {
+              const int lim = a.band_lim ? a.band_lim[u] : a.bcap;
+              int pos = atomicAdd(&a.band_cnt[u], __popc(hit));
+              const size_t base = a.band_off ? (size_t)a.band_off[u] : (size_t)u * a.bcap;
+              if (pos >= lim) {
+                if (a.band_v) my_thr = CUDART_INF_F;  // past the band: what more there is need not be counted
+              } else {
+#pragma unroll
+                for (int cc = 0; cc < 32; ++cc)
+                  if ((hit >> cc) & 1u) {
+                    if (pos < lim) {
+                      if (a.band_v) a.band_v[base + pos] = v[cc];
+                      a.band_i[base + pos] = cb + cc;
+                    }
+                    ++pos;
+                  }
               }
             }
           }
