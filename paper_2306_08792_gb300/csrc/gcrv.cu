@@ -263,9 +263,10 @@ __global__ void __launch_bounds__(256) norm_means_kernel(const float* __restrict
           float4 x[kMeanBatch];
 #pragma unroll
           for (int j = 0; j < kMeanBatch; ++j) {
-            const int64_t f = min(f0 + j, e - 1);
-            s[j] = inv[f];
-            x[j] = *reinterpret_cast<const float4*>(src + f * d);
+            if (f0 + j < e) {
+              s[j] = inv[f0 + j];
+              x[j] = *reinterpret_cast<const float4*>(src + (f0 + j) * d);
+            }
           }
 #pragma unroll
           for (int j = 0; j < kMeanBatch; ++j) {
@@ -318,16 +319,16 @@ void launch_means(const float* F, int d, const int64_t* off, const int* perm, in
   else norm_means_kernel<4, NORMS><<<rows, 256, 0, st>>>(F, d, off, perm, inv, mu);
 }
 
-// C tracklets of F frames, a block each. Few tracklets leave most of the chip idle while their frames'
-// norms are taken, eight at a time with a barrier on either side: then the norms of all frames come
-// first, a warp each over the whole chip, and the means read them (the frames a second time, from L2
-// where they fit). One pass and two: 8 tracklets of 3,000 frames of d = 1,024 1,405 and 329 us, 64 of
-// 937 504 and 207, 200 of 300 250 and 150. From two blocks per SM on, or where the rows are long, one
-// pass is as fast as the separate kernels were: 304 of 197 172 against 184, 8 of 3,000 of d = 1,536
-// 2,168 against 2,216.
+// C tracklets of nf frames, a block each. Long tracklets that together leave the chip partly idle, or
+// whose frames stay in L2, wait longest for their own norms, taken eight frames at a time with a
+// barrier on either side: then the norms of all frames come first, a warp each over the whole chip, and
+// the means read the frames again. Short ones, and many of long rows, gain from the one pass. Two passes
+// and one, us: 8 tracklets of 3,000 frames of d = 1,024 329 and 1,405, 320 of 300 229 and 487, 700 of 50
+// 98 and 120, 2,000 of 50 230 and 220; 40 of 300 of d = 2,048 135 and 269, 700 of 50 133 and 137, 2,000
+// of 50 296 and 246; 2,000 of 300 of d = 32 894 and 1,042, 700 of 6 34 and 31.
 void launch_norm_means(const float* F, int64_t nf, int d, const int64_t* off, const int* perm, int C, int rows,
                        float* inv, float* mu, cudaStream_t st) {
-  if ((d <= 1024 && C < 2 * kSMs) || (long)C * d < 8192) {
+  if (nf >= 16 * (int64_t)C && (int64_t)C * d <= 1500000) {
     frame_inv_norm_kernel<<<(unsigned)((nf + 7) / 8), 256, 0, st>>>(F, nf, d, inv);
     launch_means<false>(F, d, off, perm, rows, inv, mu, st);
   } else {
