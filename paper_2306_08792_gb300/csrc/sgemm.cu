@@ -214,18 +214,27 @@ sgemm_band_kernel(const float* __restrict__ X, const float* __restrict__ Bm, int
       const int kind = band_kind[u];
       const float thr = band_thr[u];
       const int rc = cam ? cam[row] : 0;
+      // the row's hits first, then one atomic for all of them (see the BAND mode of umma.cu)
+      uint32_t hit = 0u;
 #pragma unroll
       for (int j = 0; j < TN; ++j) {
         const int cc = acc_col(tid, j);
         const int col = col0 + cc;
         if (cc >= brows || (self_excl && col == row) || acc[i][j] < thr) continue;
         if (kind == 1 && cam[col] == rc) continue;
-        int pos = atomicAdd(&band_cnt[u], 1);
-        if (pos < bcap) {
-          band_v[(size_t)u * bcap + pos] = acc[i][j];
-          band_i[(size_t)u * bcap + pos] = col;
-        }
+        hit |= 1u << j;
       }
+      if (!hit) continue;
+      int pos = atomicAdd(&band_cnt[u], __popc(hit));
+#pragma unroll
+      for (int j = 0; j < TN; ++j)
+        if ((hit >> j) & 1u) {
+          if (pos < bcap) {
+            band_v[(size_t)u * bcap + pos] = acc[i][j];
+            band_i[(size_t)u * bcap + pos] = col0 + acc_col(tid, j);
+          }
+          ++pos;
+        }
     }
   }
 }
